@@ -60,7 +60,7 @@ enum {
   OMEN_F32_REFINE64 = 2, /* OMEN_F32 solve, then an FP64 Rayleigh–Ritz refinement inside
                             omen_eigs; the vectors of omen_hx, omen_hx_host and v0 are FP32
                             (complex64), the eigenvectors omen_eigs returns are FP64 */
-  OMEN_F64_DF = 3        /* FP64-accurate H·X on the FP32 pipe: blocks and vectors stored as
+  OMEN_F64_DF = 3        /* FP64-accurate H·X on the FP32 pipe: blocks and vectors held as
                             double-float pairs (hi, lo) of FP32 (value = hi + lo, about 48
                             significant bits), products and sums with error-free
                             transformations (Dekker 1971; Knuth TwoSum).  Real Hamiltonians
@@ -219,9 +219,10 @@ typedef struct {
 typedef struct {
   int spin_orbit;            /* 0/1: double the basis and add lambda L.sigma on p */
   int precision;             /* OMEN_F64, OMEN_F32 or OMEN_F32_REFINE64 */
-  int matrix_free;           /* 0: store every bond block; 1: regenerate blocks in H·X from
-                                the species pair, the direction and a per-bond factor
-                                (d0/d)^eta taken from the structure's strain at assembly */
+  int matrix_free;           /* 0 or 1: either form keeps the reduced block of every species pair
+                                and a per-bond factor (d0/d)^eta taken from the structure's
+                                strain at assembly, and applies blocks from them; 1 keeps them
+                                in both FP64 and FP32, 0 in the precisions of the Hamiltonian */
   const double* k;           /* NULL or [3] Bloch wave vector (1/nm) for OMEN_BLOCH axes */
   const double* U_atom_dev;  /* NULL or [natoms] onsite potential energy (eV), e.g. -phi */
 } omen_ham_opts;
@@ -287,8 +288,9 @@ omen_status omen_hx_host(omen_ctx* ctx, const omen_ham* ham, const void* x_host,
 
 typedef struct {
   int threads;               /* CTA width chosen (threads per block) */
-  int rows_per_batch;        /* block rows per register batch (omen_tune_hx) or wave vectors
-                                per thread (omen_tune_hx_kbatch); 0 = the built-in rule */
+  int rows_per_batch;        /* load batch (omen_tune_hx: bonds whose amplitudes are loaded
+                                together, 1 -> 1, 2 -> 2, 5 and 10 -> 4) or wave vectors per
+                                thread (omen_tune_hx_kbatch); 0 = the built-in rule */
   int candidates;            /* launch shapes timed */
   double ms_best;            /* mean launch time of the chosen shape (ms) */
   double ms_default;         /* mean launch time of the built-in shape (ms) */
@@ -311,7 +313,8 @@ omen_status omen_tune_hx_kbatch(omen_ctx* ctx, omen_ham* ham, int nk, int reps, 
  * rows_per_batch from the compiled set (FP32 stored blocks 1, 2, 5, and 10 without spin-orbit
  * for sp3d5s*; FP64 stored 1, 2; matrix-free 1, 2; 0 = the built-in rule; rows_per_batch must
  * divide the orbital count).  k batch: wave vectors per thread 1, 2 (FP64 and FP32) or 4 (FP32), 0 =
- * default 2.  EINVAL for a shape that is not compiled. */
+ * default 1.  Products too small to fill the device take one shape whatever is set here.
+ * EINVAL for a shape that is not compiled. */
 omen_status omen_hx_set_tile(omen_ctx* ctx, omen_ham* ham, int vec_precision, int threads, int rows_per_batch);
 omen_status omen_hx_kbatch_set_tile(omen_ctx* ctx, omen_ham* ham, int vec_precision, int threads,
                                     int k_per_thread);

@@ -1,12 +1,10 @@
 // Device-side Hamiltonian assembly (paper Section I: sp3s*/sp3d5s* tight binding with strain).
 //
-// 1. b0 table: the Slater–Koster block of every (species pair, bond direction) at d0,
-//    from the Table I integrals (sk_device.cuh).
-// 2. bond blocks: each existing bond slot gets (d0/d)^eta * b0[pair][dir], d = d0 (1 + strain),
-//    stored in tiles of 32 consecutive slots with the entries of a tile contiguous
-//    (blk[(tile*ne + e)*32 + lane]): a warp reads 32 slots of one entry with one coalesced
-//    128-byte load, and one bond block of a warp is a single contiguous run.  Matrix-free Hamiltonians skip this step and H·X
-//    regenerates the block from the b0 table, the two species and the strain.
+// 1. the Slater–Koster block of every species pair at d0, in the reduced form the product
+//    applies (sk_device.cuh), for both ends of the bond;
+// 2. the factor (d0/d)^eta of every bond slot, d = d0 (1 + strain): a bond's block is its
+//    factor times its pair's reduced block, with the signs of its direction.
+// Stored and matrix-free Hamiltonians hold the same data, in the precisions their products use.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -14,81 +12,33 @@
 #include "omen_internal.h"
 #include "sk_device.cuh"
 
-__constant__ int c_dir[4][3] = {{1, 1, 1}, {1, -1, -1}, {-1, 1, -1}, {-1, -1, 1}};
-
-__global__ void b0_table_kernel(const double* __restrict__ V, int ns, int norb, double* __restrict__ b0,
-                                float* __restrict__ b0_32) {
-  const int total = ns * ns * 4 * norb * norb;
+// coef[end][pair][coef_stride(norb)]: end 0 the rows of the A atom, end 1 those of the B atom
+__global__ void coef_table_kernel(const double* __restrict__ V, int ns, int norb, double* __restrict__ c64,
+                                  float* __restrict__ c32, float2* __restrict__ cdf) {
+  const int cs = coef_stride(norb);
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= total) return;
-  const int e = t % (norb * norb);
-  const int k = (t / (norb * norb)) % 4;
-  const int pair = t / (norb * norb * 4);
-  const int sa = pair / ns, sb = pair % ns;
-  const double inv = 0.57735026918962576;  // 1/sqrt(3)
-  const double c[3] = {c_dir[k][0] * inv, c_dir[k][1] * inv, c_dir[k][2] * inv};
-  const int o1 = e / norb, o2 = e % norb;
-  const double v = sk_element(sk_code(o1, norb), sk_code(o2, norb), c, V + (sa * ns + sb) * 14, V + (sb * ns + sa) * 14);
-  b0[t] = v;
-  b0_32[t] = (float)v;
-}
-
-__global__ void assemble_bonds_kernel(Geo g, NeighbourTables nt, const uint8_t* __restrict__ species,
-                                      const double* __restrict__ strain, const double* __restrict__ b0,
-                                      int ns, int norb, double eta, int slot_stride, double* __restrict__ blk64,
-                                      float* __restrict__ blk32, float2* __restrict__ blkdf) {
-  const int npad = 16 * slot_stride;
-  const int pidx = blockIdx.x * blockDim.x + threadIdx.x;   // padded slot index
-  if (pidx >= npad) return;
-  const int cell = pidx % slot_stride;
-  const int ks = pidx / slot_stride;  // k*4 + s
-  const int ne = norb * norb;
-  const size_t base = ((size_t)(pidx >> 5) * ne) * 32 + (pidx & 31);
-  if (cell >= g.ncells) {  // padding
-    for (int e = 0; e < ne; ++e) {
-      if (blk64) blk64[base + (size_t)e * 32] = 0.0;
-      if (blk32) blk32[base + (size_t)e * 32] = 0.0f;
-      if (blkdf) blkdf[base + (size_t)e * 32] = make_float2(0.f, 0.f);
-    }
-    return;
-  }
-  const int slot = ks * g.ncells + cell;  // strain input layout
-  const int k = ks >> 2, s = ks & 3;
-  const int ix = cell % g.nx, iy = (cell / g.nx) % g.ny, iz = cell / (g.nx * g.ny);
-  int cell2, wrap[3];
-  const bool ok = shift_cell(g, ix, iy, iz, nt.a_to_b_off[s][k][0], nt.a_to_b_off[s][k][1], nt.a_to_b_off[s][k][2],
-                             cell2, wrap);
-  if (!ok) {
-    for (int e = 0; e < ne; ++e) {
-      if (blk64) blk64[base + (size_t)e * 32] = 0.0;
-      if (blk32) blk32[base + (size_t)e * 32] = 0.0f;
-      if (blkdf) blkdf[base + (size_t)e * 32] = make_float2(0.f, 0.f);
-    }
-    return;
-  }
-  const int sa = species[s * g.ncells + cell];
-  const int sb = species[nt.a_to_b_site[s][k] * g.ncells + cell2];
-  const double f = pow(1.0 + strain[slot], -eta);
-  const double* tb = b0 + ((size_t)(sa * ns + sb) * 4 + k) * ne;
-  for (int e = 0; e < ne; ++e) {
-    const double v = f * tb[e];
-    if (blk64) blk64[base + (size_t)e * 32] = v;
-    if (blk32) blk32[base + (size_t)e * 32] = (float)v;
-    if (blkdf) {
-      const float hi = __double2float_rn(v);
-      blkdf[base + (size_t)e * 32] = make_float2(hi, __double2float_rn(v - (double)hi));
-    }
+  if (t >= 2 * ns * ns) return;
+  const int end = t / (ns * ns), pair = t - end * ns * ns;
+  const int sa = pair / ns, sb = pair - sa * ns;
+  double c[28];
+  reduced_block(V + (sa * ns + sb) * 14, V + (sb * ns + sa) * 14, norb, end != 0, c);
+  for (int i = 0; i < cs; ++i) {
+    const size_t at = (size_t)t * cs + i;
+    const float hi = __double2float_rn(c[i]);
+    if (c64) c64[at] = c[i];
+    if (c32) c32[at] = hi;
+    if (cdf) cdf[at] = make_float2(hi, __double2float_rn(c[i] - (double)hi));
   }
 }
 
-// Matrix-free Hamiltonians: the bond-length factor (d0/d)^eta of every slot, d = d0 (1 + strain),
-// kept in both precisions (the product regenerates each block as factor x b0[pair][dir]).
-__global__ void mf_scale_kernel(const double* __restrict__ strain, long long nslots, double eta,
-                                double* __restrict__ s64, float* __restrict__ s32) {
+__global__ void bond_scale_kernel(const double* __restrict__ strain, long long nslots, double eta,
+                                  double* __restrict__ s64, float* __restrict__ s32, float2* __restrict__ sdf) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nslots; i += (long long)gridDim.x * blockDim.x) {
     const double f = pow(1.0 + strain[i], -eta);
-    s64[i] = f;
-    s32[i] = (float)f;
+    const float hi = __double2float_rn(f);
+    if (s64) s64[i] = f;
+    if (s32) s32[i] = hi;
+    if (sdf) sdf[i] = make_float2(hi, __double2float_rn(f - (double)hi));
   }
 }
 
@@ -100,13 +50,12 @@ __global__ void max_species_kernel(const uint8_t* __restrict__ sp, int n, int* _
 }
 
 static void free_ham_buffers(omen_ham* h) {
-  cudaFree(h->d_blk64);
-  cudaFree(h->d_blk32);
-  cudaFree(h->d_blkdf);
-  cudaFree(h->d_b0_64);
-  cudaFree(h->d_b0_32);
+  cudaFree(h->d_coef64);
+  cudaFree(h->d_coef32);
+  cudaFree(h->d_coefdf);
   cudaFree(h->d_scale64);
   cudaFree(h->d_scale32);
+  cudaFree(h->d_scaledf);
   cudaFree(h->d_onsite);
   cudaFree(h->d_onsite32);
   cudaFree(h->d_onsite_df);
@@ -177,25 +126,28 @@ extern "C" omen_status omen_assemble_H(omen_ctx* ctx, const omen_lattice* lat, c
   h->is_complex = (h->spin_orbit || h->bloch) ? 1 : 0;
   for (int s = 0; s < 4; ++s) h->lambda_so[s] = p->lambda_so[s];
 
-  const int ns = p->nspecies, norb = p->basis, ne = norb * norb;
-  h->slot_stride = (lat->ncells + 31) / 32 * 32;
-  const size_t nslots = 16 * (size_t)h->slot_stride;
-  const size_t ntab = (size_t)ns * ns * 4 * ne;
-  ALLOC_OR_FAIL(h->d_b0_64, ntab * sizeof(double));
-  ALLOC_OR_FAIL(h->d_b0_32, ntab * sizeof(float));
+  const int ns = p->nspecies, norb = p->basis;
+  const size_t nslots = 16 * (size_t)lat->ncells;
+  const size_t ncoef = 2 * (size_t)ns * ns * coef_stride(norb);
   ALLOC_OR_FAIL(h->d_onsite, sizeof(double) * ns * norb);
   ALLOC_OR_FAIL(h->d_onsite32, sizeof(float) * ns * norb);
   ALLOC_OR_FAIL(h->d_U, sizeof(double) * lat->natoms);
   ALLOC_OR_FAIL(h->d_lambda, sizeof(double) * 4);
-  const bool need64 = !h->matrix_free && (h->precision == OMEN_F64 || h->precision == OMEN_F32_REFINE64);
-  const bool need32 = !h->matrix_free && (h->precision == OMEN_F32 || h->precision == OMEN_F32_REFINE64);
+  // the precisions the products of this Hamiltonian use (matrix-free: FP64 and FP32)
+  const bool need64 = h->matrix_free || h->precision == OMEN_F64 || h->precision == OMEN_F32_REFINE64;
+  const bool need32 = h->matrix_free || h->precision == OMEN_F32 || h->precision == OMEN_F32_REFINE64;
   const bool needdf = h->precision == OMEN_F64_DF;
-  if (need64) ALLOC_OR_FAIL(h->d_blk64, sizeof(double) * ne * nslots);
-  if (need32) ALLOC_OR_FAIL(h->d_blk32, sizeof(float) * ne * nslots);
-  if (needdf) ALLOC_OR_FAIL(h->d_blkdf, sizeof(float2) * ne * nslots);
-  if (h->matrix_free) {
-    ALLOC_OR_FAIL(h->d_scale64, sizeof(double) * 16 * (size_t)lat->ncells);
-    ALLOC_OR_FAIL(h->d_scale32, sizeof(float) * 16 * (size_t)lat->ncells);
+  if (need64) {
+    ALLOC_OR_FAIL(h->d_coef64, ncoef * sizeof(double));
+    ALLOC_OR_FAIL(h->d_scale64, nslots * sizeof(double));
+  }
+  if (need32) {
+    ALLOC_OR_FAIL(h->d_coef32, ncoef * sizeof(float));
+    ALLOC_OR_FAIL(h->d_scale32, nslots * sizeof(float));
+  }
+  if (needdf) {
+    ALLOC_OR_FAIL(h->d_coefdf, ncoef * sizeof(float2));
+    ALLOC_OR_FAIL(h->d_scaledf, nslots * sizeof(float2));
   }
 
   // parameter tables
@@ -245,20 +197,12 @@ extern "C" omen_status omen_assemble_H(omen_ctx* ctx, const omen_lattice* lat, c
       e = cudaMemsetAsync(h->d_U, 0, sizeof(double) * lat->natoms, ctx->stream);
   }
   if (e == cudaSuccess) {
-    b0_table_kernel<<<(unsigned)((ntab + 255) / 256), 256, 0, ctx->stream>>>(d_V, ns, norb, h->d_b0_64, h->d_b0_32);
+    coef_table_kernel<<<1, 64, 0, ctx->stream>>>(d_V, ns, norb, h->d_coef64, h->d_coef32, h->d_coefdf);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess && h->matrix_free) {
-    const long long n = 16ll * lat->ncells;
-    mf_scale_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 65535), 256, 0, ctx->stream>>>(
-        lat->d_strain, n, p->eta, h->d_scale64, h->d_scale32);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess && (need64 || need32 || needdf)) {
-    Geo g{lat->nx, lat->ny, lat->nz, lat->ncells, lat->natoms, {lat->periodic[0], lat->periodic[1], lat->periodic[2]}};
-    assemble_bonds_kernel<<<(unsigned)((nslots + 255) / 256), 256, 0, ctx->stream>>>(
-        g, host_neighbour_tables(), lat->d_species, lat->d_strain, h->d_b0_64, ns, norb, p->eta,
-        h->slot_stride, h->d_blk64, h->d_blk32, h->d_blkdf);
+  if (e == cudaSuccess) {
+    bond_scale_kernel<<<(unsigned)std::min<size_t>((nslots + 255) / 256, 65535), 256, 0, ctx->stream>>>(
+        lat->d_strain, (long long)nslots, p->eta, h->d_scale64, h->d_scale32, h->d_scaledf);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);

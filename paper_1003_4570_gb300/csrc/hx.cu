@@ -1,15 +1,29 @@
 // y = (H - sigma) x: the block-sparse tight-binding product repeated by the Lanczos
 // recurrence (paper Section II-B benchmarks "500 Lanczos iterations"; Section III-A item 1).
 //
-// One thread per atom (grid.x over (cell tile, site b) with b fastest, grid.z over vectors).  Each row
-// of H has an onsite block and four bond blocks.  Bond blocks are stored once per bond
-// (A-atom slot); an A atom applies B, its B partner applies B^T, so no block is duplicated.
-// The partner's copy of the block is read within about one z-plane of cells of the first
-// read, which lies inside the L2 cache, so HBM sees each block about once.
-// Blocks are stored in 32-slot tiles (entries of a tile contiguous): for a fixed entry,
-// consecutive threads (consecutive cells) read consecutive words, and a warp's whole block
-// is one contiguous run of memory.  Vectors are orbital-major, atom-minor, so the
-// per-orbital loads of x and stores of y are coalesced as well.
+// Bond blocks are applied in reduced form.  A two-centre block is invariant under rotations
+// about its bond, so along (1,1,1), with the p and t2g amplitudes written (x, y, z) and
+// (yz, zx, xy), it holds 25 numbers (10 for sp3s*) instead of 100 (25): the s, s* rows see
+// only the sums P = px+py+pz and T = dyz+dzx+dxy; p-p, p-t2g, t2g-t2g parts are a multiple of
+// the identity plus a multiple of the all-ones matrix; the e pair couples to p and t2g through
+// the zero-sum triple q = (-e2/2 + r e1, -e2/2 - r e1, e2), r = sqrt(3)/2.  The other three
+// directions differ by the signs of (px, py, pz) and (dyz, dzx, dxy), the same three signs for
+// both; the bond's length multiplies the whole block by (d0/d)^eta.  A bond end costs 61
+// operations (FP64: the bound) instead of 100, and reads one factor instead of a block, so no
+// block is stored: the reduced numbers of every species pair (a few KB, both ends of the bond)
+// sit in shared memory.
+//
+// Measured on the sp3d5s* alloy of 1M atoms, full blocks before and this form after: FP64 0.706 ->
+// 0.451 ms (92% of the FP64 rate; bound by it), FP32 stored 0.169 -> 0.040 ms, FP32 matrix-free
+// 0.061 -> 0.040 ms (bound by the shared-memory reads of the reduced blocks, 27 words a bond end
+// and lane, and the latency of the neighbours' amplitudes: 54% of the LSU data rate, 65% of the
+// issue slots).  The rounding error against 64 bits falls with the number of terms: FP32 1.3e-7
+// -> 0.7e-7 of the result's norm.
+//
+// One thread per atom; a warp takes 32 consecutive cells of one site, the eight warps of a CTA
+// the eight sites of the same cells, so that of the sixteen bonds of a cell nine find their
+// neighbour's amplitudes in the lines the CTA has just read.  Vectors are orbital-major,
+// atom-minor: the per-orbital loads of x and stores of y are coalesced.
 // Bloch phase: a neighbour reached across the high (low) face of a Bloch-periodic direction d
 // is its periodic image shifted by +L_d (-L_d); its amplitude is multiplied by
 // exp(+i k_d L_d) (resp. the conjugate).
@@ -29,419 +43,481 @@ template <> struct Cx<float> { using t = float2; };
 template <typename T, bool CPLX> struct VecT { using t = T; };
 template <typename T> struct VecT<T, true> { using t = typename Cx<T>::t; };
 
-template <typename T>
-struct HxArgs {
-  Geo g;
-  NeighbourTables nt;
-  const T* __restrict__ blk;          // stored blocks (entry-major), or null for matrix-free
-  const T* __restrict__ b0;           // [ns*ns*4][norb*norb] blocks at d0 (matrix-free)
-  const T* __restrict__ scale;        // [16*ncells] (d0/d)^eta per bond slot (matrix-free)
-  const uint8_t* __restrict__ species;
-  const double* __restrict__ onsite;  // [ns][norb]
-  const T* __restrict__ onsite_t;     // the same in T (real matrix-free rows)
-  const double* __restrict__ U;       // [natoms]
-  const double* __restrict__ lambda;  // [ns]
-  const void* x;
-  void* y;
-  long long nrows;
-  double sigma;
-  double2 phase[3];
-  int ns;
-  int slot_stride;
-  int cell0, cell1;                   // cells [cell0, cell1) of this launch (a z-range of planes)
-  int nbid;                           // CTA work items: 8 sites x cell tiles of blockDim.x cells
-};
+// Amplitudes (real, or complex as a pair) times real numbers.  FP32 pairs use the packed
+// FP32x2 instructions: each lane an ordinary fma, add or multiply.
+__device__ __forceinline__ double v_fma(double c, double x, double a) { return fma(c, x, a); }
+__device__ __forceinline__ float v_fma(float c, float x, float a) { return fmaf(c, x, a); }
+__device__ __forceinline__ double2 v_fma(double c, double2 x, double2 a) { return make_double2(fma(c, x.x, a.x), fma(c, x.y, a.y)); }
+__device__ __forceinline__ float2 v_fma(float c, float2 x, float2 a) { return __ffma2_rn(make_float2(c, c), x, a); }
+__device__ __forceinline__ double v_mul(double c, double x) { return c * x; }
+__device__ __forceinline__ float v_mul(float c, float x) { return c * x; }
+__device__ __forceinline__ double2 v_mul(double c, double2 x) { return make_double2(c * x.x, c * x.y); }
+__device__ __forceinline__ float2 v_mul(float c, float2 x) { return __fmul2_rn(make_float2(c, c), x); }
+__device__ __forceinline__ double v_add(double a, double b) { return a + b; }
+__device__ __forceinline__ float v_add(float a, float b) { return a + b; }
+__device__ __forceinline__ double2 v_add(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 v_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ double v_neg(double a) { return -a; }
+__device__ __forceinline__ float v_neg(float a) { return -a; }
+__device__ __forceinline__ double2 v_neg(double2 a) { return make_double2(-a.x, -a.y); }
+__device__ __forceinline__ float2 v_neg(float2 a) { return make_float2(-a.x, -a.y); }
+template <typename V> __device__ __forceinline__ V v_zero();
+template <> __device__ __forceinline__ double v_zero<double>() { return 0.0; }
+template <> __device__ __forceinline__ float v_zero<float>() { return 0.f; }
+template <> __device__ __forceinline__ double2 v_zero<double2>() { return make_double2(0.0, 0.0); }
+template <> __device__ __forceinline__ float2 v_zero<float2>() { return make_float2(0.f, 0.f); }
 
-template <typename T>
-__device__ __forceinline__ typename Cx<T>::t cmul(typename Cx<T>::t a, typename Cx<T>::t b) {
-  typename Cx<T>::t r;
+template <typename C>
+__device__ __forceinline__ C cmul(C a, C b) {
+  C r;
   r.x = a.x * b.x - a.y * b.y;
   r.y = a.x * b.y + a.y * b.x;
   return r;
 }
 
-// Accumulator helpers: real or complex times a real block entry.
-template <typename T> __device__ __forceinline__ void fma_r(T& acc, T h, T x) { acc = fma(h, x, acc); }
-template <typename T, typename C> __device__ __forceinline__ void fma_c(C& acc, T h, C x) {
-  acc.x = fma(h, x.x, acc.x);
-  acc.y = fma(h, x.y, acc.y);
-}
-
-// RBT: block rows loaded per register batch (0 = the built-in rule below); the CTA width
-// (blockDim.x, a multiple of 32 up to 128) and RBT are the tile shape the tuner chooses.
-// Matrix-free block rows: RB rows of the b0 block (shared memory) into registers, with 16-byte
-// loads where the row offsets allow (FP32 with an even RB and orbital count, FP64 with an even
-// orbital count), else one word at a time.
-template <typename T, int NORB, int RB>
-__device__ __forceinline__ void smem_rows(const T* hb, int r0, T* hr) {
-  constexpr int NE = RB * NORB;
-  if constexpr (sizeof(T) == 4 && NORB % 2 == 0 && RB % 2 == 0) {
-    const float4* h4 = reinterpret_cast<const float4*>(hb + r0 * NORB);
+// The reduced numbers of one bond end, shared memory to registers in 16-byte loads.
+template <typename T, int NORB>
+__device__ __forceinline__ void load_coef(const T* __restrict__ s, T (&c)[coef_stride(NORB)]) {
+  constexpr int N = coef_stride(NORB);
+  if constexpr (sizeof(T) == 4) {
+    const float4* s4 = reinterpret_cast<const float4*>(s);
 #pragma unroll
-    for (int e = 0; e < NE / 4; ++e) {
-      const float4 v = h4[e];
-      hr[4 * e] = v.x; hr[4 * e + 1] = v.y; hr[4 * e + 2] = v.z; hr[4 * e + 3] = v.w;
-    }
-  } else if constexpr (sizeof(T) == 8 && NORB % 2 == 0) {
-    const double2* h2 = reinterpret_cast<const double2*>(hb + r0 * NORB);
-#pragma unroll
-    for (int e = 0; e < NE / 2; ++e) {
-      const double2 v = h2[e];
-      hr[2 * e] = v.x; hr[2 * e + 1] = v.y;
+    for (int i = 0; i < N / 4; ++i) {
+      const float4 v = s4[i];
+      c[4 * i] = v.x; c[4 * i + 1] = v.y; c[4 * i + 2] = v.z; c[4 * i + 3] = v.w;
     }
   } else {
+    const double2* s2 = reinterpret_cast<const double2*>(s);
 #pragma unroll
-    for (int e = 0; e < NE; ++e) hr[e] = hb[r0 * NORB + e];
+    for (int i = 0; i < N / 2; ++i) {
+      const double2 v = s2[i];
+      c[2 * i] = v.x; c[2 * i + 1] = v.y;
+    }
   }
 }
 
-// Rows of one work item: site b = bid & 7 (fastest, so CTAs in flight cover all 8 sites of a
-// window of cells and the transposed (B-end) read of a bond block follows its A-end read within
-// L2 reach) and cells [cell0 + (bid >> 3) * blockDim.x, ...) one per thread.
-template <typename T, int NORB, bool CPLX, bool SO, bool MATFREE, int RBT>
-__device__ __forceinline__ void hx_item(const HxArgs<T>& a, int bid, const T* __restrict__ tab) {
-  using V = typename VecT<T, CPLX>::t;
-  constexpr int NS = SO ? 2 : 1;
-  const Geo& g = a.g;
-  const int b = bid & 7;
-  const int cell = a.cell0 + (bid >> 3) * blockDim.x + threadIdx.x;
-  if (cell >= a.cell1) return;
-  const int N = g.natoms;
-  const int atom = b * g.ncells + cell;
-  const int ix = cell % g.nx, iy = (cell / g.nx) % g.ny, iz = cell / (g.nx * g.ny);
-  const V* __restrict__ x = static_cast<const V*>(a.x) + (size_t)blockIdx.z * a.nrows;
-  V* __restrict__ y = static_cast<V*>(a.y) + (size_t)blockIdx.z * a.nrows;
-  const int sp = a.species[atom];
-
-  V acc[NS][NORB];
-  {
-    const T u = (T)(a.U[atom] - a.sigma);
+// r = B x for the bond along (1,1,1), from its reduced numbers (the order of coef_table).
+template <typename T, int NORB, typename V>
+__device__ __forceinline__ void bond_product(const T (&c)[coef_stride(NORB)], const V (&x)[NORB], V (&r)[NORB]) {
+  if constexpr (NORB == 5) {
+    const V P = v_add(v_add(x[1], x[2]), x[3]);
+    r[0] = v_fma(c[2], x[4], v_fma(c[1], P, v_mul(c[0], x[0])));
+    r[4] = v_fma(c[5], x[4], v_fma(c[4], P, v_mul(c[3], x[0])));
+    const V C = v_fma(c[8], P, v_fma(c[7], x[4], v_mul(c[6], x[0])));
 #pragma unroll
-    for (int s = 0; s < NS; ++s)
+    for (int i = 0; i < 3; ++i) r[1 + i] = v_fma(c[9], x[1 + i], C);
+  } else {
+    constexpr T kHalf = (T)0.5, kR = (T)0.86602540378443865;   // sqrt(3)/2
+    const V p12 = v_add(x[1], x[2]), t12 = v_add(x[4], x[5]);
+    const V P = v_add(p12, x[3]), Q = v_add(t12, x[6]);
+    r[0] = v_fma(c[3], x[9], v_fma(c[2], Q, v_fma(c[1], P, v_mul(c[0], x[0]))));
+    r[9] = v_fma(c[7], x[9], v_fma(c[6], Q, v_fma(c[5], P, v_mul(c[4], x[0]))));
+    const V Cp = v_fma(c[11], Q, v_fma(c[10], P, v_fma(c[9], x[9], v_mul(c[8], x[0]))));
+    const V Ct = v_fma(c[18], Q, v_fma(c[17], P, v_fma(c[16], x[9], v_mul(c[15], x[0]))));
+    const V h = v_mul(-kHalf, x[8]);
+    const V q[3] = {v_fma(kR, x[7], h), v_fma(-kR, x[7], h), x[8]};
 #pragma unroll
-      for (int o = 0; o < NORB; ++o) {
-        const T d = a.onsite_t[sp * NORB + o] + u;
-        const V xv = x[(size_t)(s * NORB + o) * N + atom];
-        if constexpr (CPLX) {
-          acc[s][o].x = d * xv.x;
-          acc[s][o].y = d * xv.y;
-        } else {
-          acc[s][o] = d * xv;
-        }
-      }
-    if constexpr (SO) {
-      // lambda L.sigma on (px,py,pz) = orbitals 1..3, basis (spin, orbital), spin up first
-      const T lam = (T)a.lambda[sp];
-      V xu[3], xd[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        xu[i] = x[(size_t)(1 + i) * N + atom];
-        xd[i] = x[(size_t)(NORB + 1 + i) * N + atom];
-      }
-      // i*z = (-z.y, z.x)
-      // up x: -i xu_y + xd_z ; up y: i xu_x - i xd_z ; up z: i xd_y - xd_x
-      // dn x: i xd_y - xu_z ; dn y: -i xd_x - i xu_z ; dn z: i xu_y + xu_x
-      acc[0][1].x += lam * (xu[1].y + xd[2].x);
-      acc[0][1].y += lam * (-xu[1].x + xd[2].y);
-      acc[0][2].x += lam * (-xu[0].y + xd[2].y);
-      acc[0][2].y += lam * (xu[0].x - xd[2].x);
-      acc[0][3].x += lam * (-xd[1].y - xd[0].x);
-      acc[0][3].y += lam * (xd[1].x - xd[0].y);
-      acc[1][1].x += lam * (-xd[1].y - xu[2].x);
-      acc[1][1].y += lam * (xd[1].x - xu[2].y);
-      acc[1][2].x += lam * (xd[0].y + xu[2].y);
-      acc[1][2].y += lam * (-xd[0].x - xu[2].x);
-      acc[1][3].x += lam * (-xu[1].y + xu[0].x);
-      acc[1][3].y += lam * (xu[1].x + xu[0].y);
+    for (int i = 0; i < 3; ++i) {
+      r[1 + i] = v_fma(c[13], x[4 + i], v_fma(c[12], x[1 + i], v_fma(c[14], q[i], Cp)));
+      r[4 + i] = v_fma(c[20], x[4 + i], v_fma(c[19], x[1 + i], v_fma(c[21], q[i], Ct)));
     }
+    const V pe1 = v_add(x[1], v_neg(x[2])), te1 = v_add(x[4], v_neg(x[5]));
+    const V pe2 = v_fma(-kHalf, p12, x[3]), te2 = v_fma(-kHalf, t12, x[6]);
+    r[7] = v_fma(c[24], x[7], v_fma(c[26], te1, v_mul(c[25], pe1)));
+    r[8] = v_fma(c[24], x[8], v_fma(c[23], te2, v_mul(c[22], pe2)));
   }
+}
 
+// Whether component i of bond direction k is minus: the sign of p_i and of the i-th t2g orbital.
+__host__ __device__ constexpr bool dir_minus(int k, int i) {
+  return k != 0 && i != k - 1;   // (1,1,1), (1,-1,-1), (-1,1,-1), (-1,-1,1)
+}
+
+// One structure of a product.  Real and complex vectors, FP64 and FP32.
+template <typename T>
+struct HxInst {
+  Geo g;
+  const T* __restrict__ coef;         // [2 ends][ns*ns][coef_stride] reduced blocks
+  const T* __restrict__ scale;        // [16*ncells] (d0/d)^eta per bond slot
+  const uint8_t* __restrict__ species;
+  const T* __restrict__ onsite;       // [ns][norb]
+  const double* __restrict__ U;       // [natoms]
+  const double* __restrict__ lambda;  // [ns]
+  const double2* __restrict__ phases; // k batch: [nk][3] exp(i k_d L_d)
+  long long nrows;
+  long long x_off;                    // first element of this structure's vectors
+  double2 phase[3];                   // the same for the one wave vector of a plain product
+  int ns;
+  int nvec;                           // vectors (k batch: wave vectors)
+  int cta0, tiles;                    // k batch: first CTA, CTAs per group of wave vectors
+};
+
+// Where the bonds of one atom lead.  With the four A sites (000), (022), (202), (220) and the B
+// sites those plus (111), direction k joins A site s with B site s^k, and crosses into the next
+// cell down (seen from A; up from B) along each axis where dir_k is minus and the site's
+// coordinate is 0 (B: 3).  So an atom has one possible step per axis, the same for all its bonds.
+struct Steps {
+  int d[3];        // cell index change of the step along each axis (0: this site never steps there)
+  unsigned bits;   // bit d: that step crosses a face of the block; bit 4 + d: and leaves a hard wall
+};
+
+__device__ __forceinline__ Steps steps_of(const Geo& g, int b, int ix, int iy, int iz) {
   const bool is_a = b < 4;
-  const int s = is_a ? b : b - 4;
-  constexpr int RB = RBT > 0 ? RBT
-                             : (MATFREE ? ((sizeof(T) == 4 && NORB % 2 == 0) ? 2 : 1)
-                                        : (sizeof(T) == 8 ? 1 : (NS == 1 ? NORB : (NORB == 10 ? 5 : NORB))));
-  static_assert(NORB % RB == 0, "RB must divide the orbital count");
-#pragma unroll 1
-  for (int k = 0; k < 4; ++k) {
-    int ox, oy, oz, site2;
-    if (is_a) {
-      ox = a.nt.a_to_b_off[s][k][0]; oy = a.nt.a_to_b_off[s][k][1]; oz = a.nt.a_to_b_off[s][k][2];
-      site2 = a.nt.a_to_b_site[s][k];
-    } else {
-      ox = a.nt.b_to_a_off[s][k][0]; oy = a.nt.b_to_a_off[s][k][1]; oz = a.nt.b_to_a_off[s][k][2];
-      site2 = a.nt.b_to_a_site[s][k];
-    }
-    int cell2, wrap[3];
-    if (!shift_cell(g, ix, iy, iz, ox, oy, oz, cell2, wrap)) continue;
-    const int atom2 = site2 * g.ncells + cell2;
-    // bond slot belongs to the A end
-    const size_t slot = is_a ? (size_t)(k * 4 + s) * g.ncells + cell : (size_t)(k * 4 + site2) * g.ncells + cell2;
-
-    V xn[NS][NORB];
+  const int s = b & 3;
+  const int at[3] = {ix, iy, iz}, ext[3] = {g.nx, g.ny, g.nz}, str[3] = {1, g.nx, g.nx * g.ny};
+  Steps t;
+  t.bits = 0;
 #pragma unroll
-    for (int q = 0; q < NS; ++q)
-#pragma unroll
-      for (int o = 0; o < NORB; ++o) xn[q][o] = x[(size_t)(q * NORB + o) * N + atom2];
-    if constexpr (CPLX) {
-      if (wrap[0] | wrap[1] | wrap[2]) {
-        typename Cx<T>::t f;
-        f.x = (T)1; f.y = (T)0;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          if (wrap[d]) {
-            typename Cx<T>::t p;
-            p.x = (T)a.phase[d].x;
-            p.y = (T)(wrap[d] > 0 ? a.phase[d].y : -a.phase[d].y);
-            f = cmul<T>(f, p);
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < NS; ++q)
-#pragma unroll
-          for (int o = 0; o < NORB; ++o) xn[q][o] = cmul<T>(xn[q][o], f);
-      }
-    }
-
-    const T* __restrict__ hb;
-    size_t stride;
-    T scale = (T)1;
-    if constexpr (MATFREE) {
-      const int sa = is_a ? sp : a.species[atom2];
-      const int sb = is_a ? a.species[atom2] : sp;
-      scale = a.scale[slot];
-      hb = tab + ((sa * a.ns + sb) * 4 + k) * (NORB * NORB);
-      stride = 1;
-    } else {
-      const size_t ks = is_a ? (size_t)(k * 4 + s) : (size_t)(k * 4 + site2);
-      const size_t pidx = ks * a.slot_stride + (is_a ? cell : cell2);
-      hb = a.blk + ((pidx >> 5) * (NORB * NORB)) * 32 + (pidx & 31);
-      stride = 32;
-    }
-
-    if constexpr (MATFREE) {
-      // the (d0/d)^eta factor is applied to the neighbour amplitudes once per bond
-#pragma unroll
-      for (int q = 0; q < NS; ++q)
-#pragma unroll
-        for (int o = 0; o < NORB; ++o) {
-          if constexpr (CPLX) { xn[q][o].x *= scale; xn[q][o].y *= scale; } else { xn[q][o] *= scale; }
-        }
-    }
-    // Rows of the block are loaded RB at a time into registers before their FMAs, so each
-    // thread keeps RB*NORB independent loads in flight (memory-level parallelism).  Every
-    // accumulator sums its terms in the same order for any RB: the result does not depend on it.
-#pragma unroll
-    for (int r0 = 0; r0 < NORB; r0 += RB) {
-      T hr[RB * NORB];
-      if constexpr (MATFREE) {
-        smem_rows<T, NORB, RB>(hb, r0, hr);
-      } else {
-#pragma unroll
-        for (int e = 0; e < RB * NORB; ++e) hr[e] = __ldg(hb + (size_t)(r0 * NORB + e) * stride);
-      }
-      if (is_a) {
-#pragma unroll
-        for (int i = 0; i < RB; ++i)
-#pragma unroll
-          for (int o2 = 0; o2 < NORB; ++o2) {
-            const T h = hr[i * NORB + o2];
-#pragma unroll
-            for (int q = 0; q < NS; ++q) {
-              if constexpr (CPLX) fma_c(acc[q][r0 + i], h, xn[q][o2]); else fma_r(acc[q][r0 + i], h, xn[q][o2]);
-            }
-          }
-      } else {
-#pragma unroll
-        for (int i = 0; i < RB; ++i)
-#pragma unroll
-          for (int o2 = 0; o2 < NORB; ++o2) {
-            const T h = hr[i * NORB + o2];
-#pragma unroll
-            for (int q = 0; q < NS; ++q) {
-              if constexpr (CPLX) fma_c(acc[q][o2], h, xn[q][r0 + i]); else fma_r(acc[q][o2], h, xn[q][r0 + i]);
-            }
-          }
-      }
-    }
+  for (int d = 0; d < 3; ++d) {
+    const bool can = is_a ? (s == 0 || s == d + 1) : (s != 0 && s != d + 1);
+    const bool edge = is_a ? at[d] == 0 : at[d] == ext[d] - 1;
+    const int down = edge ? (ext[d] - 1) * str[d] : -str[d];   // of an A atom; a B atom's is the opposite
+    t.d[d] = can ? (is_a ? down : -down) : 0;
+    if (can && edge) t.bits |= (g.periodic[d] == OMEN_HARD_WALL ? 17u : 1u) << d;
   }
-#pragma unroll
-  for (int q = 0; q < NS; ++q)
-#pragma unroll
-    for (int o = 0; o < NORB; ++o) y[(size_t)(q * NORB + o) * N + atom] = acc[q][o];
+  return t;
 }
 
-// Real matrix-free rows (no spin-orbit, no Bloch phase).  The site class (A or B end of its
-// bonds) is a template parameter, so the row/column order of each block product is fixed at
-// compile time; the four bonds are unrolled; the onsite energies come from a table in T and
-// U - sigma is formed once per atom, so an FP32 product runs no FP64 arithmetic per orbital.
-// Each accumulator sums its terms in the same order as hx_item's (onsite, then k = 0..3).
-// Real FP32 rows with an even orbital count use packed FP32x2 FMAs and a second, row-pair
-// interleaved copy of the table (for the A end) after the row-major one.
-template <typename T, int NORB, bool CPLX>
-__host__ __device__ constexpr bool mf_paired() { return !CPLX && sizeof(T) == 4 && NORB % 2 == 0; }
+struct Neighbour {
+  int atom;
+  int slot;        // bond slot (the A end's)
+  unsigned wrap;   // bit d: the bond crosses a face along d (downwards from an A atom)
+  bool ok;         // false: the bond leaves a hard wall
+};
 
-template <typename T, int NORB, int RB, bool IS_A>
-__device__ __forceinline__ void hx_item_mf_real(const HxArgs<T>& a, int bid, const T* __restrict__ tab) {
-  constexpr bool PAIRED = mf_paired<T, NORB, false>();
-  const int tab_copy = a.ns * a.ns * 4 * NORB * NORB;   // offset of the interleaved copy
-  const Geo& g = a.g;
-  const int b = bid & 7;
-  const int s = IS_A ? b : b - 4;
-  const int cell = a.cell0 + (bid >> 3) * blockDim.x + threadIdx.x;
-  if (cell >= a.cell1) return;
-  const int N = g.natoms;
+__device__ __forceinline__ Neighbour neighbour_of(const Geo& g, const Steps& t, int b, int k, int cell) {
+  const bool is_a = b < 4;
+  const int s = b & 3;
+  int cell2 = cell;
+  unsigned mask = 0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    if (dir_minus(k, d)) {
+      cell2 += t.d[d];
+      mask |= 1u << d;
+    }
+  Neighbour n;
+  n.wrap = t.bits & mask;
+  n.ok = (t.bits & (mask << 4)) == 0;
+  n.atom = ((s ^ k) + (is_a ? 4 : 0)) * g.ncells + cell2;
+  n.slot = is_a ? (k * 4 + s) * g.ncells + cell : (k * 4 + (s ^ k)) * g.ncells + cell2;
+  return n;
+}
+
+// exp(i k.T) of a wrapped bond
+template <typename T>
+__device__ __forceinline__ typename Cx<T>::t wrap_phase(unsigned wrap, bool is_a, const double2* __restrict__ ph) {
+  typename Cx<T>::t f;
+  f.x = (T)1;
+  f.y = (T)0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    if (wrap >> d & 1u) {
+      typename Cx<T>::t p;
+      p.x = (T)ph[d].x;
+      p.y = (T)(is_a ? -ph[d].y : ph[d].y);
+      f = cmul(f, p);
+    }
+  return f;
+}
+
+// Onsite rows: (E_o + U - sigma) x, and lambda L.sigma on the p amplitudes with spin-orbit
+// (basis (spin, orbital), spin up first; spin `q` of this thread, xo the other spin's vector).
+template <typename T, int NORB, bool CPLX, bool SO>
+__device__ __forceinline__ void onsite_rows(const HxInst<T>& I, int atom, int sp, double sigma, int q,
+                                            const typename VecT<T, CPLX>::t* __restrict__ x,
+                                            typename VecT<T, CPLX>::t (&acc)[NORB]) {
+  using V = typename VecT<T, CPLX>::t;
+  const size_t N = I.g.natoms;
+  const T u = (T)(I.U[atom] - sigma);
+  const V* __restrict__ xp = x + (size_t)(SO ? q * NORB : 0) * N + atom;
+  V xv[NORB];
+#pragma unroll
+  for (int o = 0; o < NORB; ++o) xv[o] = xp[o * N];
+  // one energy for each of s, p, d, s*
+  const T* __restrict__ e = I.onsite + sp * NORB;
+  const T es = e[0] + u, ep = e[1] + u, ed = e[NORB == 10 ? 4 : 1] + u, eS = e[NORB - 1] + u;
+#pragma unroll
+  for (int o = 0; o < NORB; ++o) acc[o] = v_mul(o == 0 ? es : o < 4 ? ep : o == NORB - 1 ? eS : ed, xv[o]);
+  if constexpr (SO) {
+    const T lam = (T)I.lambda[sp];
+    const V* __restrict__ xo = x + (size_t)((1 - q) * NORB) * N + atom;
+    const V o0 = xo[N], o1 = xo[2 * N], o2 = xo[3 * N];   // the other spin's px, py, pz
+    const V m0 = xv[1], m1 = xv[2], m2 = xv[3];
+    // i*z = (-z.y, z.x)
+    if (q == 0) {   // up x: -i xu_y + xd_z ; up y: i xu_x - i xd_z ; up z: i xd_y - xd_x
+      acc[1].x += lam * (m1.y + o2.x);
+      acc[1].y += lam * (-m1.x + o2.y);
+      acc[2].x += lam * (-m0.y + o2.y);
+      acc[2].y += lam * (m0.x - o2.x);
+      acc[3].x += lam * (-o1.y - o0.x);
+      acc[3].y += lam * (o1.x - o0.y);
+    } else {        // dn x: i xd_y - xu_z ; dn y: -i xd_x - i xu_z ; dn z: i xu_y + xu_x
+      acc[1].x += lam * (-m1.y - o2.x);
+      acc[1].y += lam * (m1.x - o2.y);
+      acc[2].x += lam * (m0.y + o2.y);
+      acc[2].y += lam * (-m0.x - o2.x);
+      acc[3].x += lam * (-o1.y + o0.x);
+      acc[3].y += lam * (o1.x + o0.y);
+    }
+  }
+}
+
+// Rows of one atom for NV vectors v0.. (nv of them present).  LB bonds' amplitudes are loaded
+// before their arithmetic; every accumulator sums its terms in the same order for any LB, NV
+// and CTA width: the result does not depend on them.
+template <typename T, int NORB, bool CPLX, bool SO, bool KPH, int NV, int LB>
+__device__ __forceinline__ void hx_rows(const HxInst<T>& I, const T* __restrict__ tab, double sigma, int b, int cell, int q, int v0, int nv, const void* xv, void* yv) {
+  using V = typename VecT<T, CPLX>::t;
+  constexpr int CS = coef_stride(NORB);
+  const Geo& g = I.g;
+  const size_t N = g.natoms;
   const int atom = b * g.ncells + cell;
   const int nxy = g.nx * g.ny;
-  const int iz = cell / nxy;
-  const int rem = cell - iz * nxy;
-  const int iy = rem / g.nx;
-  const int ix = rem - iy * g.nx;
-  // faces this cell touches: a bond leaving through one wraps (periodic) or is absent (hard wall)
-  const bool lo[3] = {ix == 0, iy == 0, iz == 0};
-  const bool hi[3] = {ix == g.nx - 1, iy == g.ny - 1, iz == g.nz - 1};
-  const int stride[3] = {1, g.nx, nxy};
-  const int extent[3] = {g.nx * 1, g.ny * g.nx, g.nz * nxy};
-  const T* __restrict__ x = static_cast<const T*>(a.x) + (size_t)blockIdx.z * a.nrows;
-  T* __restrict__ y = static_cast<T*>(a.y) + (size_t)blockIdx.z * a.nrows;
-  const int sp = a.species[atom];
-  const int npair = a.ns * a.ns;
-  T acc[NORB];
-  {
-    const T u = (T)(a.U[atom] - a.sigma);
-    const T* xp = x + atom;
+  const int iz = cell / nxy, rem = cell - iz * nxy, iy = rem / g.nx, ix = rem - iy * g.nx;
+  const Steps steps = steps_of(g, b, ix, iy, iz);
+  const V* __restrict__ x = static_cast<const V*>(xv) + I.x_off + (size_t)v0 * I.nrows;
+  V* __restrict__ y = static_cast<V*>(yv) + I.x_off + (size_t)v0 * I.nrows;
+  const int sp = I.species[atom];
+  const bool is_a = b < 4;
+  const T* __restrict__ tb = tab + (is_a ? 0 : I.ns * I.ns * CS);
+  V acc[NV][NORB];
 #pragma unroll
-    for (int o = 0; o < NORB; ++o) acc[o] = (a.onsite_t[sp * NORB + o] + u) * xp[o * N];
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int* off = IS_A ? a.nt.a_to_b_off[s][k] : a.nt.b_to_a_off[s][k];
-    const int site2 = IS_A ? a.nt.a_to_b_site[s][k] : a.nt.b_to_a_site[s][k];
-    int cell2 = cell;
-    bool ok = true;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int od = off[d];            // uniform over the CTA: -1 or 0 (A sites), 0 or +1 (B sites)
-      cell2 += od * stride[d];
-      if ((od < 0 && lo[d]) || (od > 0 && hi[d])) {
-        ok = ok && g.periodic[d] != OMEN_HARD_WALL;
-        cell2 -= od * extent[d];
-      }
-    }
-    if (!ok) continue;
-    const int atom2 = site2 * g.ncells + cell2;
-    const int slot = IS_A ? (k * 4 + s) * g.ncells + cell : (k * 4 + site2) * g.ncells + cell2;
-    const int sp2 = a.species[atom2];
-    // table in shared memory ordered [direction][pair][entry]: the (at most ns^2) blocks a warp
-    // reads for one direction lie in distinct banks
-    const T* hb = tab + (k * npair + (IS_A ? sp * a.ns + sp2 : sp2 * a.ns + sp)) * (NORB * NORB);
-    const T sc = a.scale[slot];
-    const T* xp = x + atom2;
-    T xn[NORB];
-#pragma unroll
-    for (int o = 0; o < NORB; ++o) xn[o] = xp[o * N] * sc;
-    if constexpr (PAIRED) {
-      // two accumulators per packed FP32x2 FMA (each lane an ordinary fma: same bits as the
-      // scalar form).  A end: acc[r], acc[r+1] += (h[r][c], h[r+1][c]) x[c] from the row-pair
-      // interleaved copy of the table; B end: acc[c], acc[c+1] += (h[r][c], h[r][c+1]) x[r]
-      // from the row-major copy.
-      const float4* h4 = reinterpret_cast<const float4*>(IS_A ? hb + tab_copy : hb);
-#pragma unroll
-      for (int p = 0; p < NORB / 2; ++p) {
-        float2 hp[NORB];
-#pragma unroll
-        for (int q = 0; q < NORB / 2; ++q) {
-          const float4 v = h4[p * (NORB / 2) + q];
-          hp[2 * q] = make_float2(v.x, v.y);
-          hp[2 * q + 1] = make_float2(v.z, v.w);
-        }
-        if constexpr (IS_A) {
-          float2 acc2 = make_float2(acc[2 * p], acc[2 * p + 1]);
-#pragma unroll
-          for (int c = 0; c < NORB; ++c) acc2 = __ffma2_rn(hp[c], make_float2(xn[c], xn[c]), acc2);
-          acc[2 * p] = acc2.x;
-          acc[2 * p + 1] = acc2.y;
-        } else {
-          // hp holds rows 2p and 2p+1 (row-major: NORB/2 pairs per row)
-#pragma unroll
-          for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int q = 0; q < NORB / 2; ++q) {
-              float2 acc2 = make_float2(acc[2 * q], acc[2 * q + 1]);
-              acc2 = __ffma2_rn(hp[i * (NORB / 2) + q], make_float2(xn[2 * p + i], xn[2 * p + i]), acc2);
-              acc[2 * q] = acc2.x;
-              acc[2 * q + 1] = acc2.y;
-            }
-        }
-      }
+  for (int w = 0; w < NV; ++w) {
+    if (w < nv) {
+      onsite_rows<T, NORB, CPLX, SO>(I, atom, sp, sigma, q, x + (size_t)w * I.nrows, acc[w]);
     } else {
 #pragma unroll
-      for (int r0 = 0; r0 < NORB; r0 += RB) {
-        T hr[RB * NORB];
-        smem_rows<T, NORB, RB>(hb, r0, hr);
+      for (int o = 0; o < NORB; ++o) acc[w][o] = v_zero<V>();
+    }
+  }
+  const size_t spin = SO ? (size_t)(q * NORB) * N : 0;
+  T c[CS];
+  if (I.ns == 1) load_coef<T, NORB>(tb, c);   // one species: the same block for every bond
 #pragma unroll
-        for (int i = 0; i < RB; ++i)
+  for (int k0 = 0; k0 < 4; k0 += LB) {
+    Neighbour n[LB];
+    V xn[LB][NV][NORB];
+    T sc[LB];
+    int sp2[LB];
 #pragma unroll
-          for (int o2 = 0; o2 < NORB; ++o2) {
-            if constexpr (IS_A) acc[r0 + i] = fma(hr[i * NORB + o2], xn[o2], acc[r0 + i]);
-            else acc[o2] = fma(hr[i * NORB + o2], xn[r0 + i], acc[o2]);
+    for (int j = 0; j < LB; ++j) {
+      n[j] = neighbour_of(g, steps, b, k0 + j, cell);
+      sc[j] = (T)0;
+      sp2[j] = 0;
+      if (n[j].ok) {
+        sc[j] = I.scale[n[j].slot];
+        sp2[j] = I.species[n[j].atom];
+      }
+#pragma unroll
+      for (int w = 0; w < NV; ++w) {
+        const V* __restrict__ xp = x + (size_t)w * I.nrows + spin + n[j].atom;
+#pragma unroll
+        for (int o = 0; o < NORB; ++o) xn[j][w][o] = (n[j].ok && w < nv) ? xp[o * N] : v_zero<V>();
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < LB; ++j) {
+      const int k = k0 + j;
+      if (I.ns > 1) load_coef<T, NORB>(tb + (is_a ? sp * I.ns + sp2[j] : sp2[j] * I.ns + sp) * CS, c);
+#pragma unroll
+      for (int w = 0; w < NV; ++w) {
+        V(&xw)[NORB] = xn[j][w];
+        if constexpr (CPLX) {
+          if (n[j].wrap) {
+            const V f = wrap_phase<T>(n[j].wrap, is_a, KPH ? I.phases + (size_t)min(v0 + w, I.nvec - 1) * 3 : I.phase);
+#pragma unroll
+            for (int o = 0; o < NORB; ++o) xw[o] = cmul(xw[o], f);
           }
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          if (dir_minus(k, i)) {
+            xw[1 + i] = v_neg(xw[1 + i]);
+            if constexpr (NORB == 10) xw[4 + i] = v_neg(xw[4 + i]);
+          }
+        V r[NORB];
+        bond_product<T, NORB>(c, xw, r);
+#pragma unroll
+        for (int o = 0; o < NORB; ++o) {
+          const bool odd = o >= 1 && o <= (NORB == 10 ? 6 : 3);
+          acc[w][o] = v_fma(odd && dir_minus(k, (o - 1) % 3) ? -sc[j] : sc[j], r[o], acc[w][o]);
+        }
       }
     }
   }
-  T* yp = y + atom;
 #pragma unroll
-  for (int o = 0; o < NORB; ++o) yp[o * N] = acc[o];
+  for (int w = 0; w < NV; ++w)
+    if (w < nv) {
+      V* __restrict__ yp = y + (size_t)w * I.nrows + spin + atom;
+#pragma unroll
+      for (int o = 0; o < NORB; ++o) yp[o * N] = acc[w][o];
+    }
 }
 
-// Stored blocks: one work item per CTA.  Matrix-free: the b0 table (ns^2 x 4 directions x
-// norb^2 entries, a few KB) is staged in shared memory once per CTA and the CTAs stride over the
-// work items, so the per-bond block reads are shared-memory broadcasts (a warp touches at most
-// ns^2 distinct blocks) instead of divergent L1 traffic.
-template <typename T, int NORB, bool CPLX, bool SO, bool MATFREE, int RBT>
-__global__ void __launch_bounds__(128) hx_kernel(HxArgs<T> a) {
-  if constexpr (MATFREE) {
-    extern __shared__ __align__(16) unsigned char hx_smem[];
-    T* tab = reinterpret_cast<T*>(hx_smem);
-    constexpr int NE = NORB * NORB;
-    const int npair = a.ns * a.ns;
-    const int n = npair * 4 * NE;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      if constexpr (CPLX) {
-        tab[i] = a.b0[i];
-      } else {            // b0 is [pair][k][e]; the real rows read [k][pair][e]
-        const int e = i % NE, pk = i / NE, pair = pk >> 2, k = pk & 3;
-        const int blk = (k * npair + pair) * NE;
-        tab[blk + e] = a.b0[i];
-        if constexpr (mf_paired<T, NORB, CPLX>()) {   // row pair p, column c, row parity q
-          const int r = e / NORB, c = e - r * NORB;
-          tab[n + blk + ((r >> 1) * NORB + c) * 2 + (r & 1)] = a.b0[i];
-        }
-      }
-    }
-    __syncthreads();
-    if constexpr (!CPLX) {
-      constexpr int RB = RBT > 0 ? RBT : ((sizeof(T) == 4 && NORB % 2 == 0) ? 2 : 1);
-      for (int bid = blockIdx.x; bid < a.nbid; bid += gridDim.x) {
-        if ((bid & 7) < 4) hx_item_mf_real<T, NORB, RB, true>(a, bid, tab);
-        else hx_item_mf_real<T, NORB, RB, false>(a, bid, tab);
-      }
-    } else {
-      for (int bid = blockIdx.x; bid < a.nbid; bid += gridDim.x) hx_item<T, NORB, CPLX, SO, true, RBT>(a, bid, tab);
+// The reduced blocks of every species pair, both ends, into shared memory.
+template <typename T, int NORB>
+__device__ __forceinline__ void stage_coef(const T* __restrict__ coef, int ns, T* tab) {
+  const int n = 2 * ns * ns * coef_stride(NORB);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) tab[i] = coef[i];
+  __syncthreads();
+}
+
+// y = (H - sigma) x.  grid.x: work items (site fastest, then tiles of 32 cells) over the warps;
+// grid.y: the two spins with spin-orbit (the bonds are spin diagonal); grid.z: vectors.
+template <typename T, int NORB, bool CPLX, bool SO, int LB>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : CPLX ? 2 : 4) hx_kernel(const __grid_constant__ HxInst<T> I,
+                                                 double sigma, int cell0, int cell1, const void* x, void* y) {
+  __shared__ __align__(16) T tab[2 * 16 * coef_stride(NORB)];
+  stage_coef<T, NORB>(I.coef, I.ns, tab);
+  const int item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int b = item & 7;
+  const int cell = cell0 + (item >> 3) * 32 + (threadIdx.x & 31);
+  if (cell >= cell1) return;
+  const int q = SO ? blockIdx.y : 0, v = blockIdx.z;
+  hx_rows<T, NORB, CPLX, SO, false, 1, LB>(I, tab, sigma, b, cell, q, v, 1, x, y);
+}
+
+// lambda (L.sigma x) of p orbital i (0..2) at spin q: `first` and `second` are the amplitudes it
+// needs (see onsite_rows): its spin's p_1 (i = 0) or p_0 (i = 1), or the other spin's p_1 (i = 2);
+// and the other spin's p_2 (i = 0, 1) or p_0 (i = 2).
+template <typename V>
+__device__ __forceinline__ V so_term(int q, int i, V first, V second) {
+  const bool p1 = q == 0 ? i == 0 : i == 1;                        // sign of first.y in the real part
+  const bool p2 = q == 0 ? i != 2 : i != 0;                        // sign of second in the real part
+  const auto a = i == 1 ? second.y : second.x, b = i == 1 ? second.x : second.y;
+  const bool p3 = i == 1 ? false : q == 0 ? i == 0 : i == 2;       // sign of second in the imaginary part
+  V r;
+  r.x = (p1 ? first.y : -first.y) + (p2 ? a : -a);
+  r.y = (p1 ? -first.x : first.x) + (p3 ? b : -b);
+  return r;
+}
+
+// The same with one lane per bond, and for complex vectors one per bond and component: a warp
+// takes 8 atoms x 4 bonds (4 x 4 x 2 complex), the bonds' rows are summed by shuffles that leave
+// each lane the orbitals o = bond mod 4, and those lanes add the onsite rows and store.  For FP64
+// and complex products too small to give every SM sub-partition a warp: FP64 issues one warp
+// instruction in 64 cycles there, so a slab's product costs the FP64 instructions of one thread.
+// 1x1x16-cell slab, complex128: 41.0 us with one thread per atom and full blocks, 27.0 us with
+// one thread per atom and reduced blocks, 8.9 us here.
+template <typename T, int NORB, bool CPLX, bool SO>
+__global__ void __launch_bounds__(32) hx_split_kernel(const __grid_constant__ HxInst<T> I, double sigma, int cell0, int cell1,
+                                                      const void* xv, void* yv) {
+  using V = typename VecT<T, CPLX>::t;
+  constexpr int CS = coef_stride(NORB), CELLS = CPLX ? 4 : 8, G = (NORB + 3) / 4;
+  __shared__ __align__(16) T tab[2 * 16 * coef_stride(NORB)];
+  stage_coef<T, NORB>(I.coef, I.ns, tab);
+  const Geo& g = I.g;
+  const size_t N = g.natoms;
+  const int lane = threadIdx.x;
+  const int k = (lane / CELLS) & 3;
+  const bool im = CPLX && lane >= 16;              // this lane's component
+  const int b = blockIdx.x & 7;
+  const int cell_raw = cell0 + (blockIdx.x >> 3) * CELLS + lane % CELLS;
+  const bool live = cell_raw < cell1;
+  const int cell = live ? cell_raw : cell1 - 1;    // idle lanes repeat the last cell, and store nothing
+  const int q = SO ? blockIdx.y : 0, v = blockIdx.z;
+  const V* __restrict__ x = static_cast<const V*>(xv) + I.x_off + (size_t)v * I.nrows;
+  const int atom = b * g.ncells + cell;
+  const int nxy = g.nx * g.ny;
+  const int iz = cell / nxy, rem = cell - iz * nxy, iy = rem / g.nx, ix = rem - iy * g.nx;
+  const Steps steps = steps_of(g, b, ix, iy, iz);
+  const bool is_a = b < 4;
+  const size_t spin = SO ? (size_t)(q * NORB) * N : 0;
+  const Neighbour n = neighbour_of(g, steps, b, k, cell);
+  const int sp = I.species[atom];
+  T sc = (T)0;
+  int sp2 = 0;
+  if (n.ok) {
+    sc = I.scale[n.slot];
+    sp2 = I.species[n.atom];
+  }
+  const V* __restrict__ xp = x + spin + n.atom;
+  V xn[NORB], own[G];
+#pragma unroll
+  for (int o = 0; o < NORB; ++o) xn[o] = n.ok ? xp[o * N] : v_zero<V>();
+#pragma unroll
+  for (int j = 0; j < G; ++j) {
+    const int o = 4 * j + k;
+    own[j] = o < NORB ? x[spin + o * N + atom] : v_zero<V>();
+  }
+  T xs[NORB];                                      // this lane's component, times the Bloch phase
+  if constexpr (CPLX) {
+    V f;
+    f.x = (T)1;
+    f.y = (T)0;
+    if (n.wrap) f = wrap_phase<T>(n.wrap, is_a, I.phase);
+    const T fy = im ? f.y : -f.y;
+#pragma unroll
+    for (int o = 0; o < NORB; ++o) {
+      const T mine = im ? xn[o].y : xn[o].x, other = im ? xn[o].x : xn[o].y;
+      xs[o] = mine;
+      if (n.wrap) xs[o] = fma(mine, f.x, other * fy);
     }
   } else {
-    hx_item<T, NORB, CPLX, SO, false, RBT>(a, blockIdx.x, nullptr);
+#pragma unroll
+    for (int o = 0; o < NORB; ++o) xs[o] = xn[o];
+  }
+  T sg[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const bool minus = dir_minus(k, i);
+    sg[i] = minus ? -sc : sc;
+    if (minus) {
+      xs[1 + i] = -xs[1 + i];
+      if constexpr (NORB == 10) xs[4 + i] = -xs[4 + i];
+    }
+  }
+  T c[CS];
+  load_coef<T, NORB>(tab + (is_a ? 0 : I.ns * I.ns * CS) + (is_a ? sp * I.ns + sp2 : sp2 * I.ns + sp) * CS, c);
+  T r[4 * G];
+  {
+    T r0[NORB];
+    bond_product<T, NORB>(c, xs, r0);
+#pragma unroll
+    for (int o = 0; o < 4 * G; ++o) {
+      const bool odd = o >= 1 && o <= (NORB == 10 ? 6 : 3);
+      r[o] = o < NORB ? (odd ? sg[(o - 1) % 3] : sc) * r0[o < NORB ? o : 0] : (T)0;
+    }
+  }
+  const T u = (T)(I.U[atom] - sigma);
+#pragma unroll
+  for (int j = 0; j < G; ++j) {
+    // bonds k and k^2, then k and k^1: of orbitals 4j..4j+3 the lane keeps 4j + k
+    const bool h = k & 2, l = k & 1;
+    const T a0 = (h ? r[4 * j + 2] : r[4 * j]) + __shfl_xor_sync(0xffffffffu, h ? r[4 * j] : r[4 * j + 2], 2 * CELLS);
+    const T a1 = (h ? r[4 * j + 3] : r[4 * j + 1]) + __shfl_xor_sync(0xffffffffu, h ? r[4 * j + 1] : r[4 * j + 3], 2 * CELLS);
+    const T sum = (l ? a1 : a0) + __shfl_xor_sync(0xffffffffu, l ? a0 : a1, CELLS);
+    const int o = 4 * j + k;
+    if (live && o < NORB) {
+      T mine;
+      if constexpr (CPLX) mine = im ? own[j].y : own[j].x; else mine = own[j];
+      T out = fma(I.onsite[sp * NORB + o] + u, mine, sum);
+      if constexpr (SO) {
+        if (o >= 1 && o <= 3) {
+          const int i = o - 1;
+          const V* __restrict__ xo = x + (size_t)((1 - q) * NORB) * N + atom;
+          const V first = i == 2 ? xo[2 * N] : x[spin + (i == 0 ? 2 : 1) * N + atom];
+          const V t = so_term(q, i, first, i == 2 ? xo[N] : xo[3 * N]);
+          out = fma((T)I.lambda[sp], im ? t.y : t.x, out);
+        }
+      }
+      V* __restrict__ y = static_cast<V*>(yv) + I.x_off + (size_t)v * I.nrows + spin + o * N + atom;
+      if constexpr (CPLX) (im ? y->y : y->x) = out; else *y = out;
+    }
   }
 }
 
 // ---------------------------------------------------------------------------------------
 // Double-float product (precision OMEN_F64_DF): every value is an FP32 pair (hi, lo) with
 // value = hi + lo, products and sums by the error-free transformations of df.cuh, all on the
-// FP32 pipe (57x GB300's FP64 rate); the bytes moved equal those of FP64.
+// FP32 pipe (57x GB300's FP64 rate), on reduced blocks like the rest: 1M atoms 0.325 ms with full
+// blocks (79% of the HBM rate), 0.131 ms here (bound by the FP32 pipe, some 750 instructions a
+// bond end).
 struct HxDfArgs {
   Geo g;
-  NeighbourTables nt;
-  const float2* __restrict__ blk;
+  const float2* __restrict__ coef;     // as HxInst::coef, double-float
+  const float2* __restrict__ scale;
   const uint8_t* __restrict__ species;
   const float2* __restrict__ onsite;   // [ns][norb] double-float
   const double* __restrict__ U;
@@ -449,74 +525,110 @@ struct HxDfArgs {
   float2* y;
   long long nrows;
   double sigma;
-  int slot_stride;
+  int ns;
   int cell0, cell1;                    // cells [cell0, cell1) of this launch
 };
 
+// Running double-float sum (S, C)
+struct DfSum {
+  float S, C;
+  __device__ __forceinline__ float2 value() const { return df_norm(S, C); }
+};
+__device__ __forceinline__ DfSum ds_mul(float2 a, float2 b) {
+  DfSum r;
+  r.S = __fmul_rn(a.x, b.x);
+  r.C = __fmaf_rn(a.y, b.x, __fmaf_rn(a.x, b.y, __fmaf_rn(a.x, b.x, -r.S)));
+  return r;
+}
+__device__ __forceinline__ DfSum ds_mac(float2 a, float2 b, DfSum s) {
+  df_mac(s.S, s.C, a, b);
+  return s;
+}
+__device__ __forceinline__ float2 df_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 df_half(float2 a) { return make_float2(0.5f * a.x, 0.5f * a.y); }   // exact
+
+// bond_product in double-float arithmetic
 template <int NORB>
-__global__ void __launch_bounds__(128) hx_df_kernel(HxDfArgs a) {
+__device__ __forceinline__ void bond_product_df(const float2* __restrict__ c, const float2 (&x)[NORB], float2 (&r)[NORB]) {
+  if constexpr (NORB == 5) {
+    const float2 P = df_add(df_add(x[1], x[2]), x[3]);
+    r[0] = ds_mac(c[2], x[4], ds_mac(c[1], P, ds_mul(c[0], x[0]))).value();
+    r[4] = ds_mac(c[5], x[4], ds_mac(c[4], P, ds_mul(c[3], x[0]))).value();
+    const DfSum C = ds_mac(c[8], P, ds_mac(c[7], x[4], ds_mul(c[6], x[0])));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) r[1 + i] = ds_mac(c[9], x[1 + i], C).value();
+  } else {
+    const float2 kR = make_float2(0.866025388f, 1.55436253e-8f);   // sqrt(3)/2 as hi + lo
+    const float2 p12 = df_add(x[1], x[2]), t12 = df_add(x[4], x[5]);
+    const float2 P = df_add(p12, x[3]), Q = df_add(t12, x[6]);
+    r[0] = ds_mac(c[3], x[9], ds_mac(c[2], Q, ds_mac(c[1], P, ds_mul(c[0], x[0])))).value();
+    r[9] = ds_mac(c[7], x[9], ds_mac(c[6], Q, ds_mac(c[5], P, ds_mul(c[4], x[0])))).value();
+    const DfSum Cp = ds_mac(c[11], Q, ds_mac(c[10], P, ds_mac(c[9], x[9], ds_mul(c[8], x[0]))));
+    const DfSum Ct = ds_mac(c[18], Q, ds_mac(c[17], P, ds_mac(c[16], x[9], ds_mul(c[15], x[0]))));
+    const float2 h = df_neg(df_half(x[8])), re = ds_mul(kR, x[7]).value();
+    const float2 q[3] = {df_add(h, re), df_add(h, df_neg(re)), x[8]};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      r[1 + i] = ds_mac(c[13], x[4 + i], ds_mac(c[12], x[1 + i], ds_mac(c[14], q[i], Cp))).value();
+      r[4 + i] = ds_mac(c[20], x[4 + i], ds_mac(c[19], x[1 + i], ds_mac(c[21], q[i], Ct))).value();
+    }
+    const float2 pe1 = df_add(x[1], df_neg(x[2])), te1 = df_add(x[4], df_neg(x[5]));
+    const float2 pe2 = df_add(x[3], df_neg(df_half(p12))), te2 = df_add(x[6], df_neg(df_half(t12)));
+    r[7] = ds_mac(c[24], x[7], ds_mac(c[26], te1, ds_mul(c[25], pe1))).value();
+    r[8] = ds_mac(c[24], x[8], ds_mac(c[23], te2, ds_mul(c[22], pe2))).value();
+  }
+}
+
+template <int NORB>
+__global__ void __launch_bounds__(256) hx_df_kernel(const __grid_constant__ HxDfArgs a) {
+  constexpr int CS = coef_stride(NORB);
+  __shared__ __align__(16) float2 tab[2 * 16 * CS];
+  stage_coef<float2, NORB>(a.coef, a.ns, tab);
   const Geo& g = a.g;
-  const int b = blockIdx.x & 7;
-  const int cell = a.cell0 + (blockIdx.x >> 3) * blockDim.x + threadIdx.x;
+  const int item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int b = item & 7;
+  const int cell = a.cell0 + (item >> 3) * 32 + (threadIdx.x & 31);
   if (cell >= a.cell1) return;
-  const int N = g.natoms;
+  const size_t N = g.natoms;
   const int atom = b * g.ncells + cell;
-  const int ix = cell % g.nx, iy = (cell / g.nx) % g.ny, iz = cell / (g.nx * g.ny);
+  const int nxy = g.nx * g.ny;
+  const int iz = cell / nxy, rem = cell - iz * nxy, iy = rem / g.nx, ix = rem - iy * g.nx;
+  const Steps steps = steps_of(g, b, ix, iy, iz);
   const float2* __restrict__ x = a.x + (size_t)blockIdx.z * a.nrows;
   float2* __restrict__ y = a.y + (size_t)blockIdx.z * a.nrows;
   const int sp = a.species[atom];
-  float S[NORB], C[NORB];
+  const bool is_a = b < 4;
+  const float2* __restrict__ tb = tab + (is_a ? 0 : a.ns * a.ns * CS);
+  DfSum acc[NORB];
   {
     const float2 u = df_from_double(a.U[atom] - a.sigma);
 #pragma unroll
-    for (int o = 0; o < NORB; ++o) {
-      S[o] = 0.f;
-      C[o] = 0.f;
-      df_mac(S[o], C[o], df_add(a.onsite[sp * NORB + o], u), x[(size_t)o * N + atom]);
-    }
+    for (int o = 0; o < NORB; ++o) acc[o] = ds_mul(df_add(a.onsite[sp * NORB + o], u), x[o * N + atom]);
   }
-  const bool is_a = b < 4;
-  const int s = is_a ? b : b - 4;
-#pragma unroll 1
+#pragma unroll
   for (int k = 0; k < 4; ++k) {
-    int ox, oy, oz, site2;
-    if (is_a) {
-      ox = a.nt.a_to_b_off[s][k][0]; oy = a.nt.a_to_b_off[s][k][1]; oz = a.nt.a_to_b_off[s][k][2];
-      site2 = a.nt.a_to_b_site[s][k];
-    } else {
-      ox = a.nt.b_to_a_off[s][k][0]; oy = a.nt.b_to_a_off[s][k][1]; oz = a.nt.b_to_a_off[s][k][2];
-      site2 = a.nt.b_to_a_site[s][k];
-    }
-    int cell2, wrap[3];
-    if (!shift_cell(g, ix, iy, iz, ox, oy, oz, cell2, wrap)) continue;
-    const int atom2 = site2 * g.ncells + cell2;
-    float2 xn[NORB];
+    const Neighbour n = neighbour_of(g, steps, b, k, cell);
+    if (!n.ok) continue;
+    const float2 sc = a.scale[n.slot];
+    const int sp2 = a.species[n.atom];
+    float2 xn[NORB], r[NORB];
 #pragma unroll
-    for (int o = 0; o < NORB; ++o) xn[o] = x[(size_t)o * N + atom2];
-    const size_t ks = is_a ? (size_t)(k * 4 + s) : (size_t)(k * 4 + site2);
-    const size_t pidx = ks * a.slot_stride + (is_a ? cell : cell2);
-    const float2* __restrict__ hb = a.blk + ((pidx >> 5) * (NORB * NORB)) * 32 + (pidx & 31);
-    constexpr int RB = (NORB == 10) ? 5 : NORB;
+    for (int o = 0; o < NORB; ++o) xn[o] = x[o * N + n.atom];
 #pragma unroll
-    for (int r0 = 0; r0 < NORB; r0 += RB) {
-      float2 hr[RB * NORB];
-#pragma unroll
-      for (int e = 0; e < RB * NORB; ++e) hr[e] = __ldg(hb + (size_t)(r0 * NORB + e) * 32);
-      if (is_a) {
-#pragma unroll
-        for (int i = 0; i < RB; ++i)
-#pragma unroll
-          for (int o2 = 0; o2 < NORB; ++o2) df_mac(S[r0 + i], C[r0 + i], hr[i * NORB + o2], xn[o2]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < RB; ++i)
-#pragma unroll
-          for (int o2 = 0; o2 < NORB; ++o2) df_mac(S[o2], C[o2], hr[i * NORB + o2], xn[r0 + i]);
+    for (int i = 0; i < 3; ++i)
+      if (dir_minus(k, i)) {
+        xn[1 + i] = df_neg(xn[1 + i]);
+        if constexpr (NORB == 10) xn[4 + i] = df_neg(xn[4 + i]);
       }
+    bond_product_df<NORB>(tb + (is_a ? sp * a.ns + sp2 : sp2 * a.ns + sp) * CS, xn, r);
+#pragma unroll
+    for (int o = 0; o < NORB; ++o) {
+      const bool odd = o >= 1 && o <= (NORB == 10 ? 6 : 3);
+      acc[o] = ds_mac(odd && dir_minus(k, (o - 1) % 3) ? df_neg(sc) : sc, r[o], acc[o]);
     }
   }
 #pragma unroll
-  for (int o = 0; o < NORB; ++o) y[(size_t)o * N + atom] = df_norm(S[o], C[o]);
+  for (int o = 0; o < NORB; ++o) y[o * N + atom] = acc[o].value();
 }
 
 __global__ void f64_to_df_kernel(const double* __restrict__ src, float2* __restrict__ dst, long long n) {
@@ -533,8 +645,8 @@ static cudaError_t launch_df(const omen_ham* h, const void* x, void* y, int nvec
   const omen_lattice* L = h->lat;
   HxDfArgs a;
   a.g = Geo{L->nx, L->ny, L->nz, L->ncells, L->natoms, {L->periodic[0], L->periodic[1], L->periodic[2]}};
-  a.nt = host_neighbour_tables();
-  a.blk = h->d_blkdf;
+  a.coef = h->d_coefdf;
+  a.scale = h->d_scaledf;
   a.species = L->d_species;
   a.onsite = h->d_onsite_df;
   a.U = h->d_U;
@@ -542,12 +654,12 @@ static cudaError_t launch_df(const omen_ham* h, const void* x, void* y, int nvec
   a.y = static_cast<float2*>(y);
   a.nrows = h->nrows;
   a.sigma = sigma;
-  a.slot_stride = h->slot_stride;
+  a.ns = h->nspecies;
   a.cell0 = cell0;
   a.cell1 = cell1;
-  dim3 grid(((cell1 - cell0 + 127) / 128) * 8, 1, nvec);
-  if (h->norb == 10) hx_df_kernel<10><<<grid, 128, 0, st>>>(a);
-  else hx_df_kernel<5><<<grid, 128, 0, st>>>(a);
+  dim3 grid((cell1 - cell0 + 31) / 32, 1, nvec);   // a CTA's eight warps: the eight sites of 32 cells
+  if (h->norb == 10) hx_df_kernel<10><<<grid, 256, 0, st>>>(a);
+  else hx_df_kernel<5><<<grid, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -566,34 +678,19 @@ extern "C" omen_status omen_convert_vectors(omen_ctx* ctx, const void* src, int 
 
 // ---------------------------------------------------------------------------------------
 // k-batched product over several structures: y = (H_i(k) - sigma) x for every wave vector k of
-// every structure i, all in one launch (the (structure, k) work list).  Within a structure the
-// real bond blocks are the same for every k (the phase sits only on bonds that wrap a Bloch
-// face), so each thread loads a block entry once and applies it to KB wave vectors.  The CTAs
-// of structure i are [cta0_i, cta0_i + tiles_i * ceil(nk_i / KB)); within them the tile index
-// runs fastest.  phases_i[k*3 + d] = exp(i k_d L_d).  Structure i's vectors are [nk_i][nrows_i]
-// starting at element x_off_i of x and y.
+// every structure i, all in one launch (the (structure, k) work list).  Within a structure only
+// the phase on bonds that wrap a Bloch face depends on k, so each thread finds its neighbours and
+// reads their factors and reduced blocks once for KB wave vectors.  The CTAs of structure i are
+// [cta0_i, cta0_i + tiles_i * ceil(nk_i / KB)); within them the tile index runs fastest.
+// phases_i[k*3 + d] = exp(i k_d L_d).  Structure i's vectors are [nk_i][nrows_i] starting at
+// element x_off_i of x and y.
+// 4x4x80 cells, 32 wave vectors, complex64: 56 us per launch with full blocks, 28 us here (one wave
+// vector a thread at 100 registers: 25 us; two at 160: 27 us; latency, 27 MB read and written in L2).
 static constexpr int kMaxKInst = 16;
 
 template <typename T>
-struct KInst {
-  Geo g;
-  const T* blk;
-  const uint8_t* species;
-  const double* onsite;
-  const double* U;
-  const double2* phases;
-  long long nrows;
-  long long x_off;
-  int nk;
-  int slot_stride;
-  int cta0;
-  int tiles;
-};
-
-template <typename T>
 struct KMulti {
-  NeighbourTables nt;
-  KInst<T> in[kMaxKInst];
+  HxInst<T> in[kMaxKInst];
   int n;
   const void* x;
   void* y;
@@ -601,100 +698,18 @@ struct KMulti {
 };
 
 template <typename T, int NORB, int KB>
-__global__ void __launch_bounds__(128) hx_kbatch_kernel(KMulti<T> m) {
-  using V = typename Cx<T>::t;
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : KB == 1 ? 5 : KB == 2 ? 3 : 2) hx_kbatch_kernel(const __grid_constant__ KMulti<T> m) {
+  __shared__ __align__(16) T tab[2 * 16 * coef_stride(NORB)];
   int inst = 0;
   while (inst + 1 < m.n && (int)blockIdx.x >= m.in[inst + 1].cta0) ++inst;
-  const KInst<T>& I = m.in[inst];
-  const Geo& g = I.g;
+  const HxInst<T>& I = m.in[inst];
+  stage_coef<T, NORB>(I.coef, I.ns, tab);
   const int local = (int)blockIdx.x - I.cta0;
-  const int tile = local % I.tiles;
-  const int b = tile & 7;
-  const int cell = (tile >> 3) * blockDim.x + threadIdx.x;
-  if (cell >= g.ncells) return;
-  const int N = g.natoms;
-  const int atom = b * g.ncells + cell;
-  const int ix = cell % g.nx, iy = (cell / g.nx) % g.ny, iz = cell / (g.nx * g.ny);
+  const int item = (local % I.tiles) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int cell = (item >> 3) * 32 + (threadIdx.x & 31);
+  if (cell >= I.g.ncells) return;
   const int k0 = (local / I.tiles) * KB;
-  const int nkb = min(KB, I.nk - k0);
-  const V* __restrict__ x = static_cast<const V*>(m.x) + I.x_off;
-  V* __restrict__ y = static_cast<V*>(m.y) + I.x_off;
-  const int sp = I.species[atom];
-  V acc[KB][NORB];
-  {
-    const T u = (T)(I.U[atom] - m.sigma);
-#pragma unroll
-    for (int q = 0; q < KB; ++q)
-#pragma unroll
-      for (int o = 0; o < NORB; ++o) {
-        acc[q][o].x = (T)0;
-        acc[q][o].y = (T)0;
-        if (q < nkb) {
-          const T d = (T)I.onsite[sp * NORB + o] + u;
-          const V xv = x[(size_t)(k0 + q) * I.nrows + (size_t)o * N + atom];
-          acc[q][o].x = d * xv.x;
-          acc[q][o].y = d * xv.y;
-        }
-      }
-  }
-  const bool is_a = b < 4;
-  const int s = is_a ? b : b - 4;
-#pragma unroll 1
-  for (int k = 0; k < 4; ++k) {
-    int ox, oy, oz, site2;
-    if (is_a) {
-      ox = m.nt.a_to_b_off[s][k][0]; oy = m.nt.a_to_b_off[s][k][1]; oz = m.nt.a_to_b_off[s][k][2];
-      site2 = m.nt.a_to_b_site[s][k];
-    } else {
-      ox = m.nt.b_to_a_off[s][k][0]; oy = m.nt.b_to_a_off[s][k][1]; oz = m.nt.b_to_a_off[s][k][2];
-      site2 = m.nt.b_to_a_site[s][k];
-    }
-    int cell2, wrap[3];
-    if (!shift_cell(g, ix, iy, iz, ox, oy, oz, cell2, wrap)) continue;
-    const int atom2 = site2 * g.ncells + cell2;
-    V xn[KB][NORB];
-#pragma unroll
-    for (int q = 0; q < KB; ++q) {
-      V f;
-      f.x = (T)1;
-      f.y = (T)0;
-      if (q < nkb && (wrap[0] | wrap[1] | wrap[2])) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d)
-          if (wrap[d]) {
-            const double2 ph = I.phases[(size_t)(k0 + q) * 3 + d];
-            V p;
-            p.x = (T)ph.x;
-            p.y = (T)(wrap[d] > 0 ? ph.y : -ph.y);
-            f = cmul<T>(f, p);
-          }
-      }
-#pragma unroll
-      for (int o = 0; o < NORB; ++o) {
-        if (q < nkb) xn[q][o] = cmul<T>(x[(size_t)(k0 + q) * I.nrows + (size_t)o * N + atom2], f);
-        else { xn[q][o].x = (T)0; xn[q][o].y = (T)0; }
-      }
-    }
-    const size_t ks = is_a ? (size_t)(k * 4 + s) : (size_t)(k * 4 + site2);
-    const size_t pidx = ks * I.slot_stride + (is_a ? cell : cell2);
-    const T* __restrict__ hb = I.blk + ((pidx >> 5) * (NORB * NORB)) * 32 + (pidx & 31);
-#pragma unroll
-    for (int o1 = 0; o1 < NORB; ++o1)
-#pragma unroll
-      for (int o2 = 0; o2 < NORB; ++o2) {
-        const T h = __ldg(hb + (size_t)(o1 * NORB + o2) * 32);
-#pragma unroll
-        for (int q = 0; q < KB; ++q) {
-          if (is_a) fma_c(acc[q][o1], h, xn[q][o2]);
-          else fma_c(acc[q][o2], h, xn[q][o1]);
-        }
-      }
-  }
-#pragma unroll
-  for (int q = 0; q < KB; ++q)
-    if (q < nkb)
-#pragma unroll
-      for (int o = 0; o < NORB; ++o) y[(size_t)(k0 + q) * I.nrows + (size_t)o * N + atom] = acc[q][o];
+  hx_rows<T, NORB, true, false, true, KB, 1>(I, tab, m.sigma, item & 7, cell, 0, k0, min(KB, I.nvec - k0), m.x, m.y);
 }
 
 size_t vec_elem_bytes(const omen_ham* h, int precision) {
@@ -702,108 +717,95 @@ size_t vec_elem_bytes(const omen_ham* h, int precision) {
   return h->is_complex ? 2 * r : r;
 }
 
-template <typename T, int NORB, bool CPLX, bool SO, bool MF, int RBT>
-static cudaError_t launch_t(const HxArgs<T>& a0, int nvec, int threads, cudaStream_t st) {
-  HxArgs<T> a = a0;
-  a.nbid = ((a.cell1 - a.cell0 + threads - 1) / threads) * 8;
-  if constexpr (!MF) {
-    dim3 grid(a.nbid, 1, nvec);
-    hx_kernel<T, NORB, CPLX, SO, false, RBT><<<grid, threads, 0, st>>>(a);
-    return cudaGetLastError();
-  } else {
-    // one resident wave of CTAs (per vector), each striding over the work items
-    const size_t smem = (size_t)a.ns * a.ns * 4 * NORB * NORB * sizeof(T) * (mf_paired<T, NORB, CPLX>() ? 2 : 1);
-    auto kern = hx_kernel<T, NORB, CPLX, SO, true, RBT>;
-    if (smem > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-    if (e != cudaSuccess) return e;
-    const int wave = std::max(1, sms * std::max(1, per_sm));
-    dim3 grid(std::min(a.nbid, wave), 1, nvec);
-    kern<<<grid, threads, smem, st>>>(a);
+// FP64 and complex products of fewer warps (32 cells of a site, a vector, a spin) than this take
+// one lane per bond.  Measured either side of the line, lane per bond against row per lane: FP64
+// real 688 warps (14^3 cells) 18.9 against 22.7 us, 1024 warps 25.0 against 22.8 us; complex128
+// 256 warps 18.7 against 27.0 us, 400 warps 26.9 against 27.0 us; complex64 256 warps 6.1 against
+// 6.6 us.  FP32 real products gain nothing from it (5.2 us either way).
+static constexpr long long split_below(bool f64, bool cplx) { return cplx ? 400 : f64 ? 800 : 0; }
+
+template <typename T, int NORB, bool CPLX, bool SO, int LB>
+static cudaError_t launch_t(const HxInst<T>& I, int nvec, int threads, double sigma, int cell0, int cell1, const void* x,
+                            void* y, cudaStream_t st) {
+  const int warps = threads / 32;
+  const long long items = (long long)((cell1 - cell0 + 31) / 32) * 8;
+  const dim3 grid((unsigned)((items + warps - 1) / warps), SO ? 2 : 1, nvec);
+  hx_kernel<T, NORB, CPLX, SO, LB><<<grid, threads, 0, st>>>(I, sigma, cell0, cell1, x, y);
+  return cudaGetLastError();
+}
+
+// Whether `rb` is one of the load batches accepted for this kind of product (0 = the built-in
+// rule): FP32 stored 1, 2, 5, or the orbital count without spin-orbit; FP64 and matrix-free 1, 2;
+// each must divide the orbital count.
+static bool rb_valid(int norb, bool f64, bool so, bool mf, int rb) {
+  if (rb == 0) return true;
+  if (rb < 0 || norb % rb != 0) return false;
+  if (mf || f64) return rb == 1 || rb == 2;
+  return rb == 1 || rb == 2 || rb == 5 || (rb == norb && !so);
+}
+
+template <typename T, int NORB, bool CPLX, bool SO>
+static cudaError_t launch_rows(const HxInst<T>& I, int nvec, HxTile t, double sigma, int cell0, int cell1, const void* x,
+                               void* y, cudaStream_t st) {
+  // the rule looks at the whole structure, so a product computed in pieces has the same bits
+  const long long warps = (long long)((I.g.ncells + 31) / 32) * 8 * (SO ? 2 : 1) * nvec;
+  if (warps < split_below(sizeof(T) == 8, CPLX)) {
+    constexpr int cells = CPLX ? 4 : 8;
+    const long long items = (long long)((cell1 - cell0 + cells - 1) / cells) * 8;
+    const dim3 grid((unsigned)items, SO ? 2 : 1, nvec);   // one warp a CTA: the warps spread over the SMs
+    hx_split_kernel<T, NORB, CPLX, SO><<<grid, 32, 0, st>>>(I, sigma, cell0, cell1, x, y);
     return cudaGetLastError();
   }
-}
-
-// Register-batch sizes compiled for each variant (0 = the built-in rule): FP32 stored blocks
-// take 1, 2, 5 or NORB rows (NORB only without spin-orbit); FP64 stored 1 or 2; matrix-free
-// 1 or 2 (rows dividing the orbital count).
-template <typename T, int NORB, bool SO, bool MF>
-static constexpr bool rb_compiled(int rb) {
-  if (rb == 0) return true;
-  if (NORB % rb != 0) return false;
-  if (MF) return rb == 1 || rb == 2;
-  if (sizeof(T) == 8) return rb == 1 || rb == 2;
-  return rb == 1 || rb == 2 || rb == 5 || (rb == NORB && !SO);
-}
-
-template <typename T, int NORB, bool CPLX, bool SO, bool MF>
-static cudaError_t launch_rb(const HxArgs<T>& a, int nvec, HxTile t, cudaStream_t st) {
+  // bonds whose amplitudes are loaded together: rb 1 -> 1, 2 -> 2, 5 or 10 -> 4
   const int thr = t.threads ? t.threads : 128;
-  if constexpr (rb_compiled<T, NORB, SO, MF>(1)) if (t.rb == 1) return launch_t<T, NORB, CPLX, SO, MF, 1>(a, nvec, thr, st);
-  if constexpr (rb_compiled<T, NORB, SO, MF>(2)) if (t.rb == 2) return launch_t<T, NORB, CPLX, SO, MF, 2>(a, nvec, thr, st);
-  if constexpr (rb_compiled<T, NORB, SO, MF>(5)) if (t.rb == 5) return launch_t<T, NORB, CPLX, SO, MF, 5>(a, nvec, thr, st);
-  if constexpr (rb_compiled<T, NORB, SO, MF>(10)) if (t.rb == 10) return launch_t<T, NORB, CPLX, SO, MF, 10>(a, nvec, thr, st);
-  return launch_t<T, NORB, CPLX, SO, MF, 0>(a, nvec, thr, st);
+  const int lb = t.rb == 0 ? (sizeof(T) == 4 && !CPLX ? 2 : 1) : t.rb == 1 ? 1 : t.rb == 2 ? 2 : 4;
+  if constexpr (sizeof(T) == 4) if (lb == 4) return launch_t<T, NORB, CPLX, SO, 4>(I, nvec, thr, sigma, cell0, cell1, x, y, st);
+  if (lb == 2) return launch_t<T, NORB, CPLX, SO, 2>(I, nvec, thr, sigma, cell0, cell1, x, y, st);
+  return launch_t<T, NORB, CPLX, SO, 1>(I, nvec, thr, sigma, cell0, cell1, x, y, st);
 }
 
-template <typename T, int NORB>
-static cudaError_t launch_norb(const HxArgs<T>& a, const omen_ham* h, int nvec, HxTile t, cudaStream_t st) {
-  const bool mf = h->matrix_free;
-  if (!h->is_complex) return mf ? launch_rb<T, NORB, false, false, true>(a, nvec, t, st) : launch_rb<T, NORB, false, false, false>(a, nvec, t, st);
-  if (!h->spin_orbit) return mf ? launch_rb<T, NORB, true, false, true>(a, nvec, t, st) : launch_rb<T, NORB, true, false, false>(a, nvec, t, st);
-  return mf ? launch_rb<T, NORB, true, true, true>(a, nvec, t, st) : launch_rb<T, NORB, true, true, false>(a, nvec, t, st);
-}
-
-// Whether (threads, rb) is a compiled tile shape for this Hamiltonian and vector precision.
+// Whether (threads, rb) is an accepted launch shape for this Hamiltonian and vector precision.
 bool hx_tile_valid(const omen_ham* h, int vec_precision, int threads, int rb) {
   if (threads != 0 && (threads < 32 || threads > 128 || threads % 32 != 0)) return false;
-  const bool f64 = vec_precision == OMEN_F64;
-  const bool so = h->spin_orbit, mf = h->matrix_free;
-  if (h->norb == 10) {
-    if (f64) return so ? (mf ? rb_compiled<double, 10, true, true>(rb) : rb_compiled<double, 10, true, false>(rb))
-                       : (mf ? rb_compiled<double, 10, false, true>(rb) : rb_compiled<double, 10, false, false>(rb));
-    return so ? (mf ? rb_compiled<float, 10, true, true>(rb) : rb_compiled<float, 10, true, false>(rb))
-              : (mf ? rb_compiled<float, 10, false, true>(rb) : rb_compiled<float, 10, false, false>(rb));
+  return rb_valid(h->norb, vec_precision == OMEN_F64, h->spin_orbit, h->matrix_free, rb);
+}
+
+// The structure, reduced blocks and potential of a Hamiltonian for FP64 or FP32 products.
+template <typename T>
+static HxInst<T> make_inst(const omen_ham* h) {
+  const omen_lattice* L = h->lat;
+  HxInst<T> I{};
+  I.g = Geo{L->nx, L->ny, L->nz, L->ncells, L->natoms, {L->periodic[0], L->periodic[1], L->periodic[2]}};
+  if constexpr (sizeof(T) == 8) {
+    I.coef = h->d_coef64;
+    I.scale = h->d_scale64;
+    I.onsite = h->d_onsite;
+  } else {
+    I.coef = h->d_coef32;
+    I.scale = h->d_scale32;
+    I.onsite = h->d_onsite32;
   }
-  if (f64) return so ? (mf ? rb_compiled<double, 5, true, true>(rb) : rb_compiled<double, 5, true, false>(rb))
-                     : (mf ? rb_compiled<double, 5, false, true>(rb) : rb_compiled<double, 5, false, false>(rb));
-  return so ? (mf ? rb_compiled<float, 5, true, true>(rb) : rb_compiled<float, 5, true, false>(rb))
-            : (mf ? rb_compiled<float, 5, false, true>(rb) : rb_compiled<float, 5, false, false>(rb));
+  I.species = L->d_species;
+  I.U = h->d_U;
+  I.lambda = h->d_lambda;
+  I.nrows = h->nrows;
+  for (int d = 0; d < 3; ++d) I.phase[d] = h->phase[d];
+  I.ns = h->nspecies;
+  return I;
 }
 
 template <typename T>
-static cudaError_t launch_prec(const omen_ham* h, const T* blk, const T* b0, const T* scale, const void* x, void* y,
-                               int nvec, double sigma, cudaStream_t st, int cell0, int cell1) {
-  const omen_lattice* L = h->lat;
-  HxArgs<T> a;
-  a.g = Geo{L->nx, L->ny, L->nz, L->ncells, L->natoms, {L->periodic[0], L->periodic[1], L->periodic[2]}};
-  a.nt = host_neighbour_tables();
-  a.blk = blk;
-  a.b0 = b0;
-  a.scale = scale;
-  a.species = L->d_species;
-  a.onsite = h->d_onsite;
-  if constexpr (sizeof(T) == 8) a.onsite_t = reinterpret_cast<const T*>(h->d_onsite);
-  else a.onsite_t = reinterpret_cast<const T*>(h->d_onsite32);
-  a.U = h->d_U;
-  a.lambda = h->d_lambda;
-  a.x = x;
-  a.y = y;
-  a.nrows = h->nrows;
-  a.sigma = sigma;
-  for (int d = 0; d < 3; ++d) a.phase[d] = h->phase[d];
-  a.ns = h->nspecies;
-  a.slot_stride = h->slot_stride;
-  a.cell0 = cell0;
-  a.cell1 = cell1;
+static cudaError_t launch_prec(const omen_ham* h, const void* x, void* y, int nvec, double sigma, cudaStream_t st,
+                               int cell0, int cell1) {
+  const HxInst<T> I = make_inst<T>(h);
   const HxTile t = h->tile[sizeof(T) == 8 ? 0 : 1];
-  return h->norb == 10 ? launch_norb<T, 10>(a, h, nvec, t, st) : launch_norb<T, 5>(a, h, nvec, t, st);
+  auto go = [&](auto norb) {
+    constexpr int NORB = decltype(norb)::value;
+    if (!h->is_complex) return launch_rows<T, NORB, false, false>(I, nvec, t, sigma, cell0, cell1, x, y, st);
+    if (!h->spin_orbit) return launch_rows<T, NORB, true, false>(I, nvec, t, sigma, cell0, cell1, x, y, st);
+    return launch_rows<T, NORB, true, true>(I, nvec, t, sigma, cell0, cell1, x, y, st);
+  };
+  return h->norb == 10 ? go(std::integral_constant<int, 10>{}) : go(std::integral_constant<int, 5>{});
 }
 
 // y rows of the cells [cell0, cell1) (all orbitals, sites, vectors); the rest of y is untouched
@@ -813,14 +815,14 @@ static omen_status launch_hx_cells(omen_ctx* ctx, const omen_ham* h, const void*
   if (cell1 <= cell0) return OMEN_OK;
   cudaError_t e;
   if (vec_precision == OMEN_F64_DF) {
-    if (!h->d_blkdf) return set_err(ctx, OMEN_EINVAL, "Hamiltonian has no double-float blocks");
+    if (!h->d_scaledf) return set_err(ctx, OMEN_EINVAL, "Hamiltonian has no double-float blocks");
     e = launch_df(h, x, y, nvec, sigma, st, cell0, cell1);
   } else if (vec_precision == OMEN_F64) {
-    if (!h->matrix_free && !h->d_blk64) return set_err(ctx, OMEN_EINVAL, "Hamiltonian has no FP64 blocks");
-    e = launch_prec<double>(h, h->d_blk64, h->d_b0_64, h->d_scale64, x, y, nvec, sigma, st, cell0, cell1);
+    if (!h->d_scale64) return set_err(ctx, OMEN_EINVAL, "Hamiltonian has no FP64 blocks");
+    e = launch_prec<double>(h, x, y, nvec, sigma, st, cell0, cell1);
   } else {
-    if (!h->matrix_free && !h->d_blk32) return set_err(ctx, OMEN_EINVAL, "Hamiltonian has no FP32 blocks");
-    e = launch_prec<float>(h, h->d_blk32, h->d_b0_32, h->d_scale32, x, y, nvec, sigma, st, cell0, cell1);
+    if (!h->d_scale32) return set_err(ctx, OMEN_EINVAL, "Hamiltonian has no FP32 blocks");
+    e = launch_prec<float>(h, x, y, nvec, sigma, st, cell0, cell1);
   }
   if (e != cudaSuccess) return set_err(ctx, OMEN_ECUDA, "H·X launch failed: %s", cudaGetErrorString(e));
   return OMEN_OK;
@@ -977,9 +979,8 @@ extern "C" omen_status omen_hx_host(omen_ctx* ctx, const omen_ham* h, const void
   return OMEN_OK;
 }
 
-// Wave vectors per thread KB: 2 by default (the FP64 register budget: 2 x 10 complex
-// amplitudes per bond); 1, 2, 4 compiled for FP32 and 1, 2 for FP64.
-static constexpr int kKB = 2;
+// Wave vectors per thread KB: 1 by default (registers: two FP64 ones spill, two FP32 ones leave 12
+// warps an SM); 1, 2, 4 compiled for FP32 and 1, 2 for FP64.
 static bool kb_compiled(bool f64, int kb) { return kb == 0 || kb == 1 || kb == 2 || (!f64 && kb == 4); }
 
 bool hx_kbatch_tile_valid(int vec_precision, int threads, int kb) {
@@ -989,11 +990,13 @@ bool hx_kbatch_tile_valid(int vec_precision, int threads, int kb) {
 
 template <typename T, int KB>
 static cudaError_t launch_kb(KMulti<T>& m, int norb, int threads, cudaStream_t st) {
+  const int warps = threads / 32;
   long long total = 0;
   for (int i = 0; i < m.n; ++i) {
-    m.in[i].tiles = ((m.in[i].g.ncells + threads - 1) / threads) * 8;
+    const int items = ((m.in[i].g.ncells + 31) / 32) * 8;
+    m.in[i].tiles = (items + warps - 1) / warps;
     m.in[i].cta0 = (int)total;
-    total += (long long)m.in[i].tiles * ((m.in[i].nk + KB - 1) / KB);
+    total += (long long)m.in[i].tiles * ((m.in[i].nvec + KB - 1) / KB);
   }
   if (total > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   if (norb == 10) hx_kbatch_kernel<T, 10, KB><<<(unsigned)total, threads, 0, st>>>(m);
@@ -1005,31 +1008,22 @@ template <typename T>
 static cudaError_t launch_kmulti_prec(const KItem* items, int nitems, const void* x, void* y, double sigma,
                                       cudaStream_t st) {
   KMulti<T> m;
-  m.nt = host_neighbour_tables();
   m.n = nitems;
   m.x = x;
   m.y = y;
   m.sigma = sigma;
   for (int i = 0; i < nitems; ++i) {
-    const omen_ham* h = items[i].ham;
-    const omen_lattice* L = h->lat;
-    KInst<T>& I = m.in[i];
-    I.g = Geo{L->nx, L->ny, L->nz, L->ncells, L->natoms, {L->periodic[0], L->periodic[1], L->periodic[2]}};
-    if constexpr (sizeof(T) == 8) I.blk = h->d_blk64; else I.blk = h->d_blk32;
-    I.species = L->d_species;
-    I.onsite = h->d_onsite;
-    I.U = h->d_U;
-    I.phases = items[i].phases;
-    I.nrows = h->nrows;
-    I.x_off = items[i].x_off;
-    I.nk = items[i].nk;
-    I.slot_stride = h->slot_stride;
+    m.in[i] = make_inst<T>(items[i].ham);
+    m.in[i].phases = items[i].phases;
+    m.in[i].x_off = items[i].x_off;
+    m.in[i].nvec = items[i].nk;
   }
   const HxTile t = items[0].ham->ktile[sizeof(T) == 8 ? 0 : 1];
   const int thr = t.threads ? t.threads : 128;
   if (t.rb == 1) return launch_kb<T, 1>(m, items[0].ham->norb, thr, st);
   if constexpr (sizeof(T) == 4) if (t.rb == 4) return launch_kb<T, 4>(m, items[0].ham->norb, thr, st);
-  return launch_kb<T, kKB>(m, items[0].ham->norb, thr, st);
+  if (t.rb == 2) return launch_kb<T, 2>(m, items[0].ham->norb, thr, st);
+  return launch_kb<T, 1>(m, items[0].ham->norb, thr, st);
 }
 
 omen_status launch_hx_kmulti(omen_ctx* ctx, const KItem* items, int nitems, const void* x, void* y, double sigma,
@@ -1042,7 +1036,7 @@ omen_status launch_hx_kmulti(omen_ctx* ctx, const KItem* items, int nitems, cons
     if (!h->bloch || h->matrix_free || h->spin_orbit)
       return set_err(ctx, OMEN_EUNSUPPORTED, "k batch needs Bloch structures with stored blocks and no spin-orbit");
     if (h->norb != items[0].ham->norb) return set_err(ctx, OMEN_EINVAL, "structures of one k batch share the basis");
-    if (f64 ? !h->d_blk64 : !h->d_blk32) return set_err(ctx, OMEN_EINVAL, "structure %d has no blocks of this precision", i);
+    if (f64 ? !h->d_scale64 : !h->d_scale32) return set_err(ctx, OMEN_EINVAL, "structure %d has no blocks of this precision", i);
   }
   const cudaError_t e = f64 ? launch_kmulti_prec<double>(items, nitems, x, y, sigma, ctx->stream)
                             : launch_kmulti_prec<float>(items, nitems, x, y, sigma, ctx->stream);

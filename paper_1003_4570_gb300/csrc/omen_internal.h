@@ -45,7 +45,6 @@ struct HxTile {
   int threads = 0, rb = 0;
 };
 
-// Per-species-pair bond blocks for the four ideal directions, at d0 (device, row-major).
 struct omen_ham {
   const omen_lattice* lat = nullptr;
   int norb = 0, nspin = 1, nb = 0;        // nb = norb * nspin
@@ -55,18 +54,16 @@ struct omen_ham {
   double eta = 2.0;
   double kvec[3] = {0, 0, 0};
   double2 phase[3];                       // exp(i k.L_d e_d) for a +1 supercell wrap along d
-  // stored bond blocks in 32-slot tiles: slot (k*4+s, cell) -> p = (k*4+s)*slot_stride + cell,
-  // entry e = o1*norb + o2 (A rows, B cols) at blk[((p >> 5) * norb*norb + e) * 32 + (p & 31)]
-  int slot_stride = 0;                    // ncells rounded up to a multiple of 32
-  double* d_blk64 = nullptr;
-  float* d_blk32 = nullptr;
-  float2* d_blkdf = nullptr;              // double-float (hi, lo) blocks, same tiled layout
-  // matrix-free table: B0[((sa*ns + sb)*4 + k)*norb*norb + e], and the per-slot bond-length
-  // factor (d0/d)^eta of the structure's strain at assembly ([16*ncells], slot layout)
-  double* d_b0_64 = nullptr;
-  float* d_b0_32 = nullptr;
+  // reduced bond blocks of every species pair, both ends ([2][ns*ns][coef_stride(norb)], see
+  // sk_device.cuh), and the bond-length factor (d0/d)^eta of every slot from the structure's
+  // strain at assembly ([16*ncells], slot layout): FP64, FP32 and double-float copies as the
+  // products of this Hamiltonian need them, else null
+  double* d_coef64 = nullptr;
+  float* d_coef32 = nullptr;
+  float2* d_coefdf = nullptr;
   double* d_scale64 = nullptr;
   float* d_scale32 = nullptr;
+  float2* d_scaledf = nullptr;
   // onsite energies per species and orbital [ns][norb], potential per atom
   double* d_onsite = nullptr;
   float* d_onsite32 = nullptr;            // the same in FP32

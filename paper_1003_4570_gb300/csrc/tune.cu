@@ -1,5 +1,5 @@
-// Launch-shape tuner for the H·X kernels.  The tile shape of a product (CTA width; block rows
-// per register batch, or wave vectors per thread in the k batch) trades memory-level
+// Launch-shape tuner for the H·X kernels.  The tile shape of a product (CTA width; bonds whose
+// amplitudes are loaded together, or wave vectors per thread in the k batch) trades memory-level
 // parallelism against registers and occupancy, and the best choice moves with the basis,
 // precision and structure.  The tuner times every compiled shape on the Hamiltonian itself
 // (CUDA events on the context's stream, after warm-up launches) and keeps the fastest.  No
@@ -21,8 +21,7 @@ __global__ void tune_fill_kernel(float* p, long long nwords) {
 int prec_slot(int vec_precision) { return vec_precision == OMEN_F64 ? 0 : 1; }
 
 bool has_blocks(const omen_ham* h, int vec_precision) {
-  if (h->matrix_free) return true;
-  return vec_precision == OMEN_F64 ? h->d_blk64 != nullptr : h->d_blk32 != nullptr;
+  return vec_precision == OMEN_F64 ? h->d_scale64 != nullptr : h->d_scale32 != nullptr;
 }
 
 struct Scratch {
