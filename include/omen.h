@@ -417,23 +417,28 @@ typedef struct {
 typedef struct {
   double rtol;               /* stop when ||r|| <= rtol ||b|| (b - A x in FP64 in both forms) */
   int max_iter;
-  int precision;             /* OMEN_F64: FP64 iterations.  OMEN_F32_REFINE64: FP32 iterations
-                                whose residual is replaced by the FP64 one b - A x after every
-                                10x drop (reliable updates); x, the stopping test and the answer
-                                stay FP64.  Zero-initialised options give OMEN_F64. */
+  int precision;             /* OMEN_F64: the residual tested is carried from step to step (r - A d
+                                for a direct correction d, the recurrence of CG iterations).
+                                OMEN_F32_REFINE64: the residual tested is b - A x, formed anew;
+                                CG iterations, where they are needed, run in FP32 with FP64
+                                residual replacement after every 10x drop (reliable updates).
+                                x, the stopping test and the answer are FP64 in both.
+                                Zero-initialised options give OMEN_F64. */
 } omen_cg_opts;
 
 typedef struct {
-  int iterations;
+  int iterations;            /* direct corrections and CG iterations */
   int converged;
   double rel_residual;       /* ||r|| / ||b|| at exit */
   double seconds;
 } omen_solve_info;
 
 /* Solve -div(eps0 eps_r grad phi) = rho (7-point finite differences, periodic x and y,
- * phi = 0 at both z ends) by conjugate gradients, all iterations in one cooperative launch
- * (paper: finite-difference Poisson solver, Section III-A item 3), in FP64 or with FP32
- * iterations and FP64 residual replacement (opts->precision).
+ * phi = 0 at both z ends; paper: finite-difference Poisson solver, Section III-A item 3) by direct
+ * corrections: Hartley transforms along x and y, tridiagonal solves along z, in FP64.  At most two
+ * are applied; what they leave above the tolerance, and grids with lines of more than 2,048 points
+ * or more than 1,024 planes, go to conjugate gradients in one cooperative launch, in FP64 or with
+ * FP32 iterations and FP64 residual replacement (opts->precision).
  * rho_dev: C/m^3; phi_dev: V, initial guess in, solution out (rho = 0 gives phi = 0).
  * ENOCONV at max_iter; EINVAL for a grid of 2^31 or more unknowns or another precision. */
 omen_status omen_poisson(omen_ctx* ctx, const omen_grid* grid, const double* rho_dev, double* phi_dev,

@@ -2,8 +2,11 @@
 // equation and an iterative linear solver; Aztec there, conjugate gradients here).
 //
 // -div(eps0 eps_r grad phi) = rho on a uniform grid: 7-point stencil, periodic along x and y,
-// phi = 0 on the z = 0 and z = Lz planes.  The operator is symmetric positive definite, so
-// plain CG (Hestenes & Stiefel 1952) applies.  The whole iteration runs in one cooperative
+// phi = 0 on the z = 0 and z = Lz planes.  omen_poisson solves it directly (poisson_direct.cu) and
+// iterates only for what direct corrections do not reach: lines of more than 2,048 points or 1,024
+// planes, a tolerance below the rounding of the residual, or no room for their work vectors;
+// omen_poisson_static, which may not allocate, always iterates.  The operator is symmetric positive
+// definite, so plain CG (Hestenes & Stiefel 1952) applies.  The whole iteration runs in one cooperative
 // launch: three grid-wide barriers per iteration, block partial sums reduced by every block in
 // the same order, so all blocks see bit-identical scalars and leave the loop together.
 #include <cooperative_groups.h>
@@ -13,6 +16,7 @@
 #include <cmath>
 
 #include "omen_internal.h"
+#include "poisson_direct.h"
 
 namespace cgr = cooperative_groups;
 
@@ -496,6 +500,28 @@ extern "C" omen_status omen_poisson(omen_ctx* ctx, const omen_grid* gr, const do
   g.cz = 1.0 / (hz * hz);
   g.n = (long long)g.nx * g.ny * g.nzi;
   if (g.n >= (1ll << 31)) return set_err(ctx, OMEN_EINVAL, "grid larger than 2^31 unknowns");
+  const double scale = 1.0 / (kEps0 * gr->eps_r);
+  int done = 0;
+  if (poisson_direct_fits(g)) {
+    // direct corrections; what they cannot reach (a tolerance below the rounding of b - A x) or
+    // cannot allocate is left to the iterations below
+    DirectResult dr{};
+    const omen_status s = poisson_direct(ctx, g, rho, scale, phi, o->rtol, o->max_iter, mixed, &dr);
+    if (s != OMEN_OK && s != OMEN_ENOMEM) return s;
+    if (s == OMEN_OK) {
+      if (dr.converged || dr.iterations >= o->max_iter) {
+        if (info) {
+          info->iterations = dr.iterations;
+          info->converged = dr.converged;
+          info->rel_residual = dr.rel;
+          info->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+        }
+        if (!dr.converged) return set_err(ctx, OMEN_ENOCONV, "Poisson solve stopped at %d iterations, relative residual %.3e", dr.iterations, dr.rel);
+        return OMEN_OK;
+      }
+      done = dr.iterations;
+    }
+  }
   int dev_sms = 0, per_sm = 0;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, ctx->device);
   const void* kern = mixed ? (const void*)cg_mixed_kernel : (const void*)cg_kernel;
@@ -516,9 +542,8 @@ extern "C" omen_status omen_poisson(omen_ctx* ctx, const omen_grid* gr, const do
   }
   double* part = reinterpret_cast<double*>(buf + nvec * vec);
   CGOut* out = reinterpret_cast<CGOut*>(part + 3 * blocks);
-  double scale = 1.0 / (kEps0 * gr->eps_r);
   double rtol = o->rtol;
-  int max_iter = o->max_iter;
+  int max_iter = o->max_iter - done;
   cudaError_t e;
   if (mixed) {
     const double cmax = std::max(g.cx, std::max(g.cy, g.cz));
@@ -527,13 +552,13 @@ extern "C" omen_status omen_poisson(omen_ctx* ctx, const omen_grid* gr, const do
     float* p = reinterpret_cast<float*>(buf + vec);
     float* q = reinterpret_cast<float*>(buf + 2 * vec);
     float* d = reinterpret_cast<float*>(buf + 3 * vec);
-    void* args[] = {&g, &g32, (void*)&cmax, &rho, &scale, &phi, &r, &p, &q, &d, &part, &rtol, &max_iter, &out};
+    void* args[] = {&g, &g32, (void*)&cmax, &rho, (void*)&scale, &phi, &r, &p, &q, &d, &part, &rtol, &max_iter, &out};
     e = cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(threads), args, 0, ctx->stream);
   } else {
     double* r = reinterpret_cast<double*>(buf);
     double* p = reinterpret_cast<double*>(buf + vec);
     double* q = reinterpret_cast<double*>(buf + 2 * vec);
-    void* args[] = {&g, &rho, &scale, &phi, &r, &p, &q, &part, &rtol, &max_iter, &out};
+    void* args[] = {&g, &rho, (void*)&scale, &phi, &r, &p, &q, &part, &rtol, &max_iter, &out};
     e = cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(256), args, 0, ctx->stream);
   }
   CGOut ho{};
@@ -543,12 +568,12 @@ extern "C" omen_status omen_poisson(omen_ctx* ctx, const omen_grid* gr, const do
   if (e != cudaSuccess || e2 != cudaSuccess)
     return set_err(ctx, OMEN_ECUDA, "Poisson CG: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
   if (info) {
-    info->iterations = ho.iterations;
+    info->iterations = done + ho.iterations;
     info->converged = ho.converged;
     info->rel_residual = ho.rel;
     info->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   }
-  if (!ho.converged) return set_err(ctx, OMEN_ENOCONV, "CG stopped at %d iterations, relative residual %.3e", ho.iterations, ho.rel);
+  if (!ho.converged) return set_err(ctx, OMEN_ENOCONV, "CG stopped at %d iterations, relative residual %.3e", done + ho.iterations, ho.rel);
   return OMEN_OK;
 }
 
