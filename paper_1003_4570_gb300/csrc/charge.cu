@@ -134,7 +134,7 @@ extern "C" omen_status omen_density_accum(omen_ctx* ctx, const omen_ham* h, cons
   if (!ctx || !h || !psi || !occ_host || !n_atom || nstates < 0) return set_err(ctx, OMEN_EINVAL, "null argument");
   if (nstates == 0) return OMEN_OK;
   double* d_occ = nullptr;
-  if (cudaMallocAsync(&d_occ, sizeof(double) * nstates, ctx->stream) != cudaSuccess) {
+  if (ctx_alloc(ctx, &d_occ, sizeof(double) * nstates) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "occupations");
   }
@@ -188,7 +188,7 @@ extern "C" omen_status omen_deposit(omen_ctx* ctx, const omen_lattice* L, const 
   const long long plane = (long long)G.nx * G.ny;
   const long long nodes_n = plane * (G.nz + 1);
   double* nodes = nullptr;
-  if (cudaMallocAsync(&nodes, sizeof(double) * nodes_n, ctx->stream) != cudaSuccess) {
+  if (ctx_alloc(ctx, &nodes, sizeof(double) * nodes_n) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "deposit nodes");
   }

@@ -21,6 +21,17 @@ extern "C" omen_status omen_create(omen_ctx** out, int device, void* stream) {
     omen_destroy(c);
     return OMEN_ENOMEM;
   }
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = device;
+  if (cudaMemPoolCreate(&c->pool, &props) == cudaSuccess) {
+    unsigned long long keep = kPoolKeep;
+    cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  } else {
+    c->pool = nullptr;   // the device's default pool serves
+  }
+  cudaGetLastError();
   *out = c;
   return OMEN_OK;
 }
@@ -34,6 +45,7 @@ extern "C" void omen_destroy(omen_ctx* c) {
     if (st) cudaStreamDestroy(st);
   if (c->host_scratch) cudaFree(c->host_scratch);
   for (cudaEvent_t e : c->host_events) cudaEventDestroy(e);
+  if (c->pool) cudaMemPoolDestroy(c->pool);   // work still in flight keeps its part until it is freed
   delete c;
 }
 

@@ -143,7 +143,8 @@ struct HxInst {
   const T* __restrict__ onsite;       // [ns][norb]
   const double* __restrict__ U;       // [natoms]
   const double* __restrict__ lambda;  // [ns]
-  const double2* __restrict__ phases; // k batch: [nk][3] exp(i k_d L_d)
+  const double2* __restrict__ phases; // k batch: [nk][3] exp(i k_d L_d); null: with the launch,
+  int ph_at;                          // from this entry
   long long nrows;
   long long x_off;                    // first element of this structure's vectors
   double2 phase[3];                   // the same for the one wave vector of a plain product
@@ -267,7 +268,8 @@ __device__ __forceinline__ void onsite_rows(const HxInst<T>& I, int atom, int sp
 // before their arithmetic; every accumulator sums its terms in the same order for any LB, NV
 // and CTA width: the result does not depend on them.
 template <typename T, int NORB, bool CPLX, bool SO, bool KPH, int NV, int LB>
-__device__ __forceinline__ void hx_rows(const HxInst<T>& I, const T* __restrict__ tab, double sigma, int b, int cell, int q, int v0, int nv, const void* xv, void* yv) {
+__device__ __forceinline__ void hx_rows(const HxInst<T>& I, const T* __restrict__ tab, double sigma, int b, int cell, int q, int v0, int nv, const void* xv, void* yv,
+                                        const double2* __restrict__ phases = nullptr) {
   using V = typename VecT<T, CPLX>::t;
   constexpr int CS = coef_stride(NORB);
   const Geo& g = I.g;
@@ -325,7 +327,7 @@ __device__ __forceinline__ void hx_rows(const HxInst<T>& I, const T* __restrict_
         V(&xw)[NORB] = xn[j][w];
         if constexpr (CPLX) {
           if (n[j].wrap) {
-            const V f = wrap_phase<T>(n[j].wrap, is_a, KPH ? I.phases + (size_t)min(v0 + w, I.nvec - 1) * 3 : I.phase);
+            const V f = wrap_phase<T>(n[j].wrap, is_a, KPH ? phases + (size_t)min(v0 + w, I.nvec - 1) * 3 : I.phase);
 #pragma unroll
             for (int o = 0; o < NORB; ++o) xw[o] = cmul(xw[o], f);
           }
@@ -686,6 +688,8 @@ extern "C" omen_status omen_convert_vectors(omen_ctx* ctx, const void* src, int 
 // element x_off_i of x and y.
 // 4x4x80 cells, 32 wave vectors, complex64: 56 us per launch with full blocks, 28 us here (one wave
 // vector a thread at 100 registers: 25 us; two at 160: 27 us; latency, 27 MB read and written in L2).
+// Up to 128 wave vectors' phases travel as kernel parameters: allocating, copying and freeing a table
+// held a call to 42 us among others and 285 us alone; 24 and 60 us without.
 static constexpr int kMaxKInst = 16;
 
 template <typename T>
@@ -695,6 +699,7 @@ struct KMulti {
   const void* x;
   void* y;
   double sigma;
+  double2 ph[3 * kInlinePhases];      // phases of the structures whose table is null, in order
 };
 
 template <typename T, int NORB, int KB>
@@ -709,7 +714,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : KB == 1 ? 5 : KB == 
   const int cell = (item >> 3) * 32 + (threadIdx.x & 31);
   if (cell >= I.g.ncells) return;
   const int k0 = (local / I.tiles) * KB;
-  hx_rows<T, NORB, true, false, true, KB, 1>(I, tab, m.sigma, item & 7, cell, 0, k0, min(KB, I.nvec - k0), m.x, m.y);
+  hx_rows<T, NORB, true, false, true, KB, 1>(I, tab, m.sigma, item & 7, cell, 0, k0, min(KB, I.nvec - k0), m.x, m.y,
+                                              I.phases ? I.phases : m.ph + I.ph_at);
 }
 
 size_t vec_elem_bytes(const omen_ham* h, int precision) {
@@ -927,8 +933,8 @@ extern "C" omen_status omen_hx_host(omen_ctx* ctx, const omen_ham* h, const void
     // FP64 host arrays; double-float conversion on the device
     const long long n = h->nrows * nvec;
     void *dx = nullptr, *dy = nullptr, *fx = nullptr;
-    if (cudaMallocAsync(&dx, bytes, ctx->stream) != cudaSuccess || cudaMallocAsync(&dy, bytes, ctx->stream) != cudaSuccess ||
-        cudaMallocAsync(&fx, 8 * (size_t)n, ctx->stream) != cudaSuccess) {
+    if (ctx_alloc(ctx, &dx, bytes) != cudaSuccess || ctx_alloc(ctx, &dy, bytes) != cudaSuccess ||
+        ctx_alloc(ctx, &fx, 8 * (size_t)n) != cudaSuccess) {
       cudaGetLastError();
       return set_err(ctx, OMEN_ENOMEM, "device allocation of %zu bytes failed", bytes);
     }
@@ -1012,8 +1018,14 @@ static cudaError_t launch_kmulti_prec(const KItem* items, int nitems, const void
   m.x = x;
   m.y = y;
   m.sigma = sigma;
+  int ph = 0;
   for (int i = 0; i < nitems; ++i) {
     m.in[i] = make_inst<T>(items[i].ham);
+    if (!items[i].phases) {
+      m.in[i].ph_at = ph;
+      std::copy(items[i].phases_host, items[i].phases_host + 3 * items[i].nk, m.ph + ph);
+      ph += 3 * items[i].nk;
+    }
     m.in[i].phases = items[i].phases;
     m.in[i].x_off = items[i].x_off;
     m.in[i].nvec = items[i].nk;
@@ -1050,7 +1062,7 @@ omen_status launch_hx_kbatch(omen_ctx* ctx, const omen_ham* h, int nk, const dou
   return launch_hx_kmulti(ctx, &item, 1, x, y, sigma, vec_precision);
 }
 
-omen_status make_phases(omen_ctx* ctx, const omen_ham* h, int nk, const double* k_host, double2** out) {
+std::vector<double2> phase_table(const omen_ham* h, int nk, const double* k_host) {
   const omen_lattice* L = h->lat;
   std::vector<double2> ph((size_t)nk * 3);
   const int nc[3] = {L->nx, L->ny, L->nz};
@@ -1059,7 +1071,12 @@ omen_status make_phases(omen_ctx* ctx, const omen_ham* h, int nk, const double* 
       const double t = (L->periodic[d] == OMEN_BLOCH) ? k_host[q * 3 + d] * nc[d] * L->a_nm : 0.0;
       ph[(size_t)q * 3 + d] = make_double2(cos(t), sin(t));
     }
-  if (cudaMallocAsync(out, sizeof(double2) * ph.size(), ctx->stream) != cudaSuccess) {
+  return ph;
+}
+
+omen_status make_phases(omen_ctx* ctx, const omen_ham* h, int nk, const double* k_host, double2** out) {
+  const std::vector<double2> ph = phase_table(h, nk, k_host);
+  if (ctx_alloc(ctx, out, sizeof(double2) * ph.size()) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "phase table");
   }
@@ -1072,14 +1089,19 @@ extern "C" omen_status omen_hx_kbatch_multi(omen_ctx* ctx, int nitems, const ome
   if (!ctx || !it || !x || !y || nitems < 1 || nitems > kMaxKInst) return set_err(ctx, OMEN_EINVAL, "null argument or 1..%d structures", kMaxKInst);
   std::vector<KItem> items(nitems);
   std::vector<double2*> ph(nitems, nullptr);
-  long long off = 0;
+  std::vector<std::vector<double2>> inl(nitems);
+  long long off = 0, total = 0;
+  for (int i = 0; i < nitems; ++i) total += std::max(0, it[i].nk);
+  // a few wave vectors travel with the launch: no table to allocate, copy and free
+  const bool with_launch = total <= kInlinePhases;
   omen_status s = OMEN_OK;
   for (int i = 0; i < nitems && s == OMEN_OK; ++i) {
     if (!it[i].ham || !it[i].k_host || it[i].nk < 1) { s = set_err(ctx, OMEN_EINVAL, "structure %d: null argument or nk < 1", i); break; }
     if (it[i].ham->effmass) { s = set_err(ctx, OMEN_EUNSUPPORTED, "k batch runs on tight-binding Hamiltonians"); break; }
     if (!it[i].ham->bloch) { s = set_err(ctx, OMEN_EINVAL, "structure %d has no Bloch-periodic direction", i); break; }
-    s = make_phases(ctx, it[i].ham, it[i].nk, it[i].k_host, &ph[i]);
-    items[i] = KItem{it[i].ham, it[i].nk, ph[i], off};
+    if (with_launch) inl[i] = phase_table(it[i].ham, it[i].nk, it[i].k_host);
+    else s = make_phases(ctx, it[i].ham, it[i].nk, it[i].k_host, &ph[i]);
+    items[i] = KItem{it[i].ham, it[i].nk, ph[i], off, inl[i].data()};
     off += (long long)it[i].nk * it[i].ham->nrows;
   }
   if (s == OMEN_OK) {
@@ -1098,10 +1120,6 @@ extern "C" omen_status omen_hx_kbatch(omen_ctx* ctx, const omen_ham* h, int nk, 
   if (!ctx || !h || !k_host || !x || !y || nk < 1) return set_err(ctx, OMEN_EINVAL, "null argument or nk < 1");
   if (h->effmass) return set_err(ctx, OMEN_EUNSUPPORTED, "k batch runs on tight-binding Hamiltonians");
   if (!h->bloch) return set_err(ctx, OMEN_EINVAL, "k batch needs a structure with Bloch-periodic directions");
-  double2* ph = nullptr;
-  omen_status s = make_phases(ctx, h, nk, k_host, &ph);
-  if (s != OMEN_OK) return s;
-  s = launch_hx_kbatch(ctx, h, nk, ph, x, y, sigma, native_precision(h));
-  cudaFreeAsync(ph, ctx->stream);
-  return s;
+  const omen_kbatch_item item{h, nk, k_host};
+  return omen_hx_kbatch_multi(ctx, 1, &item, x, y, sigma);
 }

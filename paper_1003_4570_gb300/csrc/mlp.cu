@@ -406,7 +406,7 @@ extern "C" omen_status omen_mlp_get_params(omen_ctx* ctx, const omen_mlp* m, flo
   for (int l = 0; l < 3; ++l) {
     const size_t nw = (size_t)m->d[l + 1] * m->d[l], nb = m->d[l + 1];
     if (bf16_rounded) {
-      if (cudaMallocAsync(&tmp, nw * 4, ctx->stream) != cudaSuccess) { cudaGetLastError(); return set_err(ctx, OMEN_ENOMEM, "copy buffer"); }
+      if (ctx_alloc(ctx, &tmp, nw * 4) != cudaSuccess) { cudaGetLastError(); return set_err(ctx, OMEN_ENOMEM, "copy buffer"); }
       from_bf16_kernel<<<grid_for(nw), 256, 0, ctx->stream>>>(m->W16[l], tmp, nw);
       OMEN_CUDA(ctx, cudaMemcpyAsync(params + off, tmp, nw * 4, cudaMemcpyDeviceToHost, ctx->stream));
       cudaFreeAsync(tmp, ctx->stream);
@@ -453,7 +453,7 @@ extern "C" omen_status omen_mlp_warm_start(omen_ctx* ctx, omen_mlp* m, const ome
   s = ensure_batch(ctx, m, 1);
   if (s != OMEN_OK) return s;
   float* xy = nullptr;
-  if (cudaMallocAsync(&xy, sizeof(float) * (m->d[0] + m->d[3]), ctx->stream) != cudaSuccess) {
+  if (ctx_alloc(ctx, &xy, sizeof(float) * (m->d[0] + m->d[3])) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "warm-start buffers");
   }

@@ -261,7 +261,7 @@ extern "C" omen_status omen_state_weights(omen_ctx* ctx, const omen_ham* h, cons
   if (h->effmass || !h->lat) return set_err(ctx, OMEN_EUNSUPPORTED, "state weights need a tight-binding Hamiltonian");
   if (nstates == 0) return OMEN_OK;
   double* dw = nullptr;
-  if (cudaMallocAsync(&dw, sizeof(double) * nstates, ctx->stream) != cudaSuccess) {
+  if (ctx_alloc(ctx, &dw, sizeof(double) * nstates) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "state weights");
   }
@@ -305,7 +305,7 @@ extern "C" omen_status omen_poisson_newton(omen_ctx* ctx, const omen_lattice* L,
   });
   auto alloc = [&](size_t bytes) -> void* {
     void* p = nullptr;
-    if (cudaMallocAsync(&p, std::max<size_t>(bytes, 8), st) != cudaSuccess) {
+    if (ctx_alloc(ctx, &p, std::max<size_t>(bytes, 8)) != cudaSuccess) {
       cudaGetLastError();
       p = nullptr;
     }

@@ -28,7 +28,19 @@ struct omen_ctx {
   void* host_scratch = nullptr;
   size_t host_scratch_bytes = 0;
   std::vector<cudaEvent_t> host_events;  // the pipeline's events, created once
+  // work areas of the calls come from a pool of the context's own, which keeps up to kPoolKeep
+  // bytes mapped between calls (the default pool gives everything back at the next
+  // synchronisation, and a call then spends 0.1 to 0.4 ms mapping it again); gone with the context
+  cudaMemPool_t pool = nullptr;
 };
+constexpr unsigned long long kPoolKeep = 512ull << 20;
+
+// Stream-ordered device memory for one call on the context's stream (free with cudaFreeAsync).
+template <typename T>
+inline cudaError_t ctx_alloc(omen_ctx* ctx, T** p, size_t bytes) {
+  return ctx->pool ? cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, ctx->pool, ctx->stream)
+                   : cudaMallocAsync(reinterpret_cast<void**>(p), bytes, ctx->stream);
+}
 
 struct omen_lattice {
   int nx, ny, nz, ncells, natoms;
@@ -124,10 +136,13 @@ struct KItem {
   int nk;
   const double2* phases;
   long long x_off;
+  const double2* phases_host = nullptr;   // where `phases` is null: [nk][3], passed with the launch
 };
+constexpr int kInlinePhases = 128;        // wave vectors of a batch whose phases fit the launch
 omen_status launch_hx_kmulti(omen_ctx* ctx, const KItem* items, int nitems, const void* x, void* y, double sigma,
                              int vec_precision);
 omen_status make_phases(omen_ctx* ctx, const omen_ham* h, int nk, const double* k_host, double2** out);
+std::vector<double2> phase_table(const omen_ham* h, int nk, const double* k_host);
 
 // Krylov helpers (lanczos.cu)
 size_t vec_elem_bytes(const omen_ham* ham, int precision);

@@ -536,7 +536,7 @@ extern "C" omen_status omen_poisson(omen_ctx* ctx, const omen_grid* gr, const do
   const int nvec = mixed ? 4 : 3;
   const size_t vec = ((size_t)g.n * elem + 255) / 256 * 256;
   char* buf = nullptr;
-  if (cudaMallocAsync(&buf, nvec * vec + 3 * blocks * sizeof(double) + sizeof(CGOut) + 64, ctx->stream) != cudaSuccess) {
+  if (ctx_alloc(ctx, &buf, nvec * vec + 3 * blocks * sizeof(double) + sizeof(CGOut) + 64) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "CG work vectors");
   }

@@ -478,7 +478,7 @@ omen_status poisson_direct(omen_ctx* ctx, const PGrid& g, const double* rho, dou
   const size_t bt = pad(sizeof(double2) * (size_t)g.nx) + pad(sizeof(double2) * (size_t)g.ny);
   const size_t bytes = (planes ? 3 : 2) * bv + bc + bt + pad(sizeof(double) * 2 * (size_t)nblocks) + pad(sizeof(State));
   char* buf = nullptr;
-  if (cudaMallocAsync(&buf, bytes, st) != cudaSuccess) {
+  if (ctx_alloc(ctx, &buf, bytes) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "Poisson work vectors");
   }

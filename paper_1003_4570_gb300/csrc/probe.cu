@@ -36,7 +36,7 @@ extern "C" omen_status omen_probe_fp64_rate(omen_ctx* ctx, double* tflops) {
   const int blocks = sms * std::max(1, per_sm);
   const int iters = 4096;
   double* out = nullptr;
-  if (cudaMallocAsync(&out, sizeof(double) * blocks * 256, ctx->stream) != cudaSuccess) {
+  if (ctx_alloc(ctx, &out, sizeof(double) * blocks * 256) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "probe buffer");
   }

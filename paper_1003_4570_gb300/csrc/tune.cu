@@ -122,7 +122,7 @@ extern "C" omen_status omen_tune_hx(omen_ctx* ctx, omen_ham* h, int vec_precisio
   OMEN_CUDA(ctx, cudaSetDevice(ctx->device));
   const size_t bytes = vec_elem_bytes(h, vec_precision) * (size_t)h->nrows * nvec;
   Scratch sx{ctx}, sy{ctx};
-  if (cudaMallocAsync(&sx.p, bytes, ctx->stream) != cudaSuccess || cudaMallocAsync(&sy.p, bytes, ctx->stream) != cudaSuccess) {
+  if (ctx_alloc(ctx, &sx.p, bytes) != cudaSuccess || ctx_alloc(ctx, &sy.p, bytes) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "tuner vectors (%zu bytes each)", bytes);
   }
@@ -147,7 +147,7 @@ extern "C" omen_status omen_tune_hx_kbatch(omen_ctx* ctx, omen_ham* h, int nk, i
   OMEN_CUDA(ctx, cudaSetDevice(ctx->device));
   const size_t bytes = vec_elem_bytes(h, prec) * (size_t)h->nrows * nk;
   Scratch sx{ctx}, sy{ctx};
-  if (cudaMallocAsync(&sx.p, bytes, ctx->stream) != cudaSuccess || cudaMallocAsync(&sy.p, bytes, ctx->stream) != cudaSuccess) {
+  if (ctx_alloc(ctx, &sx.p, bytes) != cudaSuccess || ctx_alloc(ctx, &sy.p, bytes) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "tuner vectors (%zu bytes each)", bytes);
   }

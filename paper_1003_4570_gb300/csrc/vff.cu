@@ -502,7 +502,7 @@ extern "C" omen_status omen_relax_vff(omen_ctx* ctx, const omen_lattice* L, cons
   // line coefficients (4 rows), and the state record
   const size_t bytes = sizeof(double) * (3 * (size_t)n3 + 7 * (size_t)nb) + sizeof(VffState);
   char* buf = nullptr;
-  if (cudaMallocAsync((void**)&buf, bytes, ctx->stream) != cudaSuccess) {
+  if (ctx_alloc(ctx, &buf, bytes) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "VFF work vectors (%zu bytes)", bytes);
   }
