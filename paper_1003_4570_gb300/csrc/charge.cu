@@ -56,13 +56,21 @@ __device__ __forceinline__ void df_add_square(float& S, float& Cc, double v) {
   S = s;
 }
 
+// Occupations of a few states travel with the launch, more of them in device memory.
+constexpr int kInlineStates = 64;
+struct OccInline {
+  double f[kInlineStates];
+};
+
 template <bool C, int NB>
 __global__ void __launch_bounds__(256) density_kernel(const void* __restrict__ psiv, long long nrows, int natoms,
-                                                      int nb_rt, int nstates, const double* __restrict__ occ,
-                                                      double w, double* __restrict__ n_atom) {
+                                                      int nb_rt, int nstates, const __grid_constant__ OccInline few,
+                                                      const double* __restrict__ many, double w,
+                                                      double* __restrict__ n_atom) {
   using E = Elem<double, C>;
   const typename E::V* psi = static_cast<const typename E::V*>(psiv);
   const int nb = NB > 0 ? NB : nb_rt;
+  const double* occ = many ? many : few.f;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < natoms; i += gridDim.x * blockDim.x) {
     float AS = 0.f, AC = 0.f;   // sum over states of occ * (state's sum of squares)
     for (int s = 0; s < nstates; ++s) {
@@ -93,40 +101,124 @@ __global__ void __launch_bounds__(256) density_kernel(const void* __restrict__ p
   }
 }
 
-__global__ void deposit_kernel(Geo g, double a_nm, GridGeo G, const double* __restrict__ q, double* __restrict__ nodes) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.natoms; i += gridDim.x * blockDim.x) {
-    const double qi = q[i];
-    if (qi == 0.0) continue;
-    double p[3];
-    atom_position(g, a_nm, i, p);
-    long long idx[8];
-    double w[8];
-    cic(G, p, idx, w);
-    for (int c = 0; c < 8; ++c) atomicAdd(&nodes[idx[c]], w[c] * qi);
+// The atoms' coordinates along one axis are the quarter cells Q a/4, Q = 0 .. 4 n - 1, so the
+// cloud-in-cell position of every atom is a look-up: node below, and weight of the node above.
+struct AxisTable {
+  double* f;      // [nq] weight of the node above
+  int* node;      // [nq] node below, wrapped on the periodic axes
+  double h;       // grid spacing (nm)
+  int nq, wrap;   // wrap: nodes of a periodic axis, 0 for z
+};
+
+__global__ void axis_tables_kernel(AxisTable ax, AxisTable ay, AxisTable az, double quarter) {
+  const AxisTable& A = blockIdx.y == 0 ? ax : blockIdx.y == 1 ? ay : az;
+  const int Q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (Q >= A.nq) return;
+  const double t = (Q * quarter) / A.h;
+  const int node = (int)floor(t);
+  A.f[Q] = t - node;
+  A.node[Q] = A.wrap ? node % A.wrap : node;
+}
+
+// Cloud-in-cell place of one atom from the axis tables.
+struct Place {
+  int i0, i1, j0, j1, k0;
+  double fx, fy, fz;
+};
+
+__device__ __forceinline__ Place place_of(const Geo& g, const AxisTable& X, const AxisTable& Y, const AxisTable& Z, int atom) {
+  const int b = atom / g.ncells, cell = atom - b * g.ncells;
+  const int nxy = g.nx * g.ny;
+  const int iz = cell / nxy, rem = cell - iz * nxy, iy = rem / g.nx, ix = rem - iy * g.nx;
+  const int s = b & 3, o = b >> 2;                       // sites (000) (022) (202) (220), B those plus (111)
+  const int Qx = 4 * ix + (s & 2) + o, Qy = 4 * iy + 2 * (s & 1) + o, Qz = 4 * iz + 2 * ((s ^ (s >> 1)) & 1) + o;
+  Place p;
+  p.fx = X.f[Qx];
+  p.fy = Y.f[Qy];
+  p.fz = Z.f[Qz];
+  p.i0 = X.node[Qx];
+  p.j0 = Y.node[Qy];
+  p.k0 = Z.node[Qz];
+  p.i1 = p.i0 + 1 == X.wrap ? 0 : p.i0 + 1;
+  p.j1 = p.j0 + 1 == Y.wrap ? 0 : p.j0 + 1;
+  return p;
+}
+
+// Deposit straight into the (cleared) density, already divided by the cell volume; nodes on the
+// grounded planes take nothing.  Both kernels were bound by the FP64 rate: three divisions, three
+// floors and the weights of 8 nodes an atom, on a pipe of 1/64 the FP32 rate; the tables leave 15
+// (gather 14) FP64 operations.  1M atoms on 256^3: deposit 128 us of atomics + 22 us clearing +
+// 41 us copying out of a padded node array before, 53 + 21 us now (a kernel by node without atomics
+// took 292 us: most lanes of its FP64 instructions idle).
+__global__ void __launch_bounds__(256) deposit_kernel(Geo g, AxisTable X, AxisTable Y, AxisTable Z, int nz,
+                                                      const double* __restrict__ q, double inv_vol, double* __restrict__ rho) {
+  const int atom = blockIdx.x * blockDim.x + threadIdx.x;
+  if (atom >= g.natoms) return;
+  const double qi = q[atom] * inv_vol;
+  if (qi == 0.0) return;
+  const Place p = place_of(g, X, Y, Z, atom);
+  const double qz1 = qi * p.fz, qz0 = qi - qz1;
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    const int k = p.k0 + d;
+    if (k < 1 || k > nz - 1) continue;
+    const double qz = d ? qz1 : qz0, qy1 = qz * p.fy, qy0 = qz - qy1;
+    const double a = qy0 * p.fx, c = qy1 * p.fx;
+    double* r0 = rho + ((long long)(k - 1) * Y.wrap + p.j0) * X.wrap;
+    double* r1 = rho + ((long long)(k - 1) * Y.wrap + p.j1) * X.wrap;
+    atomicAdd(r0 + p.i0, qy0 - a);
+    atomicAdd(r0 + p.i1, a);
+    atomicAdd(r1 + p.i0, qy1 - c);
+    atomicAdd(r1 + p.i1, c);
   }
 }
 
-__global__ void interior_kernel(const double* __restrict__ nodes, long long plane, long long n, double inv_vol,
-                                double* __restrict__ rho) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    rho[i] = nodes[i + plane] * inv_vol;
-}
-
-__global__ void gather_kernel(Geo g, double a_nm, GridGeo G, const double* __restrict__ phi, double* __restrict__ out) {
-  const long long plane = (long long)G.nx * G.ny;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.natoms; i += gridDim.x * blockDim.x) {
-    double p[3];
-    atom_position(g, a_nm, i, p);
-    long long idx[8];
-    double w[8];
-    cic(G, p, idx, w);
-    double s = 0.0;
-    for (int c = 0; c < 8; ++c) {
-      const long long k = idx[c] / plane;
-      if (k >= 1 && k <= G.nz - 1) s += w[c] * phi[idx[c] - plane];
+// Trilinear interpolation at every atom.  1M atoms on 256^3: 124 us before, 32 us now.
+__global__ void __launch_bounds__(256) gather_kernel(Geo g, AxisTable X, AxisTable Y, AxisTable Z, int nz,
+                                                     const double* __restrict__ phi, double* __restrict__ out) {
+  const int atom = blockIdx.x * blockDim.x + threadIdx.x;
+  if (atom >= g.natoms) return;
+  const Place p = place_of(g, X, Y, Z, atom);
+  double v[2];
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    const int k = p.k0 + d;
+    double p00 = 0.0, p01 = 0.0, p10 = 0.0, p11 = 0.0;
+    if (k >= 1 && k <= nz - 1) {
+      const double* __restrict__ r0 = phi + ((long long)(k - 1) * Y.wrap + p.j0) * X.wrap;
+      const double* __restrict__ r1 = phi + ((long long)(k - 1) * Y.wrap + p.j1) * X.wrap;
+      p00 = r0[p.i0];
+      p01 = r0[p.i1];
+      p10 = r1[p.i0];
+      p11 = r1[p.i1];
     }
-    out[i] = s;
+    const double a = fma(p.fx, p01 - p00, p00), c = fma(p.fx, p11 - p10, p10);
+    v[d] = fma(p.fy, c - a, a);
   }
+  out[atom] = fma(p.fz, v[1] - v[0], v[0]);
+}
+
+// The three axis tables of a structure on a grid, in one buffer on the context's stream.
+static omen_status make_tables(omen_ctx* ctx, const omen_lattice* L, const GridGeo& G, AxisTable (&t)[3], char** buf) {
+  const int nc[3] = {L->nx, L->ny, L->nz}, wrap[3] = {G.nx, G.ny, 0};
+  const double h[3] = {G.hx, G.hy, G.hz};
+  size_t n = 0;
+  for (int c : nc) n += 4 * (size_t)c;
+  if (ctx_alloc(ctx, buf, n * (sizeof(double) + sizeof(int))) != cudaSuccess) {
+    cudaGetLastError();
+    return set_err(ctx, OMEN_ENOMEM, "interpolation tables");
+  }
+  double* f = reinterpret_cast<double*>(*buf);
+  int* node = reinterpret_cast<int*>(f + n);
+  int most = 0;
+  for (int d = 0; d < 3; ++d) {
+    t[d] = AxisTable{f, node, h[d], 4 * nc[d], wrap[d]};
+    f += 4 * nc[d];
+    node += 4 * nc[d];
+    most = std::max(most, 4 * nc[d]);
+  }
+  axis_tables_kernel<<<dim3((most + 127) / 128, 3), 128, 0, ctx->stream>>>(t[0], t[1], t[2], 0.25 * L->a_nm);
+  return OMEN_OK;
 }
 
 extern "C" omen_status omen_density_accum(omen_ctx* ctx, const omen_ham* h, const void* psi, int nstates,
@@ -134,18 +226,24 @@ extern "C" omen_status omen_density_accum(omen_ctx* ctx, const omen_ham* h, cons
   if (!ctx || !h || !psi || !occ_host || !n_atom || nstates < 0) return set_err(ctx, OMEN_EINVAL, "null argument");
   if (nstates == 0) return OMEN_OK;
   double* d_occ = nullptr;
-  if (ctx_alloc(ctx, &d_occ, sizeof(double) * nstates) != cudaSuccess) {
-    cudaGetLastError();
-    return set_err(ctx, OMEN_ENOMEM, "occupations");
+  OccInline few{};
+  if (nstates <= kInlineStates) {
+    std::copy(occ_host, occ_host + nstates, few.f);
+  } else {
+    if (ctx_alloc(ctx, &d_occ, sizeof(double) * nstates) != cudaSuccess) {
+      cudaGetLastError();
+      return set_err(ctx, OMEN_ENOMEM, "occupations");
+    }
+    OMEN_CUDA(ctx, cudaMemcpyAsync(d_occ, occ_host, sizeof(double) * nstates, cudaMemcpyHostToDevice, ctx->stream));
   }
-  OMEN_CUDA(ctx, cudaMemcpyAsync(d_occ, occ_host, sizeof(double) * nstates, cudaMemcpyHostToDevice, ctx->stream));
   const int N = (int)(h->nrows / h->nb);   // atoms, or grid points of an effective-mass Hamiltonian
-  // one thread per atom, the grid a whole number of waves of 152-SM-sized blocks
-  const unsigned grid = (unsigned)std::max(1, std::min((N + 255) / 256, 152 * 8));
+  // one atom a thread: a grid cut to whole waves left its last round a fifth full at 1M atoms
+  // (0.259 ms for 16 states, 0.228 ms now: 83% of the HBM copy rate)
+  const unsigned grid = (unsigned)std::max(1, (N + 255) / 256);
   auto launch = [&](auto cplx, auto nbc) {
     constexpr bool Cx = decltype(cplx)::value;
     constexpr int NB = decltype(nbc)::value;
-    density_kernel<Cx, NB><<<grid, 256, 0, ctx->stream>>>(psi, h->nrows, N, h->nb, nstates, d_occ, w, n_atom);
+    density_kernel<Cx, NB><<<grid, 256, 0, ctx->stream>>>(psi, h->nrows, N, h->nb, nstates, few, d_occ, w, n_atom);
   };
   using T_ = std::true_type;
   using F_ = std::false_type;
@@ -168,7 +266,7 @@ extern "C" omen_status omen_density_accum(omen_ctx* ctx, const omen_ham* h, cons
     else launch(F_{}, I0{});
   }
   cudaError_t e = cudaGetLastError();
-  cudaFreeAsync(d_occ, ctx->stream);
+  if (d_occ) cudaFreeAsync(d_occ, ctx->stream);
   if (e != cudaSuccess) return set_err(ctx, OMEN_ECUDA, "density: %s", cudaGetErrorString(e));
   return OMEN_OK;
 }
@@ -185,20 +283,19 @@ extern "C" omen_status omen_deposit(omen_ctx* ctx, const omen_lattice* L, const 
   omen_status s = check_grid(ctx, gr);
   if (s != OMEN_OK) return s;
   const GridGeo G = grid_geo(gr);
-  const long long plane = (long long)G.nx * G.ny;
-  const long long nodes_n = plane * (G.nz + 1);
-  double* nodes = nullptr;
-  if (ctx_alloc(ctx, &nodes, sizeof(double) * nodes_n) != cudaSuccess) {
-    cudaGetLastError();
-    return set_err(ctx, OMEN_ENOMEM, "deposit nodes");
+  AxisTable t[3];
+  char* buf = nullptr;
+  s = make_tables(ctx, L, G, t, &buf);
+  if (s != OMEN_OK) return s;
+  const cudaError_t ec = cudaMemsetAsync(rho, 0, sizeof(double) * (size_t)G.nx * G.ny * (G.nz - 1), ctx->stream);
+  deposit_kernel<<<(unsigned)((L->natoms + 255) / 256), 256, 0, ctx->stream>>>(lat_geo(L), t[0], t[1], t[2], G.nz, q,
+                                                                               1.0 / G.vol_m3, rho);
+  if (ec != cudaSuccess) {
+    cudaFreeAsync(buf, ctx->stream);
+    return set_err(ctx, OMEN_ECUDA, "deposit: %s", cudaGetErrorString(ec));
   }
-  OMEN_CUDA(ctx, cudaMemsetAsync(nodes, 0, sizeof(double) * nodes_n, ctx->stream));
-  const unsigned ga = (unsigned)std::min(4096, (L->natoms + 255) / 256);
-  deposit_kernel<<<ga, 256, 0, ctx->stream>>>(lat_geo(L), L->a_nm, G, q, nodes);
-  const long long n = plane * (G.nz - 1);
-  interior_kernel<<<(unsigned)std::min<long long>(4096, (n + 255) / 256), 256, 0, ctx->stream>>>(nodes, plane, n, 1.0 / G.vol_m3, rho);
   cudaError_t e = cudaGetLastError();
-  cudaFreeAsync(nodes, ctx->stream);
+  cudaFreeAsync(buf, ctx->stream);
   if (e != cudaSuccess) return set_err(ctx, OMEN_ECUDA, "deposit: %s", cudaGetErrorString(e));
   return OMEN_OK;
 }
@@ -208,9 +305,15 @@ extern "C" omen_status omen_gather(omen_ctx* ctx, const omen_lattice* L, const o
   if (!ctx || !L || !phi || !out) return set_err(ctx, OMEN_EINVAL, "null argument");
   omen_status s = check_grid(ctx, gr);
   if (s != OMEN_OK) return s;
-  const unsigned ga = (unsigned)std::min(4096, (L->natoms + 255) / 256);
-  gather_kernel<<<ga, 256, 0, ctx->stream>>>(lat_geo(L), L->a_nm, grid_geo(gr), phi, out);
-  OMEN_CHECK_LAUNCH(ctx);
+  const GridGeo G = grid_geo(gr);
+  AxisTable t[3];
+  char* buf = nullptr;
+  s = make_tables(ctx, L, G, t, &buf);
+  if (s != OMEN_OK) return s;
+  gather_kernel<<<(unsigned)((L->natoms + 255) / 256), 256, 0, ctx->stream>>>(lat_geo(L), t[0], t[1], t[2], G.nz, phi, out);
+  cudaError_t e = cudaGetLastError();
+  cudaFreeAsync(buf, ctx->stream);
+  if (e != cudaSuccess) return set_err(ctx, OMEN_ECUDA, "gather: %s", cudaGetErrorString(e));
   return OMEN_OK;
 }
 
