@@ -186,7 +186,8 @@ typedef struct {
 } omen_vff_info;
 
 /* Energy (E_host, may be NULL) and forces -dE/du (force_dev [3][natoms], may be NULL) at
- * displacements u_dev; F_host [9] row-major, NULL = identity.  Synchronous.  EINVAL for bad
+ * displacements u_dev; F_host [9] row-major, NULL = identity.  Forces allocate 12 doubles per atom
+ * on ctx's stream.  Synchronous.  EINVAL for bad
  * parameters (nspecies, a_nm <= 0, negative constants). */
 omen_status omen_vff_energy_forces(omen_ctx* ctx, const omen_lattice* lat, const omen_vff_params* p,
                                    const double* F_host, const double* u_dev, double* E_host, double* force_dev);
@@ -196,7 +197,7 @@ omen_status omen_vff_energy_forces(omen_ctx* ctx, const omen_lattice* lat, const
  * term is the square of a quadratic in the step, so the energy is a quartic whose minimum is
  * found from its derivative's coefficients (accumulated term by term, no energy differences).
  * strain_dev (or NULL) receives |r_b|/d_b - 1 per bond slot ([16*ncells], absent bonds 0), the
- * input of omen_lattice_set_strain.  Allocates its work vectors (9 doubles per atom) on ctx's
+ * input of omen_lattice_set_strain.  Allocates its work vectors (21 doubles per atom) on ctx's
  * stream; synchronous.  ENOCONV (u and strain still written) at max_iter, ENUMERIC on a
  * non-finite force. */
 omen_status omen_relax_vff(omen_ctx* ctx, const omen_lattice* lat, const omen_vff_params* p, const double* F_host,

@@ -13,10 +13,19 @@
 // ideal A->B bond vector of direction k is dir_k a/4, so r = +-F dir_k a/4 + u_n - u_i needs no
 // stored positions and no neighbour list (neighbours come from the cell index, as in H·X).
 //
-// Kernels: per-atom gradient by gathering every term that touches the atom (own bonds, own bond
-// angles, and the angles at each neighbour that use the bond back to it), so no atomics and a
-// bit-reproducible result; per-atom energy; and, for the line search of the nonlinear conjugate-
-// gradient relaxation, the coefficients of the energy along a search direction.  Every term is
+// Kernels.  Every term belongs to a vertex: the angles between the four bonds r_p of an atom, and
+// half of each bond's stretch, so with G_pq = r_p.r_q
+//   E_i = sum_p k_p (G_pp - d_p^2)^2 + sum_{p<q} k_pq (G_pq + d_p d_q / 3)^2,
+//   f_p = dE_i/dr_p = sum_q M_pq r_q,  M_pp = 4 k_p (G_pp - d_p^2),  M_pq = 2 k_pq (G_pq + d_p d_q / 3),
+// and the gradient of atom j along its bonds k to atoms n_k is -sum_k (f_k(j) - f_k(n_k)).  One kernel
+// writes the 12 numbers f of every atom, a second gathers them (no atomics, a bit-reproducible
+// result): 150 FP64 operations an atom, where gathering every term that touches an atom took some
+// 900, 40 divisions by natural lengths among them; the constants of every species triple now come
+// from a table in shared memory.  All of it is bound by the FP64 rate.  1M atoms, one iteration: gradient
+// 1.46 ms before, 0.24 + 0.09 ms now; line coefficients 0.73 -> 0.47 ms; step 0.104 -> 0.008 ms (every
+// block bisected the quartic); direction 0.032 -> 0.015 ms; 100 iterations 237 -> 84 ms.
+// For the line search of the nonlinear conjugate-gradient relaxation, a kernel accumulates the
+// coefficients of the energy along a search direction.  Every term is
 // the square of a quadratic polynomial in the step t (r is affine in t), so E(u + t p) is a
 // quartic whose derivative c1 + 2 c2 t + 3 c3 t^2 + 4 c4 t^3 is minimised exactly; c1 = g.p is
 // accumulated term by term, so no energy difference (and no cancellation) enters the step.
@@ -24,6 +33,7 @@
 #include <chrono>
 #include <cmath>
 
+#include "neighbours.cuh"
 #include "omen_internal.h"
 #include "sk_device.cuh"
 
@@ -31,47 +41,45 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// Constants of a vertex of species v: bond to species p {k_p, d_p^2}, angle between bonds to p and
+// q {k_pq, d_p d_q / 3}.
+struct VffTable {
+  double2 bond[4][4];
+  double2 angle[4][4][4];
+};
+
 struct VffArgs {
   Geo g;
-  NeighbourTables nt;
   const uint8_t* species;
   double fd[4][3];            // F dir_k a/4: deformed ideal A->B vector of direction k (nm)
   double dnat[4];             // natural bond length sqrt(3)/4 a per species (nm)
-  double alpha[4], beta[4];   // eV/nm^2
+  VffTable t;
 };
 
-// The (up to four) bonds of one atom as vectors leaving it.
-struct Bonds4 {
-  int nb[4];                  // neighbour atom, -1 where the bond leaves a hard wall
-  double r[4][3];
-  double d[4], al[4], be[4];  // natural length, stretching and bending constant of each bond
+// One atom's site, species and bonds (neighbour atoms; -1 where a bond leaves a hard wall).
+struct Vertex {
+  int sp;
+  int nb[4];
+  int sn[4];
+  double sg;                  // A atoms sit at the tail of dir_k, B atoms at its head
 };
 
-__device__ __forceinline__ void atom_cell(const Geo& g, int atom, int& b, int& cell, int& ix, int& iy, int& iz) {
-  b = atom / g.ncells;
-  cell = atom - b * g.ncells;
-  ix = cell % g.nx;
-  const int t = cell / g.nx;
-  iy = t % g.ny;
-  iz = t / g.ny;
-}
-
-// Neighbour of `atom` along direction k (-1 if the bond leaves a hard wall).
-__device__ __forceinline__ int neighbour(const VffArgs& a, int atom, int k) {
-  int b, cell, ix, iy, iz;
-  atom_cell(a.g, atom, b, cell, ix, iy, iz);
-  int ox, oy, oz, site2;
-  if (b < 4) {
-    ox = a.nt.a_to_b_off[b][k][0]; oy = a.nt.a_to_b_off[b][k][1]; oz = a.nt.a_to_b_off[b][k][2];
-    site2 = a.nt.a_to_b_site[b][k];
-  } else {
-    const int s = b - 4;
-    ox = a.nt.b_to_a_off[s][k][0]; oy = a.nt.b_to_a_off[s][k][1]; oz = a.nt.b_to_a_off[s][k][2];
-    site2 = a.nt.b_to_a_site[s][k];
+__device__ __forceinline__ Vertex vertex_of(const VffArgs& a, int atom) {
+  const Geo& g = a.g;
+  const int b = atom / g.ncells, cell = atom - b * g.ncells;
+  const int nxy = g.nx * g.ny;
+  const int iz = cell / nxy, rem = cell - iz * nxy, iy = rem / g.nx, ix = rem - iy * g.nx;
+  const Steps steps = steps_of(g, b, ix, iy, iz);
+  Vertex v;
+  v.sp = a.species[atom];
+  v.sg = b < 4 ? 1.0 : -1.0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const Neighbour n = neighbour_of(g, steps, b, k, cell);
+    v.nb[k] = n.ok ? n.atom : -1;
+    v.sn[k] = n.ok ? a.species[n.atom] : 0;
   }
-  int cell2, wrap[3];
-  if (!shift_cell(a.g, ix, iy, iz, ox, oy, oz, cell2, wrap)) return -1;
-  return site2 * a.g.ncells + cell2;
+  return v;
 }
 
 __device__ __forceinline__ void load3(const double* __restrict__ v, long long n, int i, double out[3]) {
@@ -81,33 +89,50 @@ __device__ __forceinline__ void load3(const double* __restrict__ v, long long n,
 }
 
 __device__ __forceinline__ double dot3(const double x[3], const double y[3]) {
-  return x[0] * y[0] + x[1] * y[1] + x[2] * y[2];
+  return fma(x[2], y[2], fma(x[1], y[1], x[0] * y[0]));
 }
 
-// Bonds of `atom` at displacements u ([3][natoms]).
-__device__ __forceinline__ void bonds_of(const VffArgs& a, const double* __restrict__ u, int atom, Bonds4& B) {
+// Bond vectors of a vertex at displacements u ([3][natoms]); zero for absent bonds.
+__device__ __forceinline__ void bond_vectors(const VffArgs& a, const Vertex& v, const double* __restrict__ u, int atom,
+                                             double (&r)[4][3]) {
   const long long N = a.g.natoms;
-  const double sg = atom < 4 * a.g.ncells ? 1.0 : -1.0;   // A atoms sit at the tail of dir_k
-  const int sp = a.species[atom];
   double ui[3];
   load3(u, N, atom, ui);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const int n = neighbour(a, atom, k);
-    B.nb[k] = n;
-    if (n < 0) continue;
-    double un[3];
-    load3(u, N, n, un);
+    double un[3] = {0.0, 0.0, 0.0};
+    if (v.nb[k] >= 0) load3(u, N, v.nb[k], un);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) B.r[k][c] = sg * a.fd[k][c] + un[c] - ui[c];
-    const int sn = a.species[n];
-    B.d[k] = 0.5 * (a.dnat[sp] + a.dnat[sn]);
-    B.al[k] = 0.5 * (a.alpha[sp] + a.alpha[sn]);
-    B.be[k] = 0.5 * (a.beta[sp] + a.beta[sn]);
+    for (int c = 0; c < 3; ++c) r[k][c] = v.nb[k] >= 0 ? (v.sg * a.fd[k][c] - ui[c]) + un[c] : 0.0;
   }
 }
 
-// Deterministic block sum of NV values per thread into partial[v * nblocks + block]; with
+// Constants of the pair of bonds (p, q) of a vertex; k = 0 where one of them is absent.
+__device__ __forceinline__ double2 pair_of(const VffTable& t, const Vertex& v, int p, int q) {
+  double2 k = p == q ? t.bond[v.sp][v.sn[p]] : t.angle[v.sp][v.sn[p]][v.sn[q]];
+  if (v.nb[p] < 0 || v.nb[q] < 0) k.x = 0.0;
+  return k;
+}
+
+__device__ __forceinline__ void stage_table(const VffTable& t, VffTable& sm) {
+  const double* src = reinterpret_cast<const double*>(&t);
+  double* dst = reinterpret_cast<double*>(&sm);
+  for (int i = threadIdx.x; i < (int)(sizeof(VffTable) / sizeof(double)); i += blockDim.x) dst[i] = src[i];
+  __syncthreads();
+}
+
+// Relaxation state on the device (one small record).
+struct VffState {
+  double t;          // last step length
+  double c1;         // last directional derivative g.p
+  double gg;         // g.g of the current gradient
+  double beta;       // of the next direction
+  double gmax;       // max |g_c| of the current gradient
+  int restart;       // the last direction was not a descent direction: next direction is -g
+  unsigned arrived;  // blocks of the running reduction that have left their sums
+};
+
+// Deterministic block sums of NV values per thread into partial[v * nblocks + block]; with
 // MAX_LAST the last value is reduced by max instead of sum.
 template <int NV, bool MAX_LAST>
 __device__ __forceinline__ void block_reduce(double (&v)[NV], double* __restrict__ partial) {
@@ -132,197 +157,149 @@ __device__ __forceinline__ void block_reduce(double (&v)[NV], double* __restrict
   }
 }
 
-// dE/du for every atom; partials: [0] g.g, [1] g.g_prev (0 if g_prev is null), [2] max |g_c|.
-__global__ void __launch_bounds__(kThreads) vff_grad_kernel(VffArgs a, const double* __restrict__ u,
-                                                            double* __restrict__ g, const double* __restrict__ g_prev,
-                                                            double* __restrict__ partial) {
+// The last block to leave its partials reduces all of them in block order: v valid in thread 0 of
+// that block, which alone gets true.
+template <int NV, bool MAX_LAST>
+__device__ __forceinline__ bool grid_reduce(double (&v)[NV], double* partial, VffState* st) {
+  __shared__ bool last;
+  block_reduce<NV, MAX_LAST>(v, partial);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&st->arrived, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  __shared__ double sm[NV][kThreads / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    const bool mx = MAX_LAST && q == NV - 1;
+    double x = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += kThreads) {
+      const double y = __ldcg(partial + (size_t)q * gridDim.x + i);
+      x = mx ? fmax(x, y) : x + y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double y = __shfl_down_sync(0xffffffffu, x, o);
+      x = mx ? fmax(x, y) : x + y;
+    }
+    if (lane == 0) sm[q][w] = x;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return false;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    v[q] = sm[q][0];
+    for (int i = 1; i < kThreads / 32; ++i) v[q] = (MAX_LAST && q == NV - 1) ? fmax(v[q], sm[q][i]) : v[q] + sm[q][i];
+  }
+  st->arrived = 0;
+  return true;
+}
+
+// f_k = dE_i/dr_k of every atom: f[(3 k + c) natoms + atom].
+__global__ void __launch_bounds__(kThreads) vff_vertex_kernel(const __grid_constant__ VffArgs a, const double* __restrict__ u,
+                                                              double* __restrict__ f) {
+  __shared__ VffTable t;
+  stage_table(a.t, t);
+  const long long N = a.g.natoms;
+  const int atom = blockIdx.x * blockDim.x + threadIdx.x;
+  if (atom >= N) return;
+  const Vertex v = vertex_of(a, atom);
+  double r[4][3], fk[4][3];
+  bond_vectors(a, v, u, atom, r);
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const double2 k = pair_of(t, v, p, p);
+    const double m = 4.0 * k.x * (dot3(r[p], r[p]) - k.y);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) fk[p][c] = m * r[p][c];
+  }
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = p + 1; q < 4; ++q) {
+      const double2 k = pair_of(t, v, p, q);
+      const double m = 2.0 * k.x * (dot3(r[p], r[q]) + k.y);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        fk[p][c] = fma(m, r[q][c], fk[p][c]);
+        fk[q][c] = fma(m, r[p][c], fk[q][c]);
+      }
+    }
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f[(3 * k + c) * N + atom] = fk[k][c];
+}
+
+// Gradient (times `sign`) from the vertices' f.  With a state: g.g, g.g_prev (0 if g_prev is null)
+// and max |g_c| over the structure, and from them beta of the next direction p = -g + beta p
+// (Polak–Ribière, clipped at 0; 0 on the first iteration or after a restart).
+__global__ void __launch_bounds__(kThreads) vff_gather_kernel(const __grid_constant__ VffArgs a, const double* __restrict__ f,
+                                                              double* __restrict__ g, const double* __restrict__ g_prev,
+                                                              double sign, double* partial, VffState* st) {
   const long long N = a.g.natoms;
   double acc[3] = {0.0, 0.0, 0.0};
   for (int atom = blockIdx.x * blockDim.x + threadIdx.x; atom < N; atom += gridDim.x * blockDim.x) {
-    Bonds4 B;
-    bonds_of(a, u, atom, B);
+    const Vertex v = vertex_of(a, atom);
     double gi[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      if (B.nb[k] < 0) continue;
-      // bond stretch: dE/dr = 3 alpha / (2 d^2) (r.r - d^2) r, and r = x_n - x_i
-      const double d2 = B.d[k] * B.d[k];
-      const double cst = 1.5 * B.al[k] / d2 * (dot3(B.r[k], B.r[k]) - d2);
+      if (v.nb[k] < 0) continue;                     // f_k of an absent bond is zero
+      double own[3], back[3];
+      load3(f + 3 * k * N, N, atom, own);
+      load3(f + 3 * k * N, N, v.nb[k], back);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) gi[c] -= cst * B.r[k][c];
-    }
-    // bond angles with this atom at the vertex: d(r_p.r_q)/dx_i = -(r_p + r_q)
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = p + 1; q < 4; ++q) {
-        if (B.nb[p] < 0 || B.nb[q] < 0) continue;
-        const double dd = B.d[p] * B.d[q];
-        const double w = 0.75 * 0.5 * (B.be[p] + B.be[q]) / dd * (dot3(B.r[p], B.r[q]) + dd / 3.0);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) gi[c] -= w * (B.r[p][c] + B.r[q][c]);
-      }
-    // bond angles at each neighbour j that use the bond j -> i: d(r_ji.r_jm)/dx_i = r_jm
-#pragma unroll 1
-    for (int k = 0; k < 4; ++k) {
-      const int j = B.nb[k];
-      if (j < 0) continue;
-      const double sj = j < 4 * a.g.ncells ? 1.0 : -1.0;
-      const int spj = a.species[j];
-      double uj[3], rji[3];
-      load3(u, N, j, uj);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) rji[c] = -B.r[k][c];
-#pragma unroll 1
-      for (int k2 = 0; k2 < 4; ++k2) {
-        if (k2 == k) continue;                       // j's bond along k leads back to this atom
-        const int m = neighbour(a, j, k2);
-        if (m < 0) continue;
-        double um[3], rjm[3];
-        load3(u, N, m, um);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) rjm[c] = sj * a.fd[k2][c] + um[c] - uj[c];
-        const int spm = a.species[m];
-        const double djm = 0.5 * (a.dnat[spj] + a.dnat[spm]);
-        const double bjm = 0.5 * (a.beta[spj] + a.beta[spm]);
-        const double dd = B.d[k] * djm;
-        const double w = 0.75 * 0.5 * (B.be[k] + bjm) / dd * (dot3(rji, rjm) + dd / 3.0);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) gi[c] += w * rjm[c];
-      }
+      for (int c = 0; c < 3; ++c) gi[c] += back[c] - own[c];
     }
     double gp[3] = {0.0, 0.0, 0.0};
     if (g_prev) load3(g_prev, N, atom, gp);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      g[c * N + atom] = gi[c];
-      acc[0] += gi[c] * gi[c];
-      acc[1] += gi[c] * gp[c];
+      g[c * N + atom] = sign * gi[c];
+      acc[0] = fma(gi[c], gi[c], acc[0]);
+      acc[1] = fma(gi[c], gp[c], acc[1]);
       acc[2] = fmax(acc[2], fabs(gi[c]));
     }
   }
-  block_reduce<3, true>(acc, partial);
+  if (!st) return;
+  if (grid_reduce<3, true>(acc, partial, st)) {
+    double beta = 0.0;
+    if (g_prev && !st->restart && st->gg > 0.0) beta = fmax(0.0, (acc[0] - acc[1]) / st->gg);
+    st->beta = beta;
+    st->gg = acc[0];
+    // fmax drops a NaN: the sum of squares carries it
+    st->gmax = acc[0] == acc[0] ? acc[2] : acc[0];
+  }
 }
 
-// Energy: each bond counted at its A atom, each angle at its vertex.
-__global__ void __launch_bounds__(kThreads) vff_energy_kernel(VffArgs a, const double* __restrict__ u,
+// Energy of every vertex.
+__global__ void __launch_bounds__(kThreads) vff_energy_kernel(const __grid_constant__ VffArgs a, const double* __restrict__ u,
                                                               double* __restrict__ partial) {
+  __shared__ VffTable t;
+  stage_table(a.t, t);
   const long long N = a.g.natoms;
   double acc[1] = {0.0};
   for (int atom = blockIdx.x * blockDim.x + threadIdx.x; atom < N; atom += gridDim.x * blockDim.x) {
-    Bonds4 B;
-    bonds_of(a, u, atom, B);
-    const bool is_a = atom < 4 * a.g.ncells;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (B.nb[k] < 0 || !is_a) continue;
-      const double d2 = B.d[k] * B.d[k];
-      const double q = dot3(B.r[k], B.r[k]) - d2;
-      acc[0] += 0.375 * B.al[k] / d2 * q * q;
-    }
+    const Vertex v = vertex_of(a, atom);
+    double r[4][3];
+    bond_vectors(a, v, u, atom, r);
 #pragma unroll
     for (int p = 0; p < 4; ++p)
 #pragma unroll
-      for (int q = p + 1; q < 4; ++q) {
-        if (B.nb[p] < 0 || B.nb[q] < 0) continue;
-        const double dd = B.d[p] * B.d[q];
-        const double c = dot3(B.r[p], B.r[q]) + dd / 3.0;
-        acc[0] += 0.375 * 0.5 * (B.be[p] + B.be[q]) / dd * c * c;
+      for (int q = p; q < 4; ++q) {
+        const double2 k = pair_of(t, v, p, q);
+        const double x = p == q ? dot3(r[p], r[p]) - k.y : dot3(r[p], r[q]) + k.y;
+        acc[0] = fma(k.x * x, x, acc[0]);
       }
   }
   block_reduce<1, false>(acc, partial);
 }
 
-// Coefficients c1..c4 of E(u + t p) - E(u) = c1 t + c2 t^2 + c3 t^3 + c4 t^4.  A term
-// K (q0 + q1 t + q2 t^2)^2 contributes 2K q0 q1, K (q1^2 + 2 q0 q2), 2K q1 q2, K q2^2.
-__global__ void __launch_bounds__(kThreads) vff_line_kernel(VffArgs a, const double* __restrict__ u,
-                                                            const double* __restrict__ p, double* __restrict__ partial) {
-  const long long N = a.g.natoms;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int atom = blockIdx.x * blockDim.x + threadIdx.x; atom < N; atom += gridDim.x * blockDim.x) {
-    Bonds4 B;
-    bonds_of(a, u, atom, B);
-    double s[4][3];                                  // change of each bond vector per unit step
-    double pi[3];
-    load3(p, N, atom, pi);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (B.nb[k] < 0) continue;
-      double pn[3];
-      load3(p, N, B.nb[k], pn);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) s[k][c] = pn[c] - pi[c];
-    }
-    const bool is_a = atom < 4 * a.g.ncells;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (B.nb[k] < 0 || !is_a) continue;
-      const double d2 = B.d[k] * B.d[k];
-      const double K = 0.375 * B.al[k] / d2;
-      const double q0 = dot3(B.r[k], B.r[k]) - d2, q1 = 2.0 * dot3(B.r[k], s[k]), q2 = dot3(s[k], s[k]);
-      acc[0] += 2.0 * K * q0 * q1;
-      acc[1] += K * (q1 * q1 + 2.0 * q0 * q2);
-      acc[2] += 2.0 * K * q1 * q2;
-      acc[3] += K * q2 * q2;
-    }
-#pragma unroll
-    for (int pp = 0; pp < 4; ++pp)
-#pragma unroll
-      for (int q = pp + 1; q < 4; ++q) {
-        if (B.nb[pp] < 0 || B.nb[q] < 0) continue;
-        const double dd = B.d[pp] * B.d[q];
-        const double K = 0.375 * 0.5 * (B.be[pp] + B.be[q]) / dd;
-        const double q0 = dot3(B.r[pp], B.r[q]) + dd / 3.0;
-        const double q1 = dot3(B.r[pp], s[q]) + dot3(s[pp], B.r[q]);
-        const double q2 = dot3(s[pp], s[q]);
-        acc[0] += 2.0 * K * q0 * q1;
-        acc[1] += K * (q1 * q1 + 2.0 * q0 * q2);
-        acc[2] += 2.0 * K * q1 * q2;
-        acc[3] += K * q2 * q2;
-      }
-  }
-  block_reduce<4, false>(acc, partial);
-}
-
-// Relaxation state on the device (one small record).
-struct VffState {
-  double t;          // last step length
-  double c1;         // last directional derivative g.p
-  double gg[2];      // g.g of the current gradient, by iteration parity
-  double gmax;       // max |g_c| of the current gradient
-  int restart;       // the last direction was not a descent direction: next direction is -g
-  int pad;
-};
-
-// Sum of `nb` partials of row q, in a fixed order (every block computes the same value).
-__device__ double sum_partials(const double* __restrict__ part, int q, int nb, double* sm) {
-  double x = 0.0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) x += part[(size_t)q * nb + i];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = x;
-  __syncthreads();
-  double s = 0.0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += sm[i];
-  __syncthreads();
-  return s;
-}
-
-__device__ double max_partials(const double* __restrict__ part, int q, int nb, double* sm) {
-  double x = 0.0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) x = fmax(x, part[(size_t)q * nb + i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_down_sync(0xffffffffu, x, o));
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = x;
-  __syncthreads();
-  double s = 0.0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s = fmax(s, sm[i]);
-  __syncthreads();
-  return s;
-}
-
 // Step length minimising the quartic along the line: the first sign change of its derivative
-// c1 + 2 c2 t + 3 c3 t^2 + 4 c4 t^3 (c1 < 0) bracketed by doubling, then bisected to rounding.
+// c1 + 2 c2 t + 3 c3 t^2 + 4 c4 t^3 (c1 < 0) bracketed by doubling, then Newton's method kept
+// inside the bracket (bisection where it leaves it), to rounding.
 __device__ double quartic_step(double c1, double c2, double c3, double c4) {
   if (!(c1 < 0.0)) return 0.0;
   auto dE = [&](double t) { return c1 + t * (2.0 * c2 + t * (3.0 * c3 + t * 4.0 * c4)); };
@@ -333,56 +310,79 @@ __device__ double quartic_step(double c1, double c2, double c3, double c4) {
     ++n;
   }
   if (!(dE(hi) > 0.0)) return 0.0;                 // no minimum along the line: restart
-  double lo = 0.0;
+  double lo = 0.0, t = n ? 0.5 * hi : hi;
   for (int i = 0; i < 200 && hi - lo > 1e-16 * hi; ++i) {
-    const double m = 0.5 * (lo + hi);
-    if (dE(m) > 0.0) hi = m; else lo = m;
+    const double d = dE(t);
+    if (d > 0.0) hi = t; else lo = t;
+    const double slope = 2.0 * c2 + t * (6.0 * c3 + t * 12.0 * c4);
+    double next = t - d / slope;
+    if (!(next > lo && next < hi)) next = 0.5 * (lo + hi);
+    if (fabs(next - t) <= 1e-16 * t) break;
+    t = next;
   }
-  return 0.5 * (lo + hi);
+  return t;
 }
 
-// u += t p with t from the line coefficients (every block solves the same cubic).
-__global__ void __launch_bounds__(kThreads) vff_step_kernel(double* __restrict__ u, const double* __restrict__ p,
-                                                            long long n3, const double* __restrict__ line_part, int nb,
-                                                            VffState* st) {
-  __shared__ double sm[kThreads / 32];
-  __shared__ double t_sh;
-  const double c1 = sum_partials(line_part, 0, nb, sm);
-  const double c2 = sum_partials(line_part, 1, nb, sm);
-  const double c3 = sum_partials(line_part, 2, nb, sm);
-  const double c4 = sum_partials(line_part, 3, nb, sm);
-  if (threadIdx.x == 0) t_sh = quartic_step(c1, c2, c3, c4);
-  __syncthreads();
-  const double t = t_sh;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    st->t = t;
-    st->c1 = c1;
-    st->restart = t > 0.0 ? 0 : 1;
+// Coefficients c1..c4 of E(u + t p) - E(u) = c1 t + c2 t^2 + c3 t^3 + c4 t^4, and the step they
+// give.  A term K (q0 + q1 t + q2 t^2)^2 contributes 2K q0 q1, K (q1^2 + 2 q0 q2), 2K q1 q2, K q2^2.
+__global__ void __launch_bounds__(kThreads) vff_line_kernel(const __grid_constant__ VffArgs a, const double* __restrict__ u,
+                                                            const double* __restrict__ p, double* partial, VffState* st) {
+  __shared__ VffTable t;
+  stage_table(a.t, t);
+  const long long N = a.g.natoms;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};              // c1 / 2, c2, c3 / 2, c4
+  for (int atom = blockIdx.x * blockDim.x + threadIdx.x; atom < N; atom += gridDim.x * blockDim.x) {
+    const Vertex v = vertex_of(a, atom);
+    double r[4][3], s[4][3], pi[3];                  // bond vectors and their change per unit step
+    bond_vectors(a, v, u, atom, r);
+    load3(p, N, atom, pi);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      double pn[3] = {pi[0], pi[1], pi[2]};
+      if (v.nb[k] >= 0) load3(p, N, v.nb[k], pn);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) s[k][c] = pn[c] - pi[c];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = i; q < 4; ++q) {
+        const double2 k = pair_of(t, v, i, q);
+        const double q0 = i == q ? dot3(r[i], r[i]) - k.y : dot3(r[i], r[q]) + k.y;
+        const double q1 = i == q ? 2.0 * dot3(r[i], s[i])
+                                 : fma(s[i][2], r[q][2], fma(s[i][1], r[q][1], fma(s[i][0], r[q][0], dot3(r[i], s[q]))));
+        const double q2 = dot3(s[i], s[q]);
+        const double k0 = k.x * q0, k1 = k.x * q1;
+        acc[0] = fma(k0, q1, acc[0]);
+        acc[1] = fma(k1, q1, fma(k0 + k0, q2, acc[1]));
+        acc[2] = fma(k1, q2, acc[2]);
+        acc[3] = fma(k.x * q2, q2, acc[3]);
+      }
   }
+  if (grid_reduce<4, false>(acc, partial, st)) {
+    const double c1 = 2.0 * acc[0];
+    const double step = quartic_step(c1, acc[1], 2.0 * acc[2], acc[3]);
+    st->t = step;
+    st->c1 = c1;
+    st->restart = step > 0.0 ? 0 : 1;
+  }
+}
+
+// u += t p with the step of the line kernel.
+__global__ void __launch_bounds__(kThreads) vff_step_kernel(double* __restrict__ u, const double* __restrict__ p,
+                                                            long long n3, const VffState* __restrict__ st) {
+  const double t = st->t;
   if (t == 0.0) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n3; i += (long long)gridDim.x * blockDim.x)
-    u[i] += t * p[i];
+    u[i] = fma(t, p[i], u[i]);
 }
 
-// New direction p = -g + beta p (Polak–Ribière, clipped at 0; beta = 0 on the first iteration or
-// after a restart).  Parity selects which gg slot holds the previous g.g.
+// New direction p = -g + beta p.
 __global__ void __launch_bounds__(kThreads) vff_dir_kernel(const double* __restrict__ g, double* __restrict__ p,
-                                                           long long n3, const double* __restrict__ grad_part, int nb,
-                                                           VffState* st, int first, int parity) {
-  __shared__ double sm[kThreads / 32];
-  const double gg = sum_partials(grad_part, 0, nb, sm);
-  const double gprev = sum_partials(grad_part, 1, nb, sm);
-  const double gmax = max_partials(grad_part, 2, nb, sm);
-  const double gg_old = st->gg[parity];
-  double beta = 0.0;
-  if (!first && !st->restart && gg_old > 0.0) beta = fmax(0.0, (gg - gprev) / gg_old);
-  __syncthreads();                                   // every block has read the state
+                                                           long long n3, const VffState* __restrict__ st, int first) {
+  const double beta = st->beta;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n3; i += (long long)gridDim.x * blockDim.x)
-    p[i] = -g[i] + beta * p[i];
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    st->gg[parity ^ 1] = gg;
-    st->gmax = gmax;
-  }
+    p[i] = first ? -g[i] : fma(beta, p[i], -g[i]);
 }
 
 __global__ void vff_strain_kernel(VffArgs a, const double* __restrict__ u, double* __restrict__ strain) {
@@ -393,8 +393,11 @@ __global__ void vff_strain_kernel(VffArgs a, const double* __restrict__ u, doubl
     const int cell = (int)(sl - (long long)ks * a.g.ncells);
     const int k = ks >> 2, s = ks & 3;
     const int atom = s * a.g.ncells + cell;
-    const int n = neighbour(a, atom, k);
-    if (n < 0) {
+    const int nxy = a.g.nx * a.g.ny;
+    const int iz = cell / nxy, rem = cell - iz * nxy, iy = rem / a.g.nx, ix = rem - iy * a.g.nx;
+    const Neighbour to = neighbour_of(a.g, steps_of(a.g, s, ix, iy, iz), s, k, cell);
+    const int n = to.atom;
+    if (!to.ok) {
       strain[sl] = 0.0;
       continue;
     }
@@ -408,11 +411,6 @@ __global__ void vff_strain_kernel(VffArgs a, const double* __restrict__ u, doubl
   }
 }
 
-__global__ void vff_negate_kernel(double* __restrict__ v, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    v[i] = -v[i];
-}
-
 omen_status make_args(omen_ctx* ctx, const omen_lattice* L, const omen_vff_params* vp, const double* F, VffArgs& a) {
   if (!vp) return set_err(ctx, OMEN_EINVAL, "null VFF parameters");
   if (vp->nspecies < 1 || vp->nspecies > 4) return set_err(ctx, OMEN_EINVAL, "nspecies must be 1..4");
@@ -422,7 +420,6 @@ omen_status make_args(omen_ctx* ctx, const omen_lattice* L, const omen_vff_param
   a.g.nx = L->nx; a.g.ny = L->ny; a.g.nz = L->nz;
   a.g.ncells = L->ncells; a.g.natoms = L->natoms;
   for (int d = 0; d < 3; ++d) a.g.periodic[d] = L->periodic[d];
-  a.nt = host_neighbour_tables();
   a.species = L->d_species;
   static const int dir[4][3] = {{1, 1, 1}, {1, -1, -1}, {-1, 1, -1}, {-1, -1, 1}};
   const double q4 = 0.25 * L->a_nm;
@@ -432,12 +429,22 @@ omen_status make_args(omen_ctx* ctx, const omen_lattice* L, const omen_vff_param
       for (int c = 0; c < 3; ++c) x += (F ? F[r * 3 + c] : (r == c ? 1.0 : 0.0)) * dir[k][c];
       a.fd[k][r] = x * q4;
     }
+  double alpha[4], beta[4];
   for (int s = 0; s < 4; ++s) {
     const int t = s < vp->nspecies ? s : 0;
     a.dnat[s] = 0.25 * std::sqrt(3.0) * vp->a_nm[t];
-    a.alpha[s] = vp->alpha[t];
-    a.beta[s] = vp->beta[t];
+    alpha[s] = vp->alpha[t];
+    beta[s] = vp->beta[t];
   }
+  for (int v = 0; v < 4; ++v)
+    for (int p = 0; p < 4; ++p) {
+      const double dp = 0.5 * (a.dnat[v] + a.dnat[p]), bp = 0.5 * (beta[v] + beta[p]);
+      a.t.bond[v][p] = make_double2(0.5 * 0.375 * 0.5 * (alpha[v] + alpha[p]) / (dp * dp), dp * dp);
+      for (int q = 0; q < 4; ++q) {
+        const double dd = dp * 0.5 * (a.dnat[v] + a.dnat[q]), bq = 0.5 * (beta[v] + beta[q]);
+        a.t.angle[v][p][q] = make_double2(0.375 * 0.5 * (bp + bq) / dd, dd / 3.0);
+      }
+    }
   return OMEN_OK;
 }
 
@@ -447,6 +454,8 @@ int reduce_blocks(omen_ctx* ctx, long long n) {
   const long long want = (n + kThreads - 1) / kThreads;
   return (int)std::max<long long>(1, std::min<long long>(want, 4ll * std::max(1, sms)));
 }
+
+unsigned blocks_of(long long n) { return (unsigned)((n + kThreads - 1) / kThreads); }
 
 // Host sum of the partials of one row, in block order.
 double host_sum(const std::vector<double>& h, int q, int nb, bool take_max = false) {
@@ -470,11 +479,17 @@ extern "C" omen_status omen_vff_energy_forces(omen_ctx* ctx, const omen_lattice*
   double* part = ctx->d_work;
   std::vector<double> h((size_t)3 * nb);
   if (force_dev) {
-    vff_grad_kernel<<<nb, kThreads, 0, ctx->stream>>>(a, u_dev, force_dev, nullptr, part);
-    OMEN_CHECK_LAUNCH(ctx);
+    double* f = nullptr;
+    if (ctx_alloc(ctx, &f, sizeof(double) * 12 * (size_t)N) != cudaSuccess) {
+      cudaGetLastError();
+      return set_err(ctx, OMEN_ENOMEM, "VFF work vectors");
+    }
+    vff_vertex_kernel<<<blocks_of(N), kThreads, 0, ctx->stream>>>(a, u_dev, f);
     // force = -dE/du
-    vff_negate_kernel<<<nb, kThreads, 0, ctx->stream>>>(force_dev, 3 * N);
-    OMEN_CHECK_LAUNCH(ctx);
+    vff_gather_kernel<<<nb, kThreads, 0, ctx->stream>>>(a, f, force_dev, nullptr, -1.0, nullptr, nullptr);
+    const cudaError_t e = cudaGetLastError();
+    cudaFreeAsync(f, ctx->stream);
+    if (e != cudaSuccess) return set_err(ctx, OMEN_ECUDA, "VFF forces: %s", cudaGetErrorString(e));
   }
   if (E_host) {
     vff_energy_kernel<<<nb, kThreads, 0, ctx->stream>>>(a, u_dev, part);
@@ -498,9 +513,9 @@ extern "C" omen_status omen_relax_vff(omen_ctx* ctx, const omen_lattice* L, cons
   const long long N = L->natoms, n3 = 3 * N;
   const int nb = reduce_blocks(ctx, N);
   const int check = 10;                                 // iterations between host convergence checks
-  // work: two gradients (ping-pong), the direction, partials of the gradient (3 rows) and of the
-  // line coefficients (4 rows), and the state record
-  const size_t bytes = sizeof(double) * (3 * (size_t)n3 + 7 * (size_t)nb) + sizeof(VffState);
+  // work: two gradients (ping-pong), the direction, the vertices' f, partials of the gradient (3
+  // rows) and of the line coefficients (4 rows), and the state record
+  const size_t bytes = sizeof(double) * (7 * (size_t)n3 + 7 * (size_t)nb) + sizeof(VffState);
   char* buf = nullptr;
   if (ctx_alloc(ctx, &buf, bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -508,7 +523,8 @@ extern "C" omen_status omen_relax_vff(omen_ctx* ctx, const omen_lattice* L, cons
   }
   double* g[2] = {reinterpret_cast<double*>(buf), reinterpret_cast<double*>(buf) + n3};
   double* p = g[1] + n3;
-  double* gpart = p + n3;
+  double* f = p + n3;
+  double* gpart = f + 4 * n3;
   double* lpart = gpart + 3 * (size_t)nb;
   VffState* st = reinterpret_cast<VffState*>(lpart + 4 * (size_t)nb);
   std::vector<double> h((size_t)nb);
@@ -524,8 +540,9 @@ extern "C" omen_status omen_relax_vff(omen_ctx* ctx, const omen_lattice* L, cons
   int cur = 0, it = 0;
   bool converged = false;
   if (e == cudaSuccess) {
-    vff_grad_kernel<<<nb, kThreads, 0, ctx->stream>>>(a, u_dev, g[cur], nullptr, gpart);
-    vff_dir_kernel<<<nb, kThreads, 0, ctx->stream>>>(g[cur], p, n3, gpart, nb, st, 1, 0);
+    vff_vertex_kernel<<<blocks_of(N), kThreads, 0, ctx->stream>>>(a, u_dev, f);
+    vff_gather_kernel<<<nb, kThreads, 0, ctx->stream>>>(a, f, g[cur], nullptr, 1.0, gpart, st);
+    vff_dir_kernel<<<nb, kThreads, 0, ctx->stream>>>(g[cur], p, n3, st, 1);
     e = cudaGetLastError();
   }
   while (e == cudaSuccess) {
@@ -540,12 +557,13 @@ extern "C" omen_status omen_relax_vff(omen_ctx* ctx, const omen_lattice* L, cons
       }
       if (it == o->max_iter) break;
     }
-    vff_line_kernel<<<nb, kThreads, 0, ctx->stream>>>(a, u_dev, p, lpart);
-    vff_step_kernel<<<nb, kThreads, 0, ctx->stream>>>(u_dev, p, n3, lpart, nb, st);
-    vff_grad_kernel<<<nb, kThreads, 0, ctx->stream>>>(a, u_dev, g[cur ^ 1], g[cur], gpart);
+    vff_line_kernel<<<nb, kThreads, 0, ctx->stream>>>(a, u_dev, p, lpart, st);
+    vff_step_kernel<<<nb, kThreads, 0, ctx->stream>>>(u_dev, p, n3, st);
+    vff_vertex_kernel<<<blocks_of(N), kThreads, 0, ctx->stream>>>(a, u_dev, f);
+    vff_gather_kernel<<<nb, kThreads, 0, ctx->stream>>>(a, f, g[cur ^ 1], g[cur], 1.0, gpart, st);
     cur ^= 1;
     ++it;
-    vff_dir_kernel<<<nb, kThreads, 0, ctx->stream>>>(g[cur], p, n3, gpart, nb, st, 0, it & 1);
+    vff_dir_kernel<<<nb, kThreads, 0, ctx->stream>>>(g[cur], p, n3, st, 0);
     e = cudaGetLastError();
   }
   double E1 = 0.0;
