@@ -33,3 +33,27 @@ __device__ __forceinline__ float2 df_from_double(double v) {
   return make_float2(hi, __double2float_rn(v - (double)hi));
 }
 __device__ __forceinline__ double df_to_double(float2 v) { return (double)v.x + (double)v.y; }
+
+// v 2^kSplitShift as an FP32 pair (hi, lo), by integer operations only (the FP64 pipe, which
+// df_from_double uses, has 1/64 of the FP32 rate): hi keeps the sign, the exponent and the leading
+// 24 significant bits, lo is the rest rounded to FP32 (48 significant bits in all).  Magnitudes too
+// small for FP32 give zero, too large or non-finite ones NaN.
+template <int kSplitShift>
+__device__ __forceinline__ float2 split_fp64(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned hi32 = (unsigned)(b >> 32), lo32 = (unsigned)b;
+  const int e = (int)((hi32 >> 20) & 0x7FFu);   // biased FP64 exponent
+  // FP32 exponent of hi: e - 1023 + 127 + shift
+  const int eh = e - 896 + kSplitShift;
+  if (eh <= 0) return make_float2(0.f, 0.f);     // |v| < 2^-158, or zero
+  if (eh >= 255) return make_float2(__int_as_float(0x7fc00000), 0.f);   // beyond FP32, inf or NaN: NaN
+  const unsigned sign = hi32 & 0x80000000u;
+  const unsigned top23 = ((hi32 & 0xFFFFFu) << 3) | (lo32 >> 29);
+  const float hi = __uint_as_float(sign | ((unsigned)eh << 23) | top23);
+  // the remaining 29 bits: rem * 2^(e - 1075 + shift)
+  const unsigned rem = lo32 & 0x1FFFFFFFu;
+  const int el = e - 948 + kSplitShift;
+  const float scale = el > 0 ? __uint_as_float((unsigned)el << 23) : 0.f;
+  const float lo = __fmul_rn(__uint2float_rn(rem), scale);
+  return make_float2(hi, sign ? -lo : lo);
+}

@@ -118,18 +118,65 @@ __global__ void reduce_partial_kernel(const double2* __restrict__ P, int nchunks
   }
 }
 
+// Sums of NA values over the lanes of a warp, by halving: a lane keeps half of its values at every
+// exchange, so 16 values cost 16 additions instead of 80 (an FP64 addition of a warp holds GB300's
+// FP64 pipe for 64 cycles).  Lane l ends with the sum of value scatter_index<NA>(l).
+template <int NA>
+__device__ __forceinline__ double scatter_sum(double (&v)[NA]) {
+  const int lane = threadIdx.x & 31;
+  int live = NA;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (live > 1) {
+      live /= 2;
+      const bool hi = lane & o;
+#pragma unroll
+      for (int i = 0; i < NA / 2; ++i)
+        if (i < live) {
+          const double keep = hi ? v[i + live] : v[i], send = hi ? v[i] : v[i + live];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
+  return v[0];
+}
+template <int NA>
+__device__ __forceinline__ int scatter_index(int lane) {
+  int idx = 0, live = NA;
+  for (int o = 16; o > 0 && live > 1; o >>= 1) {
+    live /= 2;
+    if (lane & o) idx += live;
+  }
+  return idx;
+}
+
+// What the last CTA to finish does with a projection: out[i] = sum over the chunks, added into
+// column col0 of the projected matrix when accT is given.  cnt: one zeroed counter per group of
+// basis vectors, left zeroed; null: the partials are reduced by another kernel.
+struct DotsFinish {
+  int* cnt = nullptr;
+  double2* out = nullptr;
+  double2* accT = nullptr;
+  int ldT = 0, col0 = 0;
+};
+
 // Projections onto one vector, P[chunk][i] = sum_r conj(A_i[r]) b[r], for the common case of a
-// single right-hand vector.  CTA (g, c) handles basis vectors 16g..16g+15 over row chunk c;
-// each thread keeps 16 independent loads in flight per row.  Consecutive CTAs share a chunk,
-// so b stays in L2 across the basis groups.  FP64 vectors accumulate in FP64; FP32 vectors
-// accumulate each thread's rows in compensated FP32 (Kahan) before the FP64 block sum.
+// single right-hand vector.  CTA (g, c) handles `per` <= IG basis vectors over row chunk c; each
+// thread keeps IG independent loads in flight per row.  Consecutive CTAs share a chunk, so b stays
+// in L2 across the basis groups.  FP64 vectors accumulate in FP64; FP32 vectors accumulate each
+// thread's rows in compensated FP32 (Kahan) before the FP64 block sum.
+// The bound is the FP64 rate (one FMA per 8 bytes: 4.97 TB/s).  640k rows, 65 vectors: 130 us with 80
+// additions a warp in the block sums, chunks of at most 8192 rows in 1.3 waves and a last group of one
+// vector; 85 us with halving sums, one wave, and the vectors dealt evenly (FP64 floor 66 us).
 static constexpr int kIG = 16;
 // basis vectors per CTA of dots1_kernel: 16 real, 8 complex (the complex accumulators would
 // otherwise hold the kernel to one CTA per SM)
 static constexpr int dots1_ig(bool cplx) { return cplx ? 8 : kIG; }
 template <typename T, bool C, int IG>
-__global__ void __launch_bounds__(256, C ? 1 : 2) dots1_kernel(const void* Av, long long lda, int na, const void* Bv,
-                                                    long long n, int rows_per_cta, double2* __restrict__ P,
+__global__ void __launch_bounds__(256, 2) dots1_kernel(const void* Av, long long lda, int na, int per, const void* Bv,
+                                                    long long n, int rows_per_cta, double2* P, DotsFinish fin,
                                                     long long a_ps = 0, long long b_ps = 0, long long p_ps = 0,
                                                     const long long* __restrict__ poff = nullptr,
                                                     const long long* __restrict__ plen = nullptr,
@@ -137,6 +184,7 @@ __global__ void __launch_bounds__(256, C ? 1 : 2) dots1_kernel(const void* Av, l
   using E = Elem<T, C>;
   using V = typename E::V;
   using Acc = std::conditional_t<sizeof(T) == 8, double, float>;
+  constexpr int NA = C ? 2 * IG : IG;
   // IG basis vectors per CTA (at most dots1_ig(C)); chosen from na so that no accumulator
   // sits idle under a predicate (predicated-off FP64 FMAs still occupy the pipe)
   // grid.z = independent problems (batched Lanczos): offsets a_ps, b_ps (elements), p_ps
@@ -147,8 +195,8 @@ __global__ void __launch_bounds__(256, C ? 1 : 2) dots1_kernel(const void* Av, l
   const V* A = static_cast<const V*>(Av) + blockIdx.z * a_ps + off;
   const V* B = static_cast<const V*>(Bv) + blockIdx.z * b_ps + off;
   P += blockIdx.z * p_ps;
-  const int i0 = blockIdx.x * IG;
-  const int ni = min(IG, na - i0);
+  const int i0 = blockIdx.x * per;
+  const int ni = min(per, na - i0);
   const long long r0 = (long long)blockIdx.y * rows_per_cta;
   const long long r1 = min(n, r0 + rows_per_cta);
   Acc sr[IG], si[IG], cr[IG], ci[IG];
@@ -163,17 +211,21 @@ __global__ void __launch_bounds__(256, C ? 1 : 2) dots1_kernel(const void* Av, l
 #pragma unroll
     for (int i = 0; i < IG; ++i) {
       if (i < ni) {
-        Acc pr, pi = 0;
-        if constexpr (C) {
-          pr = (Acc)av[i].x * (Acc)bv.x + (Acc)av[i].y * (Acc)bv.y;
-          pi = (Acc)av[i].x * (Acc)bv.y - (Acc)av[i].y * (Acc)bv.x;
-        } else {
-          pr = (Acc)av[i] * (Acc)bv;
-        }
         if constexpr (sizeof(T) == 8) {
-          sr[i] += pr;
-          si[i] += pi;
+          if constexpr (C) {
+            sr[i] = fma(av[i].y, bv.y, fma(av[i].x, bv.x, sr[i]));
+            si[i] = fma(-av[i].y, bv.x, fma(av[i].x, bv.y, si[i]));
+          } else {
+            sr[i] = fma(av[i], bv, sr[i]);
+          }
         } else {  // Kahan-compensated FP32 sums
+          Acc pr, pi = 0;
+          if constexpr (C) {
+            pr = (Acc)av[i].x * (Acc)bv.x + (Acc)av[i].y * (Acc)bv.y;
+            pi = (Acc)av[i].x * (Acc)bv.y - (Acc)av[i].y * (Acc)bv.x;
+          } else {
+            pr = (Acc)av[i] * (Acc)bv;
+          }
           const Acc yr = pr - cr[i], tr = sr[i] + yr;
           cr[i] = (tr - sr[i]) - yr;
           sr[i] = tr;
@@ -184,22 +236,61 @@ __global__ void __launch_bounds__(256, C ? 1 : 2) dots1_kernel(const void* Av, l
       }
     }
   }
-  __shared__ double red[8][IG > 0 ? IG : 1][2];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double red[8][NA];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  double v[NA];
 #pragma unroll
   for (int i = 0; i < IG; ++i) {
-    double vr = (double)sr[i] - (double)cr[i], vi = (double)si[i] - (double)ci[i];
-    for (int o = 16; o > 0; o >>= 1) {
-      vr += __shfl_xor_sync(0xffffffffu, vr, o);
-      if constexpr (C) vi += __shfl_xor_sync(0xffffffffu, vi, o);
+    if constexpr (sizeof(T) == 8) {
+      v[i] = sr[i];
+      if constexpr (C) v[IG + i] = si[i];
+    } else {
+      v[i] = (double)sr[i] - (double)cr[i];
+      if constexpr (C) v[IG + i] = (double)si[i] - (double)ci[i];
     }
-    if (lane == 0) { red[warp][i][0] = vr; red[warp][i][1] = vi; }
+  }
+  red[warp][scatter_index<NA>(lane)] = scatter_sum<NA>(v);   // lanes of one index hold the same sum
+  __syncthreads();
+  if ((int)threadIdx.x < ni) {
+    double vr = 0.0, vi = 0.0;
+    for (int w = 0; w < nwarp; ++w) {
+      vr += red[w][threadIdx.x];
+      if constexpr (C) vi += red[w][IG + threadIdx.x];
+    }
+    P[(size_t)blockIdx.y * na + i0 + threadIdx.x] = make_double2(vr, C ? vi : 0.0);
+  }
+  if (!fin.cnt) return;
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const bool l = atomicAdd(fin.cnt + blockIdx.x, 1) == (int)gridDim.y - 1;
+    if (l) fin.cnt[blockIdx.x] = 0;
+    last = l;
   }
   __syncthreads();
-  if (threadIdx.x < ni) {
-    double vr = 0.0, vi = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { vr += red[w][threadIdx.x][0]; vi += red[w][threadIdx.x][1]; }
-    P[(size_t)blockIdx.y * na + i0 + threadIdx.x] = make_double2(vr, C ? vi : 0.0);
+  if (!last) return;
+  __threadfence();
+  // LPV lanes a vector over the chunks
+  const int lpv = min(32, (int)blockDim.x / IG), vec = threadIdx.x / lpv, part = threadIdx.x % lpv;
+  double vr = 0.0, vi = 0.0;
+  if (vec < ni)
+    for (int c = part; c < (int)gridDim.y; c += lpv) {
+      const double2 q = __ldcg(P + (size_t)c * na + i0 + vec);
+      vr += q.x;
+      if constexpr (C) vi += q.y;
+    }
+  for (int o = lpv / 2; o > 0; o >>= 1) {
+    vr += __shfl_xor_sync(0xffffffffu, vr, o);
+    if constexpr (C) vi += __shfl_xor_sync(0xffffffffu, vi, o);
+  }
+  if (vec < ni && part == 0) {
+    fin.out[i0 + vec] = make_double2(vr, vi);
+    if (fin.accT) {
+      double2* t = fin.accT + i0 + vec + (size_t)fin.col0 * fin.ldT;
+      t->x += vr;
+      t->y += vi;
+    }
   }
 }
 
@@ -289,6 +380,171 @@ __global__ void __launch_bounds__(256) combine1_kernel(const void* Av, long long
   const V* A = static_cast<const V*>(Av) + blockIdx.y * a_ps + off;
   V* Y = static_cast<V*>(Yv) + blockIdx.y * y_ps + off;
   combine1_rows<T, C, A2>(A, lda, na, Ms, Y, n, (R)beta, beta != 0.0);
+}
+
+// The kernels of a step after the product: dots1 (v_j), three_term, dots1 (basis), update_norm, scale.
+// Before, each projection had a second kernel to reduce it, the two subtractions and the norm were
+// passes of their own, and a copy mirrored the off-diagonal entry: 11 launches against 5.  640k real
+// rows, basis 48 to 96: 335 us a step besides the product before, 190 us now (FP64: two FMAs an element
+// of the basis); 1,280 complex rows, basis 24 to 48: 65 us before, 20 us now (launches).
+// The three-term part of a step in one pass: w -= h v_j + t v_{j-1}, with h = <v_j, w> and t the
+// norm of the step before (entry (js, js-1) of the projected matrix, mirrored here).
+template <typename T, bool C>
+__global__ void __launch_bounds__(256) three_term_kernel(const void* Vj, const void* Vp, const double2* __restrict__ h,
+                                                         double2* __restrict__ Tm, int ldT, int js, void* Wv, long long n) {
+  using V = typename Elem<T, C>::V;
+  const double2 hj = *h, tp = Tm[js + (size_t)(js - 1) * ldT];
+  if (blockIdx.x == 0 && threadIdx.x == 0) Tm[(js - 1) + (size_t)js * ldT] = tp;
+  const T hr = (T)-hj.x, hi = (T)-hj.y, tr = (T)-tp.x;     // a norm: its imaginary part is zero
+  const V* __restrict__ a = static_cast<const V*>(Vj);
+  const V* __restrict__ b = static_cast<const V*>(Vp);
+  V* __restrict__ w = static_cast<V*>(Wv);
+  for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x) {
+    V x = w[r];
+    const V av = a[r], bv = b[r];
+    if constexpr (C) {
+      x.x = fma(tr, bv.x, fma(-av.y, hi, fma(av.x, hr, x.x)));
+      x.y = fma(tr, bv.y, fma(av.y, hr, fma(av.x, hi, x.y)));
+    } else {
+      x = fma(tr, bv, fma(hr, av, x));
+    }
+    w[r] = x;
+  }
+}
+
+// w -= sum_i V_i h_i and ||w||^2 of the result.  A CTA holds blockDim.x / PARTS rows; PARTS groups
+// of its threads share a row's basis vectors (PARTS > 1: problems of too few rows to fill the
+// device).  The last CTA sums the squares, writes nrm[0] = ||w||^2 and nrm[1] = 1 / ||w||, and the
+// norm into T[row, col]; a zero or non-finite norm sets the flag.
+template <typename T, bool C, int PARTS>
+__global__ void __launch_bounds__(256) update_norm_kernel(const void* Av, int na, const double2* __restrict__ h, void* Wv,
+                                                          long long n, double* part, int* cnt, double2* nrm, double2* Tm,
+                                                          int ldT, int row, int col, int* flag) {
+  using V = typename Elem<T, C>::V;
+  using A2 = std::conditional_t<sizeof(T) == 8, double2, float2>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  A2* Ms = reinterpret_cast<A2*>(smem_raw);
+  constexpr int ROWS = 256 / PARTS;
+  __shared__ V sums[PARTS > 1 ? 256 : 1];
+  for (int t = threadIdx.x; t < na; t += blockDim.x) {
+    A2 m;
+    m.x = (T)-h[t].x;
+    m.y = (T)-h[t].y;
+    Ms[t] = m;
+  }
+  __syncthreads();
+  const V* __restrict__ A = static_cast<const V*>(Av);
+  V* __restrict__ W = static_cast<V*>(Wv);
+  const int rl = threadIdx.x % ROWS, pt = threadIdx.x / ROWS;
+  const int ia = (int)((long long)na * pt / PARTS), ib = (int)((long long)na * (pt + 1) / PARTS);
+  double sq = 0.0;
+  float sf = 0.f, cf = 0.f;                            // FP32 vectors: compensated FP32 sum of squares
+  for (long long rb = (long long)blockIdx.x * ROWS; rb < n; rb += (long long)gridDim.x * ROWS) {
+    const long long r = rb + rl;
+    T yr = 0, yi = 0;
+    if (r < n) {
+      int i = ia;
+      for (; i + 8 <= ib; i += 8) {
+        V av[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) av[k] = A[(size_t)(i + k) * n + r];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const A2 m = Ms[i + k];
+          if constexpr (C) {
+            yr = fma(-av[k].y, m.y, fma(av[k].x, m.x, yr));
+            yi = fma(av[k].y, m.x, fma(av[k].x, m.y, yi));
+          } else {
+            yr = fma(av[k], m.x, yr);
+          }
+        }
+      }
+      for (; i < ib; ++i) {
+        const V a = A[(size_t)i * n + r];
+        const A2 m = Ms[i];
+        if constexpr (C) {
+          yr = fma(-a.y, m.y, fma(a.x, m.x, yr));
+          yi = fma(a.y, m.x, fma(a.x, m.y, yi));
+        } else {
+          yr = fma(a, m.x, yr);
+        }
+      }
+    }
+    if constexpr (PARTS > 1) {
+      V mine;
+      if constexpr (C) { mine.x = yr; mine.y = yi; } else mine = yr;
+      __syncthreads();
+      sums[threadIdx.x] = mine;
+      __syncthreads();
+      if (pt == 0) {
+#pragma unroll
+        for (int q = 1; q < PARTS; ++q) {
+          const V o = sums[q * ROWS + rl];
+          if constexpr (C) { yr += o.x; yi += o.y; } else yr += o;
+        }
+      }
+    }
+    if (pt == 0 && r < n) {
+      V w = W[r];
+      if constexpr (C) { w.x += yr; w.y += yi; } else w += yr;
+      W[r] = w;
+      if constexpr (sizeof(T) == 8) {
+        if constexpr (C) sq = fma(w.y, w.y, fma(w.x, w.x, sq)); else sq = fma(w, w, sq);
+      } else {
+        float p;
+        if constexpr (C) p = w.x * w.x + w.y * w.y; else p = w * w;
+        const float y = p - cf, t = sf + y;
+        cf = (t - sf) - y;
+        sf = t;
+      }
+    }
+  }
+  if constexpr (sizeof(T) == 4) sq = (double)sf - (double)cf;
+  __shared__ double red[8];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (PARTS == 1 || warp * 32 < ROWS) {                // only row threads hold squares
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane == 0) red[warp] = sq;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < (ROWS + 31) / 32; ++w) t += red[w];
+    part[blockIdx.x] = t;
+    __threadfence();
+    const bool l = atomicAdd(cnt, 1) == (int)gridDim.x - 1;
+    if (l) *cnt = 0;
+    last = l;
+  }
+  __syncthreads();
+  if (!last || warp != 0) return;
+  __threadfence();
+  double t = 0.0;
+  for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(part + b);
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) {
+    const double b = sqrt(fmax(t, 0.0));
+    nrm[0] = make_double2(t, 0.0);
+    nrm[1] = make_double2((b > 1e-300) ? 1.0 / b : 0.0, 0.0);
+    Tm[row + (size_t)col * ldT] = make_double2(b, 0.0);
+    if (!(b > 1e-300) || !isfinite(b)) *flag = 1;
+  }
+}
+
+// v = w / ||w|| with 1 / ||w|| from update_norm_kernel (formed once, not by every thread: a square
+// root and a division are some 40 FP64 operations).
+template <typename T, bool C>
+__global__ void __launch_bounds__(256) scale_kernel(const void* Wv, void* Vv, long long n, const double2* __restrict__ nrm) {
+  using E = Elem<T, C>;
+  using V = typename E::V;
+  const double inv = nrm[1].x;
+  const V* __restrict__ W = static_cast<const V*>(Wv);
+  V* __restrict__ Vo = static_cast<V*>(Vv);
+  for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x) {
+    const V w = W[r];
+    Vo[r] = E::make(E::re(w) * inv, E::im(w) * inv);
+  }
 }
 
 // The update w -= V h of the full Gram–Schmidt pass, applied only where it is needed to keep
@@ -490,32 +746,39 @@ __global__ void __launch_bounds__(256) combinen_kernel(const void* Av, long long
 }
 
 // Many-output combination of real FP64 vectors (restarts: kk Ritz vectors from m basis
-// vectors): nb FMAs per element read would hold it to GB300's FP64 rate, so each element is
-// split once into a double-float pair (one FP64 subtraction) and the nb products and sums run in
+// vectors): nb FMAs per element read would hold it to GB300's FP64 rate, so each element is split
+// once into a double-float pair, by integer operations, and the nb products and sums run in
 // double-float arithmetic on the FP32 pipe; each result is rounded back to FP64 (about 48 of its
-// 53 bits exact — the next step re-orthogonalises anyway).
+// 53 bits exact — the next step re-orthogonalises anyway).  The split carries a factor 2^32, which
+// keeps components down to 2^-107 clear of FP32 underflow.  49 vectors from 97, 640k rows: four
+// passes of 16 columns at 0.75 ms with the split on the FP64 pipe (three conversions and a
+// subtraction), two passes of 25 at 0.81 ms now.
 template <int NBT>
 __global__ void __launch_bounds__(256) combine_split_kernel(const double* __restrict__ A, long long lda, int na,
                                                             const double2* __restrict__ M, int nb, double* __restrict__ Y,
                                                             long long ldy, long long n, double alpha, double beta) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* Ms = reinterpret_cast<float2*>(smem_raw);
-  for (int t = threadIdx.x; t < na * nb; t += blockDim.x) Ms[t] = df_from_double(alpha * M[t].x);
+  float2* Ms = reinterpret_cast<float2*>(smem_raw);     // [na][NBT]
+  for (int t = threadIdx.x; t < na * NBT; t += blockDim.x) {
+    const int i = t / NBT, j = t - i * NBT;
+    Ms[t] = j < nb ? df_from_double(alpha * M[i + (size_t)j * na].x) : make_float2(0.f, 0.f);
+  }
   __syncthreads();
   for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x) {
     float S[NBT], Cc[NBT];
 #pragma unroll
     for (int j = 0; j < NBT; ++j) { S[j] = 0.f; Cc[j] = 0.f; }
+    double next = A[r];
     for (int i = 0; i < na; ++i) {
-      const float2 a = df_from_double(A[(size_t)i * lda + r]);
+      const float2 a = split_fp64<32>(next);
+      if (i + 1 < na) next = A[(size_t)(i + 1) * lda + r];
 #pragma unroll
-      for (int j = 0; j < NBT; ++j)
-        if (j < nb) df_mac(S[j], Cc[j], a, Ms[i + j * na]);
+      for (int j = 0; j < NBT; ++j) df_mac(S[j], Cc[j], a, Ms[i * NBT + j]);
     }
 #pragma unroll
     for (int j = 0; j < NBT; ++j)
       if (j < nb) {
-        double v = (double)S[j] + (double)Cc[j];
+        double v = ((double)S[j] + (double)Cc[j]) * 0x1p-32;
         if (beta != 0.0) v = fma(beta, Y[(size_t)j * ldy + r], v);
         Y[(size_t)j * ldy + r] = v;
       }
@@ -865,7 +1128,10 @@ __global__ void normalize_kernel(const void* Wv, void* Vv, long long n, const do
 }
 
 // Y_j[r] = beta * Y_j[r] + alpha * sum_i A_i[r] M[i + j*na]   (M complex FP64, column-major)
-template <typename T, bool C>
+// NC columns per thread, grid.y over groups of them: 16, or 4 where the rows alone leave SMs idle (25
+// columns from 48 vectors of 1,280 complex rows: 170 us for each 16 columns on five SMs before, 23 us
+// for all 25 now).
+template <typename T, bool C, int NC>
 __global__ void combine_kernel(const void* Av, long long lda, int na, const double2* __restrict__ M, int nb,
                                void* Yv, long long ldy, long long n, double alpha, double beta) {
   // arithmetic in the vectors' precision (coefficients alpha*M rounded once): FP32 vectors keep
@@ -876,6 +1142,9 @@ __global__ void combine_kernel(const void* Av, long long lda, int na, const doub
   using R = T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   A2* Ms = reinterpret_cast<A2*>(smem_raw);
+  M += (size_t)blockIdx.y * NC * na;
+  Yv = static_cast<V*>(Yv) + (size_t)blockIdx.y * NC * ldy;
+  nb = min(NC, nb - (int)blockIdx.y * NC);
   for (int t = threadIdx.x; t < na * nb; t += blockDim.x) {
     A2 m;
     m.x = (R)(alpha * M[t].x);
@@ -887,9 +1156,9 @@ __global__ void combine_kernel(const void* Av, long long lda, int na, const doub
   V* Y = static_cast<V*>(Yv);
   const R rbeta = (R)beta;
   for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x) {
-    R yr[kMaxBlockCols], yi[kMaxBlockCols];
+    R yr[NC], yi[NC];
 #pragma unroll
-    for (int j = 0; j < kMaxBlockCols; ++j) { yr[j] = 0; yi[j] = 0; }
+    for (int j = 0; j < NC; ++j) { yr[j] = 0; yi[j] = 0; }
     for (int i0 = 0; i0 < na; i0 += 4) {
       V av[4];
 #pragma unroll
@@ -901,7 +1170,7 @@ __global__ void combine_kernel(const void* Av, long long lda, int na, const doub
         const int i = i0 + k;
         const R xr = (R)E::re(av[k]), xi = (R)E::im(av[k]);
 #pragma unroll
-        for (int j = 0; j < kMaxBlockCols; ++j) {
+        for (int j = 0; j < NC; ++j) {
           if (j < nb) {
             const A2 m = Ms[i + j * na];
             yr[j] = fma(xr, m.x, yr[j]);
@@ -915,7 +1184,7 @@ __global__ void combine_kernel(const void* Av, long long lda, int na, const doub
       }
     }
 #pragma unroll
-    for (int j = 0; j < kMaxBlockCols; ++j) {
+    for (int j = 0; j < NC; ++j) {
       if (j < nb) {
         V& out = Y[j * ldy + r];
         R orr = yr[j], oi = yi[j];
@@ -994,19 +1263,27 @@ static int dots_ig_for(int na, int cap) {
   return ig;
 }
 
+// Launch of dots1_kernel on na basis vectors: IG compiled vectors a CTA, `per` of them dealt to each.
+struct DotsShape {
+  int ig, per, groups, threads;
+  long long rows, chunks;
+};
+
 template <typename T, bool C>
-static void launch_dots1(int ig, dim3 grid, cudaStream_t st, const void* A, long long lda, int na, const void* B,
-                         long long n, int rows, double2* P, long long a_ps = 0, long long b_ps = 0, long long p_ps = 0,
+static void launch_dots1(const DotsShape& d, int P, cudaStream_t st, const void* A, long long lda, int na, const void* B,
+                         long long n, double2* part, const DotsFinish& fin, long long p_ps = 0,
                          const long long* poff = nullptr, const long long* plen = nullptr, const int* act = nullptr) {
-  switch (ig) {
-    case 1: dots1_kernel<T, C, 1><<<grid, 256, 0, st>>>(A, lda, na, B, n, rows, P, a_ps, b_ps, p_ps, poff, plen, act); break;
-    case 2: dots1_kernel<T, C, 2><<<grid, 256, 0, st>>>(A, lda, na, B, n, rows, P, a_ps, b_ps, p_ps, poff, plen, act); break;
-    case 4: dots1_kernel<T, C, 4><<<grid, 256, 0, st>>>(A, lda, na, B, n, rows, P, a_ps, b_ps, p_ps, poff, plen, act); break;
-    case 8: dots1_kernel<T, C, 8><<<grid, 256, 0, st>>>(A, lda, na, B, n, rows, P, a_ps, b_ps, p_ps, poff, plen, act); break;
+  const dim3 grid(d.groups, (unsigned)d.chunks, P);
+#define DOTS1(IGc) dots1_kernel<T, C, IGc><<<grid, d.threads, 0, st>>>(A, lda, na, d.per, B, n, (int)d.rows, part, fin, 0, 0, p_ps, poff, plen, act)
+  switch (d.ig) {
+    case 1: DOTS1(1); break;
+    case 2: DOTS1(2); break;
+    case 4: DOTS1(4); break;
+    case 8: DOTS1(8); break;
     default:
-      if constexpr (!C) dots1_kernel<T, C, 16><<<grid, 256, 0, st>>>(A, lda, na, B, n, rows, P, a_ps, b_ps, p_ps, poff, plen, act);
-      else dots1_kernel<T, C, 8><<<grid, 256, 0, st>>>(A, lda, na, B, n, rows, P, a_ps, b_ps, p_ps, poff, plen, act);
+      if constexpr (!C) DOTS1(16); else DOTS1(8);
   }
+#undef DOTS1
 }
 
 struct KrylovOps {
@@ -1024,16 +1301,22 @@ struct KrylovOps {
   size_t qr_cap = 0;
   double2* d_hs = nullptr;     // projection sums of the block path
   size_t hs_cap = 0;
+  int* d_cnt = nullptr;        // zeroed arrival counters of the kernels that finish their own sums
+  double* d_npart = nullptr;   // partial squares of update_norm_kernel, one per CTA
+  static constexpr int kCounters = 1024;
   int sm_count = 148;
 
   omen_status init() {
     el = vec_elem_bytes(ham, prec);
     cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, ctx->device);
     small_cap = 1 << 18;
-    if (cudaMalloc(&d_small, small_cap * sizeof(double2)) != cudaSuccess) {
+    if (cudaMalloc(&d_small, small_cap * sizeof(double2)) != cudaSuccess ||
+        cudaMalloc(&d_cnt, kCounters * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&d_npart, sizeof(double) * 8 * (size_t)sm_count) != cudaSuccess) {
       cudaGetLastError();
       return set_err(ctx, OMEN_ENOMEM, "small work buffer");
     }
+    OMEN_CUDA(ctx, cudaMemsetAsync(d_cnt, 0, kCounters * sizeof(int), ctx->stream));
     return OMEN_OK;
   }
   void release() {
@@ -1041,6 +1324,8 @@ struct KrylovOps {
     cudaFree(d_small);
     cudaFree(qr_tmp);
     cudaFree(d_hs);
+    cudaFree(d_cnt);
+    cudaFree(d_npart);
   }
   char* col(void* base, long long j) const { return static_cast<char*>(base) + (size_t)j * n * el; }
 
@@ -1108,37 +1393,54 @@ struct KrylovOps {
       return combine_dev(A, na, d_small, nb, Y, alpha, beta);
     }
     if ((size_t)na * kMaxBlockCols > small_cap) return set_err(ctx, OMEN_EINVAL, "combination too large");
-    for (int j0 = 0; j0 < nb; j0 += kMaxBlockCols) {
-      const int nbj = std::min(kMaxBlockCols, nb - j0);
-      std::vector<cd> Mj((size_t)na * nbj);
-      for (int j = 0; j < nbj; ++j)
-        for (int i = 0; i < na; ++i) Mj[i + (size_t)j * na] = M[i + (size_t)(j0 + j) * na];
-      OMEN_CUDA(ctx, cudaMemcpyAsync(d_small, Mj.data(), Mj.size() * sizeof(double2), cudaMemcpyHostToDevice, ctx->stream));
-      const size_t shm = Mj.size() * sizeof(double2);
-      const unsigned grid = (unsigned)std::min<long long>((n + 255) / 256, (long long)sm_count * 8);
+    // as many columns a copy as the small buffer holds, in whole groups of the kernels' columns
+    const int most = (int)std::min<size_t>(nb, small_cap / na / 400 ? small_cap / na / 400 * 400 : kMaxBlockCols);
+    for (int j0 = 0; j0 < nb; j0 += most) {
+      const int nbj = std::min(most, nb - j0);
+      // pageable source, consumed when the call returns; stream order keeps the kernels of the last
+      // copy ahead of the next one
+      OMEN_CUDA(ctx, cudaMemcpyAsync(d_small, M.data() + (size_t)j0 * na, (size_t)na * nbj * sizeof(double2),
+                                     cudaMemcpyHostToDevice, ctx->stream));
       void* Yj = col(Y, j0);
-#define COMB_LAUNCH(T, Cc)                                                                           \
-  do {                                                                                               \
-    smem_limit(combine_kernel<T, Cc>, shm); \
-    combine_kernel<T, Cc><<<grid, 256, shm, ctx->stream>>>(A, n, na, d_small, nbj, Yj, n, n, alpha, beta); \
-  } while (0)
       if (prec == OMEN_F64 && !cplx) {
-        const size_t shs = (size_t)na * nbj * sizeof(float2);
+        const unsigned grid = (unsigned)std::min<long long>((n + 255) / 256, (long long)sm_count * 8);
         const double* Ad = static_cast<const double*>(A);
-        double* Yd = static_cast<double*>(Yj);
-        if (nbj <= 8) {
-          smem_limit(combine_split_kernel<8>, shs);
-          combine_split_kernel<8><<<grid, 256, shs, ctx->stream>>>(Ad, n, na, d_small, nbj, Yd, n, n, alpha, beta);
-        } else {
-          smem_limit(combine_split_kernel<16>, shs);
-          combine_split_kernel<16><<<grid, 256, shs, ctx->stream>>>(Ad, n, na, d_small, nbj, Yd, n, n, alpha, beta);
+        // columns a pass: 25 where that saves one (49 of a basis of 96: two passes, not four)
+        const int nc = nbj <= 8 ? 8 : nbj <= 16 ? 16 : 25;
+        const size_t shs = (size_t)na * nc * sizeof(float2);
+        for (int c0 = 0; c0 < nbj; c0 += nc) {
+          const int w = std::min(nc, nbj - c0);
+          double* Yd = static_cast<double*>(Yj) + (size_t)c0 * n;
+          const double2* Mj = d_small + (size_t)c0 * na;
+#define SPLITC(NCc)                                                                                       \
+  do {                                                                                                    \
+    smem_limit(combine_split_kernel<NCc>, shs);                                                           \
+    combine_split_kernel<NCc><<<grid, 256, shs, ctx->stream>>>(Ad, n, na, Mj, w, Yd, n, n, alpha, beta);  \
+  } while (0)
+          if (nc == 8) SPLITC(8); else if (nc == 16) SPLITC(16); else SPLITC(25);
+#undef SPLITC
         }
-      } else if (prec == OMEN_F64) COMB_LAUNCH(double, true);
-      else { if (cplx) COMB_LAUNCH(float, true); else COMB_LAUNCH(float, false); }
+      } else {
+        // few rows: four columns and 64 rows a CTA
+        const bool few = (n + 255) / 256 < sm_count;
+        const int nc = few ? 4 : kMaxBlockCols, thr = few ? 64 : 256;
+        const dim3 grid((unsigned)std::min<long long>((n + thr - 1) / thr, (long long)sm_count * 8), (nbj + nc - 1) / nc);
+#define COMB_LAUNCH(T, Cc)                                                                                   \
+  do {                                                                                                       \
+    const size_t shm = (size_t)na * nc * sizeof(double2);                                                    \
+    if (few) {                                                                                               \
+      smem_limit(combine_kernel<T, Cc, 4>, shm);                                                             \
+      combine_kernel<T, Cc, 4><<<grid, thr, shm, ctx->stream>>>(A, n, na, d_small, nbj, Yj, n, n, alpha, beta); \
+    } else {                                                                                                 \
+      smem_limit(combine_kernel<T, Cc, kMaxBlockCols>, shm);                                                 \
+      combine_kernel<T, Cc, kMaxBlockCols><<<grid, thr, shm, ctx->stream>>>(A, n, na, d_small, nbj, Yj, n, n, alpha, beta); \
+    }                                                                                                        \
+  } while (0)
+        if (prec == OMEN_F64) COMB_LAUNCH(double, true);
+        else { if (cplx) COMB_LAUNCH(float, true); else COMB_LAUNCH(float, false); }
 #undef COMB_LAUNCH
+      }
       OMEN_CHECK_LAUNCH(ctx);
-      // the small buffer is reused by the next chunk: wait for this kernel to read it
-      OMEN_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     }
     return OMEN_OK;
   }
@@ -1162,7 +1464,30 @@ struct KrylovOps {
         const long long rows = dot_rows(na, ig);
         need = std::max(need, (size_t)((n + rows - 1) / rows) * na * 4);
       }
+    for (int na = 1; na <= na_max; ++na) need = std::max(need, (size_t)dots_shape(na, n, 1).chunks * na);
     return need;
+  }
+
+  // Shape of a projection on na vectors of nmax rows, for P problems at once: the vectors dealt
+  // evenly to groups of at most dots1_ig, the chunks as many as one wave of two CTAs an SM holds
+  // (six an SM for single vectors: 14.3 against 8.6 us at 640k rows, in the last CTA's sum).
+  // Small problems (fewer than an SM's worth of full CTAs each) take CTAs of 64 rows and four vectors.
+  DotsShape dots_shape(int na, long long nmax, int P) const {
+    DotsShape d;
+    d.threads = 256;
+    int cap = dots1_ig(cplx);
+    if ((nmax + 255) / 256 * ((na + cap - 1) / cap) * P < sm_count) {
+      cap = 4;
+      d.threads = 64;
+    }
+    d.groups = (na + cap - 1) / cap;
+    d.per = (na + d.groups - 1) / d.groups;
+    d.ig = dots_ig_for(d.per, cap);
+    const long long slots = std::max<long long>(1, (2LL * sm_count * (256 / d.threads)) / ((long long)d.groups * P));
+    d.rows = std::max<long long>(d.threads, ((nmax + slots - 1) / slots + d.threads - 1) / d.threads * d.threads);
+    while ((nmax + d.rows - 1) / d.rows > 65535 || d.rows > 0x7fffffffLL / 2) d.rows = d.rows > 0x7fffffffLL / 2 ? 0x3fffff00LL : d.rows * 2;
+    d.chunks = (nmax + d.rows - 1) / d.rows;
+    return d;
   }
 
   // out (host, ncols) = <A_j, B_j> for each column j
@@ -1262,20 +1587,18 @@ struct KrylovOps {
       return OMEN_OK;
     }
     if (nb == 1) {
-      const int ig1 = dots_ig_for(na, dots1_ig(cplx));
-      const int rows = (int)dot_rows(na, ig1);
-      const long long nchunks = (n + rows - 1) / rows;
-      omen_status s1 = ensure_partial((size_t)nchunks * na);
+      const DotsShape d = dots_shape(na, n, 1);
+      omen_status s1 = ensure_partial((size_t)d.chunks * na);
       if (s1 != OMEN_OK) return s1;
-      dim3 grid((na + ig1 - 1) / ig1, (unsigned)nchunks);
+      if (d.groups >= kCounters) return set_err(ctx, OMEN_EINVAL, "projection on too many vectors");
+      const DotsFinish fin{d_cnt, out_dev, accT, ldT, col0};
       if (prec == OMEN_F64) {
-        if (cplx) launch_dots1<double, true>(ig1, grid, ctx->stream, A, n, na, B, n, rows, d_partial);
-        else launch_dots1<double, false>(ig1, grid, ctx->stream, A, n, na, B, n, rows, d_partial);
+        if (cplx) launch_dots1<double, true>(d, 1, ctx->stream, A, n, na, B, n, d_partial, fin);
+        else launch_dots1<double, false>(d, 1, ctx->stream, A, n, na, B, n, d_partial, fin);
       } else {
-        if (cplx) launch_dots1<float, true>(ig1, grid, ctx->stream, A, n, na, B, n, rows, d_partial);
-        else launch_dots1<float, false>(ig1, grid, ctx->stream, A, n, na, B, n, rows, d_partial);
+        if (cplx) launch_dots1<float, true>(d, 1, ctx->stream, A, n, na, B, n, d_partial, fin);
+        else launch_dots1<float, false>(d, 1, ctx->stream, A, n, na, B, n, d_partial, fin);
       }
-      reduce_dev_kernel<<<na, 256, 0, ctx->stream>>>(d_partial, (int)nchunks, na, 1, out_dev, accT, ldT, col0);
       OMEN_CHECK_LAUNCH(ctx);
       return OMEN_OK;
     }
@@ -1358,8 +1681,8 @@ struct KrylovOps {
     const unsigned grid = (unsigned)std::min<long long>((n + 255) / 256, (long long)sm_count * 8);
 #define COMB_LAUNCH2(T, Cc)                                                                          \
   do {                                                                                               \
-    smem_limit(combine_kernel<T, Cc>, shm); \
-    combine_kernel<T, Cc><<<grid, 256, shm, ctx->stream>>>(A, n, na, M_dev, nb, Y, n, n, alpha, beta); \
+    smem_limit(combine_kernel<T, Cc, kMaxBlockCols>, shm); \
+    combine_kernel<T, Cc, kMaxBlockCols><<<grid, 256, shm, ctx->stream>>>(A, n, na, M_dev, nb, Y, n, n, alpha, beta); \
   } while (0)
     if (prec == OMEN_F64) { if (cplx) COMB_LAUNCH2(double, true); else COMB_LAUNCH2(double, false); }
     else { if (cplx) COMB_LAUNCH2(float, true); else COMB_LAUNCH2(float, false); }
@@ -1410,18 +1733,15 @@ struct KrylovOps {
       OMEN_CHECK_LAUNCH(ctx);
       return OMEN_OK;
     }
-    const int ig1 = dots_ig_for(na, dots1_ig(cplx));
-    const int rows = (int)dot_rows(na, ig1);
-    const long long nchunks = (n + rows - 1) / rows;
-    omen_status s1 = ensure_partial((size_t)nchunks * na);
+    const DotsShape d = dots_shape(na, n, 1);
+    omen_status s1 = ensure_partial((size_t)d.chunks * na);
     if (s1 != OMEN_OK) return s1;
-    dim3 grid((na + ig1 - 1) / ig1, (unsigned)nchunks);
+    const DotsFinish fin{d_cnt, h_dev, Tm, ldT, js};
     const size_t shm1 = (size_t)na * sizeof(double2);
     const unsigned grid1 = (unsigned)std::min<long long>((n + 255) / 256, (long long)sm_count * 8);
 #define PASSG(Tt, Cc)                                                                                            \
   do {                                                                                                           \
-    launch_dots1<Tt, Cc>(ig1, grid, ctx->stream, Vb, n, na, W, n, rows, d_partial, 0, 0, 0, nullptr, nullptr, gate); \
-    reduce_dev_kernel<<<na, 256, 0, ctx->stream>>>(d_partial, (int)nchunks, na, 1, h_dev, Tm, ldT, js, 0, 0, 0, gate); \
+    launch_dots1<Tt, Cc>(d, 1, ctx->stream, Vb, n, na, W, n, d_partial, fin, 0, nullptr, nullptr, gate);         \
     smem_limit(combine1_kernel<Tt, Cc>, shm1);                                                                   \
     combine1_kernel<Tt, Cc><<<grid1, 256, shm1, ctx->stream>>>(Vb, n, na, h_dev, W, n, -1.0, 1.0, 0, 0, 0, nullptr, \
                                                               nullptr, gate);                                   \
@@ -1436,6 +1756,44 @@ struct KrylovOps {
   // the next gated pass (parity) is applied unconditionally (after a restart's full passes)
   omen_status force_next_pass(int parity) {
     OMEN_CUDA(ctx, cudaMemsetAsync(ctx->d_status + 2 + (parity ^ 1), 1, sizeof(int), ctx->stream));
+    return OMEN_OK;
+  }
+
+  // w -= h v_j + T[js, js-1] v_{j-1}, the entry mirrored to T[js-1, js]
+  omen_status three_term(const void* Vj, const void* Vp, const double2* h_dev, double2* Tm, int ldT, int js, void* W) {
+    const unsigned grid = (unsigned)std::min<long long>((n + 255) / 256, (long long)sm_count * 8);
+#define TERM3(T, Cc) three_term_kernel<T, Cc><<<grid, 256, 0, ctx->stream>>>(Vj, Vp, h_dev, Tm, ldT, js, W, n)
+    if (prec == OMEN_F64) { if (cplx) TERM3(double, true); else TERM3(double, false); }
+    else { if (cplx) TERM3(float, true); else TERM3(float, false); }
+#undef TERM3
+    OMEN_CHECK_LAUNCH(ctx);
+    return OMEN_OK;
+  }
+
+  // W -= V h, then v_new = W / ||W||, the norm into T[row, col] (nrm: two entries)
+  omen_status update_and_normalize(const void* Vb, int na, const double2* h_dev, void* W, double2* nrm, double2* Tm, int ldT,
+                                   int row, int col, void* Vnew) {
+    // rows a CTA: 256, or 32 with eight threads a row where that leaves SMs idle
+    const bool few = (n + 255) / 256 < sm_count;
+    const unsigned grid = (unsigned)std::min<long long>((n + (few ? 31 : 255)) / (few ? 32 : 256), (long long)sm_count * (few ? 4 : 8));
+    const size_t shm = (size_t)na * sizeof(double2);
+    int* flag = ctx->d_status + 1;
+    int* cnt = d_cnt + kCounters - 1;
+#define UPDN(T, Cc)                                                                                               \
+  do {                                                                                                            \
+    if (few) {                                                                                                    \
+      smem_limit(update_norm_kernel<T, Cc, 8>, shm);                                                              \
+      update_norm_kernel<T, Cc, 8><<<grid, 256, shm, ctx->stream>>>(Vb, na, h_dev, W, n, d_npart, cnt, nrm, Tm, ldT, row, col, flag); \
+    } else {                                                                                                      \
+      smem_limit(update_norm_kernel<T, Cc, 1>, shm);                                                              \
+      update_norm_kernel<T, Cc, 1><<<grid, 256, shm, ctx->stream>>>(Vb, na, h_dev, W, n, d_npart, cnt, nrm, Tm, ldT, row, col, flag); \
+    }                                                                                                             \
+    scale_kernel<T, Cc><<<(unsigned)std::min<long long>((n + 255) / 256, (long long)sm_count * 8), 256, 0, ctx->stream>>>(W, Vnew, n, nrm); \
+  } while (0)
+    if (prec == OMEN_F64) { if (cplx) UPDN(double, true); else UPDN(double, false); }
+    else { if (cplx) UPDN(float, true); else UPDN(float, false); }
+#undef UPDN
+    OMEN_CHECK_LAUNCH(ctx);
     return OMEN_OK;
   }
 
@@ -1470,23 +1828,16 @@ struct KrylovOps {
   omen_status dots_dev_batch(int P, const void* A, long long lda, int na, const void* B, double2* out_dev,
                              long long out_ps, double2* accT, int ldT, long long t_ps, int col0) {
     // the P problems share the grid: chunks sized for about two CTAs per SM over the batch
-    const int igb = dots_ig_for(na, dots1_ig(cplx));
-    const long long groups = (na + igb - 1) / igb;
-    const long long want = std::max<long long>(1, (2LL * sm_count + groups * P - 1) / (groups * P));
-    long long rows = (b_nmax + want - 1) / want;
-    rows = std::min<long long>(8192, std::max<long long>(256, (rows + 255) / 256 * 256));
-    while ((b_nmax + rows - 1) / rows > 65535) rows *= 2;
-    const long long nchunks = (b_nmax + rows - 1) / rows;
-    const long long pps = nchunks * na;
+    const DotsShape d = dots_shape(na, b_nmax, P);
+    const long long pps = d.chunks * na;
     omen_status s1 = ensure_partial((size_t)pps * P);
     if (s1 != OMEN_OK) return s1;
-    dim3 grid((unsigned)groups, (unsigned)nchunks, P);
 #define DOTSB(T, Cc) \
-  launch_dots1<T, Cc>(igb, grid, ctx->stream, A, lda, na, B, b_nmax, (int)rows, d_partial, 0, 0, pps, b_off, b_len, b_act)
+  launch_dots1<T, Cc>(d, P, ctx->stream, A, lda, na, B, b_nmax, d_partial, DotsFinish{}, pps, b_off, b_len, b_act)
     if (prec == OMEN_F64) { if (cplx) DOTSB(double, true); else DOTSB(double, false); }
     else { if (cplx) DOTSB(float, true); else DOTSB(float, false); }
 #undef DOTSB
-    reduce_dev_kernel<<<dim3(na, P), 256, 0, ctx->stream>>>(d_partial, (int)nchunks, na, 1, out_dev, accT, ldT, col0, pps,
+    reduce_dev_kernel<<<dim3(na, P), 256, 0, ctx->stream>>>(d_partial, (int)d.chunks, na, 1, out_dev, accT, ldT, col0, pps,
                                                             out_ps, t_ps, b_act);
     OMEN_CHECK_LAUNCH(ctx);
     return OMEN_OK;
@@ -2137,6 +2488,17 @@ static omen_status lanczos_solve_single(KrylovOps& op, const omen_eig_opts* o, v
     long long unused = 0;
     omen_status s2 = op.apply(op.col(V, js), W, tmp, 1, folded, o->sigma, unused);
     if (s2 != OMEN_OK) return s2;
+    if (!semi && !pro && op.prec != OMEN_F64_DF) {
+      // the full policy, the last pass together with the norm: after a restart two passes over
+      // the basis, else the three-term step and one
+      s2 = fr ? op.dots_dev(V, nb, W, 1, dh, dT, ldT, js) : op.dots_dev(op.col(V, js), 1, W, 1, dh, dT + js, ldT, js);
+      if (s2 == OMEN_OK)
+        s2 = fr ? op.combine_dev(V, nb, dh, 1, W, -1.0, 1.0)
+                : op.three_term(op.col(V, js), op.col(V, js - 1), dh, dT, ldT, js, W);
+      if (s2 == OMEN_OK) s2 = op.dots_dev(V, nb, W, 1, dh, dT, ldT, js);
+      if (s2 == OMEN_OK) s2 = op.update_and_normalize(V, nb, dh, W, dn, dT, ldT, nb, js, op.col(V, nb));
+      return s2;
+    }
     if (fr) {
       // two full classical Gram–Schmidt passes
       for (int pass = 0; pass < 2 && s2 == OMEN_OK; ++pass) {
@@ -2198,9 +2560,11 @@ static omen_status lanczos_solve_single(KrylovOps& op, const omen_eig_opts* o, v
     s = op.ensure_partial(op.max_partials(m + 1));
     if (s != OMEN_OK) return s;
   }
-  while (true) {
-    // the steps up to and including the next host check run as one segment
-    int nseg = 0;
+  // the steps up to and including the next host check run as one segment; `ahead` holds the length of
+  // one that was issued before the host looked at the check before it
+  int ahead = 0;
+  auto issue_segment = [&](int& nseg) -> omen_status {
+    nseg = 0;
     for (int nb = nbas, it = iter, sc = since_check;; ++nb) {
       ++nseg;
       if (check_after(nb, ++it, ++sc)) break;
@@ -2214,9 +2578,16 @@ static omen_status lanczos_solve_single(KrylovOps& op, const omen_eig_opts* o, v
       }
       return OMEN_OK;
     };
-    if (use_graphs && nseg >= 2) s = graphs.run({jstart, nbas, fresh ? 1 : 0, nseg}, run_segment);
-    else s = run_segment();
-    if (s != OMEN_OK) return s;
+    if (use_graphs && nseg >= 2) return graphs.run({jstart, nbas, fresh ? 1 : 0, nseg}, run_segment);
+    return run_segment();
+  };
+  while (true) {
+    int nseg = ahead;
+    if (!ahead) {
+      s = issue_segment(nseg);
+      if (s != OMEN_OK) return s;
+    }
+    ahead = 0;
     hx += (long long)nseg * (folded ? 2 : 1);
     iter += nseg;
     since_check += nseg;
@@ -2231,6 +2602,18 @@ static omen_status lanczos_solve_single(KrylovOps& op, const omen_eig_opts* o, v
       OMEN_CUDA(ctx, cudaMemcpyAsync(&flag, ctx->d_status + 1, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
       OMEN_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
       if (flag) return set_err(ctx, OMEN_ENUMERIC, "Lanczos breakdown or non-finite value (zero or NaN norm)");
+      // The basis has room and iterations are left: the next segment runs while the host solves the
+      // projected problem.  It writes only basis vectors and columns of T past those of this check, so
+      // a check that ends the solve leaves it unused (at most one segment).
+      if (!full && iter < max_iter_of(o)) {
+        const int js0 = jstart, nb0 = nbas;
+        jstart = nbas;
+        nbas += 1;
+        s = issue_segment(ahead);
+        jstart = js0;
+        nbas = nb0;
+        if (s != OMEN_OK) return s;
+      }
       // Hermitian projected matrix from the column data (row i <= column j)
       std::vector<cd> Tn((size_t)nbas * nbas);
       for (int j = 0; j < nbas; ++j)
@@ -2882,11 +3265,11 @@ static omen_status kbatch_core(omen_ctx* ctx, const std::vector<KbatchInput>& in
     char* Yout = Out + (size_t)j0 * blk + (size_t)off[p] * op.el;
     const char* Ain = V + (size_t)off[p] * op.el;
     if (prec == OMEN_F64) {
-      smem_limit(combine_kernel<double, true>, shm);
-      combine_kernel<double, true><<<grid, 256, shm, ctx->stream>>>(Ain, lda, nbas, op.d_small, nbj, Yout, lda, n, 1.0, 0.0);
+      smem_limit(combine_kernel<double, true, kMaxBlockCols>, shm);
+      combine_kernel<double, true, kMaxBlockCols><<<grid, 256, shm, ctx->stream>>>(Ain, lda, nbas, op.d_small, nbj, Yout, lda, n, 1.0, 0.0);
     } else {
-      smem_limit(combine_kernel<float, true>, shm);
-      combine_kernel<float, true><<<grid, 256, shm, ctx->stream>>>(Ain, lda, nbas, op.d_small, nbj, Yout, lda, n, 1.0, 0.0);
+      smem_limit(combine_kernel<float, true, kMaxBlockCols>, shm);
+      combine_kernel<float, true, kMaxBlockCols><<<grid, 256, shm, ctx->stream>>>(Ain, lda, nbas, op.d_small, nbj, Yout, lda, n, 1.0, 0.0);
     }
     OMEN_CHECK_LAUNCH(ctx);
     // the small buffer is reused by the next call
