@@ -36,6 +36,7 @@
 #include "sk_device.cuh"
 #include "df.cuh"
 #include "neighbours.cuh"
+#include "pdl.cuh"
 
 template <typename T> struct Cx;
 template <> struct Cx<double> { using t = double2; };
@@ -352,6 +353,7 @@ __global__ void __launch_bounds__(32) hx_split_kernel(const __grid_constant__ Hx
   using V = typename VecT<T, CPLX>::t;
   constexpr int CS = coef_stride(NORB), CELLS = CPLX ? 4 : 8, G = (NORB + 3) / 4;
   __shared__ __align__(16) T tab[2 * 16 * coef_stride(NORB)];
+  pdl_trigger();
   stage_coef<T, NORB>(I.coef, I.ns, tab);
   const Geo& g = I.g;
   const size_t N = g.natoms;
@@ -363,7 +365,7 @@ __global__ void __launch_bounds__(32) hx_split_kernel(const __grid_constant__ Hx
   const bool live = cell_raw < cell1;
   const int cell = live ? cell_raw : cell1 - 1;    // idle lanes repeat the last cell, and store nothing
   const int q = SO ? blockIdx.y : 0, v = blockIdx.z;
-  const V* __restrict__ x = static_cast<const V*>(xv) + I.x_off + (size_t)v * I.nrows;
+  const V* x = static_cast<const V*>(xv) + I.x_off + (size_t)v * I.nrows;
   const int atom = b * g.ncells + cell;
   const int nxy = g.nx * g.ny;
   const int iz = cell / nxy, rem = cell - iz * nxy, iy = rem / g.nx, ix = rem - iy * g.nx;
@@ -378,7 +380,10 @@ __global__ void __launch_bounds__(32) hx_split_kernel(const __grid_constant__ Hx
     sc = I.scale[n.slot];
     sp2 = I.species[n.atom];
   }
-  const V* __restrict__ xp = x + spin + n.atom;
+  T c[CS];
+  load_coef<T, NORB>(tab + (is_a ? 0 : I.ns * I.ns * CS) + (is_a ? sp * I.ns + sp2 : sp2 * I.ns + sp) * CS, c);
+  pdl_wait();      // the vectors and the potential; structure and blocks do not change
+  const V* xp = x + spin + n.atom;
   V xn[NORB], own[G];
 #pragma unroll
   for (int o = 0; o < NORB; ++o) xn[o] = n.ok ? xp[o * N] : v_zero<V>();
@@ -414,8 +419,6 @@ __global__ void __launch_bounds__(32) hx_split_kernel(const __grid_constant__ Hx
       if constexpr (NORB == 10) xs[4 + i] = -xs[4 + i];
     }
   }
-  T c[CS];
-  load_coef<T, NORB>(tab + (is_a ? 0 : I.ns * I.ns * CS) + (is_a ? sp * I.ns + sp2 : sp2 * I.ns + sp) * CS, c);
   T r[4 * G];
   {
     T r0[NORB];
@@ -442,13 +445,13 @@ __global__ void __launch_bounds__(32) hx_split_kernel(const __grid_constant__ Hx
       if constexpr (SO) {
         if (o >= 1 && o <= 3) {
           const int i = o - 1;
-          const V* __restrict__ xo = x + (size_t)((1 - q) * NORB) * N + atom;
+          const V* xo = x + (size_t)((1 - q) * NORB) * N + atom;
           const V first = i == 2 ? xo[2 * N] : x[spin + (i == 0 ? 2 : 1) * N + atom];
           const V t = so_term(q, i, first, i == 2 ? xo[N] : xo[3 * N]);
           out = fma((T)I.lambda[sp], im ? t.y : t.x, out);
         }
       }
-      V* __restrict__ y = static_cast<V*>(yv) + I.x_off + (size_t)v * I.nrows + spin + o * N + atom;
+      V* y = static_cast<V*>(yv) + I.x_off + (size_t)v * I.nrows + spin + o * N + atom;
       if constexpr (CPLX) (im ? y->y : y->x) = out; else *y = out;
     }
   }
@@ -703,8 +706,7 @@ static cudaError_t launch_rows(const HxInst<T>& I, int nvec, HxTile t, double si
     constexpr int cells = CPLX ? 4 : 8;
     const long long items = (long long)((cell1 - cell0 + cells - 1) / cells) * 8;
     const dim3 grid((unsigned)items, SO ? 2 : 1, nvec);   // one warp a CTA: the warps spread over the SMs
-    hx_split_kernel<T, NORB, CPLX, SO><<<grid, 32, 0, st>>>(I, sigma, cell0, cell1, x, y);
-    return cudaGetLastError();
+    return launch_dependent(hx_split_kernel<T, NORB, CPLX, SO>, grid, dim3(32), 0, st, I, sigma, cell0, cell1, x, y);
   }
   // bonds whose amplitudes are loaded together: rb 1 -> 1, 2 -> 2, 5 or 10 -> 4
   const int thr = t.threads ? t.threads : 128;
