@@ -418,8 +418,8 @@ typedef struct {
 typedef struct {
   double rtol;               /* stop when ||r|| <= rtol ||b|| (b - A x in FP64 in both forms) */
   int max_iter;
-  int precision;             /* OMEN_F64: the residual tested is carried from step to step (r - A d
-                                for a direct correction d, the recurrence of CG iterations).
+  int precision;             /* OMEN_F64: the residual tested last is carried from step to step (r - A d
+                                of the second direct correction d, the recurrence of CG iterations).
                                 OMEN_F32_REFINE64: the residual tested is b - A x, formed anew;
                                 CG iterations, where they are needed, run in FP32 with FP64
                                 residual replacement after every 10x drop (reliable updates).

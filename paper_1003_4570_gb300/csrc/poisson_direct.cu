@@ -9,16 +9,17 @@
 // does not meet the tolerance; the test runs on the device, so nothing waits between the two.
 //
 // The transforms take two real lines as one complex line, mixed-radix Stockham stages in shared
-// memory (radix 4 and 2 in registers, other primes by their definition), and are bound by the FP64
-// rate (some 85 operations a point for four transforms of 256 points).  Planes small enough for
-// shared memory are transformed in x and y at once, two planes as one complex plane, with the
-// residual formed as they are read: three launches a correction.
+// memory: radix 4 and 2 in registers, six fused operations for every pair a +- w b; odd primes by their
+// definition, the first of them on sums and differences of mirrored inputs.  They are bound by the
+// FP64 rate (13 operations a point and transform at 256 points: 0.40 ms on 256^3, 86% of the rate).
+// Planes small enough for shared memory are transformed in x and y at once, two planes as one complex
+// plane, with the residual formed as they are read: three launches a correction.
 //
 // Measured against the conjugate gradients this takes the place of (poisson.cu, one cooperative
-// launch, three grid barriers an iteration): 11x11x217 grid to 1e-13 4.95 -> 0.157 ms (two
-// corrections; launches), 256x256x257 to 1e-10 in the mixed form 250 -> 3.41 ms (one correction
-// and its check; the FP64 rate), the error against 64-bit transforms 1.1e-15 -> 0.7e-15 and
-// 9.6e-12 -> 1.1e-14 of the norm.
+// launch, three grid barriers an iteration): 11x11x217 grid to 1e-13 4.95 -> 0.113 ms (two
+// corrections, eight launches of 6 to 20 us), 256x256x257 to 1e-10 in the mixed form 251 -> 2.59 ms (one
+// correction and its check); the error against 64-bit transforms 1.5e-15 -> 1.1e-15 and 2.3e-11 ->
+// 8e-14 of the norm.
 #include <algorithm>
 #include <cmath>
 
@@ -36,13 +37,17 @@ struct Fft {
   int rad[12];
 };
 
+// Odd primes from the largest down (the first stage, without twiddles, then takes the dearest), then
+// 4 and 2.
 Fft plan_of(int n) {
   Fft p{};
   p.n = n;
-  int m = n;
+  int odd[12], no = 0, m = n;
+  for (int r = 3; r <= m; r += 2)
+    while (m % r == 0) odd[no++] = r, m /= r;
+  while (no) p.rad[p.nf++] = odd[--no];
   while (m % 4 == 0) p.rad[p.nf++] = 4, m /= 4;
-  for (int r = 2; m > 1; ++r)
-    while (m % r == 0) p.rad[p.nf++] = r, m /= r;
+  if (m == 2) p.rad[p.nf++] = 2;
   return p;
 }
 
@@ -50,11 +55,16 @@ struct State {
   double bb, rr, stop;
   int active;          // the residual is above the stopping value
   int iterations;
+  int nonzero;         // the start has a component that is not zero
   unsigned arrived;    // blocks of the running residual pass that have left their sums
 };
 
-__device__ __forceinline__ double2 cx_mul(double2 a, double2 b) {
-  return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
+// a + w b and a - w b in six fused operations (the difference as 2 a less the sum)
+__device__ __forceinline__ void turn(double2 a, double2 w, double2 b, double2& sum, double2& dif) {
+  sum.x = fma(w.x, b.x, fma(-w.y, b.y, a.x));
+  sum.y = fma(w.x, b.y, fma(w.y, b.x, a.y));
+  dif.x = fma(2.0, a.x, -sum.x);
+  dif.y = fma(2.0, a.y, -sum.y);
 }
 
 // FFT of `count` lines of p.n points in shared memory; element e of line l at l*ls + e*es.  Ping-pong
@@ -67,6 +77,20 @@ __device__ double2* fft_lines(double2* a, double2* b, const double2* __restrict_
     const int R = p.rad[f], q = n / R, step = q / Ns;
     const int per = R == 4 || R == 2 ? q : n;        // work items of a line
     const int items = count * per;
+    const bool pairs = f == 0 && R >= 5;
+    if (pairs) {
+      // inputs t and R - t of a long odd stage as their sum and difference: half the products
+      const int h = R / 2;
+      for (int it = threadIdx.x; it < count * q * h; it += kT) {
+        const int line = it / (q * h), rem = it - line * q * h, t = rem / q + 1, j = rem - (t - 1) * q;
+        double2* x = a + line * ls + (j + t * q) * es;
+        double2* y = a + line * ls + (j + (R - t) * q) * es;
+        const double2 u = *x, w = *y;
+        *x = make_double2(u.x + w.x, u.y + w.y);
+        *y = make_double2(u.x - w.x, u.y - w.y);
+      }
+      __syncthreads();
+    }
     for (int it = threadIdx.x; it < items; it += kT) {
       int line, w;
       if (es == 1) {
@@ -79,29 +103,46 @@ __device__ double2* fft_lines(double2* a, double2* b, const double2* __restrict_
       const double2* src = a + line * ls;
       double2* dst = b + line * ls;
       if (R == 4) {
-        const int jm = w % Ns;
-        double2 v0 = src[w * es], v1 = src[(w + q) * es], v2 = src[(w + 2 * q) * es], v3 = src[(w + 3 * q) * es];
-        if (jm) {
-          const int t = jm * step;
-          v1 = cx_mul(v1, tw[t]);
-          v2 = cx_mul(v2, tw[2 * t]);
-          v3 = cx_mul(v3, tw[3 * t]);
+        // two layers of a +- w b, the twiddles 1, w, w^2, w^3 as w^2 inside both pairs and w between them
+        const int jm = w % Ns, o = (w - jm) * 4 + jm;
+        const double2 v0 = src[w * es], v1 = src[(w + q) * es], v2 = src[(w + 2 * q) * es], v3 = src[(w + 3 * q) * es];
+        double2 s02, d02, s13, d13, y0, y1, y2, y3;
+        if (Ns > 1) {   // the same for all lanes: a branch on jm would run both sides
+          const double2 w1 = tw[jm * step], w2 = tw[2 * jm * step];
+          turn(v0, w2, v2, s02, d02);
+          turn(v1, w2, v3, s13, d13);
+          turn(s02, w1, s13, y0, y2);
+          turn(d02, make_double2(w1.y, -w1.x), d13, y1, y3);                  // -i w
+        } else {
+          s02 = make_double2(v0.x + v2.x, v0.y + v2.y), d02 = make_double2(v0.x - v2.x, v0.y - v2.y);
+          s13 = make_double2(v1.x + v3.x, v1.y + v3.y), d13 = make_double2(v1.x - v3.x, v1.y - v3.y);
+          y0 = make_double2(s02.x + s13.x, s02.y + s13.y), y2 = make_double2(s02.x - s13.x, s02.y - s13.y);
+          y1 = make_double2(d02.x + d13.y, d02.y - d13.x), y3 = make_double2(d02.x - d13.y, d02.y + d13.x);
         }
-        const double2 s02 = make_double2(v0.x + v2.x, v0.y + v2.y), d02 = make_double2(v0.x - v2.x, v0.y - v2.y);
-        const double2 s13 = make_double2(v1.x + v3.x, v1.y + v3.y), d13 = make_double2(v1.x - v3.x, v1.y - v3.y);
-        const int o = (w - jm) * 4 + jm;
-        dst[o * es] = make_double2(s02.x + s13.x, s02.y + s13.y);
-        dst[(o + Ns) * es] = make_double2(d02.x + d13.y, d02.y - d13.x);       // d02 - i d13
-        dst[(o + 2 * Ns) * es] = make_double2(s02.x - s13.x, s02.y - s13.y);
-        dst[(o + 3 * Ns) * es] = make_double2(d02.x - d13.y, d02.y + d13.x);
+        dst[o * es] = y0;
+        dst[(o + Ns) * es] = y1;
+        dst[(o + 2 * Ns) * es] = y2;
+        dst[(o + 3 * Ns) * es] = y3;
       } else if (R == 2) {
-        const int jm = w % Ns;
-        const double2 v0 = src[w * es];
-        double2 v1 = src[(w + q) * es];
-        if (jm) v1 = cx_mul(v1, tw[jm * step]);
-        const int o = (w - jm) * 2 + jm;
-        dst[o * es] = make_double2(v0.x + v1.x, v0.y + v1.y);
-        dst[(o + Ns) * es] = make_double2(v0.x - v1.x, v0.y - v1.y);
+        const int jm = w % Ns, o = (w - jm) * 2 + jm;
+        const double2 v0 = src[w * es], v1 = src[(w + q) * es];
+        double2 y0, y1;
+        if (Ns > 1) turn(v0, tw[jm * step], v1, y0, y1);
+        else y0 = make_double2(v0.x + v1.x, v0.y + v1.y), y1 = make_double2(v0.x - v1.x, v0.y - v1.y);
+        dst[o * es] = y0;
+        dst[(o + Ns) * es] = y1;
+      } else if (pairs) {
+        // first stage, inputs already as sums and differences of t and R - t
+        const int i = w / q, j = w - i * q, e = i * q;
+        double2 r = src[j * es];
+        for (int t = 1, x = e; t <= R / 2; ++t) {
+          const double2 a = src[(j + t * q) * es], d = src[(j + (R - t) * q) * es], c = tw[x];
+          r.x = fma(-d.y, c.y, fma(a.x, c.x, r.x));
+          r.y = fma(d.x, c.y, fma(a.y, c.x, r.y));
+          x += e;
+          if (x >= n) x -= n;
+        }
+        dst[(j * R + i) * es] = r;
       } else {
         // one output: sum_t src[j + t q] exp(-2 pi i t e / n)
         const int i = w / q, j = w - i * q, jm = j % Ns;
@@ -126,17 +167,19 @@ __device__ double2* fft_lines(double2* a, double2* b, const double2* __restrict_
   return a;
 }
 
-// Twice the Hartley transforms of the two real lines (planes) whose complex FFT holds z at k and
-// zm at -k.
-__device__ __forceinline__ double2 hartley2(double2 z, double2 zm) {
-  return make_double2((z.x + zm.x) - (z.y - zm.y), (z.y + zm.y) + (z.x - zm.x));
+// Twice the Hartley transforms, at k and -k, of the two real lines (planes) whose complex FFT holds z
+// at k and zm at -k.
+__device__ __forceinline__ void hartley2(double2 z, double2 zm, double2& at, double2& mirror) {
+  const double s = z.x + zm.x, d = z.y - zm.y, t = z.y + zm.y, e = z.x - zm.x;
+  at = make_double2(s - d, t + e);
+  mirror = make_double2(s + d, t - e);
 }
 
 // Leaves the block's sum with the others'; the last block to arrive adds all of them in block
 // order and sets the state: the squared residual, and on the first pass ||b||^2 and the stopping
 // value.  All threads of the block call it.
 template <bool FIRST>
-__device__ void finish_residual(double lrr, double lbb, double* part, State* st, double rtol, int max_iter) {
+__device__ void finish_residual(double lrr, double lbb, double* part, State* st, double rtol, int max_iter, int blocks) {
   __shared__ double sh[32];
   __shared__ bool last;
   const double v = block_sum(lrr, sh);
@@ -144,17 +187,17 @@ __device__ void finish_residual(double lrr, double lbb, double* part, State* st,
   if constexpr (FIRST) w = block_sum(lbb, sh);
   if (threadIdx.x == 0) {
     part[blockIdx.x] = v;
-    if constexpr (FIRST) part[gridDim.x + blockIdx.x] = w;
+    if constexpr (FIRST) part[blocks + blockIdx.x] = w;
     __threadfence();
-    last = atomicAdd(&st->arrived, 1u) == gridDim.x - 1;
+    last = atomicAdd(&st->arrived, 1u) == (unsigned)blocks - 1;
   }
   __syncthreads();
   if (!last) return;
   __threadfence();
   double a = 0.0, c = 0.0;
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+  for (int b = threadIdx.x; b < blocks; b += blockDim.x) {
     a += __ldcg(part + b);
-    if constexpr (FIRST) c += __ldcg(part + gridDim.x + b);
+    if constexpr (FIRST) c += __ldcg(part + blocks + b);
   }
   a = block_sum(a, sh);
   if constexpr (FIRST) c = block_sum(c, sh);
@@ -170,8 +213,8 @@ __device__ void finish_residual(double lrr, double lbb, double* part, State* st,
   }
 }
 
-// How a residual is formed
-enum { kFromX = 0, kFromD = 1 };     // b - A x; or the residual kept so far less A d
+// How a residual is formed: b - A x, b = scale * rho; or the residual kept so far less scale * A d
+enum { kFromX = 0, kFromD = 1 };
 
 template <int HOW>
 __device__ __forceinline__ double residual_at(const PGrid& g, const double* __restrict__ rho, double scale,
@@ -182,39 +225,67 @@ __device__ __forceinline__ double residual_at(const PGrid& g, const double* __re
     return b - stencil_at(v, g, i, j, k, idx);
   } else {
     b = 0.0;
-    return r[idx] - stencil_at(v, g, i, j, k, idx);
+    return fma(-scale, stencil_at(v, g, i, j, k, idx), r[idx]);
   }
 }
 
+// Whether the start has a component that is not zero.  From the zero field, the usual start, the
+// first residual is the right-hand side: 2 FP64 operations a point instead of 16, on the pipe that
+// bounds it (256^3: 461 us; 80 + 28 us with this pass over
+// the start).
+__global__ void __launch_bounds__(kT) nonzero_kernel(const double* __restrict__ x, long long n, State* st) {
+  bool any = false;
+  for (long long i = (long long)blockIdx.x * kT + threadIdx.x; i < n; i += (long long)gridDim.x * kT)
+    any |= (__double_as_longlong(x[i]) << 1) != 0;
+  if (any) st->nonzero = 1;
+}
+
 // r = residual on the whole grid and its square sum: rows over the warps of the grid, points of a
-// row over the lanes.
+// row over the lanes, or narrow rows' points over all lanes.
 template <int HOW, bool FIRST>
 __global__ void __launch_bounds__(kT) residual_kernel(PGrid g, const double* __restrict__ rho, double scale,
                                                       const double* __restrict__ v, double* r, double* part,
                                                       State* st, double rtol, int max_iter) {
   if (!FIRST && !st->active) return;
-  const int lane = threadIdx.x & 31, nw = (gridDim.x * kT) >> 5;
-  const int rows = g.ny * g.nzi;
   double lrr = 0.0, lbb = 0.0;
-  for (int rw = (blockIdx.x * kT + threadIdx.x) >> 5; rw < rows; rw += nw) {
-    const int k = rw / g.ny, j = rw - k * g.ny;
-    const long long base = (long long)rw * g.nx;
-    for (int i = lane; i < g.nx; i += 32) {
-      double b;
-      const double ri = residual_at<HOW>(g, rho, scale, v, r, i, j, k, base + i, b);
-      r[base + i] = ri;
-      lrr = fma(ri, ri, lrr);
-      if constexpr (FIRST) lbb = fma(b, b, lbb);
+  if (FIRST && HOW == kFromX && !st->nonzero) {
+    for (long long i = (long long)blockIdx.x * kT + threadIdx.x; i < g.n; i += (long long)gridDim.x * kT) {
+      const double b = scale * rho[i];
+      r[i] = b;
+      lrr = fma(b, b, lrr);
+    }
+    finish_residual<FIRST>(lrr, lrr, part, st, rtol, max_iter, (int)gridDim.x);
+    return;
+  }
+  auto point = [&](int i, int j, int k, long long idx) {
+    double b;
+    const double ri = residual_at<HOW>(g, rho, scale, v, r, i, j, k, idx, b);
+    r[idx] = ri;
+    lrr = fma(ri, ri, lrr);
+    if constexpr (FIRST) lbb = fma(b, b, lbb);
+  };
+  if (g.nx >= 24) {
+    const int lane = threadIdx.x & 31, nw = (gridDim.x * kT) >> 5;
+    const int rows = g.ny * g.nzi;
+    for (int rw = (blockIdx.x * kT + threadIdx.x) >> 5; rw < rows; rw += nw) {
+      const int k = rw / g.ny, j = rw - k * g.ny;
+      const long long base = (long long)rw * g.nx;
+      for (int i = lane; i < g.nx; i += 32) point(i, j, k, base + i);
+    }
+  } else {   // narrow rows: points over the lanes (n < 2^31)
+    for (long long idx = (long long)blockIdx.x * kT + threadIdx.x; idx < g.n; idx += (long long)gridDim.x * kT) {
+      const unsigned t = (unsigned)idx, row = t / (unsigned)g.nx;
+      point((int)(t - row * g.nx), (int)(row % (unsigned)g.ny), (int)(row / (unsigned)g.ny), idx);
     }
   }
-  finish_residual<FIRST>(lrr, lbb, part, st, rtol, max_iter);
+  finish_residual<FIRST>(lrr, lbb, part, st, rtol, max_iter, (int)gridDim.x);
 }
 
 // Hartley transform of every row (x lines), P pairs of rows a block.  ADD: the result is the
 // correction, also added to x.
 template <bool ADD>
 __global__ void __launch_bounds__(kT) rows_kernel(const double* src, double* dst, double* __restrict__ x,
-                                                  int nrows, int P, const __grid_constant__ Fft p,
+                                                  double scale, int nrows, int P, const __grid_constant__ Fft p,
                                                   const double2* __restrict__ tw, const State* st) {
   if (!st->active) return;
   extern __shared__ __align__(16) double2 sm[];
@@ -229,15 +300,20 @@ __global__ void __launch_bounds__(kT) rows_kernel(const double* src, double* dst
   }
   __syncthreads();
   const double2* Z = fft_lines(A, B, W, p, have, 1, n);
-  for (int it = threadIdx.x; it < have * n; it += kT) {
-    const int l = it / n, e = it - l * n, ra = r0 + 2 * l;
-    const double2 h = hartley2(Z[it], Z[l * n + (e ? n - e : 0)]);
-    const long long at = (long long)ra * n + e;
-    dst[at] = h.x;
-    if constexpr (ADD) x[at] += h.x;
-    if (ra + 1 < nrows) {
-      dst[at + n] = h.y;
-      if constexpr (ADD) x[at + n] += h.y;
+  const int half = n / 2 + 1;
+  for (int it = threadIdx.x; it < have * half; it += kT) {
+    const int l = it / half, e = it - l * half, em = e ? n - e : 0, ra = r0 + 2 * l;
+    double2 h[2];
+    hartley2(Z[l * n + e], Z[l * n + em], h[0], h[1]);
+    const bool both = em != e;
+    for (int m = 0; m <= (both ? 1 : 0); ++m) {
+      const long long at = (long long)ra * n + (m ? em : e);
+      dst[at] = h[m].x;
+      if constexpr (ADD) x[at] = fma(scale, h[m].x, x[at]);
+      if (ra + 1 < nrows) {
+        dst[at + n] = h[m].y;
+        if constexpr (ADD) x[at + n] = fma(scale, h[m].y, x[at + n]);
+      }
     }
   }
 }
@@ -261,31 +337,91 @@ __global__ void __launch_bounds__(kT) columns_kernel(double* __restrict__ v, int
   }
   __syncthreads();
   const double2* Z = fft_lines(A, B, W, p, P, P, 1);
-  for (int it = threadIdx.x; it < P * n; it += kT) {
-    const int e = it / P, l = it - e * P;
-    const double2 h = hartley2(Z[it], Z[(e ? n - e : 0) * P + l]);
-    double* s = base + (long long)e * nx + 2 * l;
-    if (2 * l < cols) s[0] = h.x;
-    if (2 * l + 1 < cols) s[1] = h.y;
+  for (int it = threadIdx.x; it < P * (n / 2 + 1); it += kT) {
+    const int e = it / P, l = it - e * P, em = e ? n - e : 0;
+    double2 h[2];
+    hartley2(Z[e * P + l], Z[em * P + l], h[0], h[1]);
+    for (int m = 0; m <= (em != e ? 1 : 0); ++m) {
+      double* s = base + (long long)(m ? em : e) * nx + 2 * l;
+      if (2 * l < cols) s[0] = h[m].x;
+      if (2 * l + 1 < cols) s[1] = h[m].y;
+    }
   }
 }
+
+// The tridiagonal systems' pivots c_j = 1 / (delta - c_{j-1}), c_1 = 1 / delta, delta = 2 + lambda / cz,
+// for the (nx/2+1)(ny/2+1) different eigenvalues lambda = 4 cx sin^2(pi kx / nx) + 4 cy sin^2(pi ky / ny):
+// ctab[j-1][ky][kx].  In closed form c_j = e^-t expm1(-2 j t) / expm1(-2 (j+1) t), sinh^2(t/2) =
+// lambda / (4 cz) (j / (j+1) for lambda = 0); a thread starts from it and runs the recurrence for
+// `run` unknowns, until it stands still (most modes: after some 20 / t unknowns).
+__device__ void pivots(const PGrid& g, double* __restrict__ ctab, long long t0, long long stride, int run) {
+  const int hx = g.nx / 2 + 1, hy = g.ny / 2 + 1, modes = hx * hy;
+  const long long total = (long long)modes * ((g.nzi + run - 1) / run);
+  for (long long t = t0; t < total; t += stride) {
+    const int ch = (int)(t / modes), md = (int)(t - (long long)ch * modes);
+    const int ky = md / hx, kx = md - ky * hx;
+    const double sx = sinpi((double)kx / g.nx), sy = sinpi((double)ky / g.ny);
+    const double s = (g.cx * sx * sx + g.cy * sy * sy) / g.cz;      // lambda / (4 cz)
+    const int j0 = ch * run + 1, j1 = min(j0 + run - 1, g.nzi);
+    const double delta = fma(4.0, s, 2.0);
+    double c;
+    if (s == 0.0) {
+      c = (double)j0 / (j0 + 1);
+    } else {
+      const double th = 2.0 * asinh(sqrt(s));
+      c = exp(-th) * (expm1(-2.0 * j0 * th) / expm1(-2.0 * (j0 + 1) * th));
+    }
+    bool still = false;
+    for (int j = j0;; ++j) {
+      ctab[(long long)(j - 1) * modes + md] = c;
+      if (j == j1) break;
+      if (!still) {
+        const double next = 1.0 / (delta - c);
+        still = next == c;
+        c = next;
+      }
+    }
+  }
+}
+
+// Pivots and the twiddles of both directions, for grids whose planes are not transformed at once.
+__global__ void __launch_bounds__(kT) setup_kernel(PGrid g, double2* __restrict__ tw, double* __restrict__ ctab, int run) {
+  const long long t0 = (long long)blockIdx.x * kT + threadIdx.x, stride = (long long)gridDim.x * kT;
+  for (long long i = t0; i < g.nx + g.ny; i += stride) {
+    double s, c;
+    sincospi(i < g.nx ? -2.0 * i / g.nx : -2.0 * (i - g.nx) / g.ny, &s, &c);
+    tw[i] = make_double2(c, s);
+  }
+  if (ctab) pivots(g, ctab, t0, stride, run);
+}
+
+// Twiddles of small planes, with the launch.
+constexpr int kInlineTwiddles = 128;
+struct PlaneTwiddles {
+  double2 w[kInlineTwiddles];
+};
 
 // Small planes: two planes a block as one complex plane, x and y lines transformed together (the
 // Hartley transform over the plane, cas of the summed phase, which the operator's eigenvectors
 // share as well).  FORWARD: the residual is formed as the planes are read (and kept in r), its
-// transform written to `hat`; else `hat` is transformed back into the correction d, added to x.
-template <bool FORWARD, int HOW, bool FIRST>
+// transform written to `hat`; else `hat` is transformed back into the correction d (still to be
+// multiplied by `inv`), added to x.  The first launch forms the pivots as well, in blocks of its own.
+template <bool FORWARD, bool FIRST>
 __global__ void __launch_bounds__(kT) planes_kernel(PGrid g, const double* __restrict__ rho, double scale, double* __restrict__ x,
                                                     double* r, double* __restrict__ d, double* __restrict__ hat,
-                                                    double* part, State* st, double rtol, int max_iter,
+                                                    double* part, State* st, double rtol, int max_iter, double inv,
                                                     const __grid_constant__ Fft px, const __grid_constant__ Fft py,
-                                                    const double2* __restrict__ twx, const double2* __restrict__ twy) {
+                                                    const __grid_constant__ PlaneTwiddles tw, const double2* __restrict__ twd,
+                                                    double* __restrict__ ctab, int nplanes) {
   if (!FIRST && !st->active) return;
+  if (FIRST && (int)blockIdx.x >= nplanes) {           // the blocks past the planes form the pivots
+    pivots(g, ctab, ((long long)blockIdx.x - nplanes) * kT + threadIdx.x, (long long)(gridDim.x - nplanes) * kT, 1);
+    return;
+  }
   extern __shared__ __align__(16) double2 sm[];
   const int nx = g.nx, ny = g.ny, np = nx * ny;
   double2 *A = sm, *B = sm + np, *WX = sm + 2 * np, *WY = WX + nx;
-  for (int i = threadIdx.x; i < nx; i += kT) WX[i] = twx[i];
-  for (int i = threadIdx.x; i < ny; i += kT) WY[i] = twy[i];
+  for (int i = threadIdx.x; i < nx + ny; i += kT) WX[i] = twd ? twd[i] : tw.w[i];
   const int k0 = blockIdx.x * 2;
   const bool two = k0 + 1 < g.nzi;
   const long long base = (long long)k0 * np;
@@ -293,12 +429,11 @@ __global__ void __launch_bounds__(kT) planes_kernel(PGrid g, const double* __res
   for (int it = threadIdx.x; it < np; it += kT) {
     const int j = it / nx, i = it - j * nx;
     if constexpr (FORWARD) {
-      const double* v = HOW == kFromX ? x : d;
       double b0, b1 = 0.0, q1 = 0.0;
-      const double q0 = residual_at<HOW>(g, rho, scale, v, r, i, j, k0, base + it, b0);
+      const double q0 = residual_at<kFromX>(g, rho, scale, x, r, i, j, k0, base + it, b0);
       r[base + it] = q0;
       if (two) {
-        q1 = residual_at<HOW>(g, rho, scale, v, r, i, j, k0 + 1, base + np + it, b1);
+        q1 = residual_at<kFromX>(g, rho, scale, x, r, i, j, k0 + 1, base + np + it, b1);
         r[base + np + it] = q1;
       }
       lrr = fma(q0, q0, fma(q1, q1, lrr));
@@ -313,84 +448,42 @@ __global__ void __launch_bounds__(kT) planes_kernel(PGrid g, const double* __res
   const double2* Z = fft_lines(X, X == A ? B : A, WY, py, nx, nx, 1);
   for (int it = threadIdx.x; it < np; it += kT) {
     const int j = it / nx, i = it - j * nx;
-    const double2 h = hartley2(Z[it], Z[(j ? ny - j : 0) * nx + (i ? nx - i : 0)]);
-    if constexpr (FORWARD) {
-      hat[base + it] = h.x;
-      if (two) hat[base + np + it] = h.y;
-    } else {
-      d[base + it] = h.x;
-      x[base + it] += h.x;
-      if (two) {
-        d[base + np + it] = h.y;
-        x[base + np + it] += h.y;
-      }
-    }
-  }
-  if constexpr (FORWARD) finish_residual<FIRST>(lrr, lbb, part, st, rtol, max_iter);
-}
-
-// Twiddles of both directions, and the tridiagonal systems' pivots c_j = 1 / (delta - c_{j-1}),
-// c_1 = 1 / delta, delta = 2 + lambda / cz, for the (nx/2+1)(ny/2+1) different eigenvalues
-// lambda = 4 cx sin^2(pi kx / nx) + 4 cy sin^2(pi ky / ny): ctab[j-1][ky][kx].  In closed form
-// c_j = e^-t expm1(-2 j t) / expm1(-2 (j+1) t), sinh^2(t/2) = lambda / (4 cz) (j / (j+1) for
-// lambda = 0); a thread starts from it and runs the recurrence for kPivots unknowns.
-constexpr int kPivots = 16;
-
-__global__ void __launch_bounds__(kT) setup_kernel(PGrid g, double2* __restrict__ twx, double2* __restrict__ twy,
-                                                   double* __restrict__ ctab, State* st) {
-  const long long t0 = (long long)blockIdx.x * kT + threadIdx.x, stride = (long long)gridDim.x * kT;
-  if (t0 == 0) st->arrived = 0;
-  const int hx = g.nx / 2 + 1, hy = g.ny / 2 + 1, modes = hx * hy;
-  const int chunks = (g.nzi + kPivots - 1) / kPivots;
-  const long long total = (long long)modes * chunks;
-  for (long long t = t0; t < total + g.nx + g.ny; t += stride) {
-    if (t >= total) {
-      const int i = (int)(t - total);
-      double s, c;
-      if (i < g.nx) {
-        sincospi(-2.0 * i / g.nx, &s, &c);
-        twx[i] = make_double2(c, s);
+    const int im = (j ? ny - j : 0) * nx + (i ? nx - i : 0);
+    if (im < it) continue;                             // the lower of k and -k does both
+    double2 h[2];
+    hartley2(Z[it], Z[im], h[0], h[1]);
+    for (int m = 0; m <= (im != it ? 1 : 0); ++m) {
+      const long long at = base + (m ? im : it);
+      if constexpr (FORWARD) {
+        hat[at] = h[m].x;
+        if (two) hat[at + np] = h[m].y;
       } else {
-        sincospi(-2.0 * (i - g.nx) / g.ny, &s, &c);
-        twy[i - g.nx] = make_double2(c, s);
+        d[at] = h[m].x;
+        x[at] = fma(inv, h[m].x, x[at]);
+        if (two) {
+          d[at + np] = h[m].y;
+          x[at + np] = fma(inv, h[m].y, x[at + np]);
+        }
       }
-      continue;
-    }
-    const int ch = (int)(t / modes), md = (int)(t - (long long)ch * modes);
-    const int ky = md / hx, kx = md - ky * hx;
-    const double sx = sinpi((double)kx / g.nx), sy = sinpi((double)ky / g.ny);
-    const double s = (g.cx * sx * sx + g.cy * sy * sy) / g.cz;      // lambda / (4 cz)
-    const int j0 = ch * kPivots + 1, j1 = min(j0 + kPivots - 1, g.nzi);
-    const double delta = fma(4.0, s, 2.0);
-    double c;
-    if (s == 0.0) {
-      c = (double)j0 / (j0 + 1);
-    } else {
-      const double th = 2.0 * asinh(sqrt(s));
-      c = exp(-th) * (expm1(-2.0 * j0 * th) / expm1(-2.0 * (j0 + 1) * th));
-    }
-    ctab[(long long)(j0 - 1) * modes + md] = c;
-    for (int j = j0 + 1; j <= j1; ++j) {
-      c = 1.0 / (delta - c);
-      ctab[(long long)(j - 1) * modes + md] = c;
     }
   }
+  if constexpr (FORWARD) finish_residual<FIRST>(lrr, lbb, part, st, rtol, max_iter, nplanes);
 }
 
-// The tridiagonal systems of 32 modes (kx, ky), in place: warp s of the block takes unknowns
-// [s L, (s+1) L) of each.  Forward g_j = c_j (f_j + g_{j-1}) and backward u_j = g_j + c_j u_{j+1}
+// The tridiagonal systems of blockDim.x modes (kx, ky), in place: thread row s of the block takes
+// unknowns [s L, (s+1) L) of each.  Forward g_j = c_j (f_j + g_{j-1}) and backward u_j = g_j + c_j u_{j+1}
 // are linear in what enters a segment, so each warp first finds what its segment returns for
 // nothing entering, the segments' chain is followed by one warp, and the sweeps run with it.
 // The segment's f and c stay in registers between the sweeps: v is read and written once.
 // (L = 32 with 1024 threads, for more than 256 unknowns, spills part of them to L1.)
 template <int L, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) tridiag_kernel(PGrid g, double* __restrict__ v, const double* __restrict__ ctab,
-                                                                 double scale, State* st) {
+                                                                 State* st) {
   if (!st->active) return;
   __shared__ double out[32][33], prod[32][33];       // [segment][lane]
   const int lane = threadIdx.x, s = threadIdx.y, S = blockDim.y;
   const int np = g.nx * g.ny;
-  const int mode = blockIdx.x * 32 + lane;
+  const int mode = blockIdx.x * blockDim.x + lane;
   const bool live = mode < np;
   const int ky = live ? mode / g.nx : 0, kx = live ? mode - ky * g.nx : 0;
   const int hx = g.nx / 2 + 1, modes = hx * (g.ny / 2 + 1);
@@ -406,7 +499,7 @@ __global__ void __launch_bounds__(THREADS, 1) tridiag_kernel(PGrid g, double* __
   double e = 0.0, pr = 1.0;
 #pragma unroll
   for (int j = 0; j < L; ++j) {
-    h[j] = h[j] * scale * c[j];
+    h[j] *= c[j];
     e = fma(c[j], e, h[j]);
     pr *= c[j];
   }
@@ -475,7 +568,7 @@ omen_status poisson_direct(omen_ctx* ctx, const PGrid& g, const double* rho, dou
   const int nblocks = std::max(rblocks, pblocks);
   auto pad = [](size_t b) { return (b + 255) / 256 * 256; };
   const size_t bv = pad(sizeof(double) * (size_t)n), bc = pad(sizeof(double) * (size_t)(modes * g.nzi));
-  const size_t bt = pad(sizeof(double2) * (size_t)g.nx) + pad(sizeof(double2) * (size_t)g.ny);
+  const size_t bt = pad(sizeof(double2) * ((size_t)g.nx + g.ny));
   const size_t bytes = (planes ? 3 : 2) * bv + bc + bt + pad(sizeof(double) * 2 * (size_t)nblocks) + pad(sizeof(State));
   char* buf = nullptr;
   if (ctx_alloc(ctx, &buf, bytes) != cudaSuccess) {
@@ -488,50 +581,63 @@ omen_status poisson_direct(omen_ctx* ctx, const PGrid& g, const double* rho, dou
   double* d = reinterpret_cast<double*>(take(bv));
   double* hat = planes ? reinterpret_cast<double*>(take(bv)) : d;
   double* ctab = reinterpret_cast<double*>(take(bc));
-  double2* twx = reinterpret_cast<double2*>(take(sizeof(double2) * g.nx));
-  double2* twy = reinterpret_cast<double2*>(take(sizeof(double2) * g.ny));
+  double2* tw = reinterpret_cast<double2*>(take(bt));
   double* part = reinterpret_cast<double*>(take(sizeof(double) * 2 * nblocks));
   State* state = reinterpret_cast<State*>(take(sizeof(State)));
   const Fft px = plan_of(g.nx), py = plan_of(g.ny);
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(state, 0, sizeof(State), st);
   auto ok = [&](cudaError_t c) { if (e == cudaSuccess) e = c; };
 
-  const long long work = modes * ((g.nzi + kPivots - 1) / kPivots) + g.nx + g.ny;
-  setup_kernel<<<(unsigned)std::min<long long>((work + kT - 1) / kT, (long long)sms * 8), kT, 0, st>>>(g, twx, twy, ctab, state);
-  ok(cudaGetLastError());
+  // planes at once take their twiddles with the launch (else from a table) and form the pivots, one a
+  // thread, beside their first transform; line by line, longer runs of the recurrence cost less
+  PlaneTwiddles inl{};
+  const bool with_launch = planes && g.nx + g.ny <= kInlineTwiddles;
+  if (with_launch) {
+    for (int i = 0; i < g.nx + g.ny; ++i) {
+      const double a = i < g.nx ? -2.0 * M_PI * i / g.nx : -2.0 * M_PI * (i - g.nx) / g.ny;
+      inl.w[i] = make_double2(std::cos(a), std::sin(a));
+    }
+  } else {
+    const int run = 64;
+    const long long work = planes ? g.nx + g.ny : std::max<long long>(g.nx + g.ny, modes * ((g.nzi + run - 1) / run));
+    setup_kernel<<<(unsigned)std::min<long long>((work + kT - 1) / kT, (long long)sms * 8), kT, 0, st>>>(g, tw, planes ? nullptr : ctab, run);
+    ok(cudaGetLastError());
+  }
+  const double2* twd = with_launch ? nullptr : tw;
+  const double2 *twx = tw, *twy = tw + g.nx;
 
-  // each transform doubles (hartley2) and the inverse leaves nx ny
+  // each transform doubles (hartley2) and the inverse leaves nx ny; the factor goes in where the
+  // correction is added to x and where A d is taken from the residual
   const double inv = 1.0 / ((planes ? 4.0 : 16.0) * np * g.cz);
-  // unknowns per thread of the tridiagonal solves: long segments (fewer operations) once the modes
-  // alone give every SM a block
+  // modes a block: 32, or fewer where those blocks leave SMs idle; unknowns per thread: long segments
+  // (fewer operations) once the modes alone give every SM a block
   auto tridiag = [&]() {
-    const unsigned blocks = (unsigned)((np + 31) / 32);
-    const int L = g.nzi > 256 || blocks >= 2u * sms ? 32 : blocks >= (unsigned)sms ? 16 : 8;
-    const dim3 thr(32, (g.nzi + L - 1) / L);
-    if (g.nzi > 256) tridiag_kernel<32, 1024><<<blocks, thr, 0, st>>>(g, hat, ctab, inv, state);
-    else if (L == 32) tridiag_kernel<32, 256><<<blocks, thr, 0, st>>>(g, hat, ctab, inv, state);
-    else if (L == 16) tridiag_kernel<16, 512><<<blocks, thr, 0, st>>>(g, hat, ctab, inv, state);
-    else tridiag_kernel<8, 1024><<<blocks, thr, 0, st>>>(g, hat, ctab, inv, state);
+    const int per = np >= 32 * sms ? 32 : np >= 8 * sms ? 8 : 4;
+    const unsigned blocks = (unsigned)((np + per - 1) / per);
+    const int L = g.nzi > 256 || np >= 64 * sms ? 32 : np >= 32 * sms ? 16 : 8;
+    const dim3 thr(per, (g.nzi + L - 1) / L);
+    if (g.nzi > 256) tridiag_kernel<32, 1024><<<blocks, thr, 0, st>>>(g, hat, ctab, state);
+    else if (L == 32) tridiag_kernel<32, 256><<<blocks, thr, 0, st>>>(g, hat, ctab, state);
+    else if (L == 16) tridiag_kernel<16, 512><<<blocks, thr, 0, st>>>(g, hat, ctab, state);
+    else tridiag_kernel<8, 1024><<<blocks, thr, 0, st>>>(g, hat, ctab, state);
     ok(cudaGetLastError());
   };
   const int rounds = std::min(2, max_iter);
   if (planes) {
     const size_t smem = sizeof(double2) * (2 * (size_t)np + g.nx + g.ny);
-    ok(allow_smem(planes_kernel<true, kFromX, true>, smem));
-    ok(allow_smem(planes_kernel<true, kFromX, false>, smem));
-    ok(allow_smem(planes_kernel<true, kFromD, false>, smem));
-    ok(allow_smem(planes_kernel<false, kFromX, false>, smem));
+    ok(allow_smem(planes_kernel<true, true>, smem));
+    ok(allow_smem(planes_kernel<true, false>, smem));
+    ok(allow_smem(planes_kernel<false, false>, smem));
+    const int pivot_blocks = (int)std::min<long long>((modes * g.nzi + kT - 1) / kT, (long long)sms * 4);
+    auto plane_pass = [&](auto kernel, int blocks, double factor) {
+      kernel<<<blocks, kT, smem, st>>>(g, rho, factor, x, r, d, hat, part, state, rtol, max_iter, inv, px, py, inl, twd, ctab, pblocks);
+      ok(cudaGetLastError());
+    };
     for (int i = 0; i < rounds && e == cudaSuccess; ++i) {
-      if (i == 0)
-        planes_kernel<true, kFromX, true><<<pblocks, kT, smem, st>>>(g, rho, scale, x, r, d, hat, part, state, rtol, max_iter, px, py, twx, twy);
-      else if (true_residual)
-        planes_kernel<true, kFromX, false><<<pblocks, kT, smem, st>>>(g, rho, scale, x, r, d, hat, part, state, rtol, max_iter, px, py, twx, twy);
-      else
-        planes_kernel<true, kFromD, false><<<pblocks, kT, smem, st>>>(g, rho, scale, x, r, d, hat, part, state, rtol, max_iter, px, py, twx, twy);
-      ok(cudaGetLastError());
+      if (i == 0) plane_pass(planes_kernel<true, true>, pblocks + pivot_blocks, scale);
+      else plane_pass(planes_kernel<true, false>, pblocks, scale);
       tridiag();
-      planes_kernel<false, kFromX, false><<<pblocks, kT, smem, st>>>(g, rho, scale, x, r, d, hat, part, state, rtol, max_iter, px, py, twx, twy);
-      ok(cudaGetLastError());
+      plane_pass(planes_kernel<false, false>, pblocks, scale);
     }
   } else {
     // pairs of lines a block: up to 2048 complex points, and enough blocks for every SM
@@ -549,26 +655,26 @@ omen_status poisson_direct(omen_ctx* ctx, const PGrid& g, const double* rho, dou
     ok(allow_smem(rows_kernel<false>, smx));
     ok(allow_smem(rows_kernel<true>, smx));
     ok(allow_smem(columns_kernel, smy));
+    nonzero_kernel<<<(unsigned)(sms * 8), kT, 0, st>>>(x, n, state);
     residual_kernel<kFromX, true><<<rblocks, kT, 0, st>>>(g, rho, scale, x, r, part, state, rtol, max_iter);
     ok(cudaGetLastError());
     for (int i = 0; i < rounds && e == cudaSuccess; ++i) {
-      rows_kernel<false><<<bx, kT, smx, st>>>(r, d, x, nrows, PX, px, twx, state);
+      rows_kernel<false><<<bx, kT, smx, st>>>(r, d, x, inv, nrows, PX, px, twx, state);
       columns_kernel<<<by, kT, smy, st>>>(d, g.nx, PY, tiles, py, twy, state);
       ok(cudaGetLastError());
       tridiag();
       columns_kernel<<<by, kT, smy, st>>>(d, g.nx, PY, tiles, py, twy, state);
-      rows_kernel<true><<<bx, kT, smx, st>>>(d, d, x, nrows, PX, px, twx, state);
+      rows_kernel<true><<<bx, kT, smx, st>>>(d, d, x, inv, nrows, PX, px, twx, state);
       ok(cudaGetLastError());
       if (i + 1 < rounds) {
-        if (true_residual) residual_kernel<kFromX, false><<<rblocks, kT, 0, st>>>(g, rho, scale, x, r, part, state, rtol, max_iter);
-        else residual_kernel<kFromD, false><<<rblocks, kT, 0, st>>>(g, rho, scale, d, r, part, state, rtol, max_iter);
+        residual_kernel<kFromX, false><<<rblocks, kT, 0, st>>>(g, rho, scale, x, r, part, state, rtol, max_iter);
         ok(cudaGetLastError());
       }
     }
   }
-  if (e == cudaSuccess) {   // the residual the last correction leaves (skipped once one has passed the test)
+  if (e == cudaSuccess) {   // what the last correction leaves (skipped once one has passed the test)
     if (true_residual) residual_kernel<kFromX, false><<<rblocks, kT, 0, st>>>(g, rho, scale, x, r, part, state, rtol, max_iter);
-    else residual_kernel<kFromD, false><<<rblocks, kT, 0, st>>>(g, rho, scale, d, r, part, state, rtol, max_iter);
+    else residual_kernel<kFromD, false><<<rblocks, kT, 0, st>>>(g, rho, inv, d, r, part, state, rtol, max_iter);
     ok(cudaGetLastError());
   }
   State h{};

@@ -48,6 +48,21 @@ def test_direct_corrections_match_sparse_solve(ctx, n):
         assert info["iterations"] == 0 and torch.equal(again, phi)
 
 
+@pytest.mark.parametrize("n", [(3, 5, 8), (64, 49, 5), (33, 100, 6)], ids=["planes", "lines", "odd_lines"])
+def test_from_the_zero_field(ctx, n):
+    """The first residual from a zero start is the right-hand side; one component that is not zero
+    must send it the general way."""
+    from paper_1003_4570_gb300 import omen
+    g = poisson.Grid(*n, 0.2 * n[0], 0.2 * n[1], 0.2 * n[2])
+    rho = np.random.default_rng(5).normal(size=g.shape) * 1e6
+    ref = poisson.solve_direct(g, rho)
+    for last in (0.0, 1e6 * np.abs(ref).max()):
+        phi = torch.zeros(g.shape, dtype=torch.float64, device="cuda")
+        phi[-1, -1, -1] = last
+        omen.omen_poisson(ctx, g, torch.from_numpy(rho).cuda(), phi, rtol=1e-12)
+        np.testing.assert_allclose(phi.cpu().numpy(), ref, atol=1e-10 * np.abs(ref).max(), rtol=0)
+
+
 def test_iteration_limit_is_kept(ctx):
     from paper_1003_4570_gb300 import omen
     g = poisson.Grid(7, 6, 20, 1.4, 1.2, 4.0)
