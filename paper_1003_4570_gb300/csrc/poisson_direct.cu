@@ -368,8 +368,9 @@ __device__ void pivots(const PGrid& g, double* __restrict__ ctab, long long t0, 
     if (s == 0.0) {
       c = (double)j0 / (j0 + 1);
     } else {
-      const double th = 2.0 * asinh(sqrt(s));
-      c = exp(-th) * (expm1(-2.0 * j0 * th) / expm1(-2.0 * (j0 + 1) * th));
+      // e^-t and expm1(-2 (j+1) t) from expm1(-t) and expm1(-2 j t), without cancellation
+      const double th = 2.0 * asinh(sqrt(s)), e1 = expm1(-th), q = e1 + 1.0, ej = expm1(-2.0 * j0 * th);
+      c = q * (ej / fma(ej, q * q, e1 * (q + 1.0)));
     }
     bool still = false;
     for (int j = j0;; ++j) {
@@ -397,6 +398,7 @@ __global__ void __launch_bounds__(kT) setup_kernel(PGrid g, double2* __restrict_
 
 // Twiddles of small planes, with the launch.
 constexpr int kInlineTwiddles = 128;
+constexpr int kPivotThreads = 64;
 struct PlaneTwiddles {
   double2 w[kInlineTwiddles];
 };
@@ -414,8 +416,10 @@ __global__ void __launch_bounds__(kT) planes_kernel(PGrid g, const double* __res
                                                     const __grid_constant__ PlaneTwiddles tw, const double2* __restrict__ twd,
                                                     double* __restrict__ ctab, int nplanes) {
   if (!FIRST && !st->active) return;
-  if (FIRST && (int)blockIdx.x >= nplanes) {           // the blocks past the planes form the pivots
-    pivots(g, ctab, ((long long)blockIdx.x - nplanes) * kT + threadIdx.x, (long long)(gridDim.x - nplanes) * kT, 1);
+  if (FIRST && (int)blockIdx.x >= nplanes) {           // the blocks past the planes form the pivots,
+    if (threadIdx.x < kPivotThreads)                   // in few warps each: some 200 FP64 operations deep
+      pivots(g, ctab, ((long long)blockIdx.x - nplanes) * kPivotThreads + threadIdx.x,
+             (long long)(gridDim.x - nplanes) * kPivotThreads, 1);
     return;
   }
   extern __shared__ __align__(16) double2 sm[];
@@ -628,7 +632,7 @@ omen_status poisson_direct(omen_ctx* ctx, const PGrid& g, const double* rho, dou
     ok(allow_smem(planes_kernel<true, true>, smem));
     ok(allow_smem(planes_kernel<true, false>, smem));
     ok(allow_smem(planes_kernel<false, false>, smem));
-    const int pivot_blocks = (int)std::min<long long>((modes * g.nzi + kT - 1) / kT, (long long)sms * 4);
+    const int pivot_blocks = (int)std::min<long long>((modes * g.nzi + kPivotThreads - 1) / kPivotThreads, (long long)sms * 8);
     auto plane_pass = [&](auto kernel, int blocks, double factor) {
       kernel<<<blocks, kT, smem, st>>>(g, rho, factor, x, r, d, hat, part, state, rtol, max_iter, inv, px, py, inl, twd, ctab, pblocks);
       ok(cudaGetLastError());
