@@ -7,8 +7,10 @@ operator (H - sigma)^2 to a vector, i.e. two H·X products — the unit the fold
 Lanczos recurrence repeats (the paper times "500 Lanczos iterations").
 
 value = algorithmic bytes of the H·X products of all ranks / max-over-ranks time (GB/s).
-Algorithmic bytes per H·X: every stored bond block once (100 entries per bond), x and y once,
-one species byte and one potential word per atom.
+Algorithmic bytes per H·X: every bond block once (100 entries per bond), x and y once, one species
+byte and one potential word per atom — the unit both arms count in.  The GPU product keeps no
+blocks (one factor per bond and a table of reduced blocks); what it moves and the operations that
+bound it are in `roofline`.
 
 --impl reference: the CPU oracle (scipy CSR product from oracle/) on a bounded sample of the
 same workload, on this host's cores.
@@ -37,13 +39,9 @@ SAMPLE_NZ = 4          # CPU sample: 50 x 50 x 4 cells of the same recipe
 FP64_PEAK_TFLOPS = 1.25  # nominal GB300 FP64 rate (reported beside the DGEMM rate measured in the run)
 
 
-# DRAM bytes (read + write) per bond of one FP64 stored H·X launch, by launch shape (CTA width,
-# block rows per register batch): ncu capture of every shape on the 30^3-cell case of the alloy
-# recipe (profiles/hx_kernel_f64_shapes_sige_alloy.md), scaled to a launch by its bonds
-HX_F64_TRAFFIC_PER_BOND = {(32, 1): 1203.0, (32, 2): 922.4, (64, 1): 1190.2, (64, 2): 917.9, (96, 1): 1160.4,
-                           (96, 2): 924.9, (128, 1): 1151.1, (128, 2): 917.2}
-HX_F64_TRAFFIC_SOURCE = ("profiles/hx_kernel_f64_shapes_sige_alloy.md: ncu dram__bytes of each launch shape "
-                         "at 30^3 cells, per bond x this launch's bonds")
+# FP64 operations of a product by reduced blocks (sp3d5s*): 61 a bond end, 10 an atom for the onsite terms
+HX_OPS_PER_BOND_END = 61
+HX_OPS_PER_ATOM = 10
 
 
 def measured_peaks():
@@ -75,6 +73,18 @@ def alg_bytes_per_hx(nbonds, natoms, nrows, elem, vec_elem, matrix_free):
 
 def flops_per_hx(nbonds, natoms, norb=10):
     return 2.0 * (2 * norb * norb * nbonds + norb * natoms)
+
+
+def moved_bytes_per_hx(nbonds, natoms, nrows, elem, vec_elem):
+    """What the GPU product has to move: x and y once, one factor per bond, a species byte and a
+    potential word per atom."""
+    return 2 * nrows * vec_elem + nbonds * elem + natoms * (1 + 8)
+
+
+def reduced_flops_per_hx(nbonds, natoms):
+    """Operations of the sp3d5s* product by reduced blocks, each counted as the FMA whose slot it
+    takes (2 flops), as the measured FMA rate counts them."""
+    return 2.0 * (2 * HX_OPS_PER_BOND_END * nbonds + HX_OPS_PER_ATOM * natoms)
 
 
 class ClockSampler:
@@ -131,8 +141,8 @@ def workload_config(cells, natoms, nbonds, rows, matrix_free, world):
     return {"workload": f"Si0.7Ge0.3 alloy {cells}^3 cells ({natoms:,} atoms), hard wall, 2% bond "
                         "strain, sp3d5s*; step = folded operator (H-sigma)^2 x (two H·X)",
             "atoms": natoms, "bonds": nbonds, "rows": rows,
-            "storage": "matrix-free" if matrix_free else "stored bond blocks",
-            "l2": "no flush: H blocks exceed L2", "parallelism": f"replicas x{world}"}
+            "storage": "matrix-free" if matrix_free else "one factor per bond, table of reduced blocks",
+            "l2": "no flush: the vectors and bond factors of a step exceed L2", "parallelism": f"replicas x{world}"}
 
 
 def cpu_sample(seed=2):
@@ -350,9 +360,9 @@ def measure_m2_ladder(ctx, omen, sizes=(4, 5, 6, 8, 10), big=50, big_iters=2000,
 def measure_charge_poisson(ctx, omen, lat, ham, spec, nstates=16, ng=256):
     """Rows a9-a12 at the 1M-atom scale: electrons per atom from nstates FP64 eigenvectors
     (omen_density_accum), cloud-in-cell deposit of the atom charges on an ng x ng x ng grid over the
-    structure, the FP64 CG Poisson solve on that grid, and the trilinear gather back to the atoms.
-    Algorithmic bytes: the eigenvectors once (density); per CG iteration 8 words per unknown
-    (stencil input once, product written, x, r, p read and written)."""
+    structure, the Poisson solves on that grid (FP64, and the mixed form's call), and the trilinear
+    gather back to the atoms.  Algorithmic bytes: the eigenvectors once (density).  The iterations of
+    a direct Poisson solve are its corrections."""
     import torch
     from oracle import poisson  # grid description only (no computation)
     L = spec.nx * spec.a_nm
@@ -385,23 +395,17 @@ def measure_charge_poisson(ctx, omen, lat, ham, spec, nstates=16, ng=256):
     info = omen.omen_poisson(ctx, grid, rho_s, phi, rtol=1e-8, max_iter=50000)
     torch.cuda.synchronize()
     tp = time.perf_counter() - t0
-    nu = out["unknowns"]
-    out["poisson_cg"] = {"iterations": info["iterations"], "seconds": tp, "ms_per_iteration": tp / info["iterations"] * 1e3,
-                         "GB_per_s": 8 * 8 * nu * info["iterations"] / tp / 1e9, "rel_residual": info["rel_residual"]}
-    # FP32 iterations, FP64 residual replacement: 7 FP32 words per unknown per iteration (stencil
-    # input once; correction d, residual r and direction p read and written)
+    out["poisson"] = {"iterations": info["iterations"], "seconds": tp, "rel_residual": info["rel_residual"]}
     phi32 = torch.zeros(grid.shape, dtype=torch.float64, device="cuda")
     torch.cuda.synchronize()
     t0 = time.perf_counter()
     info = omen.omen_poisson(ctx, grid, rho_s, phi32, rtol=1e-8, max_iter=50000, precision=omen.OMEN_F32_REFINE64)
     torch.cuda.synchronize()
     tm = time.perf_counter() - t0
-    out["poisson_cg_mixed"] = {"iterations": info["iterations"], "seconds": tm,
-                               "ms_per_iteration": tm / info["iterations"] * 1e3,
-                               "GB_per_s": 7 * 4 * nu * info["iterations"] / tm / 1e9,
-                               "rel_residual": info["rel_residual"], "speedup_vs_fp64": tp / tm,
-                               "max_abs_diff_vs_fp64_V": float((phi32 - phi).abs().max()),
-                               "max_abs_phi_V": float(phi.abs().max())}
+    out["poisson_mixed"] = {"iterations": info["iterations"], "seconds": tm,
+                            "rel_residual": info["rel_residual"], "speedup_vs_fp64": tp / tm,
+                            "max_abs_diff_vs_fp64_V": float((phi32 - phi).abs().max()),
+                            "max_abs_phi_V": float(phi.abs().max())}
     del phi32
     phi_atom = torch.empty(spec.natoms, dtype=torch.float64, device="cuda")
     t = timed(lambda: omen.omen_gather(ctx, lat, grid, phi, phi_atom))
@@ -586,9 +590,8 @@ def c5_kpoints(L):
 
 
 def launch_hx_shapes(ctx, omen, cells):
-    """Profiling aid: one FP64 stored H·X launch per compiled launch shape (CTA width 32, 64, 96,
-    128 x block rows per batch 1, 2), in that order, on the alloy recipe at cells^3, so that one
-    ncu capture of the 8 launches gives each shape's DRAM traffic per bond."""
+    """Profiling aid: one FP64 H·X launch per launch shape that omen_hx_set_tile takes (CTA width 32,
+    64, 96, 128 x rows per batch 1, 2), in that order, on the alloy recipe at cells^3."""
     import torch
     spec, p = synth.config_sige_alloy(cells, seed=2)
     lat = omen.omen_build_lattice(ctx, spec)
@@ -908,28 +911,22 @@ def run_gpu(args, rank, world, local_rank):
 
     peaks = measured_peaks()
     hbm = peaks.get("hbm_gbs") or 6800.0
-    achieved_gbs = alg / (launch_ms / 1e3) / 1e9
+    moved_gbs = moved_bytes_per_hx(nbonds, natoms, ham.nrows, el, el) / (launch_ms / 1e3) / 1e9
     if prec == omen.OMEN_F64:
-        fl = flops_per_hx(nbonds, natoms)
-        achieved_tf = fl / (launch_ms / 1e3) / 1e12
-        # DRAM bytes per launch of this kernel for the chosen shape: per-bond traffic from the
-        # committed ncu capture of every shape, times this launch's bonds (not measured in this run)
-        shape = (tile["threads"], tile["rows_per_batch"] or 1) if tile else None
-        per_bond = HX_F64_TRAFFIC_PER_BOND.get(shape) if not args.matrix_free else None
-        traffic = per_bond * nbonds if per_bond else None
         # the FP64 FMA rate measured now on this device (the library's probe), nominal beside it
+        achieved_tf = reduced_flops_per_hx(nbonds, natoms) / (launch_ms / 1e3) / 1e12
         peak_tf = omen.omen_probe_fp64_rate(ctx)
         roof = {"bound": "alu", "achieved": achieved_tf, "peak": peak_tf, "unit": "TFLOP/s",
-                "frac": achieved_tf / peak_tf, "traffic": traffic,
+                "frac": achieved_tf / peak_tf, "traffic": None,
                 "frac_of_nominal_fp64": achieved_tf / FP64_PEAK_TFLOPS,
-                "traffic_source": HX_F64_TRAFFIC_SOURCE if traffic else None,
-                "kernel": "hx_kernel<double,10,real,stored>", "hbm_achieved_gbs": achieved_gbs,
-                "hbm_frac_of_measured": achieved_gbs / hbm,
+                "operations": "reduced bond blocks: 61 a bond end, 10 an atom, two flops each",
+                "kernel": "hx_kernel<double,10,real>", "hbm_achieved_gbs": moved_gbs,
+                "hbm_frac_of_measured": moved_gbs / hbm,
                 "peak_source": "measured in this run: FP64 FMA rate (omen_probe_fp64_rate)"}
     else:
-        kname = "hx_df_kernel<10>" if prec == omen.OMEN_F64_DF else "hx_kernel<float,10,real,stored>"
-        roof = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm, "unit": "GB/s",
-                "frac": achieved_gbs / hbm, "traffic": None,
+        kname = "hx_df_kernel<10>" if prec == omen.OMEN_F64_DF else "hx_kernel<float,10,real>"
+        roof = {"bound": "hbm", "achieved": moved_gbs, "peak": hbm, "unit": "GB/s",
+                "frac": moved_gbs / hbm, "traffic": None,
                 "kernel": kname, "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)"}
     result = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
               "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
