@@ -32,7 +32,6 @@ __device__ __forceinline__ float2 df_from_double(double v) {
   const float hi = __double2float_rn(v);
   return make_float2(hi, __double2float_rn(v - (double)hi));
 }
-__device__ __forceinline__ double df_to_double(float2 v) { return (double)v.x + (double)v.y; }
 
 // v 2^kSplitShift as an FP32 pair (hi, lo), by integer operations only (the FP64 pipe, which
 // df_from_double uses, has 1/64 of the FP32 rate): hi keeps the sign, the exponent and the leading

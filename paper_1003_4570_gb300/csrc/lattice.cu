@@ -2,12 +2,13 @@
 //
 // Paper Section II-A keeps, per subdomain, the atoms and their neighbour atoms without
 // global position lists.  On one GPU the whole block is resident and the neighbour of an
-// atom is computed from its cell index and the zincblende site tables below, so no
+// atom is computed from its cell index and site number (neighbours.cuh), so no
 // neighbour list is stored or read.
 #include <cstdarg>
 #include <cstring>
 #include <mutex>
 
+#include "neighbours.cuh"
 #include "omen_internal.h"
 
 omen_status set_err(omen_ctx* ctx, omen_status s, const char* fmt, ...) {
@@ -22,56 +23,12 @@ omen_status set_err(omen_ctx* ctx, omen_status s, const char* fmt, ...) {
   return s;
 }
 
-// Site positions in units of a/4: A sites, then B = A + (1,1,1).
-static const int kSite[8][3] = {{0, 0, 0}, {0, 2, 2}, {2, 0, 2}, {2, 2, 0},
-                                {1, 1, 1}, {1, 3, 3}, {3, 1, 3}, {3, 3, 1}};
-static const int kDir[4][3] = {{1, 1, 1}, {1, -1, -1}, {-1, 1, -1}, {-1, -1, 1}};
-
-static int floor_div4(int q) { return q >= 0 ? q / 4 : -((-q + 3) / 4); }
-
-static int site_at(const int p[3]) {
-  for (int b = 0; b < 8; ++b)
-    if (kSite[b][0] == p[0] && kSite[b][1] == p[1] && kSite[b][2] == p[2]) return b;
-  return -1;
-}
-
-static NeighbourTables build_tables() {
-  NeighbourTables t{};
-  for (int s = 0; s < 4; ++s)
-    for (int k = 0; k < 4; ++k) {
-      int q[3], off[3], loc[3];
-      // from A site s along +dir k to a B site
-      for (int d = 0; d < 3; ++d) {
-        q[d] = kSite[s][d] + kDir[k][d];
-        off[d] = floor_div4(q[d]);
-        loc[d] = q[d] - 4 * off[d];
-        t.a_to_b_off[s][k][d] = off[d];
-      }
-      t.a_to_b_site[s][k] = site_at(loc);
-      // from B site 4+s along -dir k to an A site
-      for (int d = 0; d < 3; ++d) {
-        q[d] = kSite[4 + s][d] - kDir[k][d];
-        off[d] = floor_div4(q[d]);
-        loc[d] = q[d] - 4 * off[d];
-        t.b_to_a_off[s][k][d] = off[d];
-      }
-      t.b_to_a_site[s][k] = site_at(loc);
-    }
-  return t;
-}
-
-const NeighbourTables& host_neighbour_tables() {
-  static NeighbourTables t = build_tables();
-  return t;
-}
-
+// Whether the bond of A site s along direction k from cell (ix, iy, iz) exists: none of its steps
+// into a next cell leaves a hard wall (neighbours.cuh has the rule of the steps).
 static bool slot_exists(const omen_lattice* L, int s, int k, int ix, int iy, int iz) {
-  const NeighbourTables& t = host_neighbour_tables();
-  const int i[3] = {ix, iy, iz}, n[3] = {L->nx, L->ny, L->nz};
-  for (int d = 0; d < 3; ++d) {
-    int j = i[d] + t.a_to_b_off[s][k][d];
-    if ((j < 0 || j >= n[d]) && L->periodic[d] == OMEN_HARD_WALL) return false;
-  }
+  const int at[3] = {ix, iy, iz};
+  for (int d = 0; d < 3; ++d)
+    if (at[d] == 0 && dir_minus(k, d) && (s == 0 || s == d + 1) && L->periodic[d] == OMEN_HARD_WALL) return false;
   return true;
 }
 

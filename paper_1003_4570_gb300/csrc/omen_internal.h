@@ -111,18 +111,6 @@ omen_status set_err(omen_ctx* ctx, omen_status s, const char* fmt, ...);
   } while (0)
 #define OMEN_CHECK_LAUNCH(ctx) OMEN_CUDA(ctx, cudaGetLastError())
 
-// geometry tables (constant memory), defined in lattice.cu --------------------------------
-// For A site s and direction k: the B site (4..7) of the neighbour and its cell offset.
-// For B site s (0..3 = b-4) and direction k: the A site of the neighbour and its cell offset.
-struct NeighbourTables {
-  int a_to_b_site[4][4];
-  int a_to_b_off[4][4][3];   // each component in {-1, 0}
-  int b_to_a_site[4][4];
-  int b_to_a_off[4][4][3];   // each component in {0, +1}
-};
-const NeighbourTables& host_neighbour_tables();
-omen_status upload_neighbour_tables(omen_ctx* ctx);
-
 // kernels launched from the C-ABI layer ------------------------------------------------------
 omen_status launch_assemble(omen_ctx* ctx, omen_ham* ham, const omen_tb_params* p);
 omen_status launch_hx(omen_ctx* ctx, const omen_ham* ham, const void* x, void* y, int nvec,

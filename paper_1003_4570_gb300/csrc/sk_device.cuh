@@ -53,27 +53,3 @@ struct Geo {
   int nx, ny, nz, ncells, natoms;
   int periodic[3];
 };
-
-// Neighbour cell of (ix,iy,iz) shifted by off (components in {-1,0,1}).  Returns false if the
-// shift leaves a hard-wall direction.  wrap_sign[d] = -1/+1 when the shift wrapped across the
-// low/high face of a periodic direction, else 0.
-__device__ __forceinline__ bool shift_cell(const Geo& g, int ix, int iy, int iz, int ox, int oy, int oz,
-                                           int& cell, int wrap_sign[3]) {
-  int j[3] = {ix + ox, iy + oy, iz + oz};
-  const int n[3] = {g.nx, g.ny, g.nz};
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    wrap_sign[d] = 0;
-    if (j[d] < 0) {
-      if (g.periodic[d] == OMEN_HARD_WALL) return false;
-      j[d] += n[d];
-      wrap_sign[d] = -1;
-    } else if (j[d] >= n[d]) {
-      if (g.periodic[d] == OMEN_HARD_WALL) return false;
-      j[d] -= n[d];
-      wrap_sign[d] = 1;
-    }
-  }
-  cell = (j[2] * g.ny + j[1]) * g.nx + j[0];
-  return true;
-}
