@@ -138,7 +138,7 @@ struct HxInst {
   const T* __restrict__ scale;        // [16*ncells] (d0/d)^eta per bond slot
   const uint8_t* __restrict__ species;
   const T* __restrict__ onsite;       // [ns][norb]
-  const double* __restrict__ U;       // [natoms]
+  const double* U;                    // [natoms]; kernels of the stream may write it (see pdl.cuh)
   const double* __restrict__ lambda;  // [ns]
   const double2* __restrict__ phases; // k batch: [nk][3] exp(i k_d L_d); null: with the launch,
   int ph_at;                          // from this entry
@@ -340,75 +340,96 @@ __device__ __forceinline__ V so_term(int q, int i, V first, V second) {
   return r;
 }
 
-// The same with one lane per bond, and for complex vectors one per bond and component: a warp
-// takes 8 atoms x 4 bonds (4 x 4 x 2 complex), the bonds' rows are summed by shuffles that leave
-// each lane the orbitals o = bond mod 4, and those lanes add the onsite rows and store.  For FP64
-// and complex products too small to give every SM sub-partition a warp: FP64 issues one warp
-// instruction in 64 cycles there, so a slab's product costs the FP64 instructions of one thread.
-// 1x1x16-cell slab, complex128: 41.0 us with one thread per atom and full blocks, 27.0 us with
-// one thread per atom and reduced blocks, 8.9 us here.
+// One lane's bond end in the products below: 8 atoms x 4 bonds a warp (complex vectors: 4 x 4 x 2
+// components).  Nothing here is written by an earlier kernel of the stream.
+template <typename T, int NORB, bool CPLX>
+struct BondLane {
+  static constexpr int kCells = CPLX ? 4 : 8;
+  int k, b, cell, atom, sp;
+  bool im, live, is_a;      // im: the lane's component
+  Neighbour n;
+  T sc;                     // (d0/d)^eta; 0 for an absent bond
+  const T* coef;            // its reduced block
+  typename Cx<T>::t f;      // Bloch phase, the imaginary part with the sign the component takes
+
+  __device__ __forceinline__ BondLane(const HxInst<T>& I, const T* tab, int item, int cell0, int cell1) {
+    const Geo& g = I.g;
+    const int lane = threadIdx.x & 31;
+    k = (lane / kCells) & 3;
+    im = CPLX && lane >= 16;
+    b = item & 7;
+    is_a = b < 4;
+    const int cell_raw = cell0 + (item >> 3) * kCells + lane % kCells;
+    live = cell_raw < cell1;
+    cell = live ? cell_raw : cell1 - 1;              // idle lanes repeat the last cell, and store nothing
+    atom = b * g.ncells + cell;
+    const int nxy = g.nx * g.ny;
+    const int iz = cell / nxy, rem = cell - iz * nxy, iy = rem / g.nx, ix = rem - iy * g.nx;
+    n = neighbour_of(g, steps_of(g, b, ix, iy, iz), b, k, cell);
+    sp = I.species[atom];
+    sc = (T)0;
+    int sp2 = 0;
+    if (n.ok) {
+      sc = I.scale[n.slot];
+      sp2 = I.species[n.atom];
+    }
+    coef = tab + ((is_a ? 0 : I.ns * I.ns) + (is_a ? sp * I.ns + sp2 : sp2 * I.ns + sp)) * coef_stride(NORB);
+    f.x = (T)1;
+    f.y = (T)0;
+    if (CPLX && n.wrap) f = wrap_phase<T>(n.wrap, is_a, I.phase);
+    if (!im) f.y = -f.y;
+  }
+
+  // the lane's component of a neighbour's amplitude, times the phase
+  __device__ __forceinline__ T component(typename VecT<T, CPLX>::t x) const {
+    if constexpr (CPLX) {
+      const T mine = im ? x.y : x.x, other = im ? x.x : x.y;
+      return n.wrap ? fma(mine, f.x, other * f.y) : mine;
+    } else {
+      return x;
+    }
+  }
+};
+
+// The same product with one lane per bond, and for complex vectors one per bond and component: a
+// warp takes 8 atoms x 4 bonds (4 x 4 x 2 complex), the bonds' rows are summed by shuffles that leave
+// each lane the orbitals o = bond mod 4, and those lanes add the onsite rows and store.  For
+// products too small to fill the chip: FP64 issues one warp instruction in 64 cycles on a
+// sub-partition, so the product of a small block costs the FP64 instructions of one thread.
+// The dependents are released after the wait, not before it: released at the start, kernel after kernel
+// of a run of products comes to sit on the SMs, and blocks go where one has just left instead of
+// spreading (8^3 cells, FP64, back to back: 8.1 against 5.2 us; 3x3x16, complex128: 9.9 against 5.6).
 template <typename T, int NORB, bool CPLX, bool SO>
 __global__ void __launch_bounds__(32) hx_split_kernel(const __grid_constant__ HxInst<T> I, double sigma, int cell0, int cell1,
                                                       const void* xv, void* yv) {
   using V = typename VecT<T, CPLX>::t;
   constexpr int CS = coef_stride(NORB), CELLS = CPLX ? 4 : 8, G = (NORB + 3) / 4;
   __shared__ __align__(16) T tab[2 * 16 * coef_stride(NORB)];
-  pdl_trigger();
   stage_coef<T, NORB>(I.coef, I.ns, tab);
-  const Geo& g = I.g;
-  const size_t N = g.natoms;
-  const int lane = threadIdx.x;
-  const int k = (lane / CELLS) & 3;
-  const bool im = CPLX && lane >= 16;              // this lane's component
-  const int b = blockIdx.x & 7;
-  const int cell_raw = cell0 + (blockIdx.x >> 3) * CELLS + lane % CELLS;
-  const bool live = cell_raw < cell1;
-  const int cell = live ? cell_raw : cell1 - 1;    // idle lanes repeat the last cell, and store nothing
+  const BondLane<T, NORB, CPLX> B(I, tab, blockIdx.x, cell0, cell1);
+  const size_t N = I.g.natoms;
+  const int k = B.k, atom = B.atom, sp = B.sp;
+  const bool im = B.im;
+  const T sc = B.sc;
   const int q = SO ? blockIdx.y : 0, v = blockIdx.z;
   const V* x = static_cast<const V*>(xv) + I.x_off + (size_t)v * I.nrows;
-  const int atom = b * g.ncells + cell;
-  const int nxy = g.nx * g.ny;
-  const int iz = cell / nxy, rem = cell - iz * nxy, iy = rem / g.nx, ix = rem - iy * g.nx;
-  const Steps steps = steps_of(g, b, ix, iy, iz);
-  const bool is_a = b < 4;
   const size_t spin = SO ? (size_t)(q * NORB) * N : 0;
-  const Neighbour n = neighbour_of(g, steps, b, k, cell);
-  const int sp = I.species[atom];
-  T sc = (T)0;
-  int sp2 = 0;
-  if (n.ok) {
-    sc = I.scale[n.slot];
-    sp2 = I.species[n.atom];
-  }
   T c[CS];
-  load_coef<T, NORB>(tab + (is_a ? 0 : I.ns * I.ns * CS) + (is_a ? sp * I.ns + sp2 : sp2 * I.ns + sp) * CS, c);
+  load_coef<T, NORB>(B.coef, c);
   pdl_wait();      // the vectors and the potential; structure and blocks do not change
-  const V* xp = x + spin + n.atom;
+  pdl_trigger();
+  const V* xp = x + spin + B.n.atom;
   V xn[NORB], own[G];
 #pragma unroll
-  for (int o = 0; o < NORB; ++o) xn[o] = n.ok ? xp[o * N] : v_zero<V>();
+  for (int o = 0; o < NORB; ++o) xn[o] = B.n.ok ? xp[o * N] : v_zero<V>();
 #pragma unroll
   for (int j = 0; j < G; ++j) {
     const int o = 4 * j + k;
     own[j] = o < NORB ? x[spin + o * N + atom] : v_zero<V>();
   }
-  T xs[NORB];                                      // this lane's component, times the Bloch phase
-  if constexpr (CPLX) {
-    V f;
-    f.x = (T)1;
-    f.y = (T)0;
-    if (n.wrap) f = wrap_phase<T>(n.wrap, is_a, I.phase);
-    const T fy = im ? f.y : -f.y;
+  T xs[NORB];
 #pragma unroll
-    for (int o = 0; o < NORB; ++o) {
-      const T mine = im ? xn[o].y : xn[o].x, other = im ? xn[o].x : xn[o].y;
-      xs[o] = mine;
-      if (n.wrap) xs[o] = fma(mine, f.x, other * fy);
-    }
-  } else {
-#pragma unroll
-    for (int o = 0; o < NORB; ++o) xs[o] = xn[o];
-  }
+  for (int o = 0; o < NORB; ++o) xs[o] = B.component(xn[o]);
   T sg[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -438,7 +459,7 @@ __global__ void __launch_bounds__(32) hx_split_kernel(const __grid_constant__ Hx
     const T a1 = (h ? r[4 * j + 3] : r[4 * j + 1]) + __shfl_xor_sync(0xffffffffu, h ? r[4 * j + 1] : r[4 * j + 3], 2 * CELLS);
     const T sum = (l ? a1 : a0) + __shfl_xor_sync(0xffffffffu, l ? a0 : a1, CELLS);
     const int o = 4 * j + k;
-    if (live && o < NORB) {
+    if (B.live && o < NORB) {
       T mine;
       if constexpr (CPLX) mine = im ? own[j].y : own[j].x; else mine = own[j];
       T out = fma(I.onsite[sp * NORB + o] + u, mine, sum);
@@ -454,6 +475,139 @@ __global__ void __launch_bounds__(32) hx_split_kernel(const __grid_constant__ Hx
       V* y = static_cast<V*>(yv) + I.x_off + (size_t)v * I.nrows + spin + o * N + atom;
       if constexpr (CPLX) (im ? y->y : y->x) = out; else *y = out;
     }
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ T flip(T v, bool minus) {
+  if constexpr (sizeof(T) == 8) return __hiloint2double(__double2hiint(v) ^ (minus ? 0x80000000 : 0), __double2loint(v));
+  else return __int_as_float(__float_as_int(v) ^ (minus ? 0x80000000 : 0));
+}
+
+// And with one warp per kind of row besides, s and s*, p, t2g, e, for the smallest products: each
+// warp reads the amplitudes of its kind, gives them the Bloch phase and the bond's signs and leaves
+// them with their sums in shared memory for the others; then it forms its rows of the bond, sums
+// them over the bonds by shuffles that leave lane k the k-th row, adds the onsite part and stores.
+// Some 30 FP64 instructions of a warp between the vectors' arrival and the result, where a lane
+// with all rows takes 100.  1x1x16 cells, complex128: 41.0 us with one thread per atom and full
+// blocks, 26.7 us with one thread per atom and reduced blocks, 5.8 us with one lane per bond, 2.5 us
+// here (back to back).
+template <typename T, int NORB, bool CPLX, bool SO>
+__global__ void __launch_bounds__(NORB == 10 ? 128 : 64) hx_kinds_kernel(const __grid_constant__ HxInst<T> I, double sigma, int cell0,
+                                                                         int cell1, const void* xv, void* yv) {
+  using V = typename VecT<T, CPLX>::t;
+  constexpr int CELLS = CPLX ? 4 : 8;
+  // what a kind leaves for the others: its amplitudes, their sum, and the zero-sum parts the e rows see
+  enum { S = 0, SS, P0, PSUM = P0 + 3, PE1, PE2, T0, TSUM = T0 + 3, TE1, TE2, Q0, kShared = Q0 + 3 };
+  __shared__ __align__(16) T tab[2 * 16 * coef_stride(NORB)];
+  __shared__ T ex[kShared][32];
+  stage_coef<T, NORB>(I.coef, I.ns, tab);
+  const BondLane<T, NORB, CPLX> B(I, tab, blockIdx.x, cell0, cell1);
+  const size_t N = I.g.natoms;
+  // the kinds' warps in a turning order: the p and t2g ones, the longer, spread over an SM's sub-partitions
+  const int lane = threadIdx.x & 31, kind = ((threadIdx.x >> 5) + blockIdx.x) & (NORB == 10 ? 3 : 1);
+  const int k = B.k;
+  const int q = SO ? blockIdx.y : 0, v = blockIdx.z;
+  const V* x = static_cast<const V*>(xv) + I.x_off + (size_t)v * I.nrows;
+  const size_t spin = SO ? (size_t)(q * NORB) * N : 0;
+  // this kind's numbers of the reduced block, and its rows: orbitals o0 + j od
+  constexpr int kS = NORB == 10 ? 8 : 6, kP = NORB == 10 ? 7 : 4;
+  const int nc = kind == 0 ? kS : kind == 3 ? 5 : kP, c0 = kind == 0 ? 0 : kind == 1 ? kS : kind == 2 ? kS + kP : kS + 2 * kP;
+  T c[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) c[i] = i < nc ? B.coef[c0 + i] : (T)0;
+  const int rows = kind == 0 || kind == 3 ? 2 : 3;
+  const int o0 = kind == 0 ? 0 : kind == 1 ? 1 : kind == 2 ? 4 : 7, od = kind == 0 ? NORB - 1 : 1;
+  bool minus[3];
+  T sg[3];                                         // the bond's factor with the row's sign
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    minus[i] = (kind == 1 || kind == 2) && dir_minus(k, i);
+    sg[i] = flip(B.sc, minus[i]);
+  }
+  const int o = o0 + min(k, rows - 1) * od;        // the row this lane stores
+  const T e0 = I.onsite[B.sp * NORB + o];
+  pdl_wait();      // the vectors and the potential; structure and blocks do not change
+  pdl_trigger();
+  const V* xp = x + spin + B.n.atom;
+  V xn[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) xn[j] = B.n.ok && j < rows ? xp[(o0 + j * od) * N] : v_zero<V>();
+  const V own = x[spin + o * N + B.atom];
+  const T u = (T)(I.U[B.atom] - sigma);
+  T a[3];                                          // this lane's component, times phase and sign
+#pragma unroll
+  for (int j = 0; j < 3; ++j) a[j] = flip(B.component(xn[j]), minus[j]);
+  constexpr T kHalf = (T)0.5, kR = (T)0.86602540378443865;   // sqrt(3)/2
+  if (kind == 0) {
+    ex[S][lane] = a[0];
+    ex[SS][lane] = a[1];
+  } else if (NORB == 5 || kind < 3) {
+    const int at = kind == 1 ? P0 : T0;
+    const T s = a[0] + a[1];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) ex[at + j][lane] = a[j];
+    ex[at + 3][lane] = s + a[2];
+    if constexpr (NORB == 10) {
+      ex[at + 4][lane] = a[0] - a[1];
+      ex[at + 5][lane] = fma(-kHalf, s, a[2]);
+    }
+  } else {
+    const T h = -kHalf * a[1];
+    ex[Q0][lane] = fma(kR, a[0], h);
+    ex[Q0 + 1][lane] = fma(-kR, a[0], h);
+    ex[Q0 + 2][lane] = a[1];
+  }
+  __syncthreads();
+  T r[3];
+  if (kind == 0) {
+    const T P = ex[PSUM][lane];
+    if constexpr (NORB == 10) {
+      const T Q = ex[TSUM][lane];
+      r[0] = fma(c[3], a[1], fma(c[2], Q, fma(c[1], P, c[0] * a[0])));
+      r[1] = fma(c[7], a[1], fma(c[6], Q, fma(c[5], P, c[4] * a[0])));
+    } else {
+      r[0] = fma(c[2], a[1], fma(c[1], P, c[0] * a[0]));
+      r[1] = fma(c[5], a[1], fma(c[4], P, c[3] * a[0]));
+    }
+    r[2] = (T)0;
+  } else if (NORB == 5) {
+    const T C = fma(c[2], ex[PSUM][lane], fma(c[1], ex[SS][lane], c[0] * ex[S][lane]));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) r[i] = fma(c[3], a[i], C);
+  } else if (kind < 3) {
+    // c: s, s*, P, T, p, t, q
+    const T C = fma(c[3], ex[TSUM][lane], fma(c[2], ex[PSUM][lane], fma(c[1], ex[SS][lane], c[0] * ex[S][lane])));
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      r[i] = fma(c[5], ex[T0 + i][lane], fma(c[4], ex[P0 + i][lane], fma(c[6], ex[Q0 + i][lane], C)));
+  } else {
+    // c: p and t of the second row, t, e, p and t of the first
+    r[0] = fma(c[2], a[0], fma(c[4], ex[TE1][lane], c[3] * ex[PE1][lane]));
+    r[1] = fma(c[2], a[1], fma(c[1], ex[TE2][lane], c[0] * ex[PE2][lane]));
+    r[2] = (T)0;
+  }
+#pragma unroll
+  for (int j = 0; j < 3; ++j) r[j] *= sg[j];
+  // bonds k and k^2, then k and k^1: of its kind's rows the lane keeps row k
+  const bool h = k & 2, l = k & 1;
+  const T a0 = (h ? r[2] : r[0]) + __shfl_xor_sync(0xffffffffu, h ? r[0] : r[2], 2 * CELLS);
+  const T a1 = (h ? (T)0 : r[1]) + __shfl_xor_sync(0xffffffffu, h ? r[1] : (T)0, 2 * CELLS);
+  const T sum = (l ? a1 : a0) + __shfl_xor_sync(0xffffffffu, l ? a0 : a1, CELLS);
+  if (B.live && k < rows) {
+    T mine;
+    if constexpr (CPLX) mine = B.im ? own.y : own.x; else mine = own;
+    T out = fma(e0 + u, mine, sum);
+    if constexpr (SO) {
+      if (kind == 1) {
+        const V* xo = x + (size_t)((1 - q) * NORB) * N + B.atom;
+        const V first = k == 2 ? xo[2 * N] : x[spin + (k == 0 ? 2 : 1) * N + B.atom];
+        const V t = so_term(q, k, first, k == 2 ? xo[N] : xo[3 * N]);
+        out = fma((T)I.lambda[B.sp], B.im ? t.y : t.x, out);
+      }
+    }
+    V* y = static_cast<V*>(yv) + I.x_off + (size_t)v * I.nrows + spin + o * N + B.atom;
+    if constexpr (CPLX) (B.im ? y->y : y->x) = out; else *y = out;
   }
 }
 
@@ -670,12 +824,23 @@ size_t vec_elem_bytes(const omen_ham* h, int precision) {
   return h->is_complex ? 2 * r : r;
 }
 
-// FP64 and complex products of fewer warps (32 cells of a site, a vector, a spin) than this take
-// one lane per bond.  Measured either side of the line, lane per bond against row per lane: FP64
-// real 688 warps (14^3 cells) 18.9 against 22.7 us, 1024 warps 25.0 against 22.8 us; complex128
-// 256 warps 18.7 against 27.0 us, 400 warps 26.9 against 27.0 us; complex64 256 warps 6.1 against
-// 6.6 us.  FP32 real products gain nothing from it (5.2 us either way).
-static constexpr long long split_below(bool f64, bool cplx) { return cplx ? 400 : f64 ? 800 : 0; }
+// Up to this many CTAs (8 cells of a site, complex 4, a vector, a spin) take a warp per kind of row,
+// and products of fewer warps (32 cells of a site, a vector, a spin) than split_below one lane per
+// bond.  Back to back, us, row per lane / lane per bond / kinds (warps, CTAs), either side of the lines:
+//   FP64    8^3 cells (128, 512) 14.4 / 4.6 / 4.4    9^3 (184, 736) 14.4 / 5.1 / 8.2
+//           15^3 (848) 22.6 / 20.4                   16^3 (1024) 22.6 / 23.3
+//   complex128  4x4x16 (64, 512) 26.7 / 5.8 / 5.9    5x5x16 (104, 800) 26.7 / 7.2 / 10.9
+//           10x10x16 (400) 26.7 / 23.4
+//   FP32    11^3 (336, 1336) 4.2 / 3.5 / 3.4         12^3 (432, 1728) 4.1 / 3.8 / 4.1
+//           14^3 (688) 6.2 / 4.8                     16^3 (1024) 6.2 / 6.2
+//   complex64   10x10x16 (400) 6.2 / 4.5             12x12x16 (576) 6.2 / 6.2
+// sp3s*: FP64 12^3 (432) 6.2 / 4.9, 14^3 (688) 10.3 / 10.6; complex128 256 warps 12.4 / 6.9, 400
+// 12.4 / 13.8.  Past 512 CTAs a sub-partition gets more than three and a half warps of the kinds, and
+// FP64 instructions of one warp after the other bind; the lane per bond spends fewer in all.
+static constexpr long long kinds_upto(bool f64, bool cplx) { return f64 || cplx ? 512 : 1336; }
+static constexpr long long split_below(bool f64, bool cplx, int norb) {
+  return norb == 5 ? (cplx ? 350 : 600) : !cplx ? 900 : f64 ? 450 : 560;
+}
 
 template <typename T, int NORB, bool CPLX, bool SO, int LB>
 static cudaError_t launch_t(const HxInst<T>& I, int nvec, int threads, double sigma, int cell0, int cell1, const void* x,
@@ -702,12 +867,14 @@ static cudaError_t launch_rows(const HxInst<T>& I, int nvec, HxTile t, double si
                                void* y, cudaStream_t st) {
   // the rule looks at the whole structure, so a product computed in pieces has the same bits
   const long long warps = (long long)((I.g.ncells + 31) / 32) * 8 * (SO ? 2 : 1) * nvec;
-  if (warps < split_below(sizeof(T) == 8, CPLX)) {
-    constexpr int cells = CPLX ? 4 : 8;
-    const long long items = (long long)((cell1 - cell0 + cells - 1) / cells) * 8;
-    const dim3 grid((unsigned)items, SO ? 2 : 1, nvec);   // one warp a CTA: the warps spread over the SMs
+  constexpr int cells = CPLX ? 4 : 8;
+  // a warp (kinds: a CTA) each; small CTAs spread over the SMs
+  const dim3 grid((unsigned)((cell1 - cell0 + cells - 1) / cells) * 8, SO ? 2 : 1, nvec);
+  const long long units = (long long)((I.g.ncells + cells - 1) / cells) * 8 * (SO ? 2 : 1) * nvec;
+  if (units <= kinds_upto(sizeof(T) == 8, CPLX))
+    return launch_dependent(hx_kinds_kernel<T, NORB, CPLX, SO>, grid, dim3(NORB == 10 ? 128 : 64), 0, st, I, sigma, cell0, cell1, x, y);
+  if (warps < split_below(sizeof(T) == 8, CPLX, NORB))
     return launch_dependent(hx_split_kernel<T, NORB, CPLX, SO>, grid, dim3(32), 0, st, I, sigma, cell0, cell1, x, y);
-  }
   // bonds whose amplitudes are loaded together: rb 1 -> 1, 2 -> 2, 5 or 10 -> 4
   const int thr = t.threads ? t.threads : 128;
   const int lb = t.rb == 0 ? (sizeof(T) == 4 && !CPLX ? 2 : 1) : t.rb == 1 ? 1 : t.rb == 2 ? 2 : 4;
