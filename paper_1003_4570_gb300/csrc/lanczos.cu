@@ -27,6 +27,7 @@
 
 #include "dense_eig.h"
 #include "omen_internal.h"
+#include "pdl.cuh"
 #include "vec.cuh"
 #include "df.cuh"
 
@@ -178,9 +179,8 @@ template <typename T, bool C, int IG>
 __global__ void __launch_bounds__(256, 2) dots1_kernel(const void* Av, long long lda, int na, int per, const void* Bv,
                                                     long long n, int rows_per_cta, double2* P, DotsFinish fin,
                                                     long long a_ps = 0, long long b_ps = 0, long long p_ps = 0,
-                                                    const long long* __restrict__ poff = nullptr,
-                                                    const long long* __restrict__ plen = nullptr,
-                                                    const int* __restrict__ act = nullptr) {
+                                                    const long long* poff = nullptr, const long long* plen = nullptr,
+                                                    const int* act = nullptr) {
   using E = Elem<T, C>;
   using V = typename E::V;
   using Acc = std::conditional_t<sizeof(T) == 8, double, float>;
@@ -189,6 +189,8 @@ __global__ void __launch_bounds__(256, 2) dots1_kernel(const void* Av, long long
   // sits idle under a predicate (predicated-off FP64 FMAs still occupy the pipe)
   // grid.z = independent problems (batched Lanczos): offsets a_ps, b_ps (elements), p_ps
   // (partials) per problem, or per-problem element offsets poff and lengths plen
+  pdl_wait();
+  pdl_trigger();
   const long long off = poff ? poff[blockIdx.z] : 0;
   if (act && !act[blockIdx.z]) return;   // a converged (frozen) problem of the batch
   if (plen) n = plen[blockIdx.z];
@@ -390,15 +392,17 @@ __global__ void __launch_bounds__(256) combine1_kernel(const void* Av, long long
 // The three-term part of a step in one pass: w -= h v_j + t v_{j-1}, with h = <v_j, w> and t the
 // norm of the step before (entry (js, js-1) of the projected matrix, mirrored here).
 template <typename T, bool C>
-__global__ void __launch_bounds__(256) three_term_kernel(const void* Vj, const void* Vp, const double2* __restrict__ h,
-                                                         double2* __restrict__ Tm, int ldT, int js, void* Wv, long long n) {
+__global__ void __launch_bounds__(256) three_term_kernel(const void* Vj, const void* Vp, const double2* h, double2* Tm, int ldT,
+                                                         int js, void* Wv, long long n) {
   using V = typename Elem<T, C>::V;
+  pdl_wait();
+  pdl_trigger();
   const double2 hj = *h, tp = Tm[js + (size_t)(js - 1) * ldT];
   if (blockIdx.x == 0 && threadIdx.x == 0) Tm[(js - 1) + (size_t)js * ldT] = tp;
   const T hr = (T)-hj.x, hi = (T)-hj.y, tr = (T)-tp.x;     // a norm: its imaginary part is zero
-  const V* __restrict__ a = static_cast<const V*>(Vj);
-  const V* __restrict__ b = static_cast<const V*>(Vp);
-  V* __restrict__ w = static_cast<V*>(Wv);
+  const V* a = static_cast<const V*>(Vj);
+  const V* b = static_cast<const V*>(Vp);
+  V* w = static_cast<V*>(Wv);
   for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x) {
     V x = w[r];
     const V av = a[r], bv = b[r];
@@ -417,7 +421,7 @@ __global__ void __launch_bounds__(256) three_term_kernel(const void* Vj, const v
 // device).  The last CTA sums the squares, writes nrm[0] = ||w||^2 and nrm[1] = 1 / ||w||, and the
 // norm into T[row, col]; a zero or non-finite norm sets the flag.
 template <typename T, bool C, int PARTS>
-__global__ void __launch_bounds__(256) update_norm_kernel(const void* Av, int na, const double2* __restrict__ h, void* Wv,
+__global__ void __launch_bounds__(256) update_norm_kernel(const void* Av, int na, const double2* h, void* Wv,
                                                           long long n, double* part, int* cnt, double2* nrm, double2* Tm,
                                                           int ldT, int row, int col, int* flag) {
   using V = typename Elem<T, C>::V;
@@ -426,6 +430,8 @@ __global__ void __launch_bounds__(256) update_norm_kernel(const void* Av, int na
   A2* Ms = reinterpret_cast<A2*>(smem_raw);
   constexpr int ROWS = 256 / PARTS;
   __shared__ V sums[PARTS > 1 ? 256 : 1];
+  pdl_wait();
+  pdl_trigger();
   for (int t = threadIdx.x; t < na; t += blockDim.x) {
     A2 m;
     m.x = (T)-h[t].x;
@@ -433,8 +439,8 @@ __global__ void __launch_bounds__(256) update_norm_kernel(const void* Av, int na
     Ms[t] = m;
   }
   __syncthreads();
-  const V* __restrict__ A = static_cast<const V*>(Av);
-  V* __restrict__ W = static_cast<V*>(Wv);
+  const V* A = static_cast<const V*>(Av);
+  V* W = static_cast<V*>(Wv);
   const int rl = threadIdx.x % ROWS, pt = threadIdx.x / ROWS;
   const int ia = (int)((long long)na * pt / PARTS), ib = (int)((long long)na * (pt + 1) / PARTS);
   double sq = 0.0;
@@ -535,12 +541,14 @@ __global__ void __launch_bounds__(256) update_norm_kernel(const void* Av, int na
 // v = w / ||w|| with 1 / ||w|| from update_norm_kernel (formed once, not by every thread: a square
 // root and a division are some 40 FP64 operations).
 template <typename T, bool C>
-__global__ void __launch_bounds__(256) scale_kernel(const void* Wv, void* Vv, long long n, const double2* __restrict__ nrm) {
+__global__ void __launch_bounds__(256) scale_kernel(const void* Wv, void* Vv, long long n, const double2* nrm) {
   using E = Elem<T, C>;
   using V = typename E::V;
+  pdl_wait();
+  pdl_trigger();
   const double inv = nrm[1].x;
-  const V* __restrict__ W = static_cast<const V*>(Wv);
-  V* __restrict__ Vo = static_cast<V*>(Vv);
+  const V* W = static_cast<const V*>(Wv);
+  V* Vo = static_cast<V*>(Vv);
   for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x) {
     const V w = W[r];
     Vo[r] = E::make(E::re(w) * inv, E::im(w) * inv);
@@ -1274,7 +1282,7 @@ static void launch_dots1(const DotsShape& d, int P, cudaStream_t st, const void*
                          long long n, double2* part, const DotsFinish& fin, long long p_ps = 0,
                          const long long* poff = nullptr, const long long* plen = nullptr, const int* act = nullptr) {
   const dim3 grid(d.groups, (unsigned)d.chunks, P);
-#define DOTS1(IGc) dots1_kernel<T, C, IGc><<<grid, d.threads, 0, st>>>(A, lda, na, d.per, B, n, (int)d.rows, part, fin, 0, 0, p_ps, poff, plen, act)
+#define DOTS1(IGc) launch_kernel(d.threads < 256, dots1_kernel<T, C, IGc>, grid, dim3(d.threads), 0, st, A, lda, na, d.per, B, n, (int)d.rows, part, fin, 0, 0, p_ps, poff, plen, act)
   switch (d.ig) {
     case 1: DOTS1(1); break;
     case 2: DOTS1(2); break;
@@ -1759,10 +1767,15 @@ struct KrylovOps {
     return OMEN_OK;
   }
 
+  // Vectors of less than an SM's worth of CTAs each: a step is launches then, and its kernels are set
+  // up while the ones before them run (1,280 complex rows: 51 -> 49 us a step; 640k rows lose 1 to 4%
+  // to blocks that wait on the SMs).
+  bool few_rows() const { return (n + 255) / 256 < sm_count; }
+
   // w -= h v_j + T[js, js-1] v_{j-1}, the entry mirrored to T[js-1, js]
   omen_status three_term(const void* Vj, const void* Vp, const double2* h_dev, double2* Tm, int ldT, int js, void* W) {
     const unsigned grid = (unsigned)std::min<long long>((n + 255) / 256, (long long)sm_count * 8);
-#define TERM3(T, Cc) three_term_kernel<T, Cc><<<grid, 256, 0, ctx->stream>>>(Vj, Vp, h_dev, Tm, ldT, js, W, n)
+#define TERM3(T, Cc) launch_kernel(few_rows(), three_term_kernel<T, Cc>, dim3(grid), dim3(256), 0, ctx->stream, Vj, Vp, h_dev, Tm, ldT, js, W, n)
     if (prec == OMEN_F64) { if (cplx) TERM3(double, true); else TERM3(double, false); }
     else { if (cplx) TERM3(float, true); else TERM3(float, false); }
 #undef TERM3
@@ -1774,7 +1787,7 @@ struct KrylovOps {
   omen_status update_and_normalize(const void* Vb, int na, const double2* h_dev, void* W, double2* nrm, double2* Tm, int ldT,
                                    int row, int col, void* Vnew) {
     // rows a CTA: 256, or 32 with eight threads a row where that leaves SMs idle
-    const bool few = (n + 255) / 256 < sm_count;
+    const bool few = few_rows();
     const unsigned grid = (unsigned)std::min<long long>((n + (few ? 31 : 255)) / (few ? 32 : 256), (long long)sm_count * (few ? 4 : 8));
     const size_t shm = (size_t)na * sizeof(double2);
     int* flag = ctx->d_status + 1;
@@ -1783,12 +1796,12 @@ struct KrylovOps {
   do {                                                                                                            \
     if (few) {                                                                                                    \
       smem_limit(update_norm_kernel<T, Cc, 8>, shm);                                                              \
-      update_norm_kernel<T, Cc, 8><<<grid, 256, shm, ctx->stream>>>(Vb, na, h_dev, W, n, d_npart, cnt, nrm, Tm, ldT, row, col, flag); \
+      launch_dependent(update_norm_kernel<T, Cc, 8>, dim3(grid), dim3(256), shm, ctx->stream, Vb, na, h_dev, W, n, d_npart, cnt, nrm, Tm, ldT, row, col, flag); \
     } else {                                                                                                      \
       smem_limit(update_norm_kernel<T, Cc, 1>, shm);                                                              \
-      update_norm_kernel<T, Cc, 1><<<grid, 256, shm, ctx->stream>>>(Vb, na, h_dev, W, n, d_npart, cnt, nrm, Tm, ldT, row, col, flag); \
+      launch_kernel(false, update_norm_kernel<T, Cc, 1>, dim3(grid), dim3(256), shm, ctx->stream, Vb, na, h_dev, W, n, d_npart, cnt, nrm, Tm, ldT, row, col, flag); \
     }                                                                                                             \
-    scale_kernel<T, Cc><<<(unsigned)std::min<long long>((n + 255) / 256, (long long)sm_count * 8), 256, 0, ctx->stream>>>(W, Vnew, n, nrm); \
+    launch_kernel(few, scale_kernel<T, Cc>, dim3((unsigned)std::min<long long>((n + 255) / 256, (long long)sm_count * 8)), dim3(256), 0, ctx->stream, W, Vnew, n, nrm); \
   } while (0)
     if (prec == OMEN_F64) { if (cplx) UPDN(double, true); else UPDN(double, false); }
     else { if (cplx) UPDN(float, true); else UPDN(float, false); }
