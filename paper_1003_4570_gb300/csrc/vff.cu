@@ -19,11 +19,11 @@
 //   f_p = dE_i/dr_p = sum_q M_pq r_q,  M_pp = 4 k_p (G_pp - d_p^2),  M_pq = 2 k_pq (G_pq + d_p d_q / 3),
 // and the gradient of atom j along its bonds k to atoms n_k is -sum_k (f_k(j) - f_k(n_k)).  One kernel
 // writes the 12 numbers f of every atom, a second gathers them (no atomics, a bit-reproducible
-// result): 150 FP64 operations an atom, where gathering every term that touches an atom took some
+// result): 140 FP64 operations an atom, where gathering every term that touches an atom took some
 // 900, 40 divisions by natural lengths among them; the constants of every species triple now come
 // from a table in shared memory.  All of it is bound by the FP64 rate.  1M atoms, one iteration: gradient
-// 1.46 ms before, 0.24 + 0.09 ms now; line coefficients 0.73 -> 0.47 ms; step 0.104 -> 0.008 ms (every
-// block bisected the quartic); direction 0.032 -> 0.015 ms; 100 iterations 237 -> 84 ms.
+// 1.46 ms before, 0.20 + 0.08 ms now; line coefficients 0.73 -> 0.42 ms (218 operations an atom); step 0.104 -> 0.008 ms (every
+// block bisected the quartic); direction 0.032 -> 0.015 ms; 100 iterations 237 -> 75 ms.
 // For the line search of the nonlinear conjugate-gradient relaxation, a kernel accumulates the
 // coefficients of the energy along a search direction.  Every term is
 // the square of a quadratic polynomial in the step t (r is affine in t), so E(u + t p) is a
@@ -91,6 +91,10 @@ __device__ __forceinline__ void load3(const double* __restrict__ v, long long n,
 __device__ __forceinline__ double dot3(const double x[3], const double y[3]) {
   return fma(x[2], y[2], fma(x[1], y[1], x[0] * y[0]));
 }
+// c + x.y
+__device__ __forceinline__ double dot3(double c, const double x[3], const double y[3]) {
+  return fma(x[2], y[2], fma(x[1], y[1], fma(x[0], y[0], c)));
+}
 
 // Bond vectors of a vertex at displacements u ([3][natoms]); zero for absent bonds.
 __device__ __forceinline__ void bond_vectors(const VffArgs& a, const Vertex& v, const double* __restrict__ u, int atom,
@@ -114,10 +118,12 @@ __device__ __forceinline__ double2 pair_of(const VffTable& t, const Vertex& v, i
   return k;
 }
 
-__device__ __forceinline__ void stage_table(const VffTable& t, VffTable& sm) {
-  const double* src = reinterpret_cast<const double*>(&t);
-  double* dst = reinterpret_cast<double*>(&sm);
-  for (int i = threadIdx.x; i < (int)(sizeof(VffTable) / sizeof(double)); i += blockDim.x) dst[i] = src[i];
+// The table to shared memory, k of the bonds and of the angles times a factor.
+__device__ __forceinline__ void stage_table(const VffTable& t, VffTable& sm, double bond = 1.0, double angle = 1.0) {
+  const double2* src = reinterpret_cast<const double2*>(&t);
+  double2* dst = reinterpret_cast<double2*>(&sm);
+  for (int i = threadIdx.x; i < (int)(sizeof(VffTable) / sizeof(double2)); i += blockDim.x)
+    dst[i] = make_double2((i < 16 ? bond : angle) * src[i].x, src[i].y);
   __syncthreads();
 }
 
@@ -201,7 +207,7 @@ __device__ __forceinline__ bool grid_reduce(double (&v)[NV], double* partial, Vf
 __global__ void __launch_bounds__(kThreads) vff_vertex_kernel(const __grid_constant__ VffArgs a, const double* __restrict__ u,
                                                               double* __restrict__ f) {
   __shared__ VffTable t;
-  stage_table(a.t, t);
+  stage_table(a.t, t, 4.0, 2.0);
   const long long N = a.g.natoms;
   const int atom = blockIdx.x * blockDim.x + threadIdx.x;
   if (atom >= N) return;
@@ -211,7 +217,7 @@ __global__ void __launch_bounds__(kThreads) vff_vertex_kernel(const __grid_const
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
     const double2 k = pair_of(t, v, p, p);
-    const double m = 4.0 * k.x * (dot3(r[p], r[p]) - k.y);
+    const double m = k.x * dot3(-k.y, r[p], r[p]);
 #pragma unroll
     for (int c = 0; c < 3; ++c) fk[p][c] = m * r[p][c];
   }
@@ -220,7 +226,7 @@ __global__ void __launch_bounds__(kThreads) vff_vertex_kernel(const __grid_const
 #pragma unroll
     for (int q = p + 1; q < 4; ++q) {
       const double2 k = pair_of(t, v, p, q);
-      const double m = 2.0 * k.x * (dot3(r[p], r[q]) + k.y);
+      const double m = k.x * dot3(k.y, r[p], r[q]);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         fk[p][c] = fma(m, r[q][c], fk[p][c]);
@@ -241,6 +247,8 @@ __global__ void __launch_bounds__(kThreads) vff_gather_kernel(const __grid_const
                                                               double sign, double* partial, VffState* st) {
   const long long N = a.g.natoms;
   double acc[3] = {0.0, 0.0, 0.0};
+  const int flip = sign < 0.0 ? 0x80000000 : 0;
+  long long gmax = 0;
   for (int atom = blockIdx.x * blockDim.x + threadIdx.x; atom < N; atom += gridDim.x * blockDim.x) {
     const Vertex v = vertex_of(a, atom);
     double gi[3] = {0.0, 0.0, 0.0};
@@ -257,13 +265,15 @@ __global__ void __launch_bounds__(kThreads) vff_gather_kernel(const __grid_const
     if (g_prev) load3(g_prev, N, atom, gp);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      g[c * N + atom] = sign * gi[c];
+      // the sign and the largest |g_c| on the integer pipe (a NaN compares as the largest)
+      g[c * N + atom] = __hiloint2double(__double2hiint(gi[c]) ^ flip, __double2loint(gi[c]));
       acc[0] = fma(gi[c], gi[c], acc[0]);
       acc[1] = fma(gi[c], gp[c], acc[1]);
-      acc[2] = fmax(acc[2], fabs(gi[c]));
+      gmax = max(gmax, __double_as_longlong(gi[c]) & 0x7fffffffffffffffll);
     }
   }
   if (!st) return;
+  acc[2] = __longlong_as_double(gmax);
   if (grid_reduce<3, true>(acc, partial, st)) {
     double beta = 0.0;
     if (g_prev && !st->restart && st->gg > 0.0) beta = fmax(0.0, (acc[0] - acc[1]) / st->gg);
@@ -290,7 +300,7 @@ __global__ void __launch_bounds__(kThreads) vff_energy_kernel(const __grid_const
 #pragma unroll
       for (int q = p; q < 4; ++q) {
         const double2 k = pair_of(t, v, p, q);
-        const double x = p == q ? dot3(r[p], r[p]) - k.y : dot3(r[p], r[q]) + k.y;
+        const double x = dot3(p == q ? -k.y : k.y, r[p], r[q]);
         acc[0] = fma(k.x * x, x, acc[0]);
       }
   }
@@ -330,7 +340,8 @@ __global__ void __launch_bounds__(kThreads) vff_line_kernel(const __grid_constan
   __shared__ VffTable t;
   stage_table(a.t, t);
   const long long N = a.g.natoms;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};              // c1 / 2, c2, c3 / 2, c4
+  // sums of K q0 q1, K q1^2, K q0 q2, K q1 q2, K q2^2
+  double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   for (int atom = blockIdx.x * blockDim.x + threadIdx.x; atom < N; atom += gridDim.x * blockDim.x) {
     const Vertex v = vertex_of(a, atom);
     double r[4][3], s[4][3], pi[3];                  // bond vectors and their change per unit step
@@ -348,20 +359,21 @@ __global__ void __launch_bounds__(kThreads) vff_line_kernel(const __grid_constan
 #pragma unroll
       for (int q = i; q < 4; ++q) {
         const double2 k = pair_of(t, v, i, q);
-        const double q0 = i == q ? dot3(r[i], r[i]) - k.y : dot3(r[i], r[q]) + k.y;
-        const double q1 = i == q ? 2.0 * dot3(r[i], s[i])
-                                 : fma(s[i][2], r[q][2], fma(s[i][1], r[q][1], fma(s[i][0], r[q][0], dot3(r[i], s[q]))));
+        const double q0 = dot3(i == q ? -k.y : k.y, r[i], r[q]);
+        const double q1 = i == q ? 2.0 * dot3(r[i], s[i]) : dot3(dot3(r[i], s[q]), s[i], r[q]);
         const double q2 = dot3(s[i], s[q]);
-        const double k0 = k.x * q0, k1 = k.x * q1;
-        acc[0] = fma(k0, q1, acc[0]);
-        acc[1] = fma(k1, q1, fma(k0 + k0, q2, acc[1]));
-        acc[2] = fma(k1, q2, acc[2]);
-        acc[3] = fma(k.x * q2, q2, acc[3]);
+        const double k1 = k.x * q1, k2 = k.x * q2;
+        acc[0] = fma(k1, q0, acc[0]);
+        acc[1] = fma(k1, q1, acc[1]);
+        acc[2] = fma(k2, q0, acc[2]);
+        acc[3] = fma(k2, q1, acc[3]);
+        acc[4] = fma(k2, q2, acc[4]);
       }
   }
-  if (grid_reduce<4, false>(acc, partial, st)) {
-    const double c1 = 2.0 * acc[0];
-    const double step = quartic_step(c1, acc[1], 2.0 * acc[2], acc[3]);
+  double c[4] = {acc[0], fma(2.0, acc[2], acc[1]), acc[3], acc[4]};   // c1 / 2, c2, c3 / 2, c4
+  if (grid_reduce<4, false>(c, partial, st)) {
+    const double c1 = 2.0 * c[0];
+    const double step = quartic_step(c1, c[1], 2.0 * c[2], c[3]);
     st->t = step;
     st->c1 = c1;
     st->restart = step > 0.0 ? 0 : 1;
