@@ -21,13 +21,13 @@
 #include <complex>
 #include <cstring>
 #include <map>
-#include <mutex>
 #include <type_traits>
 #include <vector>
 
 #include "dense_eig.h"
 #include "omen_internal.h"
 #include "pdl.cuh"
+#include "smem.cuh"
 #include "vec.cuh"
 #include "df.cuh"
 
@@ -1242,23 +1242,6 @@ __global__ void convert_kernel(const void* Xv, void* Yv, long long n) {
   typename Eo::V* Y = static_cast<typename Eo::V*>(Yv);
   for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x)
     Y[r] = Eo::make(Ei::re(X[r]), Ei::im(X[r]));
-}
-
-// cudaFuncSetAttribute costs a driver call: raise a kernel's dynamic shared-memory limit only
-// when a launch needs more than the largest value already set for it.
-template <typename K>
-static void smem_limit(K kernel, size_t bytes) {
-  static std::mutex mu;
-  static std::map<std::pair<int, const void*>, size_t> current;   // per (device, kernel)
-  if (bytes <= 48 * 1024) return;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  std::lock_guard<std::mutex> lock(mu);
-  size_t& cur = current[{dev, reinterpret_cast<const void*>(kernel)}];
-  if (bytes > cur) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    cur = bytes;
-  }
 }
 
 // ---------------------------------------------------------------------------------------

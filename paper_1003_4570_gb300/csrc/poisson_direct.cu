@@ -24,6 +24,7 @@
 #include <cmath>
 
 #include "poisson_direct.h"
+#include "smem.cuh"
 
 namespace {
 
@@ -549,11 +550,6 @@ __global__ void __launch_bounds__(THREADS, 1) tridiag_kernel(PGrid g, double* __
   if (blockIdx.x == 0 && lane == 0 && s == 0) st->iterations += 1;
 }
 
-template <typename K>
-cudaError_t allow_smem(K kernel, size_t bytes) {
-  return bytes > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : cudaSuccess;
-}
-
 }  // namespace
 
 bool poisson_direct_fits(const PGrid& g) { return g.nx <= kMaxLine && g.ny <= kMaxLine && g.nzi <= kMaxZ; }
@@ -629,9 +625,9 @@ omen_status poisson_direct(omen_ctx* ctx, const PGrid& g, const double* rho, dou
   const int rounds = std::min(2, max_iter);
   if (planes) {
     const size_t smem = sizeof(double2) * (2 * (size_t)np + g.nx + g.ny);
-    ok(allow_smem(planes_kernel<true, true>, smem));
-    ok(allow_smem(planes_kernel<true, false>, smem));
-    ok(allow_smem(planes_kernel<false, false>, smem));
+    ok(smem_limit(planes_kernel<true, true>, smem));
+    ok(smem_limit(planes_kernel<true, false>, smem));
+    ok(smem_limit(planes_kernel<false, false>, smem));
     const int pivot_blocks = (int)std::min<long long>((modes * g.nzi + kPivotThreads - 1) / kPivotThreads, (long long)sms * 8);
     auto plane_pass = [&](auto kernel, int blocks, double factor) {
       kernel<<<blocks, kT, smem, st>>>(g, rho, factor, x, r, d, hat, part, state, rtol, max_iter, inv, px, py, inl, twd, ctab, pblocks);
@@ -656,9 +652,9 @@ omen_status poisson_direct(omen_ctx* ctx, const PGrid& g, const double* rho, dou
     const int tiles = (g.nx + 2 * PY - 1) / (2 * PY);
     const unsigned by = (unsigned)tiles * g.nzi;
     const size_t smx = sizeof(double2) * (2 * (size_t)PX + 1) * g.nx, smy = sizeof(double2) * (2 * (size_t)PY + 1) * g.ny;
-    ok(allow_smem(rows_kernel<false>, smx));
-    ok(allow_smem(rows_kernel<true>, smx));
-    ok(allow_smem(columns_kernel, smy));
+    ok(smem_limit(rows_kernel<false>, smx));
+    ok(smem_limit(rows_kernel<true>, smx));
+    ok(smem_limit(columns_kernel, smy));
     nonzero_kernel<<<(unsigned)(sms * 8), kT, 0, st>>>(x, n, state);
     residual_kernel<kFromX, true><<<rblocks, kT, 0, st>>>(g, rho, scale, x, r, part, state, rtol, max_iter);
     ok(cudaGetLastError());
