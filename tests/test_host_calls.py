@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 
 import fake_runtime
+import synth
 from oracle import poisson
 from paper_1003_4570_gb300 import omen
 
@@ -27,3 +28,23 @@ def test_poisson_never_lowers_a_shared_memory_limit(watch, ctx):
             f = np.zeros((n[2] - 1, n[1], n[0]))
             omen.omen_poisson(ctx, poisson.Grid(*n, 1.0, 1.0, 1.0), f, f.copy())
     assert watch.lowered() == 0
+
+
+def hamiltonian(ctx, cells, basis=10, bloch=False, precision=omen.OMEN_F64):
+    lat = omen.omen_build_lattice(ctx, synth.lattice_spec(*cells, (2, 2, 0) if bloch else (0, 0, 0), seed=1))
+    return omen.omen_assemble_H(ctx, lat, synth.draw_tb_params(1, basis, 1), precision=precision,
+                                k=(0.1, 0.2, 0.0) if bloch else None)
+
+
+@pytest.mark.parametrize("precision", [omen.OMEN_F64, omen.OMEN_F32, omen.OMEN_F64_DF])
+@pytest.mark.parametrize("which", [omen.OMEN_LOWEST, omen.OMEN_NEAREST])
+@pytest.mark.parametrize("bloch", [False, True])
+def test_coefficients_outlive_their_copy(watch, ctx, precision, which, bloch):
+    """A pending copy may read host memory until the stream is synchronised: what a solve's restarts
+    and Ritz vectors copy from must be left alone until then (3 and 40 vectors: both of its routes)."""
+    if bloch and precision == omen.OMEN_F64_DF:
+        pytest.skip("double-float Hamiltonians are real")
+    ham = hamiltonian(ctx, (2, 3, 4), bloch=bloch, precision=precision)
+    for nev in (3, 40):
+        omen.omen_eigs(ctx, ham, nev, which, block=1, basis=96, raise_on_noconv=False)
+        assert watch.changed() == 0, nev
