@@ -48,3 +48,12 @@ def test_coefficients_outlive_their_copy(watch, ctx, precision, which, bloch):
     for nev in (3, 40):
         omen.omen_eigs(ctx, ham, nev, which, block=1, basis=96, raise_on_noconv=False)
         assert watch.changed() == 0, nev
+
+
+def test_wave_vectors_outlive_their_copy(watch, ctx):
+    ham = hamiltonian(ctx, (2, 2, 3), bloch=True)
+    k = np.random.default_rng(1).normal(size=(300, 3))
+    x = np.zeros((300, ham.nrows), complex)
+    omen.omen_hx_kbatch(ctx, ham, k, x, np.zeros_like(x))
+    omen.omen_eigs_kbatch(ctx, ham, k[:5], 4, raise_on_noconv=False)
+    assert watch.changed() == 0
