@@ -1305,9 +1305,14 @@ struct KrylovOps {
         cudaMalloc(&d_cnt, kCounters * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&d_npart, sizeof(double) * 8 * (size_t)sm_count) != cudaSuccess) {
       cudaGetLastError();
+      release();                       // callers return on a failed init
       return set_err(ctx, OMEN_ENOMEM, "small work buffer");
     }
-    OMEN_CUDA(ctx, cudaMemsetAsync(d_cnt, 0, kCounters * sizeof(int), ctx->stream));
+    const cudaError_t e = cudaMemsetAsync(d_cnt, 0, kCounters * sizeof(int), ctx->stream);
+    if (e != cudaSuccess) {
+      release();
+      return set_err(ctx, OMEN_ECUDA, "small work buffer: %s", cudaGetErrorString(e));
+    }
     return OMEN_OK;
   }
   void release() {

@@ -57,3 +57,22 @@ def test_wave_vectors_outlive_their_copy(watch, ctx):
     omen.omen_hx_kbatch(ctx, ham, k, x, np.zeros_like(x))
     omen.omen_eigs_kbatch(ctx, ham, k[:5], 4, raise_on_noconv=False)
     assert watch.changed() == 0
+
+
+@pytest.mark.parametrize("call", ["eigs", "refined", "kbatch"])
+def test_a_failed_allocation_leaves_nothing_behind(watch, ctx, call):
+    prec = omen.OMEN_F32_REFINE64 if call == "refined" else omen.OMEN_F64
+    ham = hamiltonian(ctx, (2, 2, 3), bloch=call == "kbatch", precision=prec)
+    before, failed = watch.live(), 0
+    for n in range(60):
+        watch.fail(n)
+        try:
+            if call == "kbatch":
+                omen.omen_eigs_kbatch(ctx, ham, np.zeros((3, 3)), 4, raise_on_noconv=False)
+            else:
+                omen.omen_eigs(ctx, ham, 4, block=1, basis=32, raise_on_noconv=False)
+        except omen.OmenError as e:
+            failed += e.status == omen.OMEN_ENOMEM
+        assert watch.live() == before, n
+    watch.fail(-1)
+    assert failed >= 15
