@@ -756,8 +756,8 @@ __global__ void __launch_bounds__(256) combinen_kernel(const void* Av, long long
 // Many-output combination of real FP64 vectors (restarts: kk Ritz vectors from m basis
 // vectors): nb FMAs per element read would hold it to GB300's FP64 rate, so each element is split
 // once into a double-float pair, by integer operations, and the nb products and sums run in
-// double-float arithmetic on the FP32 pipe; each result is rounded back to FP64 (about 48 of its
-// 53 bits exact — the next step re-orthogonalises anyway).  The split carries a factor 2^32, which
+// double-float arithmetic on the FP32 pipe; each result is rounded back to FP64 (elements within 2^-49,
+// sums to about 48 of the 53 bits — the next step re-orthogonalises anyway).  The split carries a factor 2^32, which
 // keeps components down to 2^-107 clear of FP32 underflow.  49 vectors from 97, 640k rows: four
 // passes of 16 columns at 0.75 ms with the split on the FP64 pipe (three conversions and a
 // subtraction), two passes of 25 at 0.81 ms now.
@@ -778,7 +778,7 @@ __global__ void __launch_bounds__(256) combine_split_kernel(const double* __rest
     for (int j = 0; j < NBT; ++j) { S[j] = 0.f; Cc[j] = 0.f; }
     double next = A[r];
     for (int i = 0; i < na; ++i) {
-      const float2 a = split_fp64<32>(next);
+      const float2 a = split_fp64<32, true>(next);
       if (i + 1 < na) next = A[(size_t)(i + 1) * lda + r];
 #pragma unroll
       for (int j = 0; j < NBT; ++j) df_mac(S[j], Cc[j], a, Ms[i * NBT + j]);
