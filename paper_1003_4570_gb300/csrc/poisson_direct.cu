@@ -352,8 +352,7 @@ __global__ void __launch_bounds__(kT) columns_kernel(double* __restrict__ v, int
 
 // The tridiagonal systems' pivots c_j = 1 / (delta - c_{j-1}), c_1 = 1 / delta, delta = 2 + lambda / cz,
 // for the (nx/2+1)(ny/2+1) different eigenvalues lambda = 4 cx sin^2(pi kx / nx) + 4 cy sin^2(pi ky / ny):
-// ctab[j-1][ky][kx].  In closed form c_j = e^-t expm1(-2 j t) / expm1(-2 (j+1) t), sinh^2(t/2) =
-// lambda / (4 cz) (j / (j+1) for lambda = 0); a thread starts from it and runs the recurrence for
+// ctab[j-1][ky][kx].  A thread starts from the closed form (pivot_at) and runs the recurrence for
 // `run` unknowns, until it stands still (most modes: after some 20 / t unknowns).
 __device__ void pivots(const PGrid& g, double* __restrict__ ctab, long long t0, long long stride, int run) {
   const int hx = g.nx / 2 + 1, hy = g.ny / 2 + 1, modes = hx * hy;
@@ -365,14 +364,7 @@ __device__ void pivots(const PGrid& g, double* __restrict__ ctab, long long t0, 
     const double s = (g.cx * sx * sx + g.cy * sy * sy) / g.cz;      // lambda / (4 cz)
     const int j0 = ch * run + 1, j1 = min(j0 + run - 1, g.nzi);
     const double delta = fma(4.0, s, 2.0);
-    double c;
-    if (s == 0.0) {
-      c = (double)j0 / (j0 + 1);
-    } else {
-      // e^-t and expm1(-2 (j+1) t) from expm1(-t) and expm1(-2 j t), without cancellation
-      const double th = 2.0 * asinh(sqrt(s)), e1 = expm1(-th), q = e1 + 1.0, ej = expm1(-2.0 * j0 * th);
-      c = q * (ej / fma(ej, q * q, e1 * (q + 1.0)));
-    }
+    double c = pivot_at(s, j0);
     bool still = false;
     for (int j = j0;; ++j) {
       ctab[(long long)(j - 1) * modes + md] = c;
