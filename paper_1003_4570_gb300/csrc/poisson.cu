@@ -4,8 +4,8 @@
 // -div(eps0 eps_r grad phi) = rho on a uniform grid: 7-point stencil, periodic along x and y,
 // phi = 0 on the z = 0 and z = Lz planes.  omen_poisson solves it directly (poisson_direct.cu) and
 // iterates only for what direct corrections do not reach: lines of more than 2,048 points or 1,024
-// planes, a tolerance below the rounding of the residual, or no room for their work vectors;
-// omen_poisson_static, which may not allocate, always iterates.  The operator is symmetric positive
+// planes, few planes of lines with large primes (where iterating is faster), a tolerance below the
+// rounding of the residual, or no room for their work vectors; omen_poisson_static, which may not allocate, always iterates.  The operator is symmetric positive
 // definite, so plain CG (Hestenes & Stiefel 1952) applies.  The whole iteration runs in one cooperative
 // launch: three grid-wide barriers per iteration, block partial sums reduced by every block in
 // the same order, so all blocks see bit-identical scalars and leave the loop together.
@@ -502,7 +502,7 @@ extern "C" omen_status omen_poisson(omen_ctx* ctx, const omen_grid* gr, const do
   if (g.n >= (1ll << 31)) return set_err(ctx, OMEN_EINVAL, "grid larger than 2^31 unknowns");
   const double scale = 1.0 / (kEps0 * gr->eps_r);
   int done = 0;
-  if (poisson_direct_fits(g)) {
+  if (poisson_direct_fits(ctx, g, o->rtol, o->max_iter, mixed)) {
     // direct corrections; what they cannot reach (a tolerance below the rounding of b - A x) or
     // cannot allocate is left to the iterations below
     DirectResult dr{};

@@ -544,7 +544,69 @@ __global__ void __launch_bounds__(THREADS, 1) tridiag_kernel(PGrid g, double* __
 
 }  // namespace
 
-bool poisson_direct_fits(const PGrid& g) { return g.nx <= kMaxLine && g.ny <= kMaxLine && g.nzi <= kMaxZ; }
+// Work items of the transforms' launches for grids that are transformed line by line.
+struct LineShape {
+  int PX, PY;              // pairs of lines a block: rows, columns
+};
+static LineShape line_shape(const PGrid& g, int sms) {
+  // up to 2048 complex points a block, and enough blocks for every SM
+  auto pairs_of = [&](int len, long long pairs) {
+    const long long most = std::max(1, kMaxLine / len);
+    return (int)std::max<long long>(1, std::min(most, (pairs + 4 * sms - 1) / (4 * sms)));
+  };
+  LineShape L;
+  L.PX = pairs_of(g.nx, ((long long)g.ny * g.nzi + 1) / 2);
+  L.PY = std::min((g.nx + 1) / 2, std::max(pairs_of(g.ny, (long long)((g.nx + 1) / 2) * g.nzi), std::min(8, std::max(1, kMaxLine / g.ny))));
+  return L;
+}
+
+// FP64 operations of the transform of a pair of lines: six for a pair a +- w b, 2 R an output for the
+// first stage of a long prime R, 4 (R - 1) for other odd ones.
+static double line_ops(int n) {
+  const Fft p = plan_of(n);
+  double s = 0.0;
+  for (int f = 0; f < p.nf; ++f) {
+    const int R = p.rad[f];
+    s += (double)n * (R == 4 ? 6 : R == 2 ? 3 : f == 0 && R >= 5 ? 2 * R : 4 * (R - 1));
+  }
+  return s;
+}
+
+// Whether direct corrections are the faster way.  A line with a large prime costs operations in
+// proportion to it, while a grid of few planes, or a loose tolerance, needs few CG iterations; so
+// both are estimated, in us, from the FP64 rate (4,130 operations a us and SM) and the times of a
+// launch and of an iteration's grid barriers.  The lines lie where these estimates cross, 15% on the
+// direct side.  Measured, direct / CG (FP64, to 1e-13): 2039x2039x2 59.2 / 5.7 ms, 1021x1021x5 29.3 /
+// 13.6, 2039x16x3 4.3 / 1.4 go to CG; 1021x1021x17 111 / 168, 509x509x33 29 / 155, 1024x1024x2 0.8 / 1.8
+// and every grid of factors 2, 3 and 5 stay.  max_iter keeps twice the estimated iterations in hand,
+// and the mixed form, whose test is b - A x, a tolerance that its iterations reach.
+static bool direct_pays(const PGrid& g, double rtol, int max_iter, bool mixed, int sms) {
+  if (mixed && rtol < 1e-12) return true;
+  constexpr double kOpsPerUs = 4130.0;
+  auto waves = [&](double blocks) { return std::max(1.0, blocks / sms); };
+  const double ox = line_ops(g.nx), oy = line_ops(g.ny);
+  double transform;                                   // x and y once
+  if ((long long)g.nx * g.ny <= kPlanePoints) {
+    transform = 1.5 * (g.ny * ox + g.nx * oy) / kOpsPerUs * waves(0.5 * g.nzi);
+  } else {
+    const LineShape L = line_shape(g, sms);
+    transform = (ox * L.PX * waves(0.5 * g.ny * g.nzi / L.PX) + oy * L.PY * waves(0.5 * g.nx * g.nzi / L.PY)) / kOpsPerUs;
+  }
+  const double direct = 80.0 + 2.0 * transform + 60.0 * g.n / (kOpsPerUs * sms);
+  // CG: error falls by (k - 1) / (k + 1) an iteration, k^2 the condition number
+  const double t = M_PI / (2.0 * (g.nzi + 1)), sn = std::sin(t), cs = std::cos(t);
+  const double k = std::sqrt((4.0 * g.cx + 4.0 * g.cy + 4.0 * g.cz * cs * cs) / (4.0 * g.cz * sn * sn));
+  const double its = k > 1.0 + 1e-6 ? std::min((double)g.n, std::log(2.0 / rtol) / std::log((k + 1.0) / (k - 1.0))) : 1.0;
+  const double cg = 200.0 + (mixed ? 1.2 : 1.0) * its * ((mixed ? 55.0 : 15.0) + (mixed ? 8.0 : 23.0) * g.n / (kOpsPerUs * sms));
+  return !(cg < 0.85 * direct && 2.0 * its < max_iter);
+}
+
+bool poisson_direct_fits(const omen_ctx* ctx, const PGrid& g, double rtol, int max_iter, bool mixed) {
+  if (g.nx > kMaxLine || g.ny > kMaxLine || g.nzi > kMaxZ) return false;
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) return true;
+  return direct_pays(g, rtol, max_iter, mixed, sms);
+}
 
 omen_status poisson_direct(omen_ctx* ctx, const PGrid& g, const double* rho, double scale, double* x, double rtol,
                            int max_iter, bool true_residual, DirectResult* res) {
@@ -632,14 +694,8 @@ omen_status poisson_direct(omen_ctx* ctx, const PGrid& g, const double* rho, dou
       plane_pass(planes_kernel<false, false>, pblocks, scale);
     }
   } else {
-    // pairs of lines a block: up to 2048 complex points, and enough blocks for every SM
-    auto pairs_of = [&](int len, long long pairs) {
-      const long long most = std::max(1, kMaxLine / len);
-      return (int)std::max<long long>(1, std::min(most, (pairs + 4 * sms - 1) / (4 * sms)));
-    };
-    const int nrows = g.ny * g.nzi;
-    const int PX = pairs_of(g.nx, (nrows + 1) / 2);
-    const int PY = std::min((g.nx + 1) / 2, std::max(pairs_of(g.ny, (long long)((g.nx + 1) / 2) * g.nzi), std::min(8, std::max(1, kMaxLine / g.ny))));
+    const LineShape L = line_shape(g, sms);
+    const int PX = L.PX, PY = L.PY, nrows = g.ny * g.nzi;
     const unsigned bx = (unsigned)((nrows + 2 * PX - 1) / (2 * PX));
     const int tiles = (g.nx + 2 * PY - 1) / (2 * PY);
     const unsigned by = (unsigned)tiles * g.nzi;

@@ -13,8 +13,8 @@ struct DirectResult {
   double rel;          // ||r|| / ||b||
 };
 
-// Whether the grid's lines fit the transforms (else the caller iterates).
-bool poisson_direct_fits(const PGrid& g);
+// Whether the grid's lines fit the transforms and these are the faster way (else the caller iterates).
+bool poisson_direct_fits(const omen_ctx* ctx, const PGrid& g, double rtol, int max_iter, bool mixed);
 
 // Up to two corrections x += A^-1 r of the solution x of A x = scale * rho, r = b - A x.  The residual
 // of the second correction, tested against rtol ||b||, is r - A d, carried like the recurrence residual

@@ -1,4 +1,8 @@
-"""Calls of omen_poisson by the form of solve they take."""
+"""Calls of omen_poisson by the form of solve they take.
+
+Checked by the residual b - A x with the oracle's matrix, whose bound does not depend on the grid's
+condition (twice the tolerance asked for: the rest is the rounding of b - A x), and against the
+oracle's sparse solve within the error that this residual allows, ||r|| / lambda_min."""
 import numpy as np
 import pytest
 
@@ -29,3 +33,32 @@ def test_lateral_spacing_far_below_the_vertical_one(ctx, n):
     b = rho.ravel() / (poisson.EPS0 * g.eps_r)
     r = b - poisson.laplacian(g) @ phi.cpu().numpy().ravel()
     assert np.linalg.norm(r) <= 2e-12 * np.linalg.norm(b)
+
+
+def residual(g, rho, phi):
+    """||b - A phi|| and ||b||."""
+    b = rho.ravel() / (poisson.EPS0 * g.eps_r)
+    return np.linalg.norm(b - poisson.laplacian(g) @ phi.cpu().numpy().ravel()), np.linalg.norm(b)
+
+
+# lines of more than 2,048 points, more than 1,024 planes, and few planes of lines with a large prime
+@pytest.mark.parametrize("n", [(1, 1, 1100), (3, 2, 1027), (2050, 1, 4), (1, 2053, 3), (2049, 3, 12), (2039, 16, 3), (1021, 64, 3)],
+                         ids=lambda n: "x".join(map(str, n)))
+def test_iterated_grids_match_sparse_solve(ctx, n):
+    """Conjugate gradients in both precisions, narrow and wide rows."""
+    from paper_1003_4570_gb300 import omen
+    g = poisson.Grid(*n, 0.21 * n[0], 0.17 * n[1], 0.3 * n[2])
+    rho = np.random.default_rng(sum(n)).normal(size=g.shape) * 1e6
+    ref = poisson.solve_direct(g, rho)
+    rho_d = torch.from_numpy(rho).cuda()
+    for rtol in (1e-10, 1e-8):
+        for prec in (omen.OMEN_F64, omen.OMEN_F32_REFINE64):
+            phi = torch.zeros(g.shape, dtype=torch.float64, device="cuda")
+            info = omen.omen_poisson(ctx, g, rho_d, phi, rtol=rtol, precision=prec)
+            assert info["converged"] == 1 and info["rel_residual"] <= rtol
+            if max(n[:2]) > 2048 or n[2] > 1025:           # else the faster form is taken
+                assert info["iterations"] > 2
+            r, b = residual(g, rho, phi)
+            assert r <= 2 * rtol * b
+            smallest = 4 * np.sin(np.pi / (2 * g.nz)) ** 2 / g.h_m[2] ** 2
+            assert np.linalg.norm(phi.cpu().numpy() - ref) <= 2 * rtol * b / smallest

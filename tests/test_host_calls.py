@@ -1,4 +1,6 @@
 """Host code of the library's calls on a stand-in for the CUDA runtime (fake_runtime.py; no GPU)."""
+import contextlib
+
 import numpy as np
 import pytest
 
@@ -76,3 +78,27 @@ def test_a_failed_allocation_leaves_nothing_behind(watch, ctx, call):
         assert watch.live() == before, n
     watch.fail(-1)
     assert failed >= 15
+
+
+ITERATED = [((2039, 2039, 2), 1e-13), ((1021, 1021, 5), 1e-13), ((2039, 16, 3), 1e-6), ((1, 2039, 3), 1e-10), ((2053, 1, 3), 1e-9),
+            ((1, 1, 1100), 1e-9)]
+DIRECT = [((1, 1, 2), 1e-13), ((11, 11, 217), 1e-13), ((16, 13, 20), 1e-13), ((251, 241, 25), 1e-10), ((24, 251, 25), 1e-10),
+          ((251, 24, 25), 1e-10), ((53, 53, 9), 1e-6), ((1024, 1024, 2), 1e-13), ((251, 251, 25), 1e-6), ((2048, 2048, 2), 1e-6),
+          ((256, 256, 25), 1e-3), ((509, 509, 33), 1e-13)]
+
+
+@pytest.mark.parametrize("precision", [omen.OMEN_F64, omen.OMEN_F32_REFINE64])
+@pytest.mark.parametrize("n, rtol", ITERATED + DIRECT)
+def test_poisson_takes_the_faster_form(watch, ctx, n, rtol, precision):
+    """Lines with a large prime and few planes are iterated, the rest is solved directly; a limit on
+    the iterations that the iterated form might not keep leaves the direct one."""
+    f = np.zeros((n[2] - 1, n[1], n[0]))
+    iterated, fits = (n, rtol) in ITERATED, n[0] <= 2048 and n[2] <= 1025
+    if precision == omen.OMEN_F32_REFINE64 and rtol < 1e-12:
+        iterated = False
+    for limit in (100000, 20):
+        watch.reset()
+        with contextlib.suppress(omen.OmenError):      # the stand-in's iterations do not converge
+            omen.omen_poisson(ctx, poisson.Grid(*n, 0.2 * n[0], 0.2 * n[1], 0.2 * n[2]), f, f.copy(), rtol=rtol, precision=precision,
+                              max_iter=limit)
+        assert (watch.launches("cg_") == 1) == (iterated and (limit > 20 or not fits)), limit
