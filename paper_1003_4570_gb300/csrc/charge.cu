@@ -24,7 +24,7 @@
 // (contributing below 2^-166) count as zero, and so do occupations below 2^-126.  Infinite or
 // NaN amplitudes (and finite ones of 2^96 or more) give NaN.
 __device__ __forceinline__ void df_add_square(float& S, float& Cc, double v) {
-  const float2 h = split_fp64<32, false>(v);
+  const float2 h = split_fp64<32>(v);
   const float p = __fmul_rn(h.x, h.x);
   float e = __fmaf_rn(h.x, h.x, -p);
   e = __fmaf_rn(__fmul_rn(2.f, h.x), h.y, e);
@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(256) density_kernel(const void* __restrict__ p
           if constexpr (C) df_add_square(S, Cc, E::im(v));
         }
       }
-      df_mac(AS, AC, df_norm(S, Cc), split_fp64<0, false>(f));
+      df_mac(AS, AC, df_norm(S, Cc), split_fp64<0>(f));
     }
     // the squares carry the factor 2^64 of the split
     n_atom[i] += w * (((double)AS + (double)AC) * 0x1p-64);

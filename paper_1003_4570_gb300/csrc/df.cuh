@@ -34,31 +34,51 @@ __device__ __forceinline__ float2 df_from_double(double v) {
 }
 
 // v 2^kSplitShift as an FP32 pair (hi, lo), by integer operations only (the FP64 pipe, which
-// df_from_double uses, has 1/64 of the FP32 rate).  kRound: hi is v rounded to 24 significant bits and
-// lo the signed rest rounded to 24, so the pair is within 2^-49 of v relatively, as df_from_double's
-// is.  Else hi is the leading 24 bits: within 2^-48, twice the error on average, in fewer
-// instructions (electrons per atom of 16 states of 1M atoms: 229 us, 260 us with rounding).
-// Magnitudes too small for FP32 give zero, too large or non-finite ones NaN.
+// df_from_double uses, has 1/64 of the FP32 rate): hi keeps the sign, the exponent and the leading
+// 24 significant bits, lo is the rest rounded to FP32 (48 significant bits in all: the pair is within
+// 2^-48 of v relatively).  Magnitudes too small for FP32 give zero, too large or non-finite ones NaN.
+template <int kSplitShift>
+__device__ __forceinline__ float2 split_fp64(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned hi32 = (unsigned)(b >> 32), lo32 = (unsigned)b;
+  const int e = (int)((hi32 >> 20) & 0x7FFu);   // biased FP64 exponent
+  // FP32 exponent of hi: e - 1023 + 127 + shift
+  const int eh = e - 896 + kSplitShift;
+  if (eh <= 0) return make_float2(0.f, 0.f);     // |v| < 2^-158, or zero
+  if (eh >= 255) return make_float2(__int_as_float(0x7fc00000), 0.f);   // beyond FP32, inf or NaN: NaN
+  const unsigned sign = hi32 & 0x80000000u;
+  const unsigned top23 = ((hi32 & 0xFFFFFu) << 3) | (lo32 >> 29);
+  const float hi = __uint_as_float(sign | ((unsigned)eh << 23) | top23);
+  // the remaining 29 bits: rem * 2^(e - 1075 + shift)
+  const unsigned rem = lo32 & 0x1FFFFFFFu;
+  const int el = e - 948 + kSplitShift;
+  const float scale = el > 0 ? __uint_as_float((unsigned)el << 23) : 0.f;
+  const float lo = __fmul_rn(__uint2float_rn(rem), scale);
+  return make_float2(hi, sign ? -lo : lo);
+}
+
+// The same with hi rounded to 24 significant bits and lo the signed rest: within 2^-49 of v, as
+// df_from_double is, with half the error on average, for some more instructions (electrons per atom
+// of 16 states of 1M atoms would take 260 us with it, 229 us with the leading bits).
 struct SplitBits {
   unsigned hi, scale;                  // hi, and the unit of the rest with v's sign, as FP32 bits
   int rest;
 };
-template <int kSplitShift, bool kRound>
-__host__ __device__ __forceinline__ SplitBits split_bits(unsigned long long b) {
+template <int kSplitShift>
+__host__ __device__ __forceinline__ SplitBits split_rounded_bits(unsigned long long b) {
+  const unsigned long long up = b + 0x10000000u;    // half of hi's last place, which may carry up to the exponent
   const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
-  const int e = (int)((unsigned)(b >> 52) & 0x7FFu);                       // biased FP64 exponent
-  // half of hi's last place, which may carry up to the exponent, leaves the bits of hi on top
-  const unsigned long long top = kRound ? b + 0x10000000u : b;
-  const int eh = (kRound ? (int)((unsigned)(top >> 52) & 0x7FFu) : e) - 896 + kSplitShift;   // FP32 exponent of hi
-  if (eh <= 0) return SplitBits{0, 0, 0};                                  // |v| < 2^-158 (shift 32), or zero
-  if (eh >= 255) return SplitBits{0x7fc00000u, 0, 0};                      // beyond FP32, inf or NaN: NaN
+  const int e = (int)((unsigned)(b >> 52) & 0x7FFu), eu = (int)((unsigned)(up >> 52) & 0x7FFu);   // biased FP64 exponents
+  const int eh = eu - 896 + kSplitShift;            // FP32 exponent of hi
+  if (eh <= 0) return SplitBits{0, 0, 0};
+  if (eh >= 255) return SplitBits{0x7fc00000u, 0, 0};
   // the rest in units of 2^(e - 1075 + shift)
   const int el = e - 948 + kSplitShift;
-  return SplitBits{sign | ((unsigned)eh << 23) | ((unsigned)(top >> 29) & 0x7FFFFFu), el > 0 ? sign | ((unsigned)el << 23) : 0u,
-                   (int)((unsigned)top & 0x1FFFFFFFu) - (kRound ? 0x10000000 : 0)};
+  return SplitBits{sign | ((unsigned)eh << 23) | ((unsigned)(up >> 29) & 0x7FFFFFu), el > 0 ? sign | ((unsigned)el << 23) : 0u,
+                   (int)((unsigned)up & 0x1FFFFFFFu) - 0x10000000};
 }
-template <int kSplitShift, bool kRound>
-__device__ __forceinline__ float2 split_fp64(double v) {
-  const SplitBits s = split_bits<kSplitShift, kRound>((unsigned long long)__double_as_longlong(v));
+template <int kSplitShift>
+__device__ __forceinline__ float2 split_fp64_rounded(double v) {
+  const SplitBits s = split_rounded_bits<kSplitShift>((unsigned long long)__double_as_longlong(v));
   return make_float2(__uint_as_float(s.hi), __fmul_rn(__int2float_rn(s.rest), __uint_as_float(s.scale)));
 }

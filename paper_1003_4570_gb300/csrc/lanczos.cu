@@ -778,7 +778,7 @@ __global__ void __launch_bounds__(256) combine_split_kernel(const double* __rest
     for (int j = 0; j < NBT; ++j) { S[j] = 0.f; Cc[j] = 0.f; }
     double next = A[r];
     for (int i = 0; i < na; ++i) {
-      const float2 a = split_fp64<32, true>(next);
+      const float2 a = split_fp64_rounded<32>(next);
       if (i + 1 < na) next = A[(size_t)(i + 1) * lda + r];
 #pragma unroll
       for (int j = 0; j < NBT; ++j) df_mac(S[j], Cc[j], a, Ms[i * NBT + j]);
