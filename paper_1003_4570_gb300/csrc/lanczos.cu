@@ -28,6 +28,7 @@
 #include "omen_internal.h"
 #include "pdl.cuh"
 #include "smem.cuh"
+#include "split_pass.h"
 #include "vec.cuh"
 #include "df.cuh"
 
@@ -1408,30 +1409,29 @@ struct KrylovOps {
       if (prec == OMEN_F64 && !cplx) {
         const unsigned grid = (unsigned)std::min<long long>((n + 255) / 256, (long long)sm_count * 8);
         const double* Ad = static_cast<const double*>(A);
-        // columns a pass: 25 where that saves one (49 of a basis of 96: two passes, not four)
-        const int nc = nbj <= 8 ? 8 : nbj <= 16 ? 16 : 25;
-        const size_t shs = (size_t)na * nc * sizeof(float2);
-        for (int c0 = 0; c0 < nbj; c0 += nc) {
-          const int w = std::min(nc, nbj - c0);
+        for (int c0 = 0; c0 < nbj;) {
+          const SplitPass ps = split_pass(na, nbj, nbj - c0);
+          const size_t shs = (size_t)na * ps.kernel * sizeof(float2);
           double* Yd = static_cast<double*>(Yj) + (size_t)c0 * n;
           const double2* Mj = d_small + (size_t)c0 * na;
-#define SPLITC(NCc)                                                                                       \
-  do {                                                                                                    \
-    smem_limit(combine_split_kernel<NCc>, shs);                                                           \
-    combine_split_kernel<NCc><<<grid, 256, shs, ctx->stream>>>(Ad, n, na, Mj, w, Yd, n, n, alpha, beta);  \
+#define SPLITC(NCc)                                                                                            \
+  do {                                                                                                         \
+    smem_limit(combine_split_kernel<NCc>, shs);                                                                \
+    combine_split_kernel<NCc><<<grid, 256, shs, ctx->stream>>>(Ad, n, na, Mj, ps.cols, Yd, n, n, alpha, beta); \
   } while (0)
-          if (nc == 8) SPLITC(8); else if (nc == 16) SPLITC(16); else SPLITC(25);
+          if (ps.kernel == 8) SPLITC(8); else if (ps.kernel == 16) SPLITC(16); else SPLITC(25);
+          c0 += ps.cols;
 #undef SPLITC
         }
       } else {
         // few rows: four columns and 64 rows a CTA
         const bool few = (n + 255) / 256 < sm_count;
-        const int nc = few ? 4 : kMaxBlockCols, thr = few ? 64 : 256;
+        const int nc = few || (size_t)na * kMaxBlockCols * sizeof(double2) > kMaxDynamicSmem ? 4 : kMaxBlockCols, thr = few ? 64 : 256;
         const dim3 grid((unsigned)std::min<long long>((n + thr - 1) / thr, (long long)sm_count * 8), (nbj + nc - 1) / nc);
 #define COMB_LAUNCH(T, Cc)                                                                                   \
   do {                                                                                                       \
-    const size_t shm = (size_t)na * nc * sizeof(double2);                                                    \
-    if (few) {                                                                                               \
+    const size_t shm = (size_t)na * std::min(nc, nbj) * sizeof(double2);                                     \
+    if (nc == 4) {                                                                                            \
       smem_limit(combine_kernel<T, Cc, 4>, shm);                                                             \
       combine_kernel<T, Cc, 4><<<grid, thr, shm, ctx->stream>>>(A, n, na, d_small, nbj, Yj, n, n, alpha, beta); \
     } else {                                                                                                 \

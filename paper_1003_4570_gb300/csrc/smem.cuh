@@ -11,6 +11,8 @@
 #include <mutex>
 #include <utility>
 
+constexpr size_t kMaxDynamicSmem = 227 * 1024;   // a block's most on sm_103
+
 template <typename K>
 inline cudaError_t smem_limit(K kernel, size_t bytes) {
   static std::mutex mu;

@@ -25,6 +25,7 @@ SOURCE = r"""
 #include <string>
 #include <vector>
 static std::mutex mu;
+static thread_local cudaError_t last = cudaSuccess;
 static std::map<void*, size_t> live;
 static long fail_at = -1, changed = 0, lowered = 0;
 static std::map<const void*, std::string> names;
@@ -61,7 +62,7 @@ static void reached() {
 static cudaError_t run(const void* f, size_t shared, void** args) {
   std::lock_guard<std::mutex> l(mu);
   auto it = limits.find(f);
-  if (shared > (size_t)(it == limits.end() ? 48 << 10 : it->second)) return cudaErrorInvalidValue;
+  if (shared > (size_t)(it == limits.end() ? 48 << 10 : it->second)) return last = cudaErrorInvalidValue;
   const std::string& name = names[f];
   ++launches[name];
   if (name.find("reduce_dev_kernel") != std::string::npos) {   // (partials, chunks, na, nb, out, ...)
@@ -98,7 +99,7 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
 cudaError_t cudaLaunchCooperativeKernel(const void* f, dim3, dim3, void** a, size_t s, cudaStream_t) { return run(f, s, a); }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute, int v) {
   std::lock_guard<std::mutex> l(mu);
-  if (v > 227 << 10) return cudaErrorInvalidValue;
+  if (v > 227 << 10) return last = cudaErrorInvalidValue;
   if (limits.count(f) && v < limits[f]) ++lowered;
   limits[f] = v;
   return cudaSuccess;
@@ -128,7 +129,7 @@ cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 152; return cudaSuccess; }
 const char* cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "no error" : "error"; }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() { const cudaError_t e = last; last = cudaSuccess; return e; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* n, const void*, int, size_t) { *n = 2; return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = 2; return cudaSuccess; }
 cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps*) { *p = (cudaMemPool_t)8; return cudaSuccess; }

@@ -102,3 +102,14 @@ def test_poisson_takes_the_faster_form(watch, ctx, n, rtol, precision):
             omen.omen_poisson(ctx, poisson.Grid(*n, 0.2 * n[0], 0.2 * n[1], 0.2 * n[2]), f, f.copy(), rtol=rtol, precision=precision,
                               max_iter=limit)
         assert (watch.launches("cg_") == 1) == (iterated and (limit > 20 or not fits)), limit
+
+
+# (Ritz vectors combined, passes of 8, 16 and 25 columns): whole passes without idle columns where that
+# costs no extra pass
+@pytest.mark.parametrize("cols, passes", [(9, (0, 1, 0)), (17, (0, 0, 1)), (32, (0, 2, 0)), (33, (1, 0, 1)), (49, (0, 0, 2)),
+                                          (51, (1, 0, 2)), (64, (0, 1, 2))])
+def test_passes_of_a_restart(watch, ctx, cols, passes):
+    ham = hamiltonian(ctx, (2, 2, 3))
+    omen.omen_set_locking_check(ctx, False)
+    omen.omen_eigs(ctx, ham, cols - 1, block=1, basis=96, raise_on_noconv=False)
+    assert tuple(watch.launches(f"combine_split_kernelILi{n}E") for n in (8, 16, 25)) == passes
