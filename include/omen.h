@@ -342,7 +342,9 @@ typedef struct {
 
 typedef struct {
   int iterations;            /* block steps taken */
-  long long hx_count;        /* single-vector H·X products */
+  long long hx_count;        /* single-vector H·X products (as iterations: of the steps used; a
+                                solve on vectors of up to 1.5 MB may run up to a check's interval
+                                of steps past its last check) */
   int restarts;
   int converged;             /* 1 if every returned pair met tol */
   double max_residual;       /* max FP64 ||H x - lambda x|| over returned pairs (eV) */

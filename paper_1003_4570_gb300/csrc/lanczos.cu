@@ -2413,6 +2413,9 @@ struct SegmentGraphs {
   }
 };
 
+// Vectors up to this size queue a segment ahead of a host check (see there for both sides).
+static constexpr size_t kAheadBytes = 3 << 19;
+
 static omen_status lanczos_solve_single(KrylovOps& op, const omen_eig_opts* o, void* X, int k_out,
                                         omen_eig_info* info, bool& converged) {
   omen_ctx* ctx = op.ctx;
@@ -2612,8 +2615,13 @@ static omen_status lanczos_solve_single(KrylovOps& op, const omen_eig_opts* o, v
       if (flag) return set_err(ctx, OMEN_ENUMERIC, "Lanczos breakdown or non-finite value (zero or NaN norm)");
       // The basis has room and iterations are left: the next segment runs while the host solves the
       // projected problem.  It writes only basis vectors and columns of T past those of this check, so
-      // a check that ends the solve leaves it unused (at most one segment).
-      if (!full && iter < max_iter_of(o)) {
+      // a check that ends the solve leaves it unused (at most one segment, which no count includes).
+      // What that hides is the host's share, 0.1 to 1 ms a check whatever the rows; what it may waste
+      // grows with them.  Whole solves without and with it: 1,280 complex rows 59.0 -> 53.7 ms, 41k rows
+      // 30.6 -> 28.2 ms, 138k rows 53.1 -> 49.5 ms, 216k rows 103.3 -> 97.5 and 43.8 -> 45.7 ms, 640k
+      // rows 178.0 -> 180.9 and, to a loose tolerance, 50.0 -> 55.8 ms, 2.7M rows 462 -> 483 ms: so
+      // vectors of up to 1.5 MB.
+      if (!full && iter < max_iter_of(o) && vbytes <= kAheadBytes) {
         const int js0 = jstart, nb0 = nbas;
         jstart = nbas;
         nbas += 1;
