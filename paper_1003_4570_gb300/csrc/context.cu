@@ -1,4 +1,6 @@
 // Context: device, stream, last error, small work buffers.
+#include <cstring>
+
 #include "omen_internal.h"
 
 extern "C" omen_status omen_create(omen_ctx** out, int device, void* stream) {
@@ -45,8 +47,35 @@ extern "C" void omen_destroy(omen_ctx* c) {
     if (st) cudaStreamDestroy(st);
   if (c->host_scratch) cudaFree(c->host_scratch);
   for (cudaEvent_t e : c->host_events) cudaEventDestroy(e);
+  if (c->stage_done) {
+    cudaEventSynchronize(c->stage_done);
+    cudaEventDestroy(c->stage_done);
+  }
+  if (c->stage) cudaFreeHost(c->stage);
   if (c->pool) cudaMemPoolDestroy(c->pool);   // work still in flight keeps its part until it is freed
   delete c;
+}
+
+omen_status copy_to_device(omen_ctx* ctx, void* dst, const void* src, size_t bytes) {
+  if (bytes <= kStageBytes && !ctx->stage) {
+    if (cudaMallocHost(&ctx->stage, kStageBytes) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->stage_done, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      if (ctx->stage) cudaFreeHost(ctx->stage);
+      ctx->stage = nullptr;
+      ctx->stage_done = nullptr;
+    }
+  }
+  if (bytes <= kStageBytes && ctx->stage) {
+    OMEN_CUDA(ctx, cudaEventSynchronize(ctx->stage_done));   // the copy before this one has left the stage
+    std::memcpy(ctx->stage, src, bytes);
+    OMEN_CUDA(ctx, cudaMemcpyAsync(dst, ctx->stage, bytes, cudaMemcpyHostToDevice, ctx->stream));
+    OMEN_CUDA(ctx, cudaEventRecord(ctx->stage_done, ctx->stream));
+    return OMEN_OK;
+  }
+  OMEN_CUDA(ctx, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, ctx->stream));
+  OMEN_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  return OMEN_OK;
 }
 
 extern "C" omen_status omen_set_reorthogonalization(omen_ctx* c, int policy) {

@@ -1382,19 +1382,10 @@ struct KrylovOps {
     return OMEN_OK;
   }
 
-  // `count` coefficients into d_small, after the kernels that read what was there.  The runtime may
-  // read pageable memory until the stream is next synchronised, and callers drop M when they return:
-  // the copy is waited for here (the kernels that use it are not).
-  omen_status upload_small(const cd* M, size_t count) {
-    OMEN_CUDA(ctx, cudaMemcpyAsync(d_small, M, count * sizeof(double2), cudaMemcpyHostToDevice, ctx->stream));
-    OMEN_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return OMEN_OK;
-  }
-
   // Y = beta*Y + alpha * A M   (M host na x nb column-major)
   omen_status combine(const void* A, int na, const std::vector<cd>& M, int nb, void* Y, double alpha, double beta) {
     if ((nb <= 4 || prec == OMEN_F64_DF) && (size_t)na * nb <= small_cap) {
-      omen_status s1 = upload_small(M.data(), (size_t)na * nb);
+      omen_status s1 = copy_to_device(ctx, d_small, M.data(), (size_t)na * nb * sizeof(double2));
       if (s1 != OMEN_OK) return s1;
       return combine_dev(A, na, d_small, nb, Y, alpha, beta);
     }
@@ -1403,7 +1394,7 @@ struct KrylovOps {
     const int most = (int)std::min<size_t>(nb, small_cap / na / 400 ? small_cap / na / 400 * 400 : kMaxBlockCols);
     for (int j0 = 0; j0 < nb; j0 += most) {
       const int nbj = std::min(most, nb - j0);
-      omen_status s1 = upload_small(M.data() + (size_t)j0 * na, (size_t)na * nbj);
+      omen_status s1 = copy_to_device(ctx, d_small, M.data() + (size_t)j0 * na, (size_t)na * nbj * sizeof(double2));
       if (s1 != OMEN_OK) return s1;
       void* Yj = col(Y, j0);
       if (prec == OMEN_F64 && !cplx) {

@@ -28,12 +28,22 @@ struct omen_ctx {
   void* host_scratch = nullptr;
   size_t host_scratch_bytes = 0;
   std::vector<cudaEvent_t> host_events;  // the pipeline's events, created once
+  // pinned host memory that small coefficient tables are copied from, and the event after the last
+  // such copy (made on first use)
+  void* stage = nullptr;
+  cudaEvent_t stage_done = nullptr;
   // work areas of the calls come from a pool of the context's own, which keeps up to kPoolKeep
   // bytes mapped between calls (the default pool gives everything back at the next
   // synchronisation, and a call then spends 0.1 to 0.4 ms mapping it again); gone with the context
   cudaMemPool_t pool = nullptr;
 };
 constexpr unsigned long long kPoolKeep = 512ull << 20;
+constexpr size_t kStageBytes = 512 << 10;
+
+// `bytes` of host memory that the caller may drop on return, to dst on the context's stream: through
+// the pinned stage, else waited for (the runtime may read pageable memory until the stream is next
+// synchronised).
+omen_status copy_to_device(omen_ctx* ctx, void* dst, const void* src, size_t bytes);
 
 // Stream-ordered device memory for one call on the context's stream (free with cudaFreeAsync).
 template <typename T>
