@@ -292,16 +292,17 @@ typedef struct {
   int rows_per_batch;        /* load batch (omen_tune_hx: bonds whose amplitudes are loaded
                                 together, 1 -> 1, 2 -> 2, 5 and 10 -> 4) or wave vectors per
                                 thread (omen_tune_hx_kbatch); 0 = the built-in rule */
-  int candidates;            /* launch shapes timed */
+  int candidates;            /* launch shapes timed, each distinct one once */
   double ms_best;            /* mean launch time of the chosen shape (ms) */
   double ms_default;         /* mean launch time of the built-in shape (ms) */
 } omen_tune_result;
 
-/* Time every compiled launch shape of omen_hx on this Hamiltonian (nvec vectors of precision
+/* Time every distinct launch shape of omen_hx on this Hamiltonian (nvec vectors of precision
  * OMEN_F64 or OMEN_F32, `reps` timed launches each after two warm-ups, CUDA events on the ctx
  * stream) and keep the fastest for later products and solves with that vector precision.
  * Allocates and frees two scratch blocks of nvec vectors; synchronises the stream.  Results
- * of the product do not depend on the shape.  out may be NULL.  EINVAL for a precision
+ * of the product do not depend on the shape.  Products too small to fill the device take one kernel
+ * whatever the shape; the built-in one is kept for them.  out may be NULL.  EINVAL for a precision
  * without blocks in this Hamiltonian. */
 omen_status omen_tune_hx(omen_ctx* ctx, omen_ham* ham, int vec_precision, int nvec, int reps,
                          omen_tune_result* out);

@@ -862,22 +862,32 @@ static bool rb_valid(int norb, bool f64, bool so, bool mf, int rb) {
   return rb == 1 || rb == 2 || rb == 5 || (rb == norb && !so);
 }
 
+// The kernel of a product, from the whole structure (so that a product computed in pieces has the same
+// bits).
+enum class HxRoute { kKinds, kSplit, kRows };
+static HxRoute hx_route(int ncells, bool f64, bool cplx, bool so, int norb, int nvec) {
+  const int cells = cplx ? 4 : 8;
+  const long long each = 8ll * (so ? 2 : 1) * nvec;
+  if ((ncells + cells - 1) / cells * each <= kinds_upto(f64, cplx)) return HxRoute::kKinds;
+  return (ncells + 31) / 32 * each < split_below(f64, cplx, norb) ? HxRoute::kSplit : HxRoute::kRows;
+}
+
+// Bonds whose amplitudes are loaded together: rb 1 -> 1, 2 -> 2, 5 or 10 -> 4.
+static int loads_of(bool f64, bool cplx, int rb) { return rb == 0 ? (!f64 && !cplx ? 2 : 1) : rb == 1 ? 1 : rb == 2 ? 2 : 4; }
+
 template <typename T, int NORB, bool CPLX, bool SO>
 static cudaError_t launch_rows(const HxInst<T>& I, int nvec, HxTile t, double sigma, int cell0, int cell1, const void* x,
                                void* y, cudaStream_t st) {
-  // the rule looks at the whole structure, so a product computed in pieces has the same bits
-  const long long warps = (long long)((I.g.ncells + 31) / 32) * 8 * (SO ? 2 : 1) * nvec;
   constexpr int cells = CPLX ? 4 : 8;
   // a warp (kinds: a CTA) each; small CTAs spread over the SMs
   const dim3 grid((unsigned)((cell1 - cell0 + cells - 1) / cells) * 8, SO ? 2 : 1, nvec);
-  const long long units = (long long)((I.g.ncells + cells - 1) / cells) * 8 * (SO ? 2 : 1) * nvec;
-  if (units <= kinds_upto(sizeof(T) == 8, CPLX))
+  const HxRoute route = hx_route(I.g.ncells, sizeof(T) == 8, CPLX, SO, NORB, nvec);
+  if (route == HxRoute::kKinds)
     return launch_dependent(hx_kinds_kernel<T, NORB, CPLX, SO>, grid, dim3(NORB == 10 ? 128 : 64), 0, st, I, sigma, cell0, cell1, x, y);
-  if (warps < split_below(sizeof(T) == 8, CPLX, NORB))
+  if (route == HxRoute::kSplit)
     return launch_dependent(hx_split_kernel<T, NORB, CPLX, SO>, grid, dim3(32), 0, st, I, sigma, cell0, cell1, x, y);
-  // bonds whose amplitudes are loaded together: rb 1 -> 1, 2 -> 2, 5 or 10 -> 4
   const int thr = t.threads ? t.threads : 128;
-  const int lb = t.rb == 0 ? (sizeof(T) == 4 && !CPLX ? 2 : 1) : t.rb == 1 ? 1 : t.rb == 2 ? 2 : 4;
+  const int lb = loads_of(sizeof(T) == 8, CPLX, t.rb);
   if constexpr (sizeof(T) == 4) if (lb == 4) return launch_t<T, NORB, CPLX, SO, 4>(I, nvec, thr, sigma, cell0, cell1, x, y, st);
   if (lb == 2) return launch_t<T, NORB, CPLX, SO, 2>(I, nvec, thr, sigma, cell0, cell1, x, y, st);
   return launch_t<T, NORB, CPLX, SO, 1>(I, nvec, thr, sigma, cell0, cell1, x, y, st);
@@ -888,6 +898,13 @@ bool hx_tile_valid(const omen_ham* h, int vec_precision, int threads, int rb) {
   if (threads != 0 && (threads < 32 || threads > 128 || threads % 32 != 0)) return false;
   return rb_valid(h->norb, vec_precision == OMEN_F64, h->spin_orbit, h->matrix_free, rb);
 }
+
+// Whether products of nvec vectors look at the launch shape (small ones take one kernel whatever is set),
+// and what distinguishes the shapes (threads, rb) there.
+bool hx_takes_tile(const omen_ham* h, int vec_precision, int nvec) {
+  return hx_route(h->lat->ncells, vec_precision == OMEN_F64, h->is_complex, h->spin_orbit, h->norb, nvec) == HxRoute::kRows;
+}
+int hx_tile_loads(const omen_ham* h, int vec_precision, int rb) { return loads_of(vec_precision == OMEN_F64, h->is_complex, rb); }
 
 // The structure, reduced blocks and potential of a Hamiltonian for FP64 or FP32 products.
 template <typename T>

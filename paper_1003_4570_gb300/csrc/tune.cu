@@ -4,11 +4,15 @@
 // precision and structure.  The tuner times every compiled shape on the Hamiltonian itself
 // (CUDA events on the context's stream, after warm-up launches) and keeps the fastest.  No
 // shape changes the result: each accumulator sums its terms in the same order.
+#include <set>
+#include <utility>
 #include <vector>
 
 #include "omen_internal.h"
 
 bool hx_tile_valid(const omen_ham* h, int vec_precision, int threads, int rb);
+bool hx_takes_tile(const omen_ham* h, int vec_precision, int nvec);
+int hx_tile_loads(const omen_ham* h, int vec_precision, int rb);
 bool hx_kbatch_tile_valid(int vec_precision, int threads, int kb);
 
 namespace {
@@ -58,9 +62,11 @@ omen_status time_launches(omen_ctx* ctx, int reps, F&& launch, double& ms) {
   return OMEN_OK;
 }
 
-// Time every candidate (threads, rb) with `launch`, set the fastest through `set`.
+// Time every candidate (threads, rb) with `launch`, set the fastest through `set`; the first is the
+// built-in shape, which stays where the launches do not depend on the shape (their times then differ
+// by noise only).
 template <typename L, typename S>
-omen_status tune_loop(omen_ctx* ctx, const std::vector<HxTile>& cand, int reps, L&& launch, S&& set,
+omen_status tune_loop(omen_ctx* ctx, const std::vector<HxTile>& cand, int reps, bool depends, L&& launch, S&& set,
                       omen_tune_result* out) {
   double best = 0.0, dflt = 0.0;
   HxTile pick;
@@ -74,7 +80,7 @@ omen_status tune_loop(omen_ctx* ctx, const std::vector<HxTile>& cand, int reps, 
       return s;
     }
     if (t.threads == 0 && t.rb == 0) dflt = ms;
-    if (timed == 0 || ms < best) {
+    if (timed == 0 || (depends && ms < best)) {
       best = ms;
       pick = t;
     }
@@ -128,13 +134,16 @@ extern "C" omen_status omen_tune_hx(omen_ctx* ctx, omen_ham* h, int vec_precisio
   }
   tune_fill_kernel<<<1216, 256, 0, ctx->stream>>>(static_cast<float*>(sx.p), (long long)(bytes / 4));
   OMEN_CHECK_LAUNCH(ctx);
+  // each (width, loads) once: several rb may name the same
   std::vector<HxTile> cand{HxTile{}};
+  std::set<std::pair<int, int>> seen{{128, hx_tile_loads(h, vec_precision, 0)}};
   for (int thr : {32, 64, 96, 128})
     for (int rb : {0, 1, 2, 5, 10})
-      if (hx_tile_valid(h, vec_precision, thr, rb)) cand.push_back(HxTile{thr, rb});
+      if (hx_tile_valid(h, vec_precision, thr, rb) && seen.insert({thr, hx_tile_loads(h, vec_precision, rb)}).second)
+        cand.push_back(HxTile{thr, rb});
   const int slot = prec_slot(vec_precision);
   return tune_loop(
-      ctx, cand, reps, [&]() { return launch_hx(ctx, h, sx.p, sy.p, nvec, 0.0, vec_precision); },
+      ctx, cand, reps, hx_takes_tile(h, vec_precision, nvec), [&]() { return launch_hx(ctx, h, sx.p, sy.p, nvec, 0.0, vec_precision); },
       [&](HxTile t) { h->tile[slot] = t; }, out);
 }
 
@@ -165,10 +174,11 @@ extern "C" omen_status omen_tune_hx_kbatch(omen_ctx* ctx, omen_ham* h, int nk, i
   std::vector<HxTile> cand{HxTile{}};
   for (int thr : {32, 64, 96, 128})
     for (int kb : {1, 2, 4})
-      if (hx_kbatch_tile_valid(prec, thr, kb)) cand.push_back(HxTile{thr, kb});
+      if ((thr != 128 || kb != 1) && hx_kbatch_tile_valid(prec, thr, kb))   // 128, 1 is the built-in shape
+        cand.push_back(HxTile{thr, kb});
   const int slot = prec_slot(prec);
   s = tune_loop(
-      ctx, cand, reps, [&]() { return launch_hx_kbatch(ctx, h, nk, ph, sx.p, sy.p, 0.0, prec); },
+      ctx, cand, reps, true, [&]() { return launch_hx_kbatch(ctx, h, nk, ph, sx.p, sy.p, 0.0, prec); },
       [&](HxTile t) { h->ktile[slot] = t; }, out);
   cudaFreeAsync(ph, ctx->stream);
   return s;

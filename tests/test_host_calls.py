@@ -125,3 +125,18 @@ def test_steps_ahead_of_a_check(watch, ctx, cells, ahead, precision):
     info = omen.omen_eigs(ctx, ham, 4, block=1, basis=48, raise_on_noconv=False)[1]
     assert info["iterations"] == 12
     assert watch.launches("update_norm_kernel") == (24 if ahead else 12)
+
+
+@pytest.mark.parametrize("cells, tuned", [((2, 2, 3), False), ((10, 10, 10), False), ((20, 20, 20), True)])
+def test_tuner_keeps_the_built_in_shape_of_small_products(watch, ctx, cells, tuned):
+    """Small products take one kernel whatever shape is set, so the times of its launches (here each
+    shorter than the one before) say nothing; of larger ones every distinct launch is timed once."""
+    ham = hamiltonian(ctx, cells, precision=omen.OMEN_F32)
+    r = omen.omen_tune_hx(ctx, ham, reps=1)
+    assert r["candidates"] == 12                       # four widths, one, two or four bonds' loads
+    if tuned:
+        assert (r["threads"], r["rows_per_batch"]) == (128, 5) and r["ms_best"] < r["ms_default"]
+        assert watch.launches("hx_kernel") == 3 * 12
+    else:
+        assert (r["threads"], r["rows_per_batch"]) == (128, 0) and r["ms_best"] == r["ms_default"]
+        assert watch.launches("hx_kernel") == 0
