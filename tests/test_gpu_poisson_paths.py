@@ -62,3 +62,19 @@ def test_iterated_grids_match_sparse_solve(ctx, n):
             assert r <= 2 * rtol * b
             smallest = 4 * np.sin(np.pi / (2 * g.nz)) ** 2 / g.h_m[2] ** 2
             assert np.linalg.norm(phi.cpu().numpy() - ref) <= 2 * rtol * b / smallest
+
+
+# line by line with several runs of 64 pivots and chains of several segments: 16 unknowns a thread, 32 a
+# thread with up to 256 and with more unknowns; planes at once with more than 256
+@pytest.mark.parametrize("n", [(64, 49, 150), (128, 81, 200), (64, 80, 300), (9, 64, 400)], ids=lambda n: "x".join(map(str, n)))
+def test_deep_grids(ctx, n):
+    from paper_1003_4570_gb300 import omen
+    g = poisson.Grid(*n, 0.21 * n[0], 0.17 * n[1], 0.3 * n[2])
+    rho = np.random.default_rng(sum(n)).normal(size=g.shape) * 1e6 + 2e5
+    rho_d = torch.from_numpy(rho).cuda()
+    for prec in (omen.OMEN_F64, omen.OMEN_F32_REFINE64):
+        phi = torch.zeros(g.shape, dtype=torch.float64, device="cuda")
+        info = omen.omen_poisson(ctx, g, rho_d, phi, rtol=1e-11, precision=prec)
+        assert info["converged"] == 1 and info["iterations"] <= 2
+        r, b = residual(g, rho, phi)
+        assert r <= 2e-11 * b
