@@ -179,8 +179,7 @@ static constexpr int dots1_ig(bool cplx) { return cplx ? 8 : kIG; }
 template <typename T, bool C, int IG>
 __global__ void __launch_bounds__(256, 2) dots1_kernel(const void* Av, long long lda, int na, int per, const void* Bv,
                                                     long long n, int rows_per_cta, double2* P, DotsFinish fin,
-                                                    long long a_ps = 0, long long b_ps = 0, long long p_ps = 0,
-                                                    const long long* poff = nullptr, const long long* plen = nullptr,
+                                                    long long p_ps = 0, const long long* poff = nullptr, const long long* plen = nullptr,
                                                     const int* act = nullptr) {
   using E = Elem<T, C>;
   using V = typename E::V;
@@ -188,15 +187,15 @@ __global__ void __launch_bounds__(256, 2) dots1_kernel(const void* Av, long long
   constexpr int NA = C ? 2 * IG : IG;
   // IG basis vectors per CTA (at most dots1_ig(C)); chosen from na so that no accumulator
   // sits idle under a predicate (predicated-off FP64 FMAs still occupy the pipe)
-  // grid.z = independent problems (batched Lanczos): offsets a_ps, b_ps (elements), p_ps
-  // (partials) per problem, or per-problem element offsets poff and lengths plen
+  // grid.z = independent problems (batched Lanczos): p_ps partials each, per-problem element offsets
+  // poff and lengths plen
   pdl_wait();
   pdl_trigger();
   const long long off = poff ? poff[blockIdx.z] : 0;
   if (act && !act[blockIdx.z]) return;   // a converged (frozen) problem of the batch
   if (plen) n = plen[blockIdx.z];
-  const V* A = static_cast<const V*>(Av) + blockIdx.z * a_ps + off;
-  const V* B = static_cast<const V*>(Bv) + blockIdx.z * b_ps + off;
+  const V* A = static_cast<const V*>(Av) + off;
+  const V* B = static_cast<const V*>(Bv) + off;
   P += blockIdx.z * p_ps;
   const int i0 = blockIdx.x * per;
   const int ni = min(per, na - i0);
@@ -1266,7 +1265,7 @@ static void launch_dots1(const DotsShape& d, int P, cudaStream_t st, const void*
                          long long n, double2* part, const DotsFinish& fin, long long p_ps = 0,
                          const long long* poff = nullptr, const long long* plen = nullptr, const int* act = nullptr) {
   const dim3 grid(d.groups, (unsigned)d.chunks, P);
-#define DOTS1(IGc) launch_kernel(d.threads < 256, dots1_kernel<T, C, IGc>, grid, dim3(d.threads), 0, st, A, lda, na, d.per, B, n, (int)d.rows, part, fin, 0, 0, p_ps, poff, plen, act)
+#define DOTS1(IGc) launch_kernel(d.threads < 256, dots1_kernel<T, C, IGc>, grid, dim3(d.threads), 0, st, A, lda, na, d.per, B, n, (int)d.rows, part, fin, p_ps, poff, plen, act)
   switch (d.ig) {
     case 1: DOTS1(1); break;
     case 2: DOTS1(2); break;

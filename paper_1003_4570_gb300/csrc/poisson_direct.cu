@@ -735,8 +735,7 @@ omen_status poisson_direct(omen_ctx* ctx, const PGrid& g, const double* rho, dou
   cudaFreeAsync(buf, st);
   if (e != cudaSuccess) return set_err(ctx, OMEN_ECUDA, "Poisson solve: %s", cudaGetErrorString(e));
   res->iterations = h.iterations;
-  res->zero = h.bb == 0.0;
-  res->converged = res->zero || h.rr <= h.stop;
+  res->converged = h.bb == 0.0 || h.rr <= h.stop;
   res->rel = h.bb > 0.0 ? std::sqrt(h.rr / h.bb) : 0.0;
   return OMEN_OK;
 }

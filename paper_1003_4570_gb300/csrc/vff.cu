@@ -130,7 +130,6 @@ __device__ __forceinline__ void stage_table(const VffTable& t, VffTable& sm, dou
 // Relaxation state on the device (one small record).
 struct VffState {
   double t;          // last step length
-  double c1;         // last directional derivative g.p
   double gg;         // g.g of the current gradient
   double beta;       // of the next direction
   double gmax;       // max |g_c| of the current gradient
@@ -375,7 +374,6 @@ __global__ void __launch_bounds__(kThreads) vff_line_kernel(const __grid_constan
     const double c1 = 2.0 * c[0];
     const double step = quartic_step(c1, c[1], 2.0 * c[2], c[3]);
     st->t = step;
-    st->c1 = c1;
     st->restart = step > 0.0 ? 0 : 1;
   }
 }
