@@ -10,6 +10,7 @@
 #include "sk_device.cuh"
 #include "vec.cuh"
 #include "cic.cuh"
+#include "param_copy.cuh"
 #include "df.cuh"
 
 // n_atom[i] += w * sum_n occ[n] * sum_o |psi_n[o*N + i]|^2
@@ -214,7 +215,11 @@ extern "C" omen_status omen_density_accum(omen_ctx* ctx, const omen_ham* h, cons
       cudaGetLastError();
       return set_err(ctx, OMEN_ENOMEM, "occupations");
     }
-    OMEN_CUDA(ctx, cudaMemcpyAsync(d_occ, occ_host, sizeof(double) * nstates, cudaMemcpyHostToDevice, ctx->stream));
+    const cudaError_t e = copy_as_params(ctx->stream, d_occ, occ_host, sizeof(double) * nstates);
+    if (e != cudaSuccess) {
+      cudaFreeAsync(d_occ, ctx->stream);
+      return set_err(ctx, OMEN_ECUDA, "occupations: %s", cudaGetErrorString(e));
+    }
   }
   const int N = (int)(h->nrows / h->nb);   // atoms, or grid points of an effective-mass Hamiltonian
   // one atom a thread: a grid cut to whole waves left its last round a fifth full at 1M atoms

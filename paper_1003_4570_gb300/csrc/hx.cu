@@ -36,6 +36,7 @@
 #include "sk_device.cuh"
 #include "df.cuh"
 #include "neighbours.cuh"
+#include "param_copy.cuh"
 #include "pdl.cuh"
 
 template <typename T> struct Cx;
@@ -1204,28 +1205,13 @@ std::vector<double2> phase_table(const omen_ham* h, int nk, const double* k_host
   return ph;
 }
 
-// A table goes to the device as parameters of launches that write it: these are read when the launch is
-// made, where a copy from the host array might still be pending when the array is gone.
-struct PhaseChunk {
-  double2 v[3 * kInlinePhases];
-};
-__global__ void __launch_bounds__(128) phases_kernel(const __grid_constant__ PhaseChunk c, int n, double2* __restrict__ out) {
-  for (int i = threadIdx.x; i < n; i += 128) out[i] = c.v[i];
-}
-
 omen_status make_phases(omen_ctx* ctx, const omen_ham* h, int nk, const double* k_host, double2** out) {
   const std::vector<double2> ph = phase_table(h, nk, k_host);
   if (ctx_alloc(ctx, out, sizeof(double2) * ph.size()) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "phase table");
   }
-  for (size_t at = 0; at < ph.size(); at += 3 * kInlinePhases) {
-    PhaseChunk c;
-    const int n = (int)std::min<size_t>(3 * kInlinePhases, ph.size() - at);
-    std::copy(ph.begin() + at, ph.begin() + at + n, c.v);
-    phases_kernel<<<1, 128, 0, ctx->stream>>>(c, n, *out + at);
-  }
-  OMEN_CHECK_LAUNCH(ctx);
+  OMEN_CUDA(ctx, copy_as_params(ctx->stream, *out, ph.data(), sizeof(double2) * ph.size()));   // ph goes on return
   return OMEN_OK;
 }
 

@@ -28,6 +28,7 @@
 #include "cic.cuh"
 #include "fd.cuh"
 #include "omen_internal.h"
+#include "param_copy.cuh"
 
 namespace cgr = cooperative_groups;
 
@@ -265,7 +266,7 @@ extern "C" omen_status omen_state_weights(omen_ctx* ctx, const omen_ham* h, cons
     cudaGetLastError();
     return set_err(ctx, OMEN_ENOMEM, "state weights");
   }
-  cudaError_t e = cudaMemcpyAsync(dw, weight_host, sizeof(double) * nstates, cudaMemcpyHostToDevice, ctx->stream);
+  cudaError_t e = copy_as_params(ctx->stream, dw, weight_host, sizeof(double) * nstates);
   const int N = h->lat->natoms;
   const long long total = (long long)nstates * N;
   const unsigned grid = (unsigned)std::min<long long>(4096, (total + 255) / 256);

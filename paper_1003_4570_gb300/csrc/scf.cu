@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "omen_internal.h"
+#include "param_copy.cuh"
 
 static constexpr double kQe = 1.602176634e-19;  // C
 
@@ -334,7 +335,7 @@ extern "C" omen_status omen_scf(omen_ctx* ctx, const omen_scf_desc* d, double* p
     }
     // ring slots hold the differences in order slot = (iteration - 1) % H; gamma is in Gram order
     // (slot order), which the update uses directly
-    OMEN_CUDA(ctx, cudaMemcpyAsync(gam.p, gamma.data(), sizeof(double) * 8, cudaMemcpyHostToDevice, ctx->stream));
+    OMEN_CUDA(ctx, copy_as_params(ctx->stream, gam.p, gamma.data(), sizeof(double) * 8));
     anderson_kernel<<<gg, 256, 0, ctx->stream>>>(phi, Fcur.d(), dXh.d(), dFh.d(), ng, h, gam.d(), d->mix, ng);
   }
   cudaError_t e = cudaStreamSynchronize(ctx->stream);

@@ -140,3 +140,20 @@ def test_tuner_keeps_the_built_in_shape_of_small_products(watch, ctx, cells, tun
     else:
         assert (r["threads"], r["rows_per_batch"]) == (128, 0) and r["ms_best"] == r["ms_default"]
         assert watch.launches("hx_kernel") == 0
+
+
+def test_host_tables_of_asynchronous_calls_may_go(watch, ctx):
+    """What a call that does not wait was given by host pointer is read when it returns."""
+    ham = hamiltonian(ctx, (2, 2, 3))
+    psi, n = np.zeros((70, ham.nrows)), np.zeros(96)
+    occ, weight = np.ones(70), np.ones(70)
+    omen.omen_density_accum(ctx, ham, psi, 70, occ, 1.0, n)
+    omen.omen_state_weights(ctx, ham, psi, 70, weight, np.zeros((70, 96)))
+    occ[:], weight[:] = 2.0, 3.0
+    assert watch.changed() == 0
+    spec = synth.lattice_spec(1, 1, 4, (2, 2, 0), seed=1)
+    g = poisson.Grid(3, 3, 12, 0.5431, 0.5431, 4 * 0.5431)
+    f = np.zeros(g.shape)
+    omen.omen_scf(ctx, omen.omen_build_lattice(ctx, spec), synth.draw_tb_params(1, 10, 1), g, f, f.copy(), 2.0, 0.01, [[0, 0, 0]],
+                  [1.0], 4, 0.0, -1.0, max_iter=4, mix_history=3, raise_on_noconv=False)
+    assert watch.changed() == 0
