@@ -1067,6 +1067,8 @@ extern "C" omen_status omen_hx_host(omen_ctx* ctx, const omen_ham* h, const void
     if (ctx_alloc(ctx, &dx, bytes) != cudaSuccess || ctx_alloc(ctx, &dy, bytes) != cudaSuccess ||
         ctx_alloc(ctx, &fx, 8 * (size_t)n) != cudaSuccess) {
       cudaGetLastError();
+      if (dx) cudaFreeAsync(dx, ctx->stream);
+      if (dy) cudaFreeAsync(dy, ctx->stream);
       return set_err(ctx, OMEN_ENOMEM, "device allocation of %zu bytes failed", bytes);
     }
     omen_status st = OMEN_OK;

@@ -61,15 +61,17 @@ def test_wave_vectors_outlive_their_copy(watch, ctx):
     assert watch.changed() == 0
 
 
-@pytest.mark.parametrize("call", ["eigs", "refined", "kbatch"])
+@pytest.mark.parametrize("call", ["eigs", "refined", "kbatch", "host"])
 def test_a_failed_allocation_leaves_nothing_behind(watch, ctx, call):
-    prec = omen.OMEN_F32_REFINE64 if call == "refined" else omen.OMEN_F64
+    prec = {"refined": omen.OMEN_F32_REFINE64, "host": omen.OMEN_F64_DF}.get(call, omen.OMEN_F64)
     ham = hamiltonian(ctx, (2, 2, 3), bloch=call == "kbatch", precision=prec)
     before, failed = watch.live(), 0
     for n in range(60):
         watch.fail(n)
         try:
-            if call == "kbatch":
+            if call == "host":
+                omen.omen_hx_host(ctx, ham, np.zeros(ham.nrows))
+            elif call == "kbatch":
                 omen.omen_eigs_kbatch(ctx, ham, np.zeros((3, 3)), 4, raise_on_noconv=False)
             else:
                 omen.omen_eigs(ctx, ham, 4, block=1, basis=32, raise_on_noconv=False)
@@ -77,7 +79,7 @@ def test_a_failed_allocation_leaves_nothing_behind(watch, ctx, call):
             failed += e.status == omen.OMEN_ENOMEM
         assert watch.live() == before, n
     watch.fail(-1)
-    assert failed >= 15
+    assert failed >= (3 if call == "host" else 15)
 
 
 ITERATED = [((2039, 2039, 2), 1e-13), ((1021, 1021, 5), 1e-13), ((2039, 16, 3), 1e-6), ((1, 2039, 3), 1e-10), ((2053, 1, 3), 1e-9),
