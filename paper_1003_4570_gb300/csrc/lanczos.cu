@@ -2403,8 +2403,10 @@ struct SegmentGraphs {
   }
 };
 
-// Vectors up to this size queue a segment ahead of a host check (see there for both sides).
+// Vectors up to kAheadBytes queue a segment ahead of every host check, larger ones while the bounds are
+// kAheadFar times the tolerance (see there for the times).
 static constexpr size_t kAheadBytes = 3 << 19;
+static constexpr double kAheadFar = 1e4;
 
 static omen_status lanczos_solve_single(KrylovOps& op, const omen_eig_opts* o, void* X, int k_out,
                                         omen_eig_info* info, bool& converged) {
@@ -2564,6 +2566,7 @@ static omen_status lanczos_solve_single(KrylovOps& op, const omen_eig_opts* o, v
   // the steps up to and including the next host check run as one segment; `ahead` holds the length of
   // one that was issued before the host looked at the check before it
   int ahead = 0;
+  double last_bound = 0.0;   // of the wanted pairs at the check before (lowest levels)
   auto issue_segment = [&](int& nseg) -> omen_status {
     nseg = 0;
     for (int nb = nbas, it = iter, sc = since_check;; ++nb) {
@@ -2607,11 +2610,13 @@ static omen_status lanczos_solve_single(KrylovOps& op, const omen_eig_opts* o, v
       // projected problem.  It writes only basis vectors and columns of T past those of this check, so
       // a check that ends the solve leaves it unused (at most one segment, which no count includes).
       // What that hides is the host's share, 0.1 to 1 ms a check whatever the rows; what it may waste
-      // grows with them.  Whole solves without and with it: 1,280 complex rows 59.0 -> 53.7 ms, 41k rows
-      // 30.6 -> 28.2 ms, 138k rows 53.1 -> 49.5 ms, 216k rows 103.3 -> 97.5 and 43.8 -> 45.7 ms, 640k
-      // rows 178.0 -> 180.9 and, to a loose tolerance, 50.0 -> 55.8 ms, 2.7M rows 462 -> 483 ms: so
-      // vectors of up to 1.5 MB.
-      if (!full && iter < max_iter_of(o) && vbytes <= kAheadBytes) {
+      // grows with them.  So larger problems do it only while the wanted pairs' bounds at the check before
+      // were far from the tolerance (lowest levels; a locking check ends otherwise).  Whole solves
+      // without, with it at every check, and so: 1,280 complex rows 59.0, 53.7 ms; 138k rows 53.1, 49.5;
+      // 216k rows 43.4, 44.2, 41.3; 640k rows 177.9, 180.7, 173.5 and, to a loose tolerance, 50.2, 55.0,
+      // 49.4; 2.7M rows 463, 484, 459; 10M rows 2867, 2871, 2862.
+      const bool far = !folded && !op.has_line && last_bound > kAheadFar * o->tol;
+      if (!full && iter < max_iter_of(o) && (vbytes <= kAheadBytes || far)) {
         const int js0 = jstart, nb0 = nbas;
         jstart = nbas;
         nbas += 1;
@@ -2669,7 +2674,8 @@ static omen_status lanczos_solve_single(KrylovOps& op, const omen_eig_opts* o, v
       if (!folded) {
         std::vector<double> lam(theta.begin(), theta.begin() + nev), res(resA.begin(), resA.begin() + nev), bd;
         error_bounds(theta, lam, res, bd);
-        done = *std::max_element(bd.begin(), bd.end()) <= o->tol;
+        last_bound = *std::max_element(bd.begin(), bd.end());
+        done = last_bound <= o->tol;
         // under partial reorthogonalisation the projected matrix is only as good as the basis's
         // orthogonality, which restarts erode: confirm on H before stopping
         if (done && pro) {

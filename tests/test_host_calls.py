@@ -120,8 +120,8 @@ def test_passes_of_a_restart(watch, ctx, cols, passes):
 @pytest.mark.parametrize("precision", [omen.OMEN_F64, omen.OMEN_F32])
 @pytest.mark.parametrize("cells, ahead", [((2, 2, 3), True), ((16, 16, 16), True), ((24, 24, 24), False)])
 def test_steps_ahead_of_a_check(watch, ctx, cells, ahead, precision):
-    """Small problems queue the next segment while the host looks at the check before it; where a step
-    costs more than the host's part, a solve runs the steps that it reports and no more."""
+    """Small problems queue the next segment while the host looks at the check before it; larger ones do
+    not where that check may end the solve: here its first one does, and only the steps reported run."""
     ham = hamiltonian(ctx, cells, basis=5, precision=precision)
     omen.omen_set_locking_check(ctx, False)
     info = omen.omen_eigs(ctx, ham, 4, block=1, basis=48, raise_on_noconv=False)[1]
