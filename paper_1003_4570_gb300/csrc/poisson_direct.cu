@@ -601,8 +601,16 @@ static bool direct_pays(const PGrid& g, double rtol, int max_iter, bool mixed, i
   return !(cg < 0.85 * direct && 2.0 * its < max_iter);
 }
 
+// Whether n has no prime factor above 31: such lines always pay.
+static bool smooth(int n) {
+  for (int p : {2, 3, 5, 7, 11, 13, 17, 19, 23, 29, 31})
+    while (n % p == 0) n /= p;
+  return n == 1;
+}
+
 bool poisson_direct_fits(const omen_ctx* ctx, const PGrid& g, double rtol, int max_iter, bool mixed) {
   if (g.nx > kMaxLine || g.ny > kMaxLine || g.nzi > kMaxZ) return false;
+  if (smooth(g.nx) && smooth(g.ny)) return true;
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) return true;
   return direct_pays(g, rtol, max_iter, mixed, sms);

@@ -29,7 +29,7 @@ omen_status poisson_direct(omen_ctx* ctx, const PGrid& g, const double* rho, dou
 // times the lateral one).
 __host__ __device__ inline double pivot_at(double s, int j) {
   if (s == 0.0) return (double)j / (j + 1);
-  const double a = sqrt(s), u = 1.0 / (a + sqrt(1.0 + s)), q = u * u;
-  const double ej = expm1(-4.0 * j * asinh(a));
+  const double a = sqrt(s), b = sqrt(1.0 + s), u = 1.0 / (a + b), q = u * u;
+  const double ej = expm1(-4.0 * j * log1p(a + s / (1.0 + b)));    // asinh(a) from the root at hand
   return q * (ej / fma(ej, q * q, -2.0 * a * u * (q + 1.0)));
 }
