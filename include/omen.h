@@ -76,7 +76,9 @@ typedef struct omen_ham omen_ham;
 /* ---- context --------------------------------------------------------------------------- */
 
 /* Create a context on CUDA device `device`, issuing work on `cuda_stream` (a cudaStream_t;
- * NULL = the legacy default stream).  Allocates small device work buffers. */
+ * NULL = the legacy default stream).  Allocates small device work buffers.  The context keeps up to
+ * 512 MB of device memory that calls have used for their work areas, mapped for the next ones, and 512
+ * KB of pinned host memory once a solve has run; omen_destroy gives everything back. */
 omen_status omen_create(omen_ctx** out, int device, void* cuda_stream);
 void omen_destroy(omen_ctx* ctx);
 const char* omen_last_error(const omen_ctx* ctx);
@@ -270,7 +272,9 @@ omen_status omen_assemble_effmass(omen_ctx* ctx, const omen_effmass_desc* desc, 
                                   omen_ham** out);
 
 /* y = (H - sigma) x for nvec vectors in the Hamiltonian's vector type (device).
- * x and y must not overlap.  This is the operation the Lanczos recurrence repeats. */
+ * x and y must not overlap.  This is the operation the Lanczos recurrence repeats.  Vectors of a small
+ * structure may be rounded differently in calls of different nvec (another kernel sums the same terms
+ * in another order). */
 omen_status omen_hx(omen_ctx* ctx, const omen_ham* ham, const void* x_dev, void* y_dev,
                     int nvec, double sigma);
 /* Convert n vector elements between OMEN_F64 (double) and OMEN_F64_DF (float2 hi, lo) on the
@@ -312,9 +316,9 @@ omen_status omen_tune_hx(omen_ctx* ctx, omen_ham* ham, int vec_precision, int nv
 omen_status omen_tune_hx_kbatch(omen_ctx* ctx, omen_ham* ham, int nk, int reps, omen_tune_result* out);
 
 /* Set a launch shape directly: threads a multiple of 32 in 32..128 (0 = default 128) and
- * rows_per_batch from the compiled set (FP32 stored blocks 1, 2, 5, and 10 without spin-orbit
- * for sp3d5s*; FP64 stored 1, 2; matrix-free 1, 2; 0 = the built-in rule; rows_per_batch must
- * divide the orbital count).  k batch: wave vectors per thread 1, 2 (FP64 and FP32) or 4 (FP32), 0 =
+ * rows_per_batch from the accepted set (FP32 Hamiltonians 1, 2, 5, and 10 without spin-orbit for
+ * sp3d5s*; FP64 1, 2; matrix-free 1, 2; 0 = the built-in rule; rows_per_batch must divide the orbital
+ * count: names from before the present kernels, which take them as bonds loaded together).  k batch: wave vectors per thread 1, 2 (FP64 and FP32) or 4 (FP32), 0 =
  * default 1.  Products too small to fill the device take one shape whatever is set here.
  * EINVAL for a shape that is not compiled. */
 omen_status omen_hx_set_tile(omen_ctx* ctx, omen_ham* ham, int vec_precision, int threads, int rows_per_batch);
@@ -344,8 +348,9 @@ typedef struct {
 typedef struct {
   int iterations;            /* block steps taken */
   long long hx_count;        /* single-vector H·X products (as iterations: of the steps used; a
-                                solve on vectors of up to 1.5 MB may run up to a check's interval
-                                of steps past its last check) */
+                                solve may run up to a check's interval of steps past its last
+                                check, on vectors above 1.5 MB only where that check converged
+                                from far off) */
   int restarts;
   int converged;             /* 1 if every returned pair met tol */
   double max_residual;       /* max FP64 ||H x - lambda x|| over returned pairs (eV) */
@@ -419,7 +424,7 @@ typedef struct {
  * phi = 0 V on the planes z = 0 and z = Lz. */
 
 typedef struct {
-  double rtol;               /* stop when ||r|| <= rtol ||b|| (b - A x in FP64 in both forms) */
+  double rtol;               /* stop when ||r|| <= rtol ||b||, r in FP64 (which r: see precision) */
   int max_iter;
   int precision;             /* OMEN_F64: the residual tested last is carried from step to step (r - A d
                                 of the second direct correction d, the recurrence of CG iterations).
@@ -433,16 +438,19 @@ typedef struct {
 typedef struct {
   int iterations;            /* direct corrections and CG iterations */
   int converged;
-  double rel_residual;       /* ||r|| / ||b|| at exit */
+  double rel_residual;       /* ||r|| / ||b|| at exit of the residual that was tested: with OMEN_F64 a
+                                carried one, which can lie far below ||b - A x|| / ||b|| once that has
+                                reached its rounding (about 1e-16 ||A|| ||x|| / ||b||) */
   double seconds;
 } omen_solve_info;
 
 /* Solve -div(eps0 eps_r grad phi) = rho (7-point finite differences, periodic x and y,
  * phi = 0 at both z ends; paper: finite-difference Poisson solver, Section III-A item 3) by direct
  * corrections: Hartley transforms along x and y, tridiagonal solves along z, in FP64.  At most two
- * are applied; what they leave above the tolerance, and grids with lines of more than 2,048 points
- * or more than 1,024 planes, go to conjugate gradients in one cooperative launch, in FP64 or with
- * FP32 iterations and FP64 residual replacement (opts->precision).
+ * are applied.  What they leave above the tolerance, grids with lines of more than 2,048 points or more
+ * than 1,024 planes, and grids of few planes whose lines have a large prime factor (where iterating is
+ * faster) go to conjugate gradients in one cooperative launch, in FP64 or with FP32 iterations and FP64
+ * residual replacement (opts->precision).  Work vectors: two or three FP64 fields and a fourth of one.
  * rho_dev: C/m^3; phi_dev: V, initial guess in, solution out (rho = 0 gives phi = 0).
  * ENOCONV at max_iter; EINVAL for a grid of 2^31 or more unknowns or another precision. */
 omen_status omen_poisson(omen_ctx* ctx, const omen_grid* grid, const double* rho_dev, double* phi_dev,
@@ -534,7 +542,8 @@ omen_status omen_density_accum(omen_ctx* ctx, const omen_ham* ham, const void* p
 
 /* Cloud-in-cell (trilinear) deposit of per-atom charge q_atom_dev (C) onto the grid nodes,
  * divided by the cell volume: rho_dev (C/m^3) is overwritten.  Charge landing on the z = 0 or
- * z = Lz planes is dropped (grounded).  Atom positions come from the structure. */
+ * z = Lz planes is dropped (grounded).  Atom positions come from the structure.  This call and the
+ * next allocate tables of 48 bytes a cell along each axis on ctx's stream. */
 omen_status omen_deposit(omen_ctx* ctx, const omen_lattice* lat, const omen_grid* grid,
                          const double* q_atom_dev, double* rho_dev);
 /* Trilinear interpolation of phi (boundary planes at 0 V) to every atom: phi_atom_dev [natoms]. */

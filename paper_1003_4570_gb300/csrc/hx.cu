@@ -14,9 +14,9 @@
 // sit in shared memory.
 //
 // Measured on the sp3d5s* alloy of 1M atoms, full blocks before and this form after: FP64 0.706 ->
-// 0.451 ms (92% of the FP64 rate; bound by it), FP32 stored 0.169 -> 0.040 ms, FP32 matrix-free
-// 0.061 -> 0.040 ms (bound by the shared-memory reads of the reduced blocks, 27 words a bond end
-// and lane, and the latency of the neighbours' amplitudes: 54% of the LSU data rate, 65% of the
+// 0.451 ms (88% of the FP64 rate in the operations needed, FP64 pipe 93% busy; bound by it), FP32
+// stored 0.169 -> 0.040 ms, FP32 matrix-free 0.061 -> 0.040 ms (bound by the shared-memory reads of the reduced blocks, 27 words a bond end
+// and lane, and the latency of the neighbours' amplitudes: 54% of the LSU data rate, 57% of the
 // issue slots).  The rounding error against 64 bits falls with the number of terms: FP32 1.3e-7
 // -> 0.7e-7 of the result's norm.
 //
@@ -854,8 +854,9 @@ static cudaError_t launch_t(const HxInst<T>& I, int nvec, int threads, double si
 }
 
 // Whether `rb` is one of the load batches accepted for this kind of product (0 = the built-in
-// rule): FP32 stored 1, 2, 5, or the orbital count without spin-orbit; FP64 and matrix-free 1, 2;
-// each must divide the orbital count.
+// rule): FP32 1, 2, 5, or the orbital count without spin-orbit; FP64 and matrix-free 1, 2; each must
+// divide the orbital count.  (The values of an earlier kernel's register batches, accepted as before;
+// loads_of says what they select.)
 static bool rb_valid(int norb, bool f64, bool so, bool mf, int rb) {
   if (rb == 0) return true;
   if (rb < 0 || norb % rb != 0) return false;

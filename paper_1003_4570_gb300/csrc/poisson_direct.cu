@@ -16,10 +16,10 @@
 // plane, with the residual formed as they are read: three launches a correction.
 //
 // Measured against the conjugate gradients this takes the place of (poisson.cu, one cooperative
-// launch, three grid barriers an iteration): 11x11x217 grid to 1e-13 4.95 -> 0.111 ms (two
-// corrections, eight launches of 6 to 14 us), 256x256x257 to 1e-10 in the mixed form 251 -> 2.59 ms (one
-// correction and its check); the error against 64-bit transforms 1.5e-15 -> 1.1e-15 and 2.3e-11 ->
-// 8e-14 of the norm.
+// launch, three grid barriers an iteration): 11x11x217 grid to 1e-13 5.07 -> 0.112 ms (two corrections,
+// seven launches of 6 to 14 us), 256x256x257 to 1e-10 in the mixed form 251 -> 2.53 ms (one correction
+// and its check); the error against 64-bit transforms 1.2e-15 -> 1.1e-15 and 4.6e-12 -> 6.2e-14 of the
+// norm.
 #include <algorithm>
 #include <cmath>
 

@@ -508,8 +508,9 @@ def grid_struct(g) -> Grid:
 
 
 def omen_poisson(ctx: Context, grid, rho_dev, phi_dev, rtol=1e-12, max_iter=100000, precision=OMEN_F64):
-    """CG solve in place on phi_dev (initial guess in).  precision OMEN_F64, or OMEN_F32_REFINE64
-    for FP32 iterations with FP64 residual replacement.  Returns the solve info dict."""
+    """Poisson solve in place on phi_dev (initial guess in): direct corrections, conjugate gradients
+    where these do not apply.  precision OMEN_F64, or OMEN_F32_REFINE64 to test b - A x itself, with
+    FP32 iterations and FP64 residual replacement.  Returns the solve info dict."""
     g = grid_struct(grid)
     o = CGOpts(float(rtol), int(max_iter), int(precision))
     info = SolveInfo()
