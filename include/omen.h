@@ -189,8 +189,8 @@ typedef struct {
 
 /* Energy (E_host, may be NULL) and forces -dE/du (force_dev [3][natoms], may be NULL) at
  * displacements u_dev; F_host [9] row-major, NULL = identity.  Forces allocate 12 doubles per atom
- * on ctx's stream.  Synchronous.  EINVAL for bad
- * parameters (nspecies, a_nm <= 0, negative constants). */
+ * on ctx's stream.  Synchronous.  EINVAL for bad parameters (nspecies, a_nm <= 0, negative constants)
+ * and for structures with a species index above 3. */
 omen_status omen_vff_energy_forces(omen_ctx* ctx, const omen_lattice* lat, const omen_vff_params* p,
                                    const double* F_host, const double* u_dev, double* E_host, double* force_dev);
 

@@ -4,6 +4,7 @@
 // global position lists.  On one GPU the whole block is resident and the neighbour of an
 // atom is computed from its cell index and site number (neighbours.cuh), so no
 // neighbour list is stored or read.
+#include <algorithm>
 #include <cstdarg>
 #include <cstring>
 #include <mutex>
@@ -49,6 +50,7 @@ extern "C" omen_status omen_build_lattice(omen_ctx* ctx, const omen_lattice_desc
   L->natoms = 8 * L->ncells;
   for (int i = 0; i < 3; ++i) L->periodic[i] = d->periodic[i];
   L->a_nm = d->a_nm;
+  L->max_species = *std::max_element(d->species_host, d->species_host + L->natoms);
   cudaError_t e1 = cudaMalloc(&L->d_species, (size_t)L->natoms);
   cudaError_t e2 = cudaMalloc(&L->d_strain, sizeof(double) * 16 * (size_t)L->ncells);
   if (e1 != cudaSuccess || e2 != cudaSuccess) {

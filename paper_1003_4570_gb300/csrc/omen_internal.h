@@ -57,6 +57,7 @@ struct omen_lattice {
   int periodic[3];
   double a_nm;
   uint8_t* d_species = nullptr;  // [natoms]
+  int max_species = 0;           // the largest of them
   double* d_strain = nullptr;    // [16*ncells]
   long long nbonds = 0;
 };

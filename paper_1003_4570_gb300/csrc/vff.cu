@@ -427,6 +427,8 @@ omen_status make_args(omen_ctx* ctx, const omen_lattice* L, const omen_vff_param
   for (int s = 0; s < vp->nspecies; ++s)
     if (!(vp->a_nm[s] > 0) || !(vp->alpha[s] >= 0) || !(vp->beta[s] >= 0))
       return set_err(ctx, OMEN_EINVAL, "species %d: a_nm must be > 0 and alpha, beta >= 0", s);
+  // the kernels look the constants up in a table of four species
+  if (L->max_species > 3) return set_err(ctx, OMEN_EINVAL, "species index %d: at most 4 species", L->max_species);
   a.g.nx = L->nx; a.g.ny = L->ny; a.g.nz = L->nz;
   a.g.ncells = L->ncells; a.g.natoms = L->natoms;
   for (int d = 0; d < 3; ++d) a.g.periodic[d] = L->periodic[d];

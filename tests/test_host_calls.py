@@ -159,3 +159,20 @@ def test_host_tables_of_asynchronous_calls_may_go(watch, ctx):
     omen.omen_scf(ctx, omen.omen_build_lattice(ctx, spec), synth.draw_tb_params(1, 10, 1), g, f, f.copy(), 2.0, 0.01, [[0, 0, 0]],
                   [1.0], 4, 0.0, -1.0, max_iter=4, mix_history=3, raise_on_noconv=False)
     assert watch.changed() == 0
+
+
+def test_relaxation_refuses_species_outside_its_table(watch, ctx):
+    """The kernels look constants up by the species of an atom: an index above 3 would leave the table."""
+    class Keating:
+        a_nm, alpha, beta = np.full(4, 0.5431), np.full(4, 300.0), np.full(4, 90.0)
+    for bad in (3, 4, 255):
+        spec = synth.lattice_spec(1, 2, 2, (0, 0, 0), seed=1)
+        spec.species[5] = bad
+        lat, u = omen.omen_build_lattice(ctx, spec), np.zeros((3, spec.natoms))
+        calls = [lambda: omen.omen_vff_energy_forces(ctx, lat, Keating, u), lambda: omen.omen_relax_vff(ctx, lat, Keating, u, max_iter=0)]
+        for call in calls:
+            if bad <= 3:
+                call()
+            else:
+                with pytest.raises(omen.OmenError, match="EINVAL"):
+                    call()
